@@ -4,13 +4,13 @@
 //
 // For every train the host selected (Train::hx_sel):
 //  1. k_hx_remove marks every particle of the train removed (the next sort drops it);
-//  2. k_hx_integrate, one warp per train, takes the train's species counts n0 as
+//  2. k_hx_integrate, one CTA per train, takes the train's species counts n0 as
 //     molecule numbers in the box volume V and integrates the reaction extents e_r
 //     (events): n(e) = n0 + nu e, de_r/dt = kappa_r n_a n_b, kappa_r = k_r / (N_A V), and
 //     (k_tab / 2) / (N_A V) for a self reaction whose tabulated value is 2k. This is Eq. 3
 //     multiplied through by N_A V. The integrator is the extrapolated linearly implicit
 //     Euler method (Deuflhard 1985; Hairer and Wanner, Solving ODEs II, Sec. IV.9) with
-//     the harmonic substep sequence 1..6 (one lane per column) and an analytic
+//     the harmonic substep sequence 1..6 (a half warp per column) and an analytic
 //     Jacobian: stiff rate equations
 //     (R9 at 1.1e11 L/mol/s) over 10 s take a few hundred steps;
 //  3. the extents are rounded to whole events without bias, E_r = floor(e_r) +
@@ -37,174 +37,166 @@ __device__ __forceinline__ int status_of_hx(const Dev& d) {
   return *reinterpret_cast<volatile int*>(&d.g->status);
 }
 
-// Kinetics of one train in molecule numbers.
-struct Kin {
-  int nt, nr;
-  int a[MAXR], b[MAXR];
-  double kappa[MAXR];
-  double nu[MAXT][MAXR];
+// One train is integrated by one CTA of three warps: each of the six extrapolation columns
+// belongs to a half warp, lane r of it to reaction r. What bounds the stage is the length
+// of its dependent chain (a few hundred steps, each a factorisation and up to six
+// substeps) and the FP64 pipe, which a warp's instruction occupies for 16 cycles however
+// many lanes are active. Rows of the matrices therefore live in the lanes' registers and
+// travel by shuffles, and the columns run side by side (two per warp, of similar length).
+// Measured, 64 trains of 500 to 20,000 species over 10 s (a whole pass with its host calls):
+// 64.1 -> 16.2 ms against one lane per column with its matrices in local memory, an FP64
+// power for the step size and the table's divisions in one lane.
+constexpr int HX_THREADS = 16 * HX_K;  // one half warp per column
+static_assert(MAXR <= 16, "a half warp holds the rows of the matrix");
+
+// Kinetics of one train in molecule numbers, and the columns' end values.
+struct HxSmem {
   double n0[MAXT];
-};
-
-__device__ void hx_numbers(const Kin& k, const double* e, double* n) {
-  for (int x = 0; x < k.nt; ++x) {
-    double v = k.n0[x];
-    for (int r = 0; r < k.nr; ++r) v += k.nu[x][r] * e[r];
-    n[x] = v;
-  }
-}
-
-__device__ void hx_rates(const Kin& k, const double* e, double* out) {
-  double n[MAXT];
-  hx_numbers(k, e, n);
-  for (int r = 0; r < k.nr; ++r) out[r] = k.kappa[r] * n[k.a[r]] * n[k.b[r]];
-}
-
-// d rate_r / d e_s = kappa_r (n_b nu[a][s] + n_a nu[b][s]) (both terms for a self reaction)
-__device__ void hx_jacobian(const Kin& k, const double* e, double (*J)[MAXR]) {
-  double n[MAXT];
-  hx_numbers(k, e, n);
-  for (int r = 0; r < k.nr; ++r) {
-    const int a = k.a[r], b = k.b[r];
-    for (int s = 0; s < k.nr; ++s) J[r][s] = k.kappa[r] * (n[b] * k.nu[a][s] + n[a] * k.nu[b][s]);
-  }
-}
-
-// In-place LU with partial pivoting of the nr x nr matrix M. False when singular.
-__device__ bool hx_lu(double (*M)[MAXR], int* piv, int nr) {
-  for (int c = 0; c < nr; ++c) {
-    int p = c;
-    double best = fabs(M[c][c]);
-    for (int r = c + 1; r < nr; ++r) {
-      if (fabs(M[r][c]) > best) { best = fabs(M[r][c]); p = r; }
-    }
-    if (!(best > 0.0)) return false;
-    piv[c] = p;
-    if (p != c) {
-      for (int q = 0; q < nr; ++q) { const double t = M[c][q]; M[c][q] = M[p][q]; M[p][q] = t; }
-    }
-    const double inv = 1.0 / M[c][c];
-    for (int r = c + 1; r < nr; ++r) {
-      const double f = M[r][c] * inv;
-      M[r][c] = f;
-      for (int q = c + 1; q < nr; ++q) M[r][q] -= f * M[c][q];
-    }
-  }
-  return true;
-}
-
-__device__ void hx_solve(const double (*M)[MAXR], const int* piv, int nr, double* x) {
-  for (int c = 0; c < nr; ++c) {
-    const int p = piv[c];
-    if (p != c) { const double t = x[c]; x[c] = x[p]; x[p] = t; }
-  }
-  for (int r = 1; r < nr; ++r) {
-    double v = x[r];
-    for (int q = 0; q < r; ++q) v -= M[r][q] * x[q];
-    x[r] = v;
-  }
-  for (int r = nr - 1; r >= 0; --r) {
-    double v = x[r];
-    for (int q = r + 1; q < nr; ++q) v -= M[r][q] * x[q];
-    x[r] = v / M[r][r];
-  }
-}
-
-// Per-warp shared memory of the integrator: the columns' end values and the step's result.
-struct HxWarpSmem {
+  double nu[MAXR][MAXT];      // change of species x per event of reaction r
+  double nu_ab[MAXR][MAXR][2];  // [s][r]: change of r's two reactants per event of s
   double col[HX_K][MAXR];
-  double y1[MAXR];
+  double e[MAXR];             // extents at the end of the integration
 };
 
-// One extrapolated step of length H from y0, taken by one warp (every lane calls it with
-// the same y0 and H): lane j - 1 integrates H with j linearly implicit Euler substeps,
-// (I - hJ) d = h f(y), y += d, with the Jacobian J of y0 (columns are independent, so the
-// six run side by side); lane 0 then applies the Aitken-Neville table, which removes the
-// error terms in h, h^2, ... (the method's expansion is in powers of h). Returns false
-// (on every lane) when a column is singular or the result is not finite; else y1 and
-// the scaled error estimate on every lane.
-__device__ bool hx_step(const Kin& k, const double* y0, double H, double* y1, double* err, HxWarpSmem& sm,
-                        int lane) {
-  const int nr = k.nr;
-  bool ok = true;
-  if (lane < HX_K) {
-    const int j = lane + 1;
-    double J[MAXR][MAXR], M[MAXR][MAXR];
-    double y[MAXR], f[MAXR];
-    int piv[MAXR];
-    hx_jacobian(k, y0, J);
-    const double h = H / j;
-    for (int r = 0; r < nr; ++r)
-      for (int s = 0; s < nr; ++s) M[r][s] = (r == s ? 1.0 : 0.0) - h * J[r][s];
-    ok = hx_lu(M, piv, nr);
-    if (ok) {
-      for (int r = 0; r < nr; ++r) y[r] = y0[r];
-      for (int i = 0; i < j; ++i) {
-        hx_rates(k, y, f);
-        for (int r = 0; r < nr; ++r) f[r] *= h;
-        hx_solve(M, piv, nr, f);
-        for (int r = 0; r < nr; ++r) y[r] += f[r];
-      }
-      for (int r = 0; r < nr; ++r) sm.col[lane][r] = y[r];
-    }
-  }
-  ok = __all_sync(0xffffffffu, ok);
-  __syncwarp();
-  if (!ok) return false;
-  double e = 0.0;
-  bool fin = true;
-  if (lane == 0) {
-    double prev[HX_K][MAXR], cur[HX_K][MAXR];
-    for (int jj = 1; jj <= HX_K; ++jj) {
-      for (int r = 0; r < nr; ++r) cur[0][r] = sm.col[jj - 1][r];
-      for (int l = 0; l + 1 < jj; ++l) {
-        const double den = static_cast<double>(jj) / static_cast<double>(jj - l - 1) - 1.0;
-        for (int r = 0; r < nr; ++r) cur[l + 1][r] = cur[l][r] + (cur[l][r] - prev[l][r]) / den;
-      }
-      for (int l = 0; l < jj; ++l)
-        for (int r = 0; r < nr; ++r) prev[l][r] = cur[l][r];
-    }
-    for (int r = 0; r < nr; ++r) {
-      const double v = cur[HX_K - 1][r];
-      fin = fin && isfinite(v);
-      sm.y1[r] = v;
-      const double sc = HX_ATOL + HX_RTOL * fmax(fabs(y0[r]), fabs(v));
-      e = fmax(e, fabs(v - cur[HX_K - 2][r]) / sc);
-    }
-  }
-  fin = __shfl_sync(0xffffffffu, fin, 0);
-  e = __shfl_sync(0xffffffffu, e, 0);
-  __syncwarp();
-  if (!fin) return false;
-  for (int r = 0; r < nr; ++r) y1[r] = sm.y1[r];
-  __syncwarp();
-  *err = e;
-  return true;
+// What a lane keeps of its reaction (lanes past the reactions: kappa 0, reactants 0).
+struct HxLane {
+  int nr, nt, r, col;
+  int a, b;
+  double kappa;
+};
+
+__device__ __forceinline__ double hx_shfl(double v, int src) {
+  return __shfl_sync(0xffffffffu, v, src, 16);
 }
 
-// Extents after T seconds from e = 0, by one warp (identical control flow on every lane).
-// Returns the accepted steps, or -1 on failure.
-__device__ long long hx_integrate(const Kin& k, double T, double* e, HxWarpSmem& sm, int lane) {
-  for (int r = 0; r < k.nr; ++r) e[r] = 0.0;
+// kappa n_a and kappa n_b of this lane's reaction and its rate, at extents y (one per lane).
+__device__ __forceinline__ double hx_rate(const HxLane& k, const HxSmem& sm, double y, double& na, double& nb) {
+  const int x = k.r & (MAXT - 1);  // lane x also carries species x (and lane x + 8 a copy)
+  double n = sm.n0[x], n2 = 0.0;
+#pragma unroll
+  for (int s = 0; s < MAXR; s += 2) {
+    if (s < k.nr) n += sm.nu[s][x] * hx_shfl(y, s);
+    if (s + 1 < k.nr) n2 += sm.nu[s + 1][x] * hx_shfl(y, s + 1);
+  }
+  n += n2;
+  na = hx_shfl(n, k.a);
+  nb = hx_shfl(n, k.b);
+  return k.kappa * na * nb;
+}
+
+// One extrapolated step of length H from y0 (one extent per lane, the same in every half
+// warp): column j takes j linearly implicit Euler substeps (I - hJ) d = h f(y), y += d,
+// h = H / j, with the Jacobian J of y0; then lane r forms the Aitken-Neville table of
+// component r, which removes the error terms in h, h^2, ... (the method's expansion is in
+// powers of h). The matrix is factored once by elimination with a pivot row per column
+// (largest element to 1 part in 2^16, rows stay where they are); a substep is one forward
+// and one backward sweep. Returns false (for the whole CTA) when a matrix is singular or
+// the result is not finite; else y1 and the scaled error estimate.
+__device__ bool hx_step(const HxLane& k, HxSmem& sm, double y0, double H, double& y1, double& err) {
+  const int nr = k.nr;
+  const double h = H / static_cast<double>(k.col + 1);
+  double na, nb;
+  double f = hx_rate(k, sm, y0, na, nb);
+  const double ka = k.kappa * nb, kb = k.kappa * na;
+  // row r of I - hJ: d rate_r / d e_s = kappa_r (n_b nu[a][s] + n_a nu[b][s])
+  double M[MAXR];
+#pragma unroll
+  for (int s = 0; s < MAXR; ++s) {
+    M[s] = 0.0;
+    if (s < nr) M[s] = (s == k.r ? 1.0 : 0.0) - h * (ka * sm.nu_ab[s][k.r][0] + kb * sm.nu_ab[s][k.r][1]);
+  }
+  int pos = MAXR;                // elimination order of this lane's row (MAXR: not yet)
+  double inv_own = 0.0;          // 1 / pivot of this lane's row
+  unsigned long long perm = 0;   // pivot lane of column c in bits 4c
+  bool ok = true;
+#pragma unroll
+  for (int c = 0; c < MAXR; ++c) {
+    if (c >= nr) break;
+    const unsigned hi = static_cast<unsigned>(__double2hiint(M[c])) & 0x7FFFFFF0u;
+    const bool free_row = pos == MAXR && k.r < nr;
+    const unsigned key = free_row ? (hi | static_cast<unsigned>(15 - k.r)) : 0u;
+    const unsigned best0 = __reduce_max_sync(0xffffffffu, (k.col & 1) ? 0u : key);
+    const unsigned best1 = __reduce_max_sync(0xffffffffu, (k.col & 1) ? key : 0u);
+    const unsigned best = (k.col & 1) ? best1 : best0;
+    const int p = 15 - static_cast<int>(best & 15u);
+    ok = ok && best >= 16u && best < 0x7FF00000u;
+    perm |= static_cast<unsigned long long>(p) << (4 * c);
+    const double inv = 1.0 / hx_shfl(M[c], p);
+    const bool mine = k.r == p;
+    if (mine) { pos = c; inv_own = inv; }
+    const double l = (free_row && !mine) ? M[c] * inv : 0.0;
+    if (free_row && !mine) M[c] = l;
+#pragma unroll
+    for (int q = c + 1; q < MAXR; ++q)
+      if (q < nr) M[q] -= l * hx_shfl(M[q], p);
+  }
+  double y = y0;
+  for (int i = 0; i <= (k.col | 1); ++i) {  // warp-uniform: as many as its longer column takes
+    if (i > 0) f = hx_rate(k, sm, y, na, nb);
+    double v = h * f, x = 0.0;
+#pragma unroll
+    for (int c = 0; c < MAXR; ++c) {
+      if (c >= nr) break;
+      const double xc = hx_shfl(v, static_cast<int>(perm >> (4 * c)) & 15);
+      if (pos > c) v -= M[c] * xc;
+    }
+#pragma unroll
+    for (int c = MAXR - 1; c >= 0; --c) {
+      if (c >= nr) continue;
+      const double xc = hx_shfl(v * inv_own, static_cast<int>(perm >> (4 * c)) & 15);
+      if (pos < c) v -= M[c] * xc;
+      if (k.r == c) x = xc;
+    }
+    if (i <= k.col) y += x;
+  }
+  sm.col[k.col][k.r] = y;
+  ok = __syncthreads_and(ok ? 1 : 0) != 0;
+  // every half warp forms the same table, so that all go on with the same values
+  double prev[HX_K], cur[HX_K];
+#pragma unroll
+  for (int j = 1; j <= HX_K; ++j) {
+    cur[0] = sm.col[j - 1][k.r];
+#pragma unroll
+    for (int l = 0; l + 1 < j; ++l)  // the weight is 1 / (j / (j - l - 1) - 1)
+      cur[l + 1] = cur[l] + (cur[l] - prev[l]) * (static_cast<double>(j - l - 1) / static_cast<double>(l + 1));
+#pragma unroll
+    for (int l = 0; l < j; ++l) prev[l] = cur[l];
+  }
+  y1 = cur[HX_K - 1];
+  const double sc = HX_ATOL + HX_RTOL * fmax(fabs(y0), fabs(y1));
+  double e = k.r < nr ? fabs(y1 - cur[HX_K - 2]) / sc : 0.0;
+  bool fin = k.r >= nr || isfinite(y1);
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) e = fmax(e, __shfl_xor_sync(0xffffffffu, e, o, 16));
+  fin = __all_sync(0xffffffffu, fin);  // (both halves hold the same components)
+  err = e;
+  if (k.r >= nr) y1 = 0.0;
+  __syncthreads();  // the columns are rewritten by the next step
+  return ok && fin;
+}
+
+// Extents after T seconds from e = 0, one per lane (identical control flow on every
+// thread). Returns the accepted steps, or -1 on failure.
+__device__ long long hx_integrate(const HxLane& k, HxSmem& sm, double T, double& e) {
+  e = 0.0;
   if (k.nr == 0 || !(T > 0.0)) return 0;
   double t = 0.0, H = fmin(T, 1e-9);
   long long accepted = 0;
-  double y1[MAXR];
   for (int it = 0; it < HX_MAX_STEPS; ++it) {
     if (t >= T) return accepted;
     const bool last = H >= T - t;
     const double Hs = last ? T - t : H;
-    double err = 0.0;
-    const bool ok = hx_step(k, e, Hs, y1, &err, sm, lane);
+    double err = 0.0, y1;
+    const bool ok = hx_step(k, sm, e, Hs, y1, err);
+    // the step-size factor needs a few digits only: FP32 power
+    const float root = (ok && err > 0.0) ? 0.9f * powf(fminf(static_cast<float>(err), 1e30f), -1.0f / HX_K) : 4.f;
     if (ok && err <= 1.0) {
-      for (int r = 0; r < k.nr; ++r) e[r] = y1[r];
+      e = y1;
       t = last ? T : t + Hs;
       ++accepted;
-      const double fac = err > 0.0 ? 0.9 * pow(err, -1.0 / HX_K) : 4.0;
-      H = Hs * fmin(4.0, fmax(0.2, fac));
+      H = Hs * static_cast<double>(fminf(4.f, fmaxf(0.2f, root)));
     } else {
-      const double fac = ok ? 0.9 * pow(err, -1.0 / HX_K) : 0.2;
-      H = Hs * fmin(0.5, fmax(0.2, fac));
+      H = Hs * static_cast<double>(ok ? fminf(0.5f, fmaxf(0.2f, root)) : 0.2f);
     }
   }
   return -1;
@@ -220,36 +212,47 @@ __global__ void k_hx_remove(Dev d) {
   }
 }
 
-constexpr int HX_WARPS = 2;  // trains per CTA, one warp each
-
-__global__ void __launch_bounds__(32 * HX_WARPS) k_hx_integrate(Dev d) {
-  __shared__ HxWarpSmem smem[HX_WARPS];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const uint32_t b = blockIdx.x * HX_WARPS + static_cast<uint32_t>(w);
-  if (b >= d.n_trains || status_of_hx(d)) return;  // warp-uniform
+__global__ void __launch_bounds__(HX_THREADS) k_hx_integrate(Dev d) {
+  __shared__ HxSmem sm;
+  const int tid = threadIdx.x;
+  const uint32_t b = blockIdx.x;
+  // one answer for the CTA (another train's CTA may raise the status meanwhile)
+  if (__syncthreads_or(status_of_hx(d))) return;
   Train& tr = d.trains[b];
   if (!tr.hx_sel) return;
   const Tables& tb = *d.tables;
-  Kin k;
+  HxLane k;
   k.nt = tb.n_types;
   k.nr = tb.n_rxn;
+  k.r = tid & 15;
+  k.col = tid >> 4;
   const double NV = HX_N_AVOGADRO * (tr.L * tr.L * tr.L * 1e-24);
-  for (int x = 0; x < MAXT; ++x) {
-    k.n0[x] = x < k.nt ? static_cast<double>(tr.counts[x]) : 0.0;
-    for (int r = 0; r < MAXR; ++r) k.nu[x][r] = 0.0;
+  for (int q = tid; q < MAXT * MAXR; q += HX_THREADS) {
+    const int x = q % MAXT, r = q / MAXT;
+    double v = 0.0;
+    if (r < k.nr && x < k.nt) {
+      if (tb.rxn_a[r] == x) v -= 1.0;
+      if (tb.rxn_b[r] == x) v -= 1.0;
+      for (int p = 0; p < tb.n_prod[r]; ++p) v += tb.prod[r][p] == x ? 1.0 : 0.0;
+    }
+    sm.nu[r][x] = v;
   }
-  for (int r = 0; r < k.nr; ++r) {
-    const int a = tb.rxn_a[r], c = tb.rxn_b[r];
-    k.a[r] = a;
-    k.b[r] = c;
-    k.kappa[r] = (a == c ? 0.5 * tb.k_tab[r] : tb.k_tab[r]) / NV;
-    k.nu[a][r] -= 1.0;
-    k.nu[c][r] -= 1.0;
-    for (int q = 0; q < tb.n_prod[r]; ++q) k.nu[tb.prod[r][q]][r] += 1.0;
+  if (tid < MAXT) sm.n0[tid] = tid < k.nt ? static_cast<double>(tr.counts[tid]) : 0.0;
+  __syncthreads();
+  k.a = k.r < k.nr ? tb.rxn_a[k.r] : 0;
+  k.b = k.r < k.nr ? tb.rxn_b[k.r] : 0;
+  k.kappa = k.r < k.nr ? (k.a == k.b ? 0.5 * tb.k_tab[k.r] : tb.k_tab[k.r]) / NV : 0.0;
+  for (int s = k.col; s < MAXR; s += HX_K) {
+    sm.nu_ab[s][k.r][0] = sm.nu[s][k.a];
+    sm.nu_ab[s][k.r][1] = sm.nu[s][k.b];
   }
-  double e[MAXR];
-  const long long steps = hx_integrate(k, tr.hx_t_end - tr.t, e, smem[w], lane);
-  if (lane != 0) return;  // the rounding and the train's record: one lane
+  __syncthreads();
+  double own;
+  const long long steps = hx_integrate(k, sm, tr.hx_t_end - tr.t, own);
+  if (tid < MAXR) sm.e[tid] = own;
+  __syncthreads();
+  if (tid != 0) return;  // the rounding and the train's record: one thread
+  const double* e = sm.e;
   if (steps < 0) {
     raise_status(d.g, CHEM_ECAPACITY);
     d.g->err_where = 0x4858u;  // integrator step limit of the homogeneous stage
@@ -267,7 +270,7 @@ __global__ void __launch_bounds__(32 * HX_WARPS) k_hx_integrate(Dev d) {
   }
   for (int x = 0; x < k.nt; ++x) {
     long long v = tr.counts[x];
-    for (int r = 0; r < k.nr; ++r) v += static_cast<long long>(k.nu[x][r]) * E[r];
+    for (int r = 0; r < k.nr; ++r) v += static_cast<long long>(sm.nu[r][x]) * E[r];
     n[x] = v;
   }
   for (;;) {
@@ -277,14 +280,14 @@ __global__ void __launch_bounds__(32 * HX_WARPS) k_hx_integrate(Dev d) {
     if (neg < 0) break;
     int rr = -1;
     for (int r = 0; r < k.nr && rr < 0; ++r)
-      if (k.nu[neg][r] < 0.0 && E[r] > 0) rr = r;
+      if (sm.nu[r][neg] < 0.0 && E[r] > 0) rr = r;
     if (rr < 0) {  // cannot happen: a negative count always has a consuming event
       raise_status(d.g, CHEM_ECAPACITY);
       tr.hx_sel = 0;
       return;
     }
     E[rr] -= 1;
-    for (int x = 0; x < k.nt; ++x) n[x] -= static_cast<long long>(k.nu[x][rr]);
+    for (int x = 0; x < k.nt; ++x) n[x] -= static_cast<long long>(sm.nu[rr][x]);
   }
   long long water = 0;
   uint32_t cum = 0;
@@ -316,7 +319,7 @@ cudaError_t enqueue_homogeneous(const Dev& d, int blocks, cudaStream_t s) {
   k_hx_remove<<<blocks, 256, 0, s>>>(d);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k_hx_integrate<<<(static_cast<int>(d.n_trains) + HX_WARPS - 1) / HX_WARPS, 32 * HX_WARPS, 0, s>>>(d);
+  k_hx_integrate<<<static_cast<int>(d.n_trains), HX_THREADS, 0, s>>>(d);
   return cudaGetLastError();
 }
 
