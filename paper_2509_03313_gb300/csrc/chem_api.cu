@@ -952,10 +952,10 @@ chem_status chem_batch_init(const chem_config* cfgs, int32_t n_trains, chem_ctx*
     d.tdx = static_cast<double*>(A(cap * 8)); d.tdy = static_cast<double*>(A(cap * 8));
     d.tdz = static_cast<double*>(A(cap * 8));
     // FP32 cell offsets of the same species for the pair search's prefilter
-    d.s4 = static_cast<float4*>(A(cap * 16));
+    d.s4 = static_cast<float4*>(A((cap + S4_SPARE) * 16));
     d.t4 = static_cast<float4*>(A(cap * 16));
   } else {
-    d.s4 = static_cast<float4*>(A(cap * 16));
+    d.s4 = static_cast<float4*>(A((cap + S4_SPARE) * 16));
     d.t4 = static_cast<float4*>(A(cap * 16));
     d.td4 = static_cast<float4*>(A(cap * 16));
     d.sd4 = static_cast<float4*>(A(cap * 16));

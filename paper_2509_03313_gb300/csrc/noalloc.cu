@@ -44,7 +44,7 @@ constexpr Layout make_layout() {
   L.sx = take(M * 8); L.sy = take(M * 8); L.sz = take(M * 8); L.stid = take(M * 4);
   L.tx = take(M * 8); L.ty = take(M * 8); L.tz = take(M * 8); L.ttid = take(M * 4);
   L.tdx = take(M * 8); L.tdy = take(M * 8); L.tdz = take(M * 8);
-  L.s4 = take(M * 16); L.t4 = take(M * 16);  // FP32 cell offsets (the search's prefilter)
+  L.s4 = take((M + S4_SPARE) * 16); L.t4 = take(M * 16);  // FP32 cell offsets (the search's prefilter)
   L.items = take((M + M / ITEM_HOME + 64) * 8);
   L.touch = take(M * 4);
   L.cell_sorted = take(M * 4);

@@ -12,12 +12,12 @@
 #include <type_traits>
 #include <math_constants.h>
 
+#include "fixed_normals.cuh"
 #include "onesweep.cuh"
 #include "sbs_device.cuh"
 
 namespace chem {
 
-constexpr double TWO_PI = 6.283185307179586;  // 2 * pi rounded to double
 constexpr double TWO_POW_M53 = 1.1102230246251565e-16;
 constexpr float TWO_POW_M24F = 5.9604644775390625e-08f;
 
@@ -63,24 +63,50 @@ __device__ __forceinline__ double sq3(double x, double y, double z) {
   return __dadd_rn(__dadd_rn(__dmul_rn(x, x), __dmul_rn(y, y)), __dmul_rn(z, z));
 }
 
+// The same for the diffused position of an FP64 species, and y = x + L/2 of the result. A
+// position still inside the box (0 <= y < L, compared on the bits: positive doubles order as
+// integers) is its own wrap, so the division is left to the few that leave it.
+__device__ __forceinline__ double wrap_box_diffused(double x, double L, double halfL, double& y) {
+  y = __dadd_rn(x, halfL);
+  const long long b = __double_as_longlong(y);
+  if (b < 0 || b >= __double_as_longlong(L)) {
+    x = wrap_box(x, L, halfL);
+    y = __dadd_rn(x, halfL);
+  }
+  return x;
+}
+
+// y >= 0 as an exact sum of two floats, hi truncated to 24 bits (0 below 2^-60).
+__device__ __forceinline__ void split_double(double y, float& hi, float& lo) {
+  const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(y));
+  const int e = static_cast<int>(b >> 52);  // y >= 0
+  const bool tiny = e < 1023 - 60;
+  hi = tiny ? 0.f : __uint_as_float((static_cast<uint32_t>(e - 896) << 23) | (static_cast<uint32_t>(b >> 29) & 0x7FFFFFu));
+  lo = tiny ? 0.f : static_cast<float>(static_cast<uint32_t>(b) & 0x1FFFFFFFu) *
+                        __uint_as_float(static_cast<uint32_t>(e - 896 - 52) << 23);
+}
+
+// v truncated to a float without the FP64 pipe (0 below 2^-126).
+__device__ __forceinline__ float truncate_double(double v) {
+  const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(v));
+  const int e = static_cast<int>((b >> 52) & 0x7FFu) - 896;
+  const uint32_t sign = static_cast<uint32_t>(b >> 32) & 0x80000000u;
+  return e <= 0 ? 0.f : __uint_as_float(sign | (static_cast<uint32_t>(e) << 23) | (static_cast<uint32_t>(b >> 29) & 0x7FFFFFu));
+}
+
 // Three standard normals for species `id` at step `step` (FP64 mode): two Philox blocks,
-// 53-bit uniforms u1 in (0,1], u2 in [0,1), Box-Muller.
+// 53-bit uniforms u1 in (0,1], u2 in [0,1), Box-Muller, its functions in fixed point
+// (fixed_normals.cuh).
 __device__ __forceinline__ void gauss3_f64(uint32_t id, uint32_t step, uint32_t k0, uint32_t k1,
                                            double& g0, double& g1, double& g2) {
   const uint4 a = philox4x32_10(make_uint4(id, step, 0u, 0u), k0, k1);
   const uint4 b = philox4x32_10(make_uint4(id, step, 0u, 1u), k0, k1);
-  const double u1 = __dmul_rn(__dadd_rn(static_cast<double>(u53(a.x, a.y)), 1.0), TWO_POW_M53);
-  const double u2 = __dmul_rn(static_cast<double>(u53(a.z, a.w)), TWO_POW_M53);
-  const double u3 = __dmul_rn(__dadd_rn(static_cast<double>(u53(b.x, b.y)), 1.0), TWO_POW_M53);
-  const double u4 = __dmul_rn(static_cast<double>(u53(b.z, b.w)), TWO_POW_M53);
-  const double r = sqrt(__dmul_rn(-2.0, log(u1)));
-  const double th = __dmul_rn(TWO_PI, u2);
+  const double r = fixedn::radius(u53(a.x, a.y));
   double s, c;
-  sincos(th, &s, &c);
+  fixedn::sincos_2pi(u53(a.z, a.w), s, c);
   g0 = __dmul_rn(r, c);
   g1 = __dmul_rn(r, s);
-  const double r2 = sqrt(__dmul_rn(-2.0, log(u3)));
-  g2 = __dmul_rn(r2, cos(__dmul_rn(TWO_PI, u4)));
+  g2 = __dmul_rn(fixedn::radius(u53(b.x, b.y)), fixedn::cos_2pi(u53(b.z, b.w)));
 }
 
 // Three standard normals (FP32-local mode): one Philox block, 24-bit uniforms.
@@ -126,6 +152,24 @@ __device__ __forceinline__ double bridge_p(double d0, double d1, double R, doubl
 __device__ __forceinline__ int cell_index(double x, double halfL, double inv_h, int n) {
   int i = static_cast<int>(floor(__dmul_rn(__dadd_rn(x, halfL), inv_h)));
   return min(max(i, 0), n - 1);
+}
+
+// Cell index of an in-box coordinate y = x + L/2 (the value of cell_index) and the offset from
+// the cell's corner as a float, on the FP32 pipe: FP32 places y within 2.5e-4 of a cell for
+// grids up to 1024, so only coordinates closer than 1e-3 to a face repeat the FP64 test. The
+// offset is within 1.5e-7 of a cell (two fused steps from the exact halves of y and h).
+__device__ __forceinline__ int cell_index_split(double y, double inv_h, int n, float hf, float hlo, float inv_hf,
+                                                float& off) {
+  float yh, yl;
+  split_double(y, yh, yl);
+  const float q = yh * inv_hf;
+  int i = static_cast<int>(q);
+  const float fr = q - static_cast<float>(i);
+  if (fr < 1e-3f || fr > 0.999f) i = static_cast<int>(floor(__dmul_rn(y, inv_h)));
+  i = min(max(i, 0), n - 1);
+  const float fi = static_cast<float>(-i);
+  off = __fmaf_rn(fi, hf, yh) + __fmaf_rn(fi, hlo, yl);
+  return i;
 }
 
 // Bits per axis of the cell index of a grid of n cells per axis: enough for the values
@@ -330,6 +374,7 @@ static __device__ void phase_begin(const Dev& d, BeginSmem& sb) {
     tr.h = h;
     tr.inv_h = inv_h;
     tr.hf = static_cast<float>(h);
+    tr.hlo = static_cast<float>(h - static_cast<double>(tr.hf));
     tr.inv_hf = static_cast<float>(inv_h);
     sb.hf[b] = static_cast<float>(h);
     if (b == 0) sb.cb0 = axis_bits(n);
@@ -608,23 +653,19 @@ __device__ void phase_diffuse(const Dev& d, uint32_t (*hist)[RADIX]) {
           gauss3_f64(tid_id(tid), tr.step, tr.key0, tr.key1, g0, g1, g2);
           const double sig = tr.sig[ty];
           const double ex = __dmul_rn(sig, g0), ey = __dmul_rn(sig, g1), ez = __dmul_rn(sig, g2);
-          const double x = wrap_box(__dadd_rn(px, ex), tr.L, tr.halfL);
-          const double y = wrap_box(__dadd_rn(py, ey), tr.L, tr.halfL);
-          const double z = wrap_box(__dadd_rn(pz, ez), tr.L, tr.halfL);
+          double yx, yy, yz;  // from the box corner
+          const double x = wrap_box_diffused(__dadd_rn(px, ex), tr.L, tr.halfL, yx);
+          const double y = wrap_box_diffused(__dadd_rn(py, ey), tr.L, tr.halfL, yy);
+          const double z = wrap_box_diffused(__dadd_rn(pz, ez), tr.L, tr.halfL, yz);
           d.tx[s] = x; d.ty[s] = y; d.tz[s] = z; d.ttid[s] = tid;
           d.tdx[s] = ex; d.tdy[s] = ey; d.tdz[s] = ez;
           const int n = tr.n;
-          const int ix = cell_index(x, tr.halfL, tr.inv_h, n);
-          const int iy = cell_index(y, tr.halfL, tr.inv_h, n);
-          const int iz = cell_index(z, tr.halfL, tr.inv_h, n);
+          float ox, oy, oz;  // FP32 offsets from the cell's corner for the pair search's prefilter
+          const int ix = cell_index_split(yx, tr.inv_h, n, tr.hf, tr.hlo, tr.inv_hf, ox);
+          const int iy = cell_index_split(yy, tr.inv_h, n, tr.hf, tr.hlo, tr.inv_hf, oy);
+          const int iz = cell_index_split(yz, tr.inv_h, n, tr.hf, tr.hlo, tr.inv_hf, oz);
           key = tr.cell_base + cell_encode(ix, iy, iz, tr.cb);
-          if (d.t4) {  // FP32 offsets from the cell's corner for the pair search's prefilter
-            d.t4[s] = make_float4(
-                static_cast<float>(__dsub_rn(__dadd_rn(x, tr.halfL), __dmul_rn(static_cast<double>(ix), tr.h))),
-                static_cast<float>(__dsub_rn(__dadd_rn(y, tr.halfL), __dmul_rn(static_cast<double>(iy), tr.h))),
-                static_cast<float>(__dsub_rn(__dadd_rn(z, tr.halfL), __dmul_rn(static_cast<double>(iz), tr.h))),
-                __uint_as_float(tid));
-          }
+          d.t4[s] = make_float4(ox, oy, oz, __uint_as_float(tid));
         } else {
           const uint32_t ftid = __float_as_uint(v.w);
           const uint32_t ty = tid_type(ftid);
@@ -785,7 +826,7 @@ __device__ void phase_gather(const Dev& d) {
         if (ok[g]) {
           const uint32_t s = s0 + static_cast<uint32_t>(g) * stride, i = idx[g];
           d.sx[s] = d.tx[i]; d.sy[s] = d.ty[i]; d.sz[s] = d.tz[i]; d.stid[s] = d.ttid[i];
-          if (d.s4) d.s4[s] = d.t4[i];
+          d.s4[s] = d.t4[i];
         }
       }
     }
@@ -977,55 +1018,49 @@ __device__ __forceinline__ bool accept_f64(double d0sq, double d1sq, int r, cons
   return u < bridge_p(sqrt(d0sq), sqrt(d1sq), tb.R[r], tr.ddt[r]);
 }
 
-// Neighbours whose loads one iteration of the per-species walk keeps in flight together.
-constexpr int TPS_UNROLL = 4;
+// FP64 mode: may the pair be rejected on FP32 values alone? f2 is the squared FP32 separation
+// of the species' cell offsets, (dx, dy, dz) the FP32 start separation; both distances are
+// within eps of the exact ones. False: undecided (or to be accepted, which needs the exact
+// separation anyway).
+__device__ __forceinline__ bool surely_rejected(float d0f, float d1f, float eps, int r, const Tables& tb,
+                                                const Train& tr, uint32_t id_lo, uint32_t id_hi) {
+  const float Rf = tb.Rf[r];
+  if (!(d1f > Rf * 1.001f + eps && d0f > Rf * 1.001f + eps)) return false;
+  const uint4 w = philox4x32_10(make_uint4(id_lo, tr.step, id_hi, 2u), tr.key0, tr.key1);
+  const float a = d0f - Rf, b = d1f - Rf, inv = tr.inv_ddt_f[r];
+  const float x = a * b * inv;
+  // accept_f64's error bound with the distances' error eps on top
+  const float err = inv * (b * (eps + 2.4e-7f * (d0f + Rf)) + a * (eps + 2.4e-7f * (d1f + Rf)) + eps * eps) +
+                    1e-6f * (1.f + x) + 4e-6f;
+  if (x > 60.f) return err < 15.f && (w.x | (w.y >> 11)) != 0u;  // p <= exp(-x + err) < 2^-53 <= u
+  if (err > 0.25f) return false;
+  const float ea = __expf(-x);
+  const float ulo = static_cast<float>(w.x >> 8) * 5.9604645e-8f;
+  if (ulo >= ea * (1.f + 2.f * err)) return true;  // p <= exp(-a)
+  const float cb = d0f * d1f * inv, cc = Rf * (d0f + d1f - Rf) * inv;
+  const float p = ea * (expm1f(-cc) / expm1f(-cb));
+  // a relative error of cb or cc is at most passed on: each has at most 2 eps / R
+  return ulo >= p * (1.f + 2.f * (err + 4.f * eps / Rf));
+}
 
-// ---- one thread per home species
-// Each lane takes one home species (warps take 32 consecutive sorted slots by work
-// stealing), keeps the forward cells its largest cutoff can reach (a 13-bit mask from
-// per-axis face gaps), collects their non-empty ranges after its own cell's later slots,
-// and walks them one range at a time, TPS_UNROLL neighbours per iteration. Lanes of one
-// cell walk the same ranges in step, so their neighbour loads are broadcasts; the loops
-// are warp-uniform (trip count = the longest walk among the lanes) and pairs inside the
-// cutoff go to the warp's pair queue.
-
+// Acceptance of one queued pair (home slot si, neighbour slot j in the forward cell k of
+// the home's cell) and, when accepted, its candidate record. kb = k | train << 8. Both
+// search mappings queue pairs that passed the FP32 cutoff test and resolve them here, one
+// pair per lane. In FP64 mode that test is against a widened cutoff, the FP32 distances
+// (error below eps = 2e-6 of a cell, the same margin) reject most pairs, and the rest are
+// formed and tested exactly in FP64: the FP64 pipe (two lanes per clock and SM) then only
+// sees the few percent that are accepted or close to a decision. The FP64 search of 1e6
+// track species (mean over 1 ps to 1 us) went from 469 to 142 us with it.
 template <bool F32L>
-struct TpsQueue;
-
-template <>
-struct TpsQueue<true> {
-  static constexpr int CAP = 64;
-  uint32_t si[CAP], j[CAP], tid_i[CAP], b[CAP];
-  float fx[CAP], fy[CAP], fz[CAP], f2[CAP];
-  uint32_t n;
-};
-
-template <>
-struct TpsQueue<false> {
-  static constexpr int CAP = 64;
-  uint32_t si[CAP], j[CAP], tid_i[CAP], b[CAP];
-  double rx[CAP], ry[CAP], rz[CAP], d2[CAP];
-  uint32_t n;
-};
-
-template <bool F32L, int W>
-struct TpsSmem {
-  using T = float;            // FP32 cutoffs (FP64 mode: widened, for its FP32 prefilter)
-  T ct[W][MAXT * MAXT];       // per warp: squared cutoffs of one train (-1: no reaction) ...
-  int ct_b[W];                // ... that train
-  uint32_t rs[W][N_FWD][32];  // per lane: its non-empty neighbour ranges [rs, re) ...
-  uint32_t re[W][N_FWD][32];
-  uint8_t rk[W][N_FWD][32];   // ... and their half-shell offsets
-  TpsQueue<F32L> q[W];
-  FwdSmem fo;                 // half-shell offsets
-};
-
-// Acceptance of one queued pair (home species given by slot and packed id/type).
-template <bool F32L>
-__device__ __forceinline__ void tps_accept(const Dev& d, const Tables& tb, const Train& tr, int b, uint32_t si,
-                                           uint32_t tid_i, uint32_t j, uint32_t tid_j, float fx, float fy,
-                                           float fz, float f2, double d1sq, double rx1, double ry1, double rz1,
-                                           const uint32_t* vf) {
+__device__ __forceinline__ void resolve_pair(const Dev& d, const Tables& tb, const FwdSmem& fo, uint32_t si,
+                                             uint32_t j, uint32_t kb, const uint32_t* vf, uint32_t& n_in_cut) {
+  const int k = static_cast<int>(kb & 255u), b = static_cast<int>(kb >> 8);
+  const Train& tr = d.trains[b];
+  const float4 hv = d.s4[si], vj = d.s4[j];
+  // the walk's separation, formed the same way
+  float fx, fy, fz;
+  const float f2 = sep_f32(fo.f[0][k], fo.f[1][k], fo.f[2][k], tr.hf, vj, hv, fx, fy, fz);
+  const uint32_t tid_i = __float_as_uint(hv.w), tid_j = __float_as_uint(vj.w);
   const uint32_t ti = tid_type(tid_i), tj = tid_type(tid_j);
   const int r = tb.pair_rxn[ti][tj];
   const uint32_t id_i = tid_id(tid_i), id_j = tid_id(tid_j);
@@ -1033,18 +1068,41 @@ __device__ __forceinline__ void tps_accept(const Dev& d, const Tables& tb, const
   const uint32_t id_lo = i_lo ? id_i : id_j, id_hi = i_lo ? id_j : id_i;
   if constexpr (F32L) {
     if (!i_lo) { fx = -fx; fy = -fy; fz = -fz; }
-    const float4 di = d.td4[vf ? vf[si] : si];
-    const float4 dj = d.td4[vf ? vf[j] : j];
+    // this step's displacements, gathered into sorted order
+    const float4 di = d.sd4[si], dj = d.sd4[j];
     const float4 dlo = i_lo ? di : dj, dhi = i_lo ? dj : di;
     const float r0x = fx - (dhi.x - dlo.x), r0y = fy - (dhi.y - dlo.y), r0z = fz - (dhi.z - dlo.z);
     const float d0sq = r0x * r0x + r0y * r0y + r0z * r0z;
     if (!accept_f32(d0sq, f2, r, tb, tr, id_lo, id_hi)) return;
     emit_candidate(d, i_lo ? si : j, i_lo ? j : si, id_lo, id_hi, r, b, static_cast<double>(f2));
   } else {
-    if (!i_lo) { rx1 = -rx1; ry1 = -ry1; rz1 = -rz1; }
-    const uint32_t tj_idx = vf ? vf[j] : j, ti_idx = vf ? vf[si] : si;
-    const double ejx = d.tdx[tj_idx], ejy = d.tdy[tj_idx], ejz = d.tdz[tj_idx];
+    const uint32_t ti_idx = vf ? vf[si] : si, tj_idx = vf ? vf[j] : j;
     const double eix = d.tdx[ti_idx], eiy = d.tdy[ti_idx], eiz = d.tdz[ti_idx];
+    const double ejx = d.tdx[tj_idx], ejy = d.tdy[tj_idx], ejz = d.tdz[tj_idx];
+    const float eps = 2e-6f * tr.hf;
+    const float d1f = sqrtf(f2);
+    const bool sure_in = d1f < sqrtf(tr.rc2f_tt[ti * MAXT + tj]) * 0.99999f - eps;
+    if (sure_in) {
+      ++n_in_cut;
+      const float r0x = fx - (truncate_double(ejx) - truncate_double(eix));
+      const float r0y = fy - (truncate_double(ejy) - truncate_double(eiy));
+      const float r0z = fz - (truncate_double(ejz) - truncate_double(eiz));
+      const float d0f = sqrtf(r0x * r0x + r0y * r0y + r0z * r0z);
+      // the displacements' truncation is relative to them, which no pair's distance bounds
+      const float big = fmaxf(fmaxf(fabsf(r0x - fx), fabsf(r0y - fy)), fabsf(r0z - fz));
+      if (surely_rejected(d0f, d1f, eps + 1e-6f * (big + d0f), r, tb, tr, id_lo, id_hi)) return;
+    }
+    // minimum image of x_j - x_i (Eq. 2), exactly as the reference forms it up to the
+    // orientation, which is negated below without rounding
+    double rx1 = min_image(__dsub_rn(d.sx[j], d.sx[si]), tr.L, tr.halfL);
+    double ry1 = min_image(__dsub_rn(d.sy[j], d.sy[si]), tr.L, tr.halfL);
+    double rz1 = min_image(__dsub_rn(d.sz[j], d.sz[si]), tr.L, tr.halfL);
+    const double d1sq = sq3(rx1, ry1, rz1);
+    if (!sure_in) {
+      if (!(d1sq < tr.rc2_tt[ti * MAXT + tj])) return;
+      ++n_in_cut;
+    }
+    if (!i_lo) { rx1 = -rx1; ry1 = -ry1; rz1 = -rz1; }
     const double elx = i_lo ? eix : ejx, ely = i_lo ? eiy : ejy, elz = i_lo ? eiz : ejz;
     const double ehx = i_lo ? ejx : eix, ehy = i_lo ? ejy : eiy, ehz = i_lo ? ejz : eiz;
     const double r0x = __dsub_rn(rx1, __dsub_rn(ehx, elx));
@@ -1055,25 +1113,63 @@ __device__ __forceinline__ void tps_accept(const Dev& d, const Tables& tb, const
   }
 }
 
-template <bool F32L>
-__device__ __forceinline__ void tps_flush(const Dev& d, const Tables& tb, TpsQueue<F32L>& q, const uint32_t* vf,
-                                          int lane) {
-  const uint32_t nq = q.n;
-  for (uint32_t e = lane; e < nq; e += 32) {
-    const uint32_t j = q.j[e];
-    const int b = static_cast<int>(q.b[e]);
-    const Train& tr = d.trains[b];
-    if constexpr (F32L)
-      tps_accept<true>(d, tb, tr, b, q.si[e], q.tid_i[e], j, __float_as_uint(d.s4[j].w), q.fx[e], q.fy[e],
-                       q.fz[e], q.f2[e], 0.0, 0.0, 0.0, 0.0, vf);
-    else
-      tps_accept<false>(d, tb, tr, b, q.si[e], q.tid_i[e], j, d.stid[j], 0.f, 0.f, 0.f, 0.f, q.d2[e], q.rx[e],
-                        q.ry[e], q.rz[e], vf);
+// Pairs queued by one warp: home slot, neighbour slot, half-shell index | train << 8.
+template <int CAP>
+struct PairQueue {
+  uint32_t si[CAP], j[CAP], kb[CAP];
+};
+
+// Resolves queued pairs [0, n), 32 at a time; with `all` unset a last part of fewer than 32
+// is kept, moved to the front. Returns the pairs kept. Called by the whole warp.
+template <bool F32L, int CAP>
+__device__ __forceinline__ uint32_t resolve_queue(const Dev& d, const Tables& tb, const FwdSmem& fo,
+                                                  PairQueue<CAP>& q, uint32_t n, bool all, const uint32_t* vf,
+                                                  int lane, uint32_t& n_in_cut) {
+  __syncwarp();
+  const uint32_t full = all ? n : n & ~31u;
+  for (uint32_t e = lane; e < full; e += 32) resolve_pair<F32L>(d, tb, fo, q.si[e], q.j[e], q.kb[e], vf, n_in_cut);
+  __syncwarp();
+  const uint32_t rest = n - full;
+  if (rest != 0u && full != 0u) {
+    uint32_t a = 0, b = 0, c = 0;
+    if (static_cast<uint32_t>(lane) < rest) { a = q.si[full + lane]; b = q.j[full + lane]; c = q.kb[full + lane]; }
+    __syncwarp();
+    if (static_cast<uint32_t>(lane) < rest) { q.si[lane] = a; q.j[lane] = b; q.kb[lane] = c; }
   }
   __syncwarp();
-  if (lane == 0) q.n = 0;
-  __syncwarp();
+  return rest;
 }
+
+// Neighbours whose loads one iteration of the per-species walk keeps in flight together. A
+// finished lane's next batch may start up to TPS_UNROLL - 1 past the last species.
+constexpr int TPS_UNROLL = 4;
+static_assert(2 * TPS_UNROLL <= S4_SPARE, "a batch past the last range stays inside s4");
+constexpr int TPS_QCAP = 32 * (TPS_UNROLL + 1);  // fewer than 32 kept pairs and one batch of a warp
+
+// ---- one thread per home species
+// Each lane takes one home species (warps take 32 consecutive sorted slots by work
+// stealing), keeps the forward cells its largest cutoff can reach (a 13-bit mask from
+// per-axis face gaps), collects their non-empty ranges after its own cell's later slots,
+// and walks them one range at a time, TPS_UNROLL neighbours per iteration. Lanes of one
+// cell walk the same ranges in step, so their neighbour loads are broadcasts; the loops
+// are warp-uniform (trip count = the longest walk among the lanes) and pairs inside the
+// cutoff go to the warp's pair queue, a whole batch with one vote per neighbour. The walk is
+// bound by instruction issue: a batch is one address and four loads at fixed offsets, and the
+// queue holds three words a pair (the separation is formed again when it is resolved). With
+// the push per neighbour, the eight-word queue and an address and zero fill per neighbour the
+// search of the 1e6-species FP32-local run (mean of 102 steps) took 146 us, now 126.
+
+template <bool F32L, int W>
+struct TpsSmem {
+  using T = float;            // FP32 cutoffs (FP64 mode: widened, for its FP32 prefilter)
+  T ct[W][MAXT * MAXT];       // per warp: squared cutoffs of one train (-1: no reaction) ...
+  int ct_b[W];                // ... that train
+  uint32_t rs[W][N_FWD][32];  // per lane: its non-empty neighbour ranges [rs, re) ...
+  uint32_t re[W][N_FWD][32];
+  uint8_t rk[W][N_FWD][32];   // ... and their half-shell offsets
+  PairQueue<TPS_QCAP> q[W];
+  FwdSmem fo;                 // half-shell offsets
+};
 
 template <bool F32L, int W>
 __device__ void phase_search_tps(const Dev& d, TpsSmem<F32L, W>& sm) {
@@ -1084,9 +1180,10 @@ __device__ void phase_search_tps(const Dev& d, TpsSmem<F32L, W>& sm) {
   const uint32_t* vf = d.g->sort_any ? (d.g->sort_parity ? d.vals1 : d.vals0) : nullptr;
   const Tables& tb = *d.tables;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  TpsQueue<F32L>& q = sm.q[wib];
+  PairQueue<TPS_QCAP>& q = sm.q[wib];
+  uint32_t qn = 0;  // queued pairs (warp-uniform)
   fwd_smem_fill(sm.fo);
-  if (lane == 0) { q.n = 0; sm.ct_b[wib] = -1; }
+  if (lane == 0) sm.ct_b[wib] = -1;
   // one status for the whole CTA (a barrier, which also publishes the offsets)
   if (!block_status_ok(d)) return;
   const FwdSmem& fo = sm.fo;
@@ -1103,17 +1200,10 @@ __device__ void phase_search_tps(const Dev& d, TpsSmem<F32L, W>& sm) {
     bool home = s < n_live;
     uint32_t tid_i = 0, cell = 0;
     float4 vi = make_float4(0.f, 0.f, 0.f, 0.f);
-    double xi = 0, yi = 0, zi = 0;
-    // FP64 mode tests pairs first on FP32 cell offsets against widened cutoffs (when the
-    // context keeps them), then exactly in FP64
-    const bool pref = F32L || d.s4 != nullptr;
     if (home) {
       cell = d.cell_sorted[s];
-      if constexpr (F32L) { vi = d.s4[s]; tid_i = __float_as_uint(vi.w); }
-      else {
-        xi = d.sx[s]; yi = d.sy[s]; zi = d.sz[s]; tid_i = d.stid[s];
-        if (pref) vi = d.s4[s];
-      }
+      vi = d.s4[s];  // FP64 mode tests pairs first on these FP32 cell offsets
+      tid_i = __float_as_uint(vi.w);
     }
     const int b = (d.n_trains == 1 || !home) ? 0 : train_of_cell(d.trains, d.n_trains, cell);
     const Train& tr = d.trains[b];
@@ -1157,14 +1247,7 @@ __device__ void phase_search_tps(const Dev& d, TpsSmem<F32L, W>& sm) {
         // cutoff of the home's type holds no partner and is not looked up (the gaps are
         // taken 1e-5 of a cell short, which covers every rounding of the offsets)
         const float hcell = tr.hf, eps = 1e-5f * tr.hf;
-        float ofx, ofy, ofz;
-        if constexpr (F32L) {
-          ofx = vi.x; ofy = vi.y; ofz = vi.z;
-        } else {
-          ofx = static_cast<float>(__dsub_rn(__dadd_rn(xi, tr.halfL), __dmul_rn(static_cast<double>(ix), tr.h)));
-          ofy = static_cast<float>(__dsub_rn(__dadd_rn(yi, tr.halfL), __dmul_rn(static_cast<double>(iy), tr.h)));
-          ofz = static_cast<float>(__dsub_rn(__dadd_rn(zi, tr.halfL), __dmul_rn(static_cast<double>(iz), tr.h)));
-        }
+        const float ofx = vi.x, ofy = vi.y, ofz = vi.z;
         float rcmax2 = -1.f;
 #pragma unroll
         for (int t = 0; t < MAXT; ++t) rcmax2 = fmaxf(rcmax2, static_cast<float>(rc2[t]));
@@ -1189,33 +1272,10 @@ __device__ void phase_search_tps(const Dev& d, TpsSmem<F32L, W>& sm) {
           if ((sx + sy) + sz <= rcmax2) kmask |= 1u << k;
         }
       }
-      // the lane's home for the walk (ranges are not moved between lanes: on clustered
-      // tracks, taking over half of a busy lane's range cost more issue slots than the
-      // idle lanes it saved; dense cells go to the cell-tile mapping instead)
-      const uint32_t hs = s, htid = tid_i;
-      const int hb = b;
-      const float4 hv = vi;
-      const double hx = xi, hy = yi, hz = zi;
-      const T* hrow = rc2;
-      const Train* htr = &tr;
-      // enqueue the pairs inside the cutoff (queue pushes are warp-wide)
-      auto push = [&](bool pass, uint32_t jj, float fx, float fy, float fz, float f2, double rx1, double ry1,
-                      double rz1, double d1sq) {
-        const uint32_t bal = __ballot_sync(0xffffffffu, pass);
-        if (bal) {
-          const uint32_t base = q.n;
-          if (pass) {
-            const uint32_t pos = base + __popc(bal & lanemask_lt);
-            q.si[pos] = hs; q.j[pos] = jj; q.tid_i[pos] = htid; q.b[pos] = static_cast<uint32_t>(hb);
-            if constexpr (F32L) { q.fx[pos] = fx; q.fy[pos] = fy; q.fz[pos] = fz; q.f2[pos] = f2; }
-            else { q.rx[pos] = rx1; q.ry[pos] = ry1; q.rz[pos] = rz1; q.d2[pos] = d1sq; }
-          }
-          __syncwarp();
-          if (lane == 0) q.n = base + __popc(bal);
-          __syncwarp();
-          if (q.n > static_cast<uint32_t>(TpsQueue<F32L>::CAP) - 32u) tps_flush<F32L>(d, tb, q, vf, lane);
-        }
-      };
+      // (ranges are not moved between lanes: on clustered tracks, taking over half of a busy
+      // lane's range cost more issue slots than the idle lanes it saved; dense cells go to the
+      // cell-tile mapping instead)
+      const float hf = tr.hf;
       int nr = 0;
       // look up only the cells within reach (warp-uniform loop over each lane's set bits:
       // at most N_FWD of them, so one pass collects them all)
@@ -1270,105 +1330,60 @@ __device__ void phase_search_tps(const Dev& d, TpsSmem<F32L, W>& sm) {
       // are in flight together; lanes of one cell stay in step (broadcast loads)
       int ri = 0;
       uint32_t j = 0, je = 0;
+      uint32_t kb_cur = 0;
       float cx = 0.f, cy = 0.f, cz = 0.f;
       auto open = [&](int r) {
         j = rs_l[32 * r];
         je = re_l[32 * r];
         const int k = rk_l[32 * r];
         cx = fo.f[0][k]; cy = fo.f[1][k]; cz = fo.f[2][k];  // in cells
+        kb_cur = static_cast<uint32_t>(k) | (static_cast<uint32_t>(b) << 8);
       };
       if (nr > 0) open(0);
       while (__any_sync(0xffffffffu, ri < nr)) {
-        // the next TPS_UNROLL neighbours of the lane's current range (one cell offset for
-        // the batch; a range's last batch may be partly empty)
-        uint32_t ju[TPS_UNROLL];
-        bool vu[TPS_UNROLL];
+        // the next TPS_UNROLL neighbours of the lane's current range (one cell offset for the
+        // batch). The whole batch is loaded, from one address; entries past the range's end
+        // belong to other cells and do not count
         const bool act = ri < nr;
-#pragma unroll
-        for (int u = 0; u < TPS_UNROLL; ++u) {
-          ju[u] = j + static_cast<uint32_t>(u);
-          vu[u] = act && ju[u] < je;
-        }
+        const uint32_t j0 = j, kb = kb_cur, left = act ? je - j : 0u;
         const float bx = cx, by = cy, bz = cz;
+        const float4* src = d.s4 + j;
+        float4 vj[TPS_UNROLL];
+#pragma unroll
+        for (int u = 0; u < TPS_UNROLL; ++u) vj[u] = src[u];
         if (act) {
           j += TPS_UNROLL;
           if (j >= je && ++ri < nr) open(ri);
         }
-        float4 vj[TPS_UNROLL];
-        uint32_t tj[TPS_UNROLL];
+        uint32_t bal[TPS_UNROLL];
 #pragma unroll
         for (int u = 0; u < TPS_UNROLL; ++u) {
-          vj[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-          tj[u] = 0u;
-          if (vu[u]) {
-            if (pref) {
-              vj[u] = d.s4[ju[u]];
-              tj[u] = __float_as_uint(vj[u].w);
-            } else {
-              tj[u] = d.stid[ju[u]];
-            }
-          }
+          float fx, fy, fz;
+          const float rc2u = static_cast<uint32_t>(u) < left ? rc2[__float_as_uint(vj[u].w) & 7u] : -1.f;
+          const bool pass = sep_f32(bx, by, bz, hf, vj[u], vi, fx, fy, fz) < rc2u;  // -1: the types do not react
+          n_tested += rc2u >= 0.f ? 1u : 0u;  // reacting type pairs only
+          if constexpr (F32L) n_in_cut += pass ? 1u : 0u;
+          bal[u] = __ballot_sync(0xffffffffu, pass);
         }
-        if constexpr (F32L) {
-          // the cutoff test for the four neighbours first; the separation is formed again,
-          // identically, for the rare pairs inside the cutoff
-          auto sep = [&](int u, float& fx, float& fy, float& fz) {
-            return sep_f32(bx, by, bz, htr->hf, vj[u], hv, fx, fy, fz);
-          };
-          bool pass[TPS_UNROLL];
-          bool any = false;
+        uint32_t any = 0u;
+#pragma unroll
+        for (int u = 0; u < TPS_UNROLL; ++u) any |= bal[u];
+        if (any != 0u) {  // the same for every lane
 #pragma unroll
           for (int u = 0; u < TPS_UNROLL; ++u) {
-            float fx, fy, fz;
-            const float rc2u = hrow[__float_as_uint(vj[u].w) & 7u];  // -1 when the types do not react
-            pass[u] = vu[u] && sep(u, fx, fy, fz) < rc2u;
-            any = any || pass[u];
-            n_tested += (vu[u] && rc2u >= 0.f) ? 1u : 0u;  // reacting type pairs only
-            n_in_cut += pass[u] ? 1u : 0u;
-          }
-          if (__any_sync(0xffffffffu, any)) {
-#pragma unroll
-            for (int u = 0; u < TPS_UNROLL; ++u) {
-              float fx = 0.f, fy = 0.f, fz = 0.f, f2 = 0.f;
-              if (pass[u]) f2 = sep(u, fx, fy, fz);
-              push(pass[u], ju[u], fx, fy, fz, f2, 0.0, 0.0, 0.0, 0.0);
+            if ((bal[u] >> lane) & 1u) {
+              const uint32_t pos = qn + __popc(bal[u] & lanemask_lt);
+              q.si[pos] = s; q.j[pos] = j0 + static_cast<uint32_t>(u); q.kb[pos] = kb;
             }
+            qn += __popc(bal[u]);
           }
-        } else {
-#pragma unroll
-          for (int u = 0; u < TPS_UNROLL; ++u) {
-            const uint32_t jj = ju[u];
-            bool pass = false;
-            double rx1 = 0, ry1 = 0, rz1 = 0, d1sq = 0;
-            if (vu[u]) {
-              const uint32_t tjj = tj[u] & 7u;
-              const float cw = hrow[tjj];  // widened FP32 bound, -1 when the types do not react
-              bool near = cw >= 0.f;
-              if (near && pref) {
-                float fx, fy, fz;
-                near = sep_f32(bx, by, bz, htr->hf, vj[u], hv, fx, fy, fz) < cw;
-              }
-              if (near) {
-                const double c2 = htr->rc2_tt[tid_type(htid) * MAXT + tjj];
-                // minimum image of x_j - x_i (Eq. 2); negated later into the reference's
-                // x_hi - x_lo orientation, which is exact for pairs inside the cutoff
-                rx1 = min_image(__dsub_rn(d.sx[jj], hx), htr->L, htr->halfL);
-                ry1 = min_image(__dsub_rn(d.sy[jj], hy), htr->L, htr->halfL);
-                rz1 = min_image(__dsub_rn(d.sz[jj], hz), htr->L, htr->halfL);
-                d1sq = sq3(rx1, ry1, rz1);
-                pass = d1sq < c2;
-              }
-            }
-            n_tested += (vu[u] && hrow[tj[u] & 7u] >= 0.f) ? 1u : 0u;  // reacting type pairs only
-            n_in_cut += pass ? 1u : 0u;
-            push(pass, jj, 0.f, 0.f, 0.f, 0.f, rx1, ry1, rz1, d1sq);
-          }
+          if (qn >= 32u) qn = resolve_queue<F32L>(d, tb, fo, q, qn, false, vf, lane, n_in_cut);
         }
       }
     }
     c_next = __shfl_sync(0xffffffffu, c_next, 0);
   }
-  tps_flush<F32L>(d, tb, q, vf, lane);
+  resolve_queue<F32L>(d, tb, fo, q, qn, true, vf, lane, n_in_cut);
   add_pair_counts(d, n_tested, n_in_cut);
 }
 

@@ -33,6 +33,7 @@ constexpr int SORT_THREADS = 512;    // threads of the per-pass sort kernel
 constexpr int PERSIST_THREADS = 256; // threads of the persistent step kernel
 constexpr int SORT_ITEMS = 15;
 constexpr int GATHER_BATCH = 4;   // slots per thread and iteration of the gather
+constexpr int S4_SPARE = 8;       // spare entries of s4 past its end: the search loads whole batches
 // the smallest sort tile (persistent kernel): sizes the look-back buffer
 constexpr int SORT_TILE_MIN = PERSIST_THREADS * SORT_ITEMS;
 constexpr int REACT_THREADS = 1024;
@@ -92,7 +93,8 @@ struct Train {
   double dt, t_next, t_start;
   int n;                   // cells per axis this step
   double h, inv_h;
-  float hf, inv_hf;
+  float hf, inv_hf;        // FP32 cell side (and 1/h); h = hf + hlo
+  float hlo;
   double rc2[MAXR];
   float rc2f[MAXR];
   double rc2_tt[MAXT * MAXT];  // squared cutoff of each type pair (-1: no reaction)

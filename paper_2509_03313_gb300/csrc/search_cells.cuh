@@ -40,10 +40,7 @@ struct ScWarp {
   uint32_t roff[SC_RANGES + 1];    // offset in the flattened list (roff[nr] = total),
   uint8_t rk[SC_RANGES + 1];       // and half-shell index
   float ct[MAXT * MAXT];           // squared cutoffs of the item's train (FP64 mode: widened)
-  uint32_t qi[SC_QCAP];            // queued pairs: home slot,
-  uint32_t qj[SC_QCAP];            // neighbour slot,
-  uint32_t qk[SC_QCAP];            // half-shell index | train << 8
-  uint32_t qn;
+  PairQueue<SC_QCAP> q;
   int ct_b;
 };
 
@@ -52,70 +49,6 @@ struct ScSmem {
   FwdSmem fo;  // half-shell offsets
   ScWarp w[W];
 };
-
-// Acceptance of one queued pair (home slot si, neighbour slot j in the forward cell k of
-// the home's cell) and, when accepted, its candidate record.
-template <bool F32L>
-__device__ __forceinline__ void sc_resolve(const Dev& d, const Tables& tb, const FwdSmem& fo, uint32_t si,
-                                           uint32_t j, uint32_t kb, const uint32_t* vf, uint32_t& n_in_cut) {
-  const int k = static_cast<int>(kb & 255u), b = static_cast<int>(kb >> 8);
-  const Train& tr = d.trains[b];
-  if constexpr (F32L) {
-    const float4 hv = d.s4[si], vj = d.s4[j];
-    // the walk's separation, formed the same way
-    float fx, fy, fz;
-    const float f2 = sep_f32(fo.f[0][k], fo.f[1][k], fo.f[2][k], tr.hf, vj, hv, fx, fy, fz);
-    const uint32_t tid_i = __float_as_uint(hv.w), tid_j = __float_as_uint(vj.w);
-    const int r = tb.pair_rxn[tid_type(tid_i)][tid_type(tid_j)];
-    const uint32_t id_i = tid_id(tid_i), id_j = tid_id(tid_j);
-    const bool i_lo = id_i < id_j;
-    const uint32_t id_lo = i_lo ? id_i : id_j, id_hi = i_lo ? id_j : id_i;
-    if (!i_lo) { fx = -fx; fy = -fy; fz = -fz; }
-    // this step's displacements, gathered into sorted order
-    const float4 di = d.sd4[si], dj = d.sd4[j];
-    const float4 dlo = i_lo ? di : dj, dhi = i_lo ? dj : di;
-    const float r0x = fx - (dhi.x - dlo.x), r0y = fy - (dhi.y - dlo.y), r0z = fz - (dhi.z - dlo.z);
-    const float d0sq = r0x * r0x + r0y * r0y + r0z * r0z;
-    if (!accept_f32(d0sq, f2, r, tb, tr, id_lo, id_hi)) return;
-    emit_candidate(d, i_lo ? si : j, i_lo ? j : si, id_lo, id_hi, r, b, static_cast<double>(f2));
-  } else {
-    const uint32_t tid_i = d.stid[si], tid_j = d.stid[j];
-    const uint32_t ti = tid_type(tid_i), tj = tid_type(tid_j);
-    // minimum image of x_j - x_i (Eq. 2), exactly as the reference forms it up to the
-    // orientation, which is negated below without rounding
-    double rx1 = min_image(__dsub_rn(d.sx[j], d.sx[si]), tr.L, tr.halfL);
-    double ry1 = min_image(__dsub_rn(d.sy[j], d.sy[si]), tr.L, tr.halfL);
-    double rz1 = min_image(__dsub_rn(d.sz[j], d.sz[si]), tr.L, tr.halfL);
-    const double d1sq = sq3(rx1, ry1, rz1);
-    if (!(d1sq < tr.rc2_tt[ti * MAXT + tj])) return;
-    ++n_in_cut;
-    const int r = tb.pair_rxn[ti][tj];
-    const uint32_t id_i = tid_id(tid_i), id_j = tid_id(tid_j);
-    const bool i_lo = id_i < id_j;
-    const uint32_t id_lo = i_lo ? id_i : id_j, id_hi = i_lo ? id_j : id_i;
-    if (!i_lo) { rx1 = -rx1; ry1 = -ry1; rz1 = -rz1; }
-    const uint32_t ti_idx = vf ? vf[si] : si, tj_idx = vf ? vf[j] : j;
-    const double eix = d.tdx[ti_idx], eiy = d.tdy[ti_idx], eiz = d.tdz[ti_idx];
-    const double ejx = d.tdx[tj_idx], ejy = d.tdy[tj_idx], ejz = d.tdz[tj_idx];
-    const double elx = i_lo ? eix : ejx, ely = i_lo ? eiy : ejy, elz = i_lo ? eiz : ejz;
-    const double ehx = i_lo ? ejx : eix, ehy = i_lo ? ejy : eiy, ehz = i_lo ? ejz : eiz;
-    const double r0x = __dsub_rn(rx1, __dsub_rn(ehx, elx));
-    const double r0y = __dsub_rn(ry1, __dsub_rn(ehy, ely));
-    const double r0z = __dsub_rn(rz1, __dsub_rn(ehz, elz));
-    if (!accept_f64(sq3(r0x, r0y, r0z), d1sq, r, tb, tr, id_lo, id_hi)) return;
-    emit_candidate(d, i_lo ? si : j, i_lo ? j : si, id_lo, id_hi, r, b, d1sq);
-  }
-}
-
-template <bool F32L>
-__device__ __forceinline__ void sc_flush(const Dev& d, const Tables& tb, const FwdSmem& fo, ScWarp& w,
-                                         const uint32_t* vf, int lane, uint32_t& n_in_cut) {
-  const uint32_t nq = w.qn;
-  for (uint32_t e = lane; e < nq; e += 32) sc_resolve<F32L>(d, tb, fo, w.qi[e], w.qj[e], w.qk[e], vf, n_in_cut);
-  __syncwarp();
-  if (lane == 0) w.qn = 0;
-  __syncwarp();
-}
 
 template <bool F32L, int W>
 __device__ void phase_search_cells(const Dev& d, ScSmem<W>& sm) {
@@ -131,7 +64,8 @@ __device__ void phase_search_cells(const Dev& d, ScSmem<W>& sm) {
   ScWarp& w = sm.w[wib];
   const FwdSmem& fo = sm.fo;
   fwd_smem_fill(sm.fo);
-  if (lane == 0) { w.qn = 0; w.ct_b = -1; }
+  if (lane == 0) w.ct_b = -1;
+  uint32_t qn = 0;  // queued pairs (warp-uniform)
   // one status for the whole CTA (a barrier, which also publishes the offsets)
   if (!block_status_ok(d)) return;
   uint32_t n_tested = 0, n_in_cut = 0;  // pair-search counters of this lane
@@ -322,28 +256,27 @@ __device__ void phase_search_cells(const Dev& d, ScSmem<W>& sm) {
           const uint32_t y = __shfl_up_sync(FULL, incl, o);
           if (lane >= o) incl += y;
         }
-        const uint32_t base = w.qn;
+        const uint32_t base = qn;
         const uint32_t want = __shfl_sync(FULL, incl, 31);
         uint32_t pos = base + incl - cnt;
         while (pass != 0u && pos < static_cast<uint32_t>(SC_QCAP)) {
           const int h = __ffs(pass) - 1;
           pass &= pass - 1u;
-          w.qi[pos] = s0 + static_cast<uint32_t>(h);
-          w.qj[pos] = j;
-          w.qk[pos] = kb;
+          w.q.si[pos] = s0 + static_cast<uint32_t>(h);
+          w.q.j[pos] = j;
+          w.q.kb[pos] = kb;
           ++pos;
         }
-        __syncwarp();
-        if (lane == 0) w.qn = min(static_cast<uint32_t>(SC_QCAP), base + want);
-        __syncwarp();
-        if (w.qn > static_cast<uint32_t>(SC_QCAP) - 32u) sc_flush<F32L>(d, tb, fo, w, vf, lane, n_in_cut);
+        qn = min(static_cast<uint32_t>(SC_QCAP), base + want);
+        if (qn > static_cast<uint32_t>(SC_QCAP) - 32u)
+          qn = resolve_queue<F32L>(d, tb, fo, w.q, qn, false, vf, lane, n_in_cut);
       }
     }
     it = it_n1;
     rec = make_uint2(__shfl_sync(FULL, rec_n1.x, 0), __shfl_sync(FULL, rec_n1.y, 0));
     it_n1 = __shfl_sync(FULL, it_n2, 0);
   }
-  sc_flush<F32L>(d, tb, fo, w, vf, lane, n_in_cut);
+  resolve_queue<F32L>(d, tb, fo, w.q, qn, true, vf, lane, n_in_cut);
   add_pair_counts(d, n_tested, n_in_cut);
 }
 
