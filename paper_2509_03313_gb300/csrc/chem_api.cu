@@ -299,6 +299,7 @@ void init_train_dynamic(Train& t, const chem_config& c, int n_max) {
   t.next_id = 0;
   t.p_head = 0;
   t.p_tail = 0;
+  t.next_arr = std::numeric_limits<double>::infinity();
   t.species_steps = 0;
   t.water = 0;
   for (int i = 0; i < MAXT; ++i) t.counts[i] = 0;
@@ -328,9 +329,11 @@ void init_train_dynamic(Train& t, const chem_config& c, int n_max) {
 
 // Kernels of one captured step: diffusion, the sort passes, gather, the search (one or
 // both mappings), fast matching, the one-CTA reaction kernel, products, and the end (or
-// end-and-next-begin) kernel.
+// end-and-next-begin) kernel; small contexts have one search kernel and one kernel for all
+// that follows it.
 int kernels_per_step(const chem_ctx* ctx) {
-  return ctx->persistent ? 0 : 6 + ctx->d.passes + (ctx->lc.search_tps == 2 ? 2 : 1);
+  if (ctx->persistent) return 0;
+  return ctx->lc.small ? 4 + ctx->d.passes : 6 + ctx->d.passes + (ctx->lc.search_tps == 2 ? 2 : 1);
 }
 
 // Radix passes for the captured graph (see chem_ctx::passes_alloc).
@@ -500,6 +503,7 @@ chem_status homogeneous_run(chem_ctx* ctx, const double* t_end) {
     const PendingBuf& buf = p.buf[p.cur];
     for (size_t i = t.p_head; i < due_end[b]; ++i) t.counts[buf.type[i]] += 1;
     t.p_head = static_cast<uint32_t>(due_end[b]);
+    t.next_arr = due_end[b] < p.size() ? buf.t[due_end[b]] : std::numeric_limits<double>::infinity();
     t.hx_sel = 1;
     t.park_n = 0;  // parked particles are removed with the others (their counts stay)
     t.hx_t_end = t_end[b];
@@ -628,6 +632,7 @@ chem_status inject_one(chem_ctx* ctx, int b, int64_t n, const int32_t* type, con
   }
   t.p_head = 0;
   t.p_tail = static_cast<uint32_t>(tot);
+  t.next_arr = tot ? dst.t[0] : std::numeric_limits<double>::infinity();
   h.E_dep += energy_eV;
   return upload_trains(ctx, tr);
 }
@@ -917,6 +922,7 @@ chem_status chem_batch_init(const chem_config* cfgs, int32_t n_trains, chem_ctx*
   ctx->lc.search_blocks = ctx->sms * 4;  // resident CTAs (launch bounds 256 x 4); items are stolen
   ctx->lc.sort_blocks = ctx->sms * sort_occ;
   ctx->lc.persistent_blocks = ctx->sms * pers_occ;
+  ctx->lc.small = n_trains == 1 && cap <= static_cast<uint64_t>(SMALL_SPECIES) ? 1 : 0;
 
   // ---- device allocations
   Dev& d = ctx->d;

@@ -69,16 +69,64 @@ __global__ void __launch_bounds__(256, 4) k_search(const __grid_constant__ Dev d
 
 constexpr int TPS_WARPS = 4;  // warps per CTA of the one-thread-per-species search
 
+template <bool F32L, int W>
+union SearchSmem {
+  TpsSmem<F32L, W> tps;
+  GrpSmem<W> grp;
+  ScSmem<W> cells;
+};
+
+// One thread per home species, or several lanes per home when the launch has two or more lanes
+// for each (the CTAs of the launch are resident together).
+template <bool F32L, int W>
+__device__ __forceinline__ void search_species(const Dev& d, SearchSmem<F32L, W>& sm) {
+  const int lg = lanes_per_home_lg(d.g->n_total - d.g->n_dead, gridDim.x * blockDim.x);
+  // warps of one CTA are a grid apart, so that few homes spread over all CTAs
+  if (lg > 0) phase_search_groups<F32L, W>(d, sm.grp, lg, (threadIdx.x >> 5) * gridDim.x + blockIdx.x, gridDim.x * W);
+  else phase_search_tps<F32L, W>(d, sm.tps);
+}
+
 template <bool F32L>
 __global__ void __launch_bounds__(32 * TPS_WARPS, F32L ? 6 : 5) k_search_tps(const __grid_constant__ Dev d) {
-  __shared__ TpsSmem<F32L, TPS_WARPS> sm;
-  phase_search_tps<F32L, TPS_WARPS>(d, sm);
+  __shared__ SearchSmem<F32L, TPS_WARPS> sm;
+  if (d.g->search_cells_now) return;  // this step runs the cell tiles (grid-uniform)
+  search_species<F32L, TPS_WARPS>(d, sm);
+}
+
+// Either mapping in one launch, for contexts of at most SMALL_SPECIES species, whose steps cost
+// their launches more than their work (on 1e6 species two kernels are the faster form: the
+// cell tiles want larger CTAs).
+template <bool F32L>
+__global__ void __launch_bounds__(32 * TPS_WARPS, F32L ? 6 : 5) k_search_any(const __grid_constant__ Dev d) {
+  __shared__ SearchSmem<F32L, TPS_WARPS> sm;
+  if (d.g->search_cells_now) phase_search_cells<F32L, TPS_WARPS>(d, sm.cells);
+  else search_species<F32L, TPS_WARPS>(d, sm);
 }
 
 template <bool F32L>
 __global__ void __launch_bounds__(256) k_products(const __grid_constant__ Dev d) {
   __shared__ ProductsSmem sm;
-  phase_products<F32L>(d, sm);
+  phase_products<F32L>(d, sm, blockIdx.x, gridDim.x);
+}
+
+// Reaction resolution, the step's end and (begin_next) the next step's begin, one CTA.
+struct alignas(16) ReactEndSmem {
+  ReactAllSmem react;
+  EndSmem end;
+  BeginSmem begin;
+};
+constexpr int REACT_END_THREADS = 512;
+constexpr size_t REACT_END_BYTES = sizeof(ReactEndSmem) + react_all_bytes(RC_CAP);
+static_assert(sizeof(ReactEndSmem) % 16 == 0, "the buffer behind it is aligned");
+static_assert(REACT_END_BYTES <= 227 * 1024, "shared memory of one CTA");
+
+template <bool F32L>
+__global__ void __launch_bounds__(REACT_END_THREADS) k_react_end(const __grid_constant__ Dev d, int begin_next) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  ReactEndSmem& sm = *reinterpret_cast<ReactEndSmem*>(smem_raw);
+  phase_react_all<F32L>(d, sm.react, reinterpret_cast<uint32_t*>(smem_raw + sizeof(ReactEndSmem)), RC_CAP);
+  phase_end_step(d, sm.end);
+  if (begin_next) phase_begin(d, sm.begin);
 }
 
 template <bool F32L>
@@ -103,11 +151,11 @@ __global__ void __launch_bounds__(PERSIST_THREADS) k_persistent(const __grid_con
       else phase_search_tps<false, 8>(d, sm.tps64);
     }
     grid_sync(d);
-    phase_match_fast(d);
+    phase_match_fast(d, blockIdx.x, gridDim.x);
     grid_sync(d);
     if (blockIdx.x == 0) phase_react_serial(d, sm.serial, nullptr);
     grid_sync(d);
-    phase_products<F32L>(d, sm.products);
+    phase_products<F32L>(d, sm.products, blockIdx.x, gridDim.x);
     grid_sync(d);
     if (blockIdx.x == 0) {
       phase_end_step(d, sm.end);
@@ -148,15 +196,20 @@ cudaError_t enqueue_phases(const Dev& d, const LaunchCfg& lc, cudaStream_t s, cu
   mark(2 * PH_GATHER + 1);
   mark(2 * PH_SEARCH);
   // one mapping, or both with the one not chosen for the step returning at once
-  if (lc.search_tps != 0) k_search_tps<F32L><<<2 * lc.search_blocks, 32 * TPS_WARPS, 0, s>>>(d);
-  if (lc.search_tps != 1) k_search<F32L><<<lc.search_blocks, 256, 0, s>>>(d);
+  if (lc.small) k_search_any<F32L><<<2 * lc.search_blocks, 32 * TPS_WARPS, 0, s>>>(d);
+  else if (lc.search_tps != 0) k_search_tps<F32L><<<2 * lc.search_blocks, 32 * TPS_WARPS, 0, s>>>(d);
+  if (!lc.small && lc.search_tps != 1) k_search<F32L><<<lc.search_blocks, 256, 0, s>>>(d);
   mark(2 * PH_SEARCH + 1);
   mark(2 * PH_REACT);
-  e = enqueue_react_head(d, lc, s);
-  if (e != cudaSuccess) return e;
-  k_products<F32L><<<lc.stream_blocks, 256, 0, s>>>(d);
-  e = last ? enqueue_end_step(d, s) : enqueue_end_begin(d, s);
-  if (e != cudaSuccess) return e;
+  if (lc.small) {
+    k_react_end<F32L><<<1, REACT_END_THREADS, REACT_END_BYTES, s>>>(d, last ? 0 : 1);
+  } else {
+    e = enqueue_react_head(d, lc, s);
+    if (e != cudaSuccess) return e;
+    k_products<F32L><<<lc.stream_blocks, 256, 0, s>>>(d);
+    e = last ? enqueue_end_step(d, s) : enqueue_end_begin(d, s);
+    if (e != cudaSuccess) return e;
+  }
   mark(2 * PH_REACT + 1);
   return cudaGetLastError();
 }
@@ -223,8 +276,11 @@ cudaError_t enqueue_persistent(const Dev& d, const LaunchCfg& lc, int n_steps, c
 
 template <bool F32L>
 cudaError_t persistent_occupancy(int* blocks_per_sm) {
-  cudaError_t e = cudaFuncSetAttribute(k_persistent<F32L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(sizeof(PhaseSmem)));
+  cudaError_t e = cudaFuncSetAttribute(k_react_end<F32L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       static_cast<int>(REACT_END_BYTES));
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(k_persistent<F32L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           static_cast<int>(sizeof(PhaseSmem)));
   if (e != cudaSuccess) return e;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_persistent<F32L>, PERSIST_THREADS,
                                                        sizeof(PhaseSmem));

@@ -16,7 +16,7 @@ __global__ void __launch_bounds__(SORT_THREADS) k_sort_pass(const __grid_constan
 }
 
 __global__ void __launch_bounds__(256) k_match_fast(const __grid_constant__ Dev d) {
-  phase_match_fast(d);
+  phase_match_fast(d, blockIdx.x, gridDim.x);
 }
 
 constexpr size_t REACT_SERIAL_DYN_SMEM = (4 * EV_SMEM_CAP * sizeof(uint32_t) > RC_SMEM_BYTES)

@@ -18,6 +18,7 @@ struct LaunchCfg {
   int persistent_blocks;  // resident CTAs of the persistent step kernel
   int search_tps;         // pair search: 1 one thread per home species, 0 cell tiles,
                           // 2 both launched, the step's choice runs (adaptive)
+  int small;              // few species: one search kernel and one reaction kernel per step
 };
 
 // kernels_exact.cu (FP64 arithmetic without contraction)
@@ -35,6 +36,7 @@ cudaError_t sort_pass_occupancy(int* blocks_per_sm);
 cudaError_t enqueue_step_f64(const Dev& d, const LaunchCfg& lc, cudaStream_t s, cudaEvent_t* ev, bool first,
                              bool last);
 cudaError_t enqueue_persistent_f64(const Dev& d, const LaunchCfg& lc, int n_steps, cudaStream_t s);
+// (also sets the shared-memory limits of the precision's kernels)
 cudaError_t persistent_occupancy_f64(int* blocks_per_sm);
 cudaError_t enqueue_set_t_end(const Dev& d, const double* t_end_dev, cudaStream_t s);
 // one device thread waits, up to limit_s, for a word nothing writes (then CHEM_ETIMEOUT)

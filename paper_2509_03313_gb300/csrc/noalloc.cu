@@ -86,7 +86,7 @@ __global__ void k_noalloc_setup(Dev d, Tables tb, Train tr) {
     *d.trains = tr;
     Global g;
     std::memset(&g, 0, sizeof(g));
-    g.item_home = ITEM_HOME;
+    g.item_home = 0;  // several lanes per home species (few species)
     *d.g = g;
   }
 }
@@ -265,6 +265,7 @@ extern "C" chem_status chem_step_noalloc(const chem_config* cfg, uint32_t step, 
   tr.t_last_release = t_s;
   tr.step = step;
   tr.next_id = next_id;
+  tr.next_arr = std::numeric_limits<double>::infinity();
   tr.n_ref = NA_CELLS_AXIS;
   tr.h_ref = cfg->L_nm / NA_CELLS_AXIS;
 
@@ -327,19 +328,21 @@ extern "C" chem_status chem_step_noalloc(const chem_config* cfg, uint32_t step, 
   d.tables = reinterpret_cast<const Tables*>(b + LAYOUT.tables);
   d.g = reinterpret_cast<Global*>(b + LAYOUT.global);
 
-  int dev = 0, sms = 0, sort_occ = 0;
+  int dev = 0, sms = 0, sort_occ = 0, pers_occ = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-      sort_pass_occupancy(&sort_occ) != cudaSuccess || sms < 1 || sort_occ < 1) {
+      sort_pass_occupancy(&sort_occ) != cudaSuccess || persistent_occupancy_f64(&pers_occ) != cudaSuccess || sms < 1 ||
+      sort_occ < 1) {
     cudaGetLastError();
     return CHEM_ECUDA;
   }
   LaunchCfg lc;
   lc.stream_blocks = std::max(1, std::min(sms * 2, (n + 255) / 256 + 1));
-  lc.search_blocks = lc.stream_blocks;
+  lc.search_blocks = sms * 4;
   lc.sort_blocks = std::min(sms * sort_occ, static_cast<int>(NA_TILES));
   lc.persistent_blocks = 1;
   lc.search_tps = 0;
+  lc.small = 1;
   cudaStream_t s = static_cast<cudaStream_t>(cfg->cuda_stream);
   // leftovers of the previous call: stale hash cells and look-back words must not match
   bool ok = cudaMemsetAsync(d.cell_info, 0xFF, (NA_CELLS + 1) * 16, s) == cudaSuccess &&

@@ -189,24 +189,30 @@ __device__ __forceinline__ void set_pair_constants(Train& tr, const Tables& tb, 
 }
 
 // ======================================================================== begin
+constexpr int BEGIN_TRAINS = 16;  // trains whose cutoffs pass through shared memory
+
 struct BeginSmem {
   Tables tb;                              // the reaction tables, read once per step
   uint32_t rel[MAX_TRAINS];
   double dt[MAX_TRAINS];
   unsigned long long rcmax_bits[MAX_TRAINS];
   float hf[MAX_TRAINS];                   // this step's cell side
+  double c[BEGIN_TRAINS];                 // cutoff factor ...
+  double rc2[BEGIN_TRAINS][MAXR];         // ... and squared cutoffs of the first trains
   int cb0;                                // train 0: key bits per axis of its cells
   uint32_t base0;                         // train 0: first global cell
   uint32_t any;
 };
 
-// One CTA. (1) per train: release count, clock step and free-jump decision; (2) per
-// (train, reaction) cutoff and bridge constants and per (train, type) step sigma, spread
-// over the threads because FP64 square roots and divisions are long on this part;
-// (3) per train: hash grid of the step; (4) per (train, type pair) cutoff tables; (5) slot
-// offsets of the releases and the step counters. The step is one short chain of
-// dependent loads: the tables, the status and the global counters are read together at
-// the start, and later stages read what earlier ones wrote from shared memory.
+// One CTA of at least MAX_TRAINS threads. (1) per train: release count, clock step and
+// free-jump decision; (2) per (train, reaction) cutoff and bridge constants and per (train,
+// type) step sigma, spread over the threads because FP64 square roots and divisions are long
+// on this part; (3) per train: hash grid of the step; (4) per (train, type pair) cutoff
+// tables; (5) slot offsets of the releases and the step counters. The phase is a chain of
+// dependent latencies on the step's critical path, so every global load is issued at the
+// start (a train's record stays in its thread's registers through (1) and (3)), later
+// stages read what earlier ones wrote from shared memory, and the pending queue is only
+// searched when its first arrival is due. With loads in every stage it took 8 us.
 static __device__ void phase_begin(const Dev& d, BeginSmem& sb) {
   const int tid = threadIdx.x, nt = blockDim.x;
   {
@@ -225,35 +231,53 @@ static __device__ void phase_begin(const Dev& d, BeginSmem& sb) {
     g_epoch = g->epoch; g_cells = g->cells_steps; g_incut = g->pairs_in_cutoff; g_mark = g->incut_mark;
     sb.any = 0;
   }
+  // train `tid`
+  const uint32_t b = static_cast<uint32_t>(tid);
+  const bool have = b < d.n_trains;
+  Train& tr = d.trains[have ? b : 0u];
+  double t = 0, t_end = 0, t_lr = 0, horizon = 0, dt_min = 0, dt_L = 0, dt_cur = 0, next_arr = 0, L = 0, inv_L = 0;
+  uint32_t p_head = 0, p_tail = 0, pend_base = 0, next_id = 0, id_limit = 0, mat = 0, parked = 0;
+  int reset = 0, tr_n_max = 0, cb_alloc = 0, n_ref = 0;
+  long long live = 0;
+  if (have) {
+    t = tr.t; t_end = tr.t_end; t_lr = tr.t_last_release; horizon = tr.horizon;
+    dt_min = tr.dt_min; dt_L = tr.dt_L; dt_cur = tr.dt_cur; next_arr = tr.next_arr;
+    p_head = tr.p_head; p_tail = tr.p_tail; pend_base = tr.pend_base;
+    next_id = tr.next_id; id_limit = tr.id_limit;
+    mat = tr.mat_n;      // survivors of a homogeneous stage (already counted)
+    parked = tr.park_n;  // species parked while the train was idle (counted)
+    reset = tr.reset_on_release;
+    L = tr.L; inv_L = tr.inv_L; tr_n_max = tr.n_max; cb_alloc = tr.cb_alloc; n_ref = tr.n_ref;
+#pragma unroll
+    for (int ty = 0; ty < MAXT; ++ty) live += tr.counts[ty];  // 0 past the context's types
+    if (b < BEGIN_TRAINS) sb.c[b] = tr.c;
+    if (b == 0) {  // the removed species' key below needs train 0's grid, idle or not
+      sb.cb0 = tr.cb;
+      sb.base0 = tr.cell_base;
+    }
+  }
   __syncthreads();
   const Tables& tb = sb.tb;
-  for (uint32_t b = tid; b < d.n_trains; b += nt) {
-    Train& tr = d.trains[b];
-    // independent loads first: the per-train work below is one short dependency chain
-    const double t = tr.t, t_end = tr.t_end, t_lr = tr.t_last_release, horizon = tr.horizon;
-    const double dt_min = tr.dt_min, dt_L = tr.dt_L;
-    double dt_cur = tr.dt_cur;
-    const uint32_t p_head = tr.p_head, p_tail = tr.p_tail, pend_base = tr.pend_base;
-    const uint32_t next_id = tr.next_id, id_limit = tr.id_limit;
-    const uint32_t mat = tr.mat_n;  // survivors of a homogeneous stage (already counted)
-    const uint32_t parked = tr.park_n;  // species parked while the train was idle (counted)
-    const int reset = tr.reset_on_release;
-    long long live = 0;
-    for (int ty = 0; ty < MAXT; ++ty) live += (ty < tb.n_types) ? tr.counts[ty] : 0;
+  double dt = 0.0;
+  int free_jump = 0;
+  if (have) {
     const bool act = (st == 0) && (t < t_end);
     // an idle train with species among the stepped slots parks them this step
     tr.park_now = (!act && d.pk_cell != nullptr && live > static_cast<long long>(parked) + mat) ? 1u : 0u;
     uint32_t rel = 0;
-    int free_jump = 0;
-    double dt = 0.0;
     sb.rcmax_bits[b] = 0ull;
     if (act) {
       // pending arrivals are sorted; release those with arrival <= t
-      uint32_t lo = p_head, hi = p_tail;
-      const double* pt = d.pt + pend_base;
-      while (lo < hi) {
-        const uint32_t mid = (lo + hi) >> 1;
-        if (pt[mid] <= t) lo = mid + 1; else hi = mid;
+      uint32_t lo = p_head;
+      if (next_arr <= t) {
+        uint32_t hi = p_tail;
+        const double* pt = d.pt + pend_base;
+        while (lo < hi) {
+          const uint32_t mid = (lo + hi) >> 1;
+          if (pt[mid] <= t) lo = mid + 1; else hi = mid;
+        }
+        next_arr = (lo < p_tail) ? pt[lo] : CUDART_INF;
+        tr.next_arr = next_arr;
       }
       rel = lo - p_head;
       double t_last = t_lr;
@@ -262,7 +286,6 @@ static __device__ void phase_begin(const Dev& d, BeginSmem& sb) {
         tr.t_last_release = t;
         if (reset) dt_cur = dt_min;
       }
-      const double next_arr = (lo < p_tail) ? pt[lo] : CUDART_INF;
       double t_next;
       if (horizon > 0.0 && __dsub_rn(t, t_last) >= horizon && next_arr > t) {
         free_jump = 1;
@@ -277,6 +300,8 @@ static __device__ void phase_begin(const Dev& d, BeginSmem& sb) {
           t_next = __dadd_rn(t, dt);
         }
       }
+      sb.dt[b] = dt;
+      sb.rel[b] = parked + rel + mat;
       tr.dt_cur = dt_cur;
       tr.dt = dt;
       tr.t_next = t_next;
@@ -297,49 +322,45 @@ static __device__ void phase_begin(const Dev& d, BeginSmem& sb) {
       if (static_cast<unsigned long long>(next_id) + rel + mat > id_limit) raise_status(d.g, CHEM_ECAPACITY);
       atomicOr(&sb.any, 1u);
     } else {
+      sb.dt[b] = 0.0;
+      sb.rel[b] = 0u;
       tr.rel_n = 0;
       tr.rel_mat = 0;
       tr.rel_park = 0;
     }
     tr.active = act ? 1 : 0;
     tr.free_jump = free_jump;
-    sb.rel[b] = act ? parked + rel + mat : 0u;
-    sb.dt[b] = act ? dt : 0.0;
   }
   __syncthreads();
   // cutoffs R + c sqrt(2 D_AB dt), bridge constants, and sigma = sqrt(2 D dt)
   const int per = MAXR + MAXT;
   for (uint32_t w = tid; w < d.n_trains * per; w += nt) {
-    const uint32_t b = w / per;
+    const uint32_t wb = w / per;
     const int q = static_cast<int>(w % per);
-    const double dt = sb.dt[b];
-    if (dt <= 0.0) continue;  // train not advancing this step
-    Train& tr = d.trains[b];
+    const double wdt = sb.dt[wb];
+    if (wdt <= 0.0) continue;  // train not advancing this step
+    Train& wt = d.trains[wb];
     if (q < MAXR) {
       if (q >= tb.n_rxn) continue;
-      const double rc = __dadd_rn(tb.R[q], __dmul_rn(tr.c, sqrt(__dmul_rn(__dmul_rn(2.0, tb.D_AB[q]), dt))));
-      tr.rc2[q] = __dmul_rn(rc, rc);
-      tr.rc2f[q] = static_cast<float>(tr.rc2[q]);
-      set_pair_constants(tr, tb, q, dt);
-      atomicMax(&sb.rcmax_bits[b], static_cast<unsigned long long>(__double_as_longlong(rc)));
+      const double c = wb < BEGIN_TRAINS ? sb.c[wb] : wt.c;
+      const double rc = __dadd_rn(tb.R[q], __dmul_rn(c, sqrt(__dmul_rn(__dmul_rn(2.0, tb.D_AB[q]), wdt))));
+      const double rc2 = __dmul_rn(rc, rc);
+      atomicMax(&sb.rcmax_bits[wb], static_cast<unsigned long long>(__double_as_longlong(rc)));
+      if (wb < BEGIN_TRAINS) sb.rc2[wb][q] = rc2;
+      wt.rc2[q] = rc2;
+      wt.rc2f[q] = static_cast<float>(rc2);
+      set_pair_constants(wt, tb, q, wdt);
     } else {
       const int ty = q - MAXR;
       if (ty >= tb.n_types) continue;
-      tr.sig[ty] = sqrt(__dmul_rn(__dmul_rn(2.0, tb.D[ty]), dt));
-      tr.sigf[ty] = static_cast<float>(tr.sig[ty]);
+      const double sig = sqrt(__dmul_rn(__dmul_rn(2.0, tb.D[ty]), wdt));
+      wt.sig[ty] = sig;
+      wt.sigf[ty] = static_cast<float>(sig);
     }
   }
   __syncthreads();
-  for (uint32_t b = tid; b < d.n_trains; b += nt) {
-    Train& tr = d.trains[b];
-    if (b == 0) {  // the removed species' key below needs train 0's grid, idle or not
-      sb.cb0 = tr.cb;
-      sb.base0 = tr.cell_base;
-    }
-    if (sb.dt[b] <= 0.0) continue;
-    const double L = tr.L, inv_L = tr.inv_L;
-    const int n_max = min(tr.n_max, (1 << tr.cb_alloc) - 1), fj = tr.free_jump;
-    int n_ref = tr.n_ref;
+  if (have && dt > 0.0) {
+    const int n_max = min(tr_n_max, (1 << cb_alloc) - 1);
     const double rcmax = __longlong_as_double(static_cast<long long>(sb.rcmax_bits[b]));
     // finest admissible grid: cells at least the largest cutoff (with slack), at least 3
     // per axis (no cell met twice among a cell's neighbours)
@@ -358,23 +379,26 @@ static __device__ void phase_begin(const Dev& d, BeginSmem& sb) {
     // keep the current grid while it is valid and at most 2x too coarse; when the
     // cutoff outgrows it, move to cells 1.2x larger than needed (fewer regrids)
     int n = n_ref;
-    if (!fj) {
+    if (!free_jump) {
       if (n > n_target) n = max(3, (5 * n_target) / 6);
       else if (2 * n < n_target) n = n_target;
     }
+    double h = __ddiv_rn(L, static_cast<double>(n));
     // the search looks one cell out: a cell must cover the largest cutoff
-    if (!fj && rcmax > 0.0) {
+    if (!free_jump && rcmax > 0.0 && n != n_target) {
       const double cut = rcmax * static_cast<double>(CELL_SLACK_F);
-      if (L / static_cast<double>(n) < cut) n = n_target;
+      if (h < cut) {
+        n = n_target;
+        h = __ddiv_rn(L, static_cast<double>(n));
+      }
     }
-    const double h = __ddiv_rn(L, static_cast<double>(n));
     const double inv_h = __dmul_rn(static_cast<double>(n), inv_L);
     tr.n = n;
     tr.cb = axis_bits(n);
     tr.h = h;
     tr.inv_h = inv_h;
     tr.hf = static_cast<float>(h);
-    tr.hlo = static_cast<float>(h - static_cast<double>(tr.hf));
+    tr.hlo = static_cast<float>(h - static_cast<double>(static_cast<float>(h)));
     tr.inv_hf = static_cast<float>(inv_h);
     sb.hf[b] = static_cast<float>(h);
     if (b == 0) sb.cb0 = axis_bits(n);
@@ -384,27 +408,27 @@ static __device__ void phase_begin(const Dev& d, BeginSmem& sb) {
   // FP32, and the FP32 one widened past any error of FP32 cell offsets (a few 1e-7 of a
   // cell per component), so that a pair the FP32 test rejects is outside the FP64 cutoff
   for (uint32_t w = tid; w < d.n_trains * (MAXT * MAXT); w += nt) {
-    const uint32_t b = w / (MAXT * MAXT);
+    const uint32_t wb = w / (MAXT * MAXT);
     const int q = static_cast<int>(w % (MAXT * MAXT));
-    if (sb.dt[b] <= 0.0) continue;
-    Train& tr = d.trains[b];
+    if (sb.dt[wb] <= 0.0) continue;
+    Train& wt = d.trains[wb];
     const int r = tb.pair_rxn[q / MAXT][q % MAXT];
-    const double c2 = r >= 0 ? tr.rc2[r] : -1.0;
+    const double c2 = r >= 0 ? (wb < BEGIN_TRAINS ? sb.rc2[wb][r] : wt.rc2[r]) : -1.0;
     const float c2f = r >= 0 ? static_cast<float>(c2) : -1.f;
-    tr.rc2_tt[q] = c2;
-    tr.rc2f_tt[q] = c2f;
+    wt.rc2_tt[q] = c2;
+    wt.rc2f_tt[q] = c2f;
     const float rc = c2f >= 0.f ? sqrtf(c2f) : -1.f;
-    const float rw = rc * 1.00001f + 2e-6f * sb.hf[b];
-    tr.rc2w_tt[q] = rc >= 0.f ? rw * rw * 1.00001f : -1.f;
+    const float rw = rc * 1.00001f + 2e-6f * sb.hf[wb];
+    wt.rc2w_tt[q] = rc >= 0.f ? rw * rw * 1.00001f : -1.f;
   }
   if (tid == 0) {
     uint32_t off = g_total;
     const uint32_t before = off;
     unsigned long long total = off;
-    for (uint32_t b = 0; b < d.n_trains; ++b) {
-      d.trains[b].rel_off = off;
-      total += sb.rel[b];
-      off += sb.rel[b];
+    for (uint32_t q = 0; q < d.n_trains; ++q) {
+      d.trains[q].rel_off = off;
+      total += sb.rel[q];
+      off += sb.rel[q];
     }
     if (total > d.cap) {
       raise_status(g, CHEM_ECAPACITY);
@@ -909,6 +933,33 @@ __device__ __forceinline__ void fwd_offset(int k, int& dx, int& dy, int& dz) {
   dz = 0; dy = 0; dx = 1;
 }
 
+// The forward cells (bits 1..13) that hold points within the squared cutoff rcmax2 of a home
+// at the offset v in its cell. A cell whose nearest point is farther holds no partner and is
+// not looked up (the gaps are taken 1e-5 of a cell short, which covers every rounding of the
+// offsets). Per axis the gap is 0 (same layer), the distance to the lower face (offset -1) or
+// to the upper face (offset +1).
+__device__ __forceinline__ uint32_t cells_in_reach(const float4& v, float hf, float rcmax2) {
+  rcmax2 *= 1.0001f;
+  const float eps = 1e-5f * hf;
+  auto gap = [&](int o, float of) {
+    const float g = o > 0 ? static_cast<float>(o) * hf - of : (o < 0 ? of + static_cast<float>(-o - 1) * hf : 0.f);
+    return fmaxf(g - eps, 0.f);
+  };
+  const float xm = gap(-1, v.x), xp = gap(1, v.x), ym = gap(-1, v.y), yp = gap(1, v.y), zp = gap(1, v.z);
+  const float xm2 = xm * xm, xp2 = xp * xp, ym2 = ym * ym, yp2 = yp * yp, zp2 = zp * zp;
+  uint32_t m = 0u;
+#pragma unroll
+  for (int k = 1; k < N_FWD; ++k) {
+    int dx, dy, dz;
+    fwd_offset(k, dx, dy, dz);
+    const float sx = dx < 0 ? xm2 : (dx > 0 ? xp2 : 0.f);
+    const float sy = dy < 0 ? ym2 : (dy > 0 ? yp2 : 0.f);
+    const float sz = dz > 0 ? zp2 : 0.f;
+    if ((sx + sy) + sz <= rcmax2) m |= 1u << k;
+  }
+  return m;
+}
+
 // FP32 separation x_j - x_i of two species held as offsets from their cells' corners,
 // the neighbour's cell lying (cfx, cfy, cfz) cells away (cell side hf), and its square.
 // Written with explicit roundings (no contraction left to the compiler) so that every
@@ -1243,34 +1294,10 @@ __device__ void phase_search_tps(const Dev& d, TpsSmem<F32L, W>& sm) {
         int ix, iy, iz;
         cell_decode(cell - tr.cell_base, tr.cb, ix, iy, iz);
         if (s + 1u < static_cast<uint32_t>(d.cell_info[cell].y)) kmask = 1u;
-        // a forward cell whose nearest point is farther from the home than the largest
-        // cutoff of the home's type holds no partner and is not looked up (the gaps are
-        // taken 1e-5 of a cell short, which covers every rounding of the offsets)
-        const float hcell = tr.hf, eps = 1e-5f * tr.hf;
-        const float ofx = vi.x, ofy = vi.y, ofz = vi.z;
         float rcmax2 = -1.f;
 #pragma unroll
         for (int t = 0; t < MAXT; ++t) rcmax2 = fmaxf(rcmax2, static_cast<float>(rc2[t]));
-        rcmax2 *= 1.0001f;
-        auto gap = [&](int o, float of) {
-          const float g = o > 0 ? static_cast<float>(o) * hcell - of
-                                : (o < 0 ? of + static_cast<float>(-o - 1) * hcell : 0.f);
-          return fmaxf(g - eps, 0.f);
-        };
-        // per axis the gap is 0 (same layer), the distance to the lower face (offset -1)
-        // or to the upper face (offset +1); the 13 offsets unrolled
-        const float xm = gap(-1, ofx), xp = gap(1, ofx), ym = gap(-1, ofy), yp = gap(1, ofy);
-        const float zp = gap(1, ofz);
-        const float xm2 = xm * xm, xp2 = xp * xp, ym2 = ym * ym, yp2 = yp * yp, zp2 = zp * zp;
-#pragma unroll
-        for (int k = 1; k < N_FWD; ++k) {
-          int dx, dy, dz;
-          fwd_offset(k, dx, dy, dz);
-          const float sx = dx < 0 ? xm2 : (dx > 0 ? xp2 : 0.f);
-          const float sy = dy < 0 ? ym2 : (dy > 0 ? yp2 : 0.f);
-          const float sz = dz > 0 ? zp2 : 0.f;
-          if ((sx + sy) + sz <= rcmax2) kmask |= 1u << k;
-        }
+        kmask |= cells_in_reach(vi, tr.hf, rcmax2);
       }
       // (ranges are not moved between lanes: on clustered tracks, taking over half of a busy
       // lane's range cost more issue slots than the idle lanes it saved; dense cells go to the
@@ -1387,6 +1414,175 @@ __device__ void phase_search_tps(const Dev& d, TpsSmem<F32L, W>& sm) {
   add_pair_counts(d, n_tested, n_in_cut);
 }
 
+// ---- several lanes per home species
+// With fewer home species than lanes on the chip, the time of a step's search is the chain
+// of one home's dependent loads and its serial walk (16 to 66 us at 2,000 to 31,000 species
+// with one lane per home, however few pairs there are; 10 to 29 us with several). Here 2^lg lanes share a home: each
+// looks up every 2^lg-th cell of the half shell with all its loads in flight together, the
+// non-empty ranges of a home are laid end to end, and its lanes take every 2^lg-th neighbour
+// of that list. The same pairs are visited and queued.
+constexpr int GRP_UNROLL = 4;    // neighbours a lane keeps in flight
+constexpr int GRP_MAX_LG = 4;
+
+// lg of the lanes per home for n species on `lanes` lanes: as many as there are spare, up to
+// 16 (a lane per cell of the half shell). 0: one thread per home species.
+__device__ __forceinline__ int lanes_per_home_lg(uint32_t n, uint32_t lanes) {
+  const uint32_t per = lanes / (n ? n : 1u);
+  return per >= 2u ? min(GRP_MAX_LG, 31 - __clz(per)) : 0;
+}
+
+template <int W>
+struct GrpSmem {
+  uint32_t rs[W][N_FWD][16];    // per home of the warp: first slot of its ranges,
+  uint32_t off[W][N_FWD][16];   // their offsets in its neighbour list,
+  uint8_t rk[W][N_FWD][16];     // and half-shell indices
+  PairQueue<32 * (GRP_UNROLL + 1)> q[W];
+  FwdSmem fo;
+};
+
+// Warp `warp` of `n_warps` (at most all of the launch) takes every n_warps-th set of homes.
+template <bool F32L, int W>
+__device__ void phase_search_groups(const Dev& d, GrpSmem<W>& sm, int lg, uint32_t warp, uint32_t n_warps) {
+  constexpr uint32_t FULL = 0xffffffffu;
+  const uint32_t n_live = d.g->n_total - d.g->n_dead;
+  const uint32_t epoch = d.g->epoch;
+  const uint32_t* vf = d.g->sort_any ? (d.g->sort_parity ? d.vals1 : d.vals0) : nullptr;
+  const Tables& tb = *d.tables;
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  const uint32_t lanemask_lt = (1u << lane) - 1u;
+  auto& q = sm.q[wib];
+  uint32_t qn = 0, n_tested = 0, n_in_cut = 0;
+  fwd_smem_fill(sm.fo);
+  if (!block_status_ok(d)) return;  // (a barrier, which also publishes the offsets)
+  const FwdSmem& fo = sm.fo;
+  const int G = 1 << lg, g = lane & (G - 1), grp = lane >> lg;
+  const uint32_t homes = 32u >> lg;
+  const uint32_t n_sets = (n_live + homes - 1u) / homes;
+  const uint32_t grp_mask = (lg == 5 ? FULL : (1u << G) - 1u) << (grp << lg);
+  for (uint32_t c = warp; c < n_sets; c += n_warps) {
+    const uint32_t s = c * homes + static_cast<uint32_t>(grp);
+    bool home = s < n_live;
+    uint32_t cell = 0;
+    float4 vi = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (home) {
+      cell = d.cell_sorted[s];
+      vi = d.s4[s];
+    }
+    const int b = (d.n_trains == 1 || !home) ? 0 : train_of_cell(d.trains, d.n_trains, cell);
+    const Train& tr = d.trains[b];
+    const uint32_t ti = tid_type(__float_as_uint(vi.w));
+    home = home && tr.active && !tr.free_jump && tb.reactive_mask[ti] != 0u;
+    const float* row = F32L ? &tr.rc2f_tt[ti * MAXT] : &tr.rc2w_tt[ti * MAXT];
+    float rc2[MAXT];
+#pragma unroll
+    for (int u = 0; u < MAXT; ++u) rc2[u] = row[u];
+    const float hf = tr.hf;
+    // the cells in reach (as in phase_search_tps), every G-th of them this lane's
+    uint32_t kmask = 0u;
+    int ix = 0, iy = 0, iz = 0;
+    const int n = tr.n;
+    if (home) {
+      cell_decode(cell - tr.cell_base, tr.cb, ix, iy, iz);
+      float rcmax2 = -1.f;
+#pragma unroll
+      for (int u = 0; u < MAXT; ++u) rcmax2 = fmaxf(rcmax2, rc2[u]);
+      kmask = 1u | cells_in_reach(vi, hf, rcmax2);
+    }
+    constexpr int MAX_MINE = N_FWD / 2;  // with two lanes per home
+    uint32_t nc[MAX_MINE], word[MAX_MINE];
+#pragma unroll
+    for (int i = 0; i < MAX_MINE; ++i) {
+      const int k = g + (i << lg);
+      nc[i] = 0u;
+      word[i] = 0u;
+      if (k < N_FWD && ((kmask >> k) & 1u)) {
+        nc[i] = tr.cell_base + cell_encode(step_cell(ix, fo.i[0][k], n), step_cell(iy, fo.i[1][k], n),
+                                           step_cell(iz, fo.i[2][k], n), tr.cb);
+        word[i] = (d.occ[nc[i] >> 5] >> (nc[i] & 31u)) & 1u;
+      }
+    }
+    uint32_t st[MAX_MINE], len[MAX_MINE];
+#pragma unroll
+    for (int i = 0; i < MAX_MINE; ++i) {
+      st[i] = 0u;
+      len[i] = 0u;
+      if (word[i]) {
+        const int4 ci = d.cell_info[nc[i]];
+        if (static_cast<uint32_t>(ci.z) == epoch) {
+          st[i] = (g + (i << lg)) == 0 ? s + 1u : static_cast<uint32_t>(ci.x);  // own cell: its later slots
+          len[i] = static_cast<uint32_t>(ci.y) > st[i] ? static_cast<uint32_t>(ci.y) - st[i] : 0u;
+        }
+      }
+    }
+    // the home's non-empty ranges end to end (the order does not matter)
+    uint32_t nr = 0, total = 0;
+#pragma unroll
+    for (int i = 0; i < MAX_MINE; ++i) {
+      if ((i << lg) >= N_FWD) break;
+      const uint32_t bal = __ballot_sync(FULL, len[i] > 0u) & grp_mask;
+      uint32_t incl = len[i];
+      for (int o = 1; o < G; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(FULL, incl, o, G);
+        if (g >= o) incl += y;
+      }
+      if (len[i] > 0u) {
+        const uint32_t at = nr + __popc(bal & lanemask_lt);
+        sm.rs[wib][at][grp] = st[i];
+        sm.off[wib][at][grp] = total + incl - len[i];
+        sm.rk[wib][at][grp] = static_cast<uint8_t>(g + (i << lg));
+      }
+      nr += __popc(bal);
+      total += __shfl_sync(FULL, incl, G - 1, G);
+    }
+    __syncwarp();
+    uint32_t r = 0, f = static_cast<uint32_t>(g);  // this lane's place in the list
+    while (__any_sync(FULL, f < total)) {
+      uint32_t ju[GRP_UNROLL], ku[GRP_UNROLL];
+      float4 vj[GRP_UNROLL];
+#pragma unroll
+      for (int u = 0; u < GRP_UNROLL; ++u) {
+        ju[u] = 0u;
+        ku[u] = 0xFFu;  // no neighbour
+        if (f < total) {
+          while (r + 1u < nr && sm.off[wib][r + 1u][grp] <= f) ++r;
+          ju[u] = sm.rs[wib][r][grp] + (f - sm.off[wib][r][grp]);
+          ku[u] = sm.rk[wib][r][grp];
+        }
+        f += static_cast<uint32_t>(G);
+      }
+#pragma unroll
+      for (int u = 0; u < GRP_UNROLL; ++u) vj[u] = d.s4[ju[u]];
+      uint32_t bal[GRP_UNROLL], any = 0u;
+#pragma unroll
+      for (int u = 0; u < GRP_UNROLL; ++u) {
+        const uint32_t k = ku[u] == 0xFFu ? 0u : ku[u];
+        const uint32_t tj = __float_as_uint(vj[u].w) & 7u;
+        const float rc2u = ku[u] == 0xFFu ? -1.f : (F32L ? tr.rc2f_tt[ti * MAXT + tj] : tr.rc2w_tt[ti * MAXT + tj]);
+        float fx, fy, fz;
+        const bool pass = sep_f32(fo.f[0][k], fo.f[1][k], fo.f[2][k], hf, vj[u], vi, fx, fy, fz) < rc2u;
+        n_tested += rc2u >= 0.f ? 1u : 0u;
+        if constexpr (F32L) n_in_cut += pass ? 1u : 0u;
+        bal[u] = __ballot_sync(FULL, pass);
+        any |= bal[u];
+      }
+      if (any != 0u) {
+#pragma unroll
+        for (int u = 0; u < GRP_UNROLL; ++u) {
+          if ((bal[u] >> lane) & 1u) {
+            const uint32_t pos = qn + __popc(bal[u] & lanemask_lt);
+            q.si[pos] = s; q.j[pos] = ju[u]; q.kb[pos] = ku[u] | (static_cast<uint32_t>(b) << 8);
+          }
+          qn += __popc(bal[u]);
+        }
+        if (qn >= 32u) qn = resolve_queue<F32L>(d, tb, fo, q, qn, false, vf, lane, n_in_cut);
+      }
+    }
+    __syncwarp();  // the next set rewrites the ranges
+  }
+  resolve_queue<F32L>(d, tb, fo, q, qn, true, vf, lane, n_in_cut);
+  add_pair_counts(d, n_tested, n_in_cut);
+}
+
 // ======================================================================== react
 // One reaction per species (Sec. 2.4: diffusion-controlled reactions, reactants react
 // on encounter):
@@ -1405,6 +1601,7 @@ __device__ void phase_search_tps(const Dev& d, TpsSmem<F32L, W>& sm) {
 struct MatchSmem {
   uint32_t n_alive, n_next;
   uint32_t n_won, won_base;
+  uint32_t n_conflict;
 };
 
 // Events ordered in shared memory by the one-CTA react kernel (4 arrays of this size).
@@ -1433,7 +1630,7 @@ struct ProductsSmem {
 };
 
 struct EndSmem {
-  uint32_t any;
+  uint32_t any, stepped;
 };
 
 // Exclusive block-wide prefix of v (one value per thread); `total` gets the block sum.
@@ -1495,11 +1692,11 @@ __device__ __forceinline__ void commit_event(const Dev& d, uint32_t c, const Can
   d.ev_v0[e] = c | (static_cast<uint32_t>(d.tables->n_prod[cd.rxn_train & 255u]) << 24);
 }
 
-static __device__ void phase_match_fast(const Dev& d) {
+static __device__ void phase_match_fast(const Dev& d, uint32_t block, uint32_t blocks) {
   const bool ok = block_status_ok(d);  // includes a barrier
   const uint32_t n_c = ok ? min(d.g->n_cand, d.cap_cand) : 0u;
-  const uint32_t stride = gridDim.x * blockDim.x;
-  for (uint32_t c0 = blockIdx.x * blockDim.x; c0 < n_c; c0 += stride) {  // uniform per block
+  const uint32_t stride = blocks * blockDim.x;
+  for (uint32_t c0 = block * blockDim.x; c0 < n_c; c0 += stride) {  // uniform per block
     const uint32_t c = c0 + threadIdx.x;
     const bool valid = c < n_c;
     Cand cd{};
@@ -1607,37 +1804,46 @@ static __device__ void phase_match_rounds(const Dev& d, MatchSmem& sm) {
 // false (nothing done) when the conflict list does not fit; the caller then runs the
 // global-memory version. `sbuf` holds RC_SMEM_BYTES.
 constexpr int RC_CAP = 1536;                 // conflict pairs
-constexpr int RC_SLOTS = 2 * RC_CAP;         // distinct slots at most
-constexpr int RC_HASH = 8192;                // >= 2 RC_SLOTS, power of two
-constexpr size_t RC_SMEM_BYTES = static_cast<size_t>(RC_CAP) * (4 + 4 + 4 + 8 + 8) +
-                                 static_cast<size_t>(RC_HASH) * 8 + static_cast<size_t>(RC_SLOTS) * (8 + 8 + 4) +
-                                 static_cast<size_t>(RC_CAP) * 8;
+__host__ __device__ constexpr uint32_t rc_hash(uint32_t n_c) {  // hash buckets: at least two per slot
+  uint32_t h = 64u;
+  while (h < 4u * n_c) h <<= 1;
+  return h;
+}
+// Bytes of sbuf for `cap` pairs (two slots each).
+__host__ __device__ constexpr size_t rc_smem_bytes(uint32_t cap) {
+  return static_cast<size_t>(cap) * (4 + 4 + 4 + 4 + 4 + 8 + 8) + static_cast<size_t>(rc_hash(cap)) * 8 +
+         static_cast<size_t>(2 * cap) * (8 + 8 + 4);
+}
+constexpr size_t RC_SMEM_BYTES = rc_smem_bytes(RC_CAP);
 
-static __device__ bool phase_match_rounds_smem(const Dev& d, MatchSmem& sm, uint32_t* sbuf) {
+// The rounds over the n_c accepted pairs list[0, n_c) (nullptr: pairs 0 .. n_c - 1, of which
+// sm.n_conflict share a species with another), sbuf of rc_smem_bytes(n_c) or more:
+// sm.n_won winners, their pairs' indices in the returned list (in sbuf).
+static __device__ const uint32_t* match_rounds_in_smem(const Dev& d, MatchSmem& sm, uint32_t* sbuf, uint32_t n_c,
+                                                       const uint32_t* list) {
   const int tid = threadIdx.x, nt = blockDim.x;
-  const bool ok = block_status_ok(d);
-  const uint32_t n_c = ok ? d.g->n_conflict : 0u;
-  if (n_c > static_cast<uint32_t>(RC_CAP)) return false;  // uniform
+  const uint32_t hash = rc_hash(n_c);
   // carve the buffer (8-byte arrays first)
   unsigned long long* kd = reinterpret_cast<unsigned long long*>(sbuf);
-  unsigned long long* kp = kd + RC_CAP;
-  unsigned long long* bd = kp + RC_CAP;
-  unsigned long long* bp = bd + RC_SLOTS;
-  uint32_t* hkey = reinterpret_cast<uint32_t*>(bp + RC_SLOTS);
-  uint32_t* hval = hkey + RC_HASH;
-  uint32_t* lo = hval + RC_HASH;
-  uint32_t* hi = lo + RC_CAP;
-  uint32_t* cix = hi + RC_CAP;
-  uint32_t* alive = cix + RC_CAP;
-  uint32_t* nxt = alive + RC_CAP;
-  uint32_t* ldead = nxt + RC_CAP;
-  for (int i = tid; i < RC_HASH; i += nt) hkey[i] = 0xFFFFFFFFu;
-  for (int i = tid; i < RC_SLOTS; i += nt) ldead[i] = 0u;
-  if (tid == 0) { sm.n_alive = n_c; sm.n_next = 0; }
+  unsigned long long* kp = kd + n_c;
+  unsigned long long* bd = kp + n_c;
+  unsigned long long* bp = bd + 2 * n_c;
+  uint32_t* hkey = reinterpret_cast<uint32_t*>(bp + 2 * n_c);
+  uint32_t* hval = hkey + hash;
+  uint32_t* lo = hval + hash;
+  uint32_t* hi = lo + n_c;
+  uint32_t* cix = hi + n_c;
+  uint32_t* alive = cix + n_c;
+  uint32_t* nxt = alive + n_c;
+  uint32_t* ldead = nxt + n_c;  // per slot: its pairs, and DEAD once it reacted
+  constexpr uint32_t DEAD = 0x80000000u;
+  for (uint32_t i = tid; i < hash; i += nt) hkey[i] = 0xFFFFFFFFu;
+  for (uint32_t i = tid; i < 2 * n_c; i += nt) ldead[i] = 0u;
+  if (tid == 0) { sm.n_alive = n_c; sm.n_next = 0; sm.n_conflict = 0; }
   __syncthreads();
   // load the pairs, reset the accepted-pair counts for the next step, insert the slots
   for (uint32_t i = tid; i < n_c; i += nt) {
-    const uint32_t c = d.alive0[i];
+    const uint32_t c = list ? list[i] : i;
     const Cand cd = d.cand[c];
     d.touch[cd.s_lo] = 0u;
     d.touch[cd.s_hi] = 0u;
@@ -1652,22 +1858,31 @@ static __device__ bool phase_match_rounds_smem(const Dev& d, MatchSmem& sm, uint
   // slot -> local index: open addressing; the thread whose CAS claims a bucket numbers it
   for (uint32_t e = tid; e < 2 * n_c; e += nt) {
     const uint32_t slot = (e & 1u) ? hi[e >> 1] : lo[e >> 1];
-    uint32_t h = (slot * 2654435761u) & (RC_HASH - 1);
-    for (int probe = 0; probe < RC_HASH; ++probe) {
+    uint32_t h = ((slot * 2654435761u) >> 8) & (hash - 1u);
+    for (uint32_t probe = 0; probe < hash; ++probe) {
       const uint32_t prev = atomicCAS(&hkey[h], 0xFFFFFFFFu, slot);
       if (prev == 0xFFFFFFFFu) { hval[h] = atomicAdd(&sm.n_next, 1u); break; }
       if (prev == slot) break;
-      h = (h + 1u) & (RC_HASH - 1);
+      h = (h + 1u) & (hash - 1u);
     }
   }
   __syncthreads();
   for (uint32_t e = tid; e < 2 * n_c; e += nt) {
     const uint32_t slot = (e & 1u) ? hi[e >> 1] : lo[e >> 1];
-    uint32_t h = (slot * 2654435761u) & (RC_HASH - 1);
-    for (int probe = 0; probe < RC_HASH && hkey[h] != slot; ++probe) h = (h + 1u) & (RC_HASH - 1);
+    uint32_t h = ((slot * 2654435761u) >> 8) & (hash - 1u);
+    for (uint32_t probe = 0; probe < hash && hkey[h] != slot; ++probe) h = (h + 1u) & (hash - 1u);
     if (e & 1u) hi[e >> 1] = hval[h]; else lo[e >> 1] = hval[h];
+    if (!list) atomicAdd(&ldead[hval[h]], 1u);
   }
   __syncthreads();
+  if (!list) {
+    for (uint32_t i0 = 0; i0 < n_c; i0 += nt) {
+      const uint32_t i = i0 + tid;
+      const uint32_t m = __ballot_sync(0xffffffffu, i < n_c && (ldead[lo[i < n_c ? i : 0u]] > 1u || ldead[hi[i < n_c ? i : 0u]] > 1u));
+      if ((tid & 31) == 0 && m) atomicAdd(&sm.n_conflict, static_cast<uint32_t>(__popc(m)));
+    }
+    __syncthreads();  // the winners below set DEAD
+  }
   // winners are listed in shared memory (the hash values are no longer needed) and
   // recorded as events after the last round with one reservation
   uint32_t* won = hval;
@@ -1706,8 +1921,8 @@ static __device__ bool phase_match_rounds_smem(const Dev& d, MatchSmem& sm, uint
       }
       const uint32_t q = warp_reserve(&sm.n_won, win);
       if (win) {
-        ldead[lo[i]] = 1u;
-        ldead[hi[i]] = 1u;
+        ldead[lo[i]] = DEAD;
+        ldead[hi[i]] = DEAD;
         won[q] = i;
       }
     }
@@ -1721,7 +1936,7 @@ static __device__ bool phase_match_rounds_smem(const Dev& d, MatchSmem& sm, uint
       uint32_t i = 0;
       if (a < na) {
         i = alive[a];
-        keep = !ldead[lo[i]] && !ldead[hi[i]];
+        keep = ldead[lo[i]] != DEAD && ldead[hi[i]] != DEAD;
       }
       const uint32_t q = warp_reserve(&sm.n_next, keep);
       if (keep) {
@@ -1735,12 +1950,20 @@ static __device__ bool phase_match_rounds_smem(const Dev& d, MatchSmem& sm, uint
     uint32_t* t = alive; alive = nxt; nxt = t;
     __syncthreads();
   }
+  for (uint32_t q = tid; q < sm.n_won; q += nt) won[q] = cix[won[q]];
+  __syncthreads();
+  return won;
+}
+
+static __device__ bool phase_match_rounds_smem(const Dev& d, MatchSmem& sm, uint32_t* sbuf) {
+  const int tid = threadIdx.x, nt = blockDim.x;
+  const bool ok = block_status_ok(d);
+  const uint32_t n_c = ok ? d.g->n_conflict : 0u;
+  if (n_c > static_cast<uint32_t>(RC_CAP)) return false;  // uniform
+  const uint32_t* won = match_rounds_in_smem(d, sm, sbuf, n_c, d.alive0);
   if (tid == 0) sm.won_base = atomicAdd(&d.g->n_events, sm.n_won);
   __syncthreads();
-  for (uint32_t q = tid; q < sm.n_won; q += nt) {
-    const uint32_t c = cix[won[q]];
-    commit_event(d, c, d.cand[c], sm.won_base + q);
-  }
+  for (uint32_t q = tid; q < sm.n_won; q += nt) commit_event(d, won[q], d.cand[won[q]], sm.won_base + q);
   __syncthreads();
   return true;
 }
@@ -1984,119 +2207,228 @@ static __device__ void phase_react_serial(const Dev& d, SerialSmem& sm, uint32_t
   products_prefix(d, sm.scan, okeys, order, order_out, pref, E, ok);
 }
 
+// Products, tallies (summed in sm) and log record of event number k (in (train, id_lo) order):
+// pair cd, first product in slot slot0 with id id0.
 template <bool F32L>
-__device__ void phase_products(const Dev& d, ProductsSmem& sm) {
-  const int tid = threadIdx.x, nt = blockDim.x;
-  const Tables& tb = *d.tables;
-  for (uint32_t b = tid; b < d.n_trains; b += nt) {
+__device__ __forceinline__ void write_event(const Dev& d, const Tables& tb, ProductsSmem& sm, const Cand& cd,
+                                            uint32_t slot0, uint32_t id0, uint32_t k) {
+  const uint32_t r = cd.rxn_train & 255u, b = cd.rxn_train >> 8;
+  const uint32_t np = static_cast<uint32_t>(tb.n_prod[r]);
+  Train& tr = d.trains[b];
+  if (slot0 + np > d.cap) {
+    raise_status(d.g, CHEM_ECAPACITY);
+    return;
+  }
+  const uint32_t tlo = tid_type(F32L ? __float_as_uint(d.s4[cd.s_lo].w) : d.stid[cd.s_lo]);
+  const uint32_t thi = tid_type(F32L ? __float_as_uint(d.s4[cd.s_hi].w) : d.stid[cd.s_hi]);
+  if (F32L) {
+    const float4 a = d.s4[cd.s_lo], c = d.s4[cd.s_hi];
+    const uint32_t ca = d.cell_sorted[cd.s_lo], cc = d.cell_sorted[cd.s_hi];
+    const int n = tr.n;
+    int ax_, ay_, az_, cx_, cy_, cz_;
+    cell_decode(ca - tr.cell_base, tr.cb, ax_, ay_, az_);
+    cell_decode(cc - tr.cell_base, tr.cb, cx_, cy_, cz_);
+    int dx = cx_ - ax_, dy = cy_ - ay_, dz = cz_ - az_;
+    // the cells of a reacting pair are at most one apart per axis (n >= 3)
+    dx = dx > 1 ? dx - n : (dx < -1 ? dx + n : dx);
+    dy = dy > 1 ? dy - n : (dy < -1 ? dy + n : dy);
+    dz = dz > 1 ? dz - n : (dz < -1 ? dz + n : dz);
+    const float w = tb.Df[tlo] / (tb.Df[tlo] + tb.Df[thi]);
+    const float px = a.x + w * (dx * tr.hf + (c.x - a.x));
+    const float py = a.y + w * (dy * tr.hf + (c.y - a.y));
+    const float pz = a.z + w * (dz * tr.hf + (c.z - a.z));
+    for (uint32_t q = 0; q < np; ++q) {
+      const uint32_t pt = static_cast<uint32_t>(tb.prod[r][q]);
+      d.s4[slot0 + q] = make_float4(px, py, pz, __uint_as_float(((id0 + q) << 3) | pt));
+      d.cell_sorted[slot0 + q] = ca;
+      d.dead[slot0 + q] = 0;
+    }
+  } else {
+    const double xa = d.sx[cd.s_lo], ya = d.sy[cd.s_lo], za = d.sz[cd.s_lo];
+    const double rx = min_image(__dsub_rn(d.sx[cd.s_hi], xa), tr.L, tr.halfL);
+    const double ry = min_image(__dsub_rn(d.sy[cd.s_hi], ya), tr.L, tr.halfL);
+    const double rz = min_image(__dsub_rn(d.sz[cd.s_hi], za), tr.L, tr.halfL);
+    const double w = __ddiv_rn(tb.D[tlo], __dadd_rn(tb.D[tlo], tb.D[thi]));
+    const double px = wrap_box(__dadd_rn(xa, __dmul_rn(w, rx)), tr.L, tr.halfL);
+    const double py = wrap_box(__dadd_rn(ya, __dmul_rn(w, ry)), tr.L, tr.halfL);
+    const double pz = wrap_box(__dadd_rn(za, __dmul_rn(w, rz)), tr.L, tr.halfL);
+    for (uint32_t q = 0; q < np; ++q) {
+      const uint32_t pt = static_cast<uint32_t>(tb.prod[r][q]);
+      d.sx[slot0 + q] = px; d.sy[slot0 + q] = py; d.sz[slot0 + q] = pz;
+      d.stid[slot0 + q] = ((id0 + q) << 3) | pt;
+      d.cell_sorted[slot0 + q] = tr.cell_base;
+      d.dead[slot0 + q] = 0;
+    }
+  }
+  atomicSub(&sm.dcount[b][tlo], 1);
+  atomicSub(&sm.dcount[b][thi], 1);
+  for (uint32_t q = 0; q < np; ++q) atomicAdd(&sm.dcount[b][tb.prod[r][q]], 1);
+  atomicAdd(&sm.devents[b][r], 1);
+  if (tb.water[r]) atomicAdd(&sm.dwater[b], tb.water[r]);
+  if (d.cap_ev_log) {
+    const uint32_t e = d.g->ev_log_n + k;
+    if (e < d.cap_ev_log) {
+      chem_event ev;
+      ev.step = tr.step; ev.rxn = static_cast<int32_t>(r); ev.id_lo = cd.id_lo; ev.id_hi = cd.id_hi;
+      ev.prod_id0 = id0; ev.n_prod = static_cast<int32_t>(np); ev.train = b; ev.reserved = 0;
+      d.ev_log[e] = ev;
+    } else {
+      raise_status(d.g, CHEM_ECAPACITY);
+    }
+  }
+}
+
+__device__ __forceinline__ void clear_products(const Dev& d, ProductsSmem& sm) {
+  for (uint32_t b = threadIdx.x; b < d.n_trains; b += blockDim.x) {
     sm.dwater[b] = 0;
     for (int q = 0; q < MAXT; ++q) sm.dcount[b][q] = 0;
     for (int q = 0; q < MAXR; ++q) sm.devents[b][q] = 0;
   }
+}
+
+// The CTA's summed tallies into the trains' records.
+__device__ __forceinline__ void add_tallies(const Dev& d, const ProductsSmem& sm) {
+  constexpr uint32_t per = MAXT + MAXR + 1;
+  for (uint32_t w = threadIdx.x; w < d.n_trains * per; w += blockDim.x) {
+    const uint32_t b = w / per;
+    const int q = static_cast<int>(w % per);
+    Train& tr = d.trains[b];
+    const int v = q < MAXT ? sm.dcount[b][q] : (q < MAXT + MAXR ? sm.devents[b][q - MAXT] : sm.dwater[b]);
+    long long* to = q < MAXT ? &tr.counts[q] : (q < MAXT + MAXR ? &tr.events[q - MAXT] : &tr.water);
+    if (v) atomicAdd(reinterpret_cast<unsigned long long*>(to), static_cast<unsigned long long>(static_cast<long long>(v)));
+  }
+}
+
+// `block` of `blocks` CTAs.
+template <bool F32L>
+__device__ void phase_products(const Dev& d, ProductsSmem& sm, uint32_t block, uint32_t blocks) {
+  const uint32_t nt = blockDim.x;
+  const Tables& tb = *d.tables;
+  clear_products(d, sm);
   const bool ok = block_status_ok(d);
   const uint32_t E = ok ? d.g->n_events : 0u;
   const uint32_t* order = d.g->ev_parity ? d.ev_v1 : d.ev_v0;
   const uint32_t* pref = d.g->ev_parity ? d.ev_k0 : d.ev_k1;
   const uint32_t n_live = d.g->n_total - d.g->n_dead;
-  for (uint32_t k = blockIdx.x * nt + tid; k < E; k += gridDim.x * nt) {
+  for (uint32_t k = block * nt + threadIdx.x; k < E; k += blocks * nt) {
     const Cand cd = d.cand[order[k] & EV_CAND_MASK];
-    const uint32_t r = cd.rxn_train & 255u, b = cd.rxn_train >> 8;
-    const uint32_t np = static_cast<uint32_t>(tb.n_prod[r]);
-    Train& tr = d.trains[b];
+    const Train& tr = d.trains[cd.rxn_train >> 8];
     const uint32_t ex = pref[k];
-    const uint32_t id0 = tr.next_id + (ex - tr.pref0);
-    const uint32_t slot0 = n_live + ex;
-    if (slot0 + np > d.cap) {
-      raise_status(d.g, CHEM_ECAPACITY);
-      continue;
-    }
-    const uint32_t tlo = tid_type(F32L ? __float_as_uint(d.s4[cd.s_lo].w) : d.stid[cd.s_lo]);
-    const uint32_t thi = tid_type(F32L ? __float_as_uint(d.s4[cd.s_hi].w) : d.stid[cd.s_hi]);
-    if (F32L) {
-      const float4 a = d.s4[cd.s_lo], c = d.s4[cd.s_hi];
-      const uint32_t ca = d.cell_sorted[cd.s_lo], cc = d.cell_sorted[cd.s_hi];
-      const int n = tr.n;
-      int ax_, ay_, az_, cx_, cy_, cz_;
-      cell_decode(ca - tr.cell_base, tr.cb, ax_, ay_, az_);
-      cell_decode(cc - tr.cell_base, tr.cb, cx_, cy_, cz_);
-      int dx = cx_ - ax_, dy = cy_ - ay_, dz = cz_ - az_;
-      // the cells of a reacting pair are at most one apart per axis (n >= 3)
-      dx = dx > 1 ? dx - n : (dx < -1 ? dx + n : dx);
-      dy = dy > 1 ? dy - n : (dy < -1 ? dy + n : dy);
-      dz = dz > 1 ? dz - n : (dz < -1 ? dz + n : dz);
-      const float w = tb.Df[tlo] / (tb.Df[tlo] + tb.Df[thi]);
-      const float px = a.x + w * (dx * tr.hf + (c.x - a.x));
-      const float py = a.y + w * (dy * tr.hf + (c.y - a.y));
-      const float pz = a.z + w * (dz * tr.hf + (c.z - a.z));
-      for (uint32_t q = 0; q < np; ++q) {
-        const uint32_t pt = static_cast<uint32_t>(tb.prod[r][q]);
-        d.s4[slot0 + q] = make_float4(px, py, pz, __uint_as_float(((id0 + q) << 3) | pt));
-        d.cell_sorted[slot0 + q] = ca;
-        d.dead[slot0 + q] = 0;
-      }
-    } else {
-      const double xa = d.sx[cd.s_lo], ya = d.sy[cd.s_lo], za = d.sz[cd.s_lo];
-      const double rx = min_image(__dsub_rn(d.sx[cd.s_hi], xa), tr.L, tr.halfL);
-      const double ry = min_image(__dsub_rn(d.sy[cd.s_hi], ya), tr.L, tr.halfL);
-      const double rz = min_image(__dsub_rn(d.sz[cd.s_hi], za), tr.L, tr.halfL);
-      const double w = __ddiv_rn(tb.D[tlo], __dadd_rn(tb.D[tlo], tb.D[thi]));
-      const double px = wrap_box(__dadd_rn(xa, __dmul_rn(w, rx)), tr.L, tr.halfL);
-      const double py = wrap_box(__dadd_rn(ya, __dmul_rn(w, ry)), tr.L, tr.halfL);
-      const double pz = wrap_box(__dadd_rn(za, __dmul_rn(w, rz)), tr.L, tr.halfL);
-      for (uint32_t q = 0; q < np; ++q) {
-        const uint32_t pt = static_cast<uint32_t>(tb.prod[r][q]);
-        d.sx[slot0 + q] = px; d.sy[slot0 + q] = py; d.sz[slot0 + q] = pz;
-        d.stid[slot0 + q] = ((id0 + q) << 3) | pt;
-        d.cell_sorted[slot0 + q] = tr.cell_base;
-        d.dead[slot0 + q] = 0;
-      }
-    }
-    atomicSub(&sm.dcount[b][tlo], 1);
-    atomicSub(&sm.dcount[b][thi], 1);
-    for (uint32_t q = 0; q < np; ++q) atomicAdd(&sm.dcount[b][tb.prod[r][q]], 1);
-    atomicAdd(&sm.devents[b][r], 1);
-    if (tb.water[r]) atomicAdd(&sm.dwater[b], tb.water[r]);
-    if (d.cap_ev_log) {
-      const uint32_t e = d.g->ev_log_n + k;
-      if (e < d.cap_ev_log) {
-        chem_event ev;
-        ev.step = tr.step; ev.rxn = static_cast<int32_t>(r); ev.id_lo = cd.id_lo; ev.id_hi = cd.id_hi;
-        ev.prod_id0 = id0; ev.n_prod = static_cast<int32_t>(np); ev.train = b; ev.reserved = 0;
-        d.ev_log[e] = ev;
-      } else {
-        raise_status(d.g, CHEM_ECAPACITY);
-      }
-    }
+    write_event<F32L>(d, tb, sm, cd, n_live + ex, tr.next_id + (ex - tr.pref0), k);
   }
   __syncthreads();
-  for (uint32_t b = 0; b < d.n_trains; ++b) {
-    Train& tr = d.trains[b];
-    for (int q = tid; q < MAXT + MAXR + 1; q += nt) {
-      if (q < MAXT) {
-        const int v = sm.dcount[b][q];
-        if (v) atomicAdd(reinterpret_cast<unsigned long long*>(&tr.counts[q]),
-                         static_cast<unsigned long long>(static_cast<long long>(v)));
-      } else if (q < MAXT + MAXR) {
-        const int v = sm.devents[b][q - MAXT];
-        if (v) atomicAdd(reinterpret_cast<unsigned long long*>(&tr.events[q - MAXT]),
-                         static_cast<unsigned long long>(static_cast<long long>(v)));
-      } else {
-        const int v = sm.dwater[b];
-        if (v) atomicAdd(reinterpret_cast<unsigned long long*>(&tr.water),
-                         static_cast<unsigned long long>(static_cast<long long>(v)));
-      }
+  add_tallies(d, sm);
+}
+
+// The whole of reaction resolution by one CTA, for steps of few accepted pairs: the rounds run
+// over all of them (no fast path and no conflict list), the winners are ordered by counting
+// the smaller keys, and each writes its products at once. One launch takes the place of four
+// whose work is a few microseconds of dependent latencies each. More accepted pairs than
+// `cap` (a crowded step) take the general phases, by this CTA alone.
+struct ReactAllSmem {
+  MatchSmem match;
+  ProductsSmem products;
+  uint32_t prods_tr[MAX_TRAINS], evs_tr[MAX_TRAINS];
+  uint32_t n_prod;
+};
+// Bytes of sbuf for steps of up to `cap` accepted pairs (the rounds and the winners' keys); a
+// crowded step uses it for its block sort and scan.
+__host__ __device__ constexpr size_t react_all_bytes(uint32_t cap) {
+  const size_t a = rc_smem_bytes(cap) + static_cast<size_t>(cap) * 8, b = sizeof(BlockSortSmem) + sizeof(ScanSmem);
+  return a > b ? a : b;
+}
+
+template <bool F32L>
+__device__ void phase_react_all(const Dev& d, ReactAllSmem& sm, uint32_t* sbuf, uint32_t cap) {
+  const int tid = threadIdx.x, nt = blockDim.x;
+  const Tables& tb = *d.tables;
+  const bool ok = block_status_ok(d);
+  Global* g = d.g;
+  const uint32_t n_c = ok ? min(g->n_cand, d.cap_cand) : 0u;
+  const uint32_t n_live = g->n_total - g->n_dead;
+  if (n_c > cap) {  // uniform
+    phase_match_fast(d, 0u, 1u);
+    __syncthreads();
+    const uint32_t n_conflict = g->n_conflict;
+    phase_match_rounds(d, sm.match);
+    const bool ok2 = block_status_ok(d);
+    const uint32_t E = ok2 ? min(g->n_events, d.cap_cand) : 0u;
+    BlockSortSmem& sort = *reinterpret_cast<BlockSortSmem*>(sbuf);
+    ScanSmem& scan = *reinterpret_cast<ScanSmem*>(sbuf + sizeof(BlockSortSmem) / 4);
+    const int p = block_sort_pairs(d.ev_k0, d.ev_v0, d.ev_k1, d.ev_v1, E, sort);
+    if (tid == 0 && ok2) {  // branch record (read by chem_get_stats)
+      g->ev_parity = static_cast<uint32_t>(p);
+      g->react_rounds_global += n_conflict > 0u ? 1u : 0u;
+      g->react_order_global += 1u;
+      g->max_conflict = max(g->max_conflict, n_conflict);
+      g->pairs_accepted += n_c;
+      g->max_events = max(g->max_events, E);
     }
+    products_prefix(d, scan, p ? d.ev_k1 : d.ev_k0, p ? d.ev_v1 : d.ev_v0, nullptr, p ? d.ev_k0 : d.ev_k1, E, ok2);
+    phase_products<F32L>(d, sm.products, 0u, 1u);
+    __syncthreads();
+    return;
   }
+  clear_products(d, sm.products);
+  for (uint32_t b = tid; b < d.n_trains; b += nt) { sm.prods_tr[b] = 0u; sm.evs_tr[b] = 0u; }
+  if (tid == 0) sm.n_prod = 0u;
+  __syncthreads();
+  uint32_t E = 0u;
+  if (n_c) {
+    const uint32_t* won = match_rounds_in_smem(d, sm.match, sbuf, n_c, nullptr);
+    E = sm.match.n_won;
+    uint32_t* key = sbuf + rc_smem_bytes(cap) / 4;  // winners' (train, id_lo) keys and
+    uint32_t* np = key + cap;                       // product counts | train << 8
+    for (uint32_t q = tid; q < E; q += nt) {
+      const Cand cd = d.cand[won[q]];
+      const uint32_t b = cd.rxn_train >> 8, n = static_cast<uint32_t>(tb.n_prod[cd.rxn_train & 255u]);
+      key[q] = event_key(d, cd);
+      np[q] = n | (b << 8);
+      atomicAdd(&sm.prods_tr[b], n);
+      atomicAdd(&sm.evs_tr[b], 1u);
+      atomicAdd(&sm.n_prod, n);
+      d.dead[cd.s_lo] = 1;
+      d.dead[cd.s_hi] = 1;
+    }
+    __syncthreads();
+    for (uint32_t q = tid; q < E; q += nt) {
+      const uint32_t mine = key[q], b = np[q] >> 8;
+      uint32_t rank = 0, before = 0, before_tr = 0;
+      for (uint32_t o = 0; o < E; ++o) {
+        const bool less = key[o] < mine;
+        const uint32_t n = less ? np[o] : 0xFFFFFF00u;
+        rank += less ? 1u : 0u;
+        before += n & 255u;
+        before_tr += (n >> 8) == b ? (n & 255u) : 0u;
+      }
+      write_event<F32L>(d, tb, sm.products, d.cand[won[q]], n_live + before, d.trains[b].next_id + before_tr, rank);
+    }
+    __syncthreads();
+    add_tallies(d, sm.products);
+  }
+  for (uint32_t b = tid; b < d.n_trains; b += nt) {
+    d.trains[b].prods_step = sm.prods_tr[b];
+    d.trains[b].n_events_step = sm.evs_tr[b];
+  }
+  if (tid == 0 && ok) {
+    g->n_events = E;
+    g->n_products = sm.n_prod;
+    g->pairs_accepted += n_c;
+    g->max_events = max(g->max_events, E);
+    if (n_c) g->max_conflict = max(g->max_conflict, sm.match.n_conflict);
+  }
+  __syncthreads();
 }
 
 static __device__ void phase_end_step(const Dev& d, EndSmem& sm) {
   const int tid = threadIdx.x, nt = blockDim.x;
-  if (tid == 0) sm.any = 0;
+  if (tid == 0) { sm.any = 0; sm.stepped = 0; }
   const bool ok = block_status_ok(d);
   const Tables& tb = *d.tables;
   for (uint32_t b = tid; b < d.n_trains; b += nt) {
     Train& tr = d.trains[b];
     if (tr.active && ok) {
+      atomicOr(&sm.stepped, 1u);
       tr.next_id += tr.prods_step;
       tr.species_steps += tr.n_live_step;
       if (d.cap_step_log) {
@@ -2122,9 +2454,7 @@ static __device__ void phase_end_step(const Dev& d, EndSmem& sm) {
   }
   __syncthreads();
   if (tid == 0) {
-    bool stepped = false;
-    for (uint32_t b = 0; b < d.n_trains; ++b) stepped |= d.trains[b].active != 0;
-    if (ok && stepped) d.g->steps_active += 1;
+    if (sm.stepped) d.g->steps_active += 1;
     if (ok) {
       const uint32_t n_live = d.g->n_total - d.g->n_dead;
       d.g->n_total = n_live + d.g->n_products;

@@ -38,6 +38,11 @@ constexpr int S4_SPARE = 8;       // spare entries of s4 past its end: the searc
 constexpr int SORT_TILE_MIN = PERSIST_THREADS * SORT_ITEMS;
 constexpr int REACT_THREADS = 1024;
 constexpr int ITEM_HOME = 32;   // most home species per pair-search work item (one cell)
+// Contexts of at most this many species run a step as few launches (one search kernel, one
+// kernel for reaction resolution and the step's end): at 2,000 to 140,000 species reaction
+// resolution to the next begin took 22 to 33 us as four kernels and takes 10 to 24 as one; the
+// 1e6-species benchmark has up to 6,800 events a step, more than one CTA should order.
+constexpr long long SMALL_SPECIES = 1ll << 18;
 constexpr int N_FWD = 14;       // own cell + 13 forward neighbour cells (half shell)
 constexpr double END_SLACK = 1.0 + 1e-6;    // last-step trim slack (relative)
 constexpr float CELL_SLACK_F = 1.0001f;    // hash cell >= cutoff * CELL_SLACK_F
@@ -82,6 +87,7 @@ struct Train {
   double t, t_end, dt_cur, t_last_release;
   uint32_t step, next_id;
   uint32_t p_head, p_tail; // pending queue [p_head, p_tail) relative to pend_base
+  double next_arr;         // arrival of its first species (infinity when empty)
   long long species_steps, water;
   long long counts[MAXT];
   long long events[MAXR];

@@ -132,30 +132,7 @@ __device__ void phase_search_cells(const Dev& d, ScSmem<W>& sm) {
         float rcmax2 = -1.f;
 #pragma unroll
         for (int u = 0; u < MAXT; ++u) rcmax2 = fmaxf(rcmax2, w.ct[t * MAXT + u]);
-        rcmax2 *= 1.0001f;
-        // a forward cell whose nearest point is farther from the home than its largest
-        // cutoff holds no partner (gaps taken 1e-5 of a cell short: no rounding drops one)
-        const float eps = 1e-5f * hf;
-        auto gap = [&](int o, float of) {
-          const float g = o > 0 ? static_cast<float>(o) * hf - of : (o < 0 ? of + static_cast<float>(-o - 1) * hf : 0.f);
-          return fmaxf(g - eps, 0.f);
-        };
-        // per axis the gap is 0 (same layer), the distance to the lower face (offset -1)
-        // or to the upper face (offset +1); the 13 offsets unrolled
-        const float xm = gap(-1, v.x), xp = gap(1, v.x), ym = gap(-1, v.y), yp = gap(1, v.y);
-        const float zp = gap(1, v.z);
-        const float xm2 = xm * xm, xp2 = xp * xp, ym2 = ym * ym, yp2 = yp * yp, zp2 = zp * zp;
-        uint32_t kr = 0u;
-#pragma unroll
-        for (int k = 1; k < N_FWD; ++k) {
-          int dx, dy, dz;
-          fwd_offset(k, dx, dy, dz);
-          const float sx = dx < 0 ? xm2 : (dx > 0 ? xp2 : 0.f);
-          const float sy = dy < 0 ? ym2 : (dy > 0 ? yp2 : 0.f);
-          const float sz = dz > 0 ? zp2 : 0.f;
-          if ((sx + sy) + sz <= rcmax2) kr |= 1u << k;
-        }
-        km |= kr & occ_mask;
+        km |= cells_in_reach(v, hf, rcmax2) & occ_mask;
       }
     }
     // a 32 x 32 bit transpose of (lane = home; bits 0..13 the half-shell cells it
