@@ -98,9 +98,10 @@ typedef struct chem_config {
   int64_t capacity_step_log;   /* >0: keep up to this many per-step records            */
   int32_t cells_per_axis_max;  /* spatial-hash resolution limit; 0 = automatic         */
   int32_t steps_per_launch;    /* steps per captured graph replay; 0 = automatic       */
-  int32_t launch_mode;         /* CHEM_LAUNCH_AUTO: persistent for batches, one kernel
-                                  per phase otherwise; CHEM_LAUNCH_PHASES;
-                                  CHEM_LAUNCH_PERSISTENT (cooperative, grid barriers)  */
+  int32_t launch_mode;         /* CHEM_LAUNCH_AUTO: by the number of species, persistent up
+                                  to some 260,000 and one kernel per phase beyond;
+                                  CHEM_LAUNCH_PHASES; CHEM_LAUNCH_PERSISTENT (many steps
+                                  per launch, CTAs resident together with barriers)    */
   void* cuda_stream;           /* cudaStream_t to run on; NULL = library-owned stream  */
   chem_alloc_fn dev_alloc;     /* NULL = cudaMalloc / cudaFree                         */
   chem_free_fn dev_free;
@@ -281,9 +282,11 @@ typedef struct chem_stats {
   int64_t phase_launches[8];/* kernel launches per phase behind phase_ms               */
   /* Which branches reaction resolution took (device counters, summed over resets). The
    * conflict rounds run in shared memory for up to 1,536 conflicting accepted pairs and
-   * in global memory beyond (always in the persistent kernel); the events of a step are
+   * in global memory beyond; the events of a step are
    * ordered in shared memory for up to 8,192 events (bucket sort, or a block radix sort
-   * when the keys cluster) and in global memory beyond. The results do not depend on the
+   * when the keys cluster) and in global memory beyond. Single trains of at most 262,144
+   * species and the persistent launches resolve up to 1,536 (persistent: 1,024) accepted
+   * pairs of a step at once in shared memory. The results do not depend on the
    * branch; these counters let tests show that each branch ran. */
   int64_t react_rounds_global;  /* steps whose conflict rounds ran in global memory     */
   int64_t react_order_global;   /* steps whose event order ran in global memory         */

@@ -64,6 +64,13 @@ struct PendingHost {
   void release() { buf[0].release(); buf[1].release(); n = 0; }
 };
 
+// Launch form by the species the next steps will work on. 64 steps of a uniform mixture and
+// whole track trajectories, ms as one cluster / one CTA per SM / per-phase kernels:
+//   2,000 species 2.04 / 2.19 / 3.36, 4,000 2.96 / 2.76 / 4.12, 32,000 7.1 / 4.3 / 5.2,
+//   200,000 - / 9.7 / 10.2; tracks 32,000 14.8 / 6.9 / 8.1, 176,000 - / 17.3 / 19.4.
+constexpr uint32_t CLUSTER_SPECIES = 2560;
+constexpr uint32_t GRID_SPECIES = 1u << 18;
+
 struct TrainHost {
   chem_config cfg;
   double E_dep = 0.0;
@@ -86,11 +93,11 @@ struct chem_ctx {
   chem_free_fn dfree = nullptr;
   void* alloc_user = nullptr;
   std::vector<std::pair<void*, size_t>> allocs;
-  cudaGraphExec_t graph = nullptr;
+  cudaGraphExec_t graph = nullptr;  // the per-phase form
   int graph_steps = 0;
   bool graph_events = false;  // the captured graph records the phase events
-  int steps_per_launch = 16;
-  bool persistent = false;
+  int steps_per_launch = 0;   // 0: automatic
+  int launch_mode = CHEM_LAUNCH_AUTO;
   int cell_factor_x100 = 1600;  // hash cells per species (x100) of the runtime grid limit
   // radix passes of the cell sort: with one train only as many as the runtime grid limit
   // needs (pass_nmax cells per axis at most, and pass_cbref bits per axis for the cells
@@ -332,7 +339,6 @@ void init_train_dynamic(Train& t, const chem_config& c, int n_max) {
 // end-and-next-begin) kernel; small contexts have one search kernel and one kernel for all
 // that follows it.
 int kernels_per_step(const chem_ctx* ctx) {
-  if (ctx->persistent) return 0;
   return ctx->lc.small ? 4 + ctx->d.passes : 6 + ctx->d.passes + (ctx->lc.search_tps == 2 ? 2 : 1);
 }
 
@@ -344,16 +350,39 @@ int sort_passes(const chem_ctx* ctx) {
   return std::max(1, std::min(ctx->passes_alloc, (3 * cb + 7) / 8));
 }
 
-chem_status capture_graph(chem_ctx* ctx) {
+// Launch form of the next steps, which will work on n species.
+enum Form { FORM_PHASES, FORM_GRID, FORM_CLUSTER };
+Form choose_form(const chem_ctx* ctx, uint32_t n) {
+  if (ctx->launch_mode == CHEM_LAUNCH_PHASES) return FORM_PHASES;
+  if (ctx->launch_mode == CHEM_LAUNCH_AUTO && (ctx->profiling || n > GRID_SPECIES)) return FORM_PHASES;
+  return ctx->lc.cluster_blocks > 0 && n <= CLUSTER_SPECIES ? FORM_CLUSTER : FORM_GRID;
+}
+
+constexpr int AUTO_STEPS = 16;
+int steps_of(const chem_ctx* ctx, Form f) {
+  if (ctx->steps_per_launch > 0) return ctx->steps_per_launch;
+  return f == FORM_PHASES ? AUTO_STEPS : 8 * AUTO_STEPS;  // (the persistent kernel ends by itself)
+}
+
+// Drops the captured graph after a change of what it holds.
+void drop_graph(chem_ctx* ctx) {
+  if (ctx->graph) cudaGraphExecDestroy(ctx->graph);
+  ctx->graph = nullptr;
+  ctx->graph_events = false;
+}
+
+// Sort passes and search kernels of the next launches.
+void set_launch_params(chem_ctx* ctx) {
   ctx->lc.search_tps = ctx->item_home == 0 ? 1 : (ctx->item_home > 0 ? 0 : 2);
   ctx->d.passes = sort_passes(ctx);
-  if (ctx->graph) {
-    cudaGraphExecDestroy(ctx->graph);
-    ctx->graph = nullptr;
-  }
-  ctx->graph_events = false;
-  const size_t n_ev = (ctx->profiling && !ctx->persistent)
-                          ? static_cast<size_t>(ctx->steps_per_launch) * 2 * N_PHASES : 0;
+}
+
+// Captures the per-phase form.
+chem_status capture_graph(chem_ctx* ctx) {
+  set_launch_params(ctx);
+  drop_graph(ctx);
+  const int steps = steps_of(ctx, FORM_PHASES);
+  const size_t n_ev = ctx->profiling ? static_cast<size_t>(steps) * 2 * N_PHASES : 0;
   while (ctx->events.size() < n_ev) {
     cudaEvent_t e;
     CK(cudaEventCreate(&e));
@@ -362,17 +391,11 @@ chem_status capture_graph(chem_ctx* ctx) {
   cudaGraph_t g = nullptr;
   CK(cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
   cudaError_t e = cudaSuccess;
-  if (ctx->persistent) {
-    e = ctx->precision == CHEM_FP64
-            ? enqueue_persistent_f64(ctx->d, ctx->lc, ctx->steps_per_launch, ctx->stream)
-            : enqueue_persistent_f32l(ctx->d, ctx->lc, ctx->steps_per_launch, ctx->stream);
-  } else {
-    for (int s = 0; s < ctx->steps_per_launch && e == cudaSuccess; ++s) {
-      cudaEvent_t* ev = n_ev ? &ctx->events[static_cast<size_t>(s) * 2 * N_PHASES] : nullptr;
-      const bool first = s == 0, last = s + 1 == ctx->steps_per_launch;
-      e = ctx->precision == CHEM_FP64 ? enqueue_step_f64(ctx->d, ctx->lc, ctx->stream, ev, first, last)
-                                      : enqueue_step_f32l(ctx->d, ctx->lc, ctx->stream, ev, first, last);
-    }
+  for (int s = 0; s < steps && e == cudaSuccess; ++s) {
+    cudaEvent_t* ev = n_ev ? &ctx->events[static_cast<size_t>(s) * 2 * N_PHASES] : nullptr;
+    const bool first = s == 0, last = s + 1 == steps;
+    e = ctx->precision == CHEM_FP64 ? enqueue_step_f64(ctx->d, ctx->lc, ctx->stream, ev, first, last)
+                                    : enqueue_step_f32l(ctx->d, ctx->lc, ctx->stream, ev, first, last);
   }
   cudaError_t e2 = cudaStreamEndCapture(ctx->stream, &g);
   if (e != cudaSuccess) {
@@ -383,8 +406,26 @@ chem_status capture_graph(chem_ctx* ctx) {
   e = cudaGraphInstantiate(&ctx->graph, g, 0);
   cudaGraphDestroy(g);
   CK(e);
-  ctx->graph_steps = ctx->steps_per_launch;
+  ctx->graph_steps = steps;
   ctx->graph_events = n_ev > 0;
+  return CHEM_OK;
+}
+
+// Queues the next steps in the form f.
+chem_status launch_steps(chem_ctx* ctx, Form f) {
+  if (f == FORM_PHASES) {
+    if (!ctx->graph) {
+      chem_status s = capture_graph(ctx);
+      if (s) return s;
+    }
+    CK(cudaGraphLaunch(ctx->graph, ctx->stream));
+    return CHEM_OK;
+  }
+  set_launch_params(ctx);
+  const bool cluster = f == FORM_CLUSTER;
+  CK(ctx->precision == CHEM_FP64
+         ? enqueue_steps_f64(ctx->d, ctx->lc, cluster, steps_of(ctx, f), steps_of(ctx, FORM_PHASES), ctx->stream)
+         : enqueue_steps_f32l(ctx->d, ctx->lc, cluster, steps_of(ctx, f), steps_of(ctx, FORM_PHASES), ctx->stream));
   return CHEM_OK;
 }
 
@@ -394,32 +435,34 @@ chem_status check_ctx(chem_ctx* ctx) {
 }
 
 chem_status run_loop(chem_ctx* ctx) {
-  if (!ctx->graph) {
-    chem_status s = capture_graph(ctx);
-    if (s) return s;
-  }
   {
     chem_status s0 = download_global(ctx);
     if (s0) return s0;
   }
   uint32_t active_before = ctx->g_pinned->steps_active;
   for (long long it = 0;; ++it) {
-    CK(cudaGraphLaunch(ctx->graph, ctx->stream));
+    const Form form = choose_form(ctx, ctx->g_pinned->n_ahead);
+    chem_status ls = launch_steps(ctx, form);
+    if (ls) return ls;
     CK(cudaMemcpyAsync(ctx->g_pinned, ctx->d.g, sizeof(Global), cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
     const Global& g = *ctx->g_pinned;
     note_device_counters(ctx, g);
-    ctx->stats.graph_replays += 1;
-    ctx->stats.steps_launched += ctx->graph_steps;
-    // per replay: one begin kernel, then every step's kernels (the end kernel of each step
-    // but the last also begins the next)
-    ctx->stats.kernel_launches += ctx->persistent ? 1 : 1 + static_cast<int64_t>(ctx->graph_steps) * kernels_per_step(ctx);
     ctx->stats.bytes_d2h += sizeof(Global);
     const uint32_t stepped = g.steps_active - active_before;
     active_before = g.steps_active;
-    if (ctx->persistent) {
+    if (form != FORM_PHASES) {
+      ctx->stats.steps_launched += stepped;
+      ctx->stats.kernel_launches += 1;
       ctx->stats.phase_launches[PH_PERSISTENT] += 1;
-    } else if (ctx->graph_events) {
+    } else {
+      // per replay: one begin kernel, then every step's kernels (the end kernel of each step
+      // but the last also begins the next)
+      ctx->stats.graph_replays += 1;
+      ctx->stats.steps_launched += ctx->graph_steps;
+      ctx->stats.kernel_launches += 1 + static_cast<int64_t>(ctx->graph_steps) * kernels_per_step(ctx);
+    }
+    if (form == FORM_PHASES && ctx->graph_events) {
       for (uint32_t st = 0; st < stepped && st < static_cast<uint32_t>(ctx->graph_steps); ++st) {
         for (int ph = 0; ph < PH_PERSISTENT; ++ph) {
           float ms = 0.f;
@@ -780,8 +823,7 @@ chem_status chem_batch_init(const chem_config* cfgs, int32_t n_trains, chem_ctx*
     delete ctx;
     return CHEM_EINVAL;
   }
-  ctx->persistent = c0.launch_mode == CHEM_LAUNCH_PERSISTENT ||
-                    (c0.launch_mode == CHEM_LAUNCH_AUTO && n_trains > 1);
+  ctx->launch_mode = c0.launch_mode;
 
   // ---- chemistry tables
   Tables& T = ctx->tables;
@@ -811,6 +853,8 @@ chem_status chem_batch_init(const chem_config* cfgs, int32_t n_trains, chem_ctx*
     T.water[r] = x.water_delta;
     T.rxn_a[r] = x.a;
     T.rxn_b[r] = x.b;
+    T.w_ab[r][0] = T.D[x.a] / (T.D[x.a] + T.D[x.b]);
+    T.w_ab[r][1] = T.D[x.b] / (T.D[x.b] + T.D[x.a]);
     T.k_tab[r] = x.k_tab;
   }
 
@@ -907,13 +951,13 @@ chem_status chem_batch_init(const chem_config* cfgs, int32_t n_trains, chem_ctx*
     *out = ctx;
     return fail(ctx, CHEM_ECUDA, "no usable CUDA device");
   }
-  int sort_occ = 0, pers_occ = 0;
+  int sort_occ = 0, pers_occ = 0, cluster = 0;
   if (sort_pass_occupancy(&sort_occ) != cudaSuccess || sort_occ < 1) {
     *out = ctx;
     return fail(ctx, CHEM_ECUDA, "sort kernel not loadable: %s", cudaGetErrorString(cudaGetLastError()));
   }
-  cudaError_t pe = ctx->precision == CHEM_FP64 ? persistent_occupancy_f64(&pers_occ)
-                                               : persistent_occupancy_f32l(&pers_occ);
+  cudaError_t pe = ctx->precision == CHEM_FP64 ? step_kernel_limits_f64(&pers_occ, &cluster)
+                                               : step_kernel_limits_f32l(&pers_occ, &cluster);
   if (pe != cudaSuccess || pers_occ < 1) {
     *out = ctx;
     return fail(ctx, CHEM_ECUDA, "step kernel not loadable: %s", cudaGetErrorString(pe));
@@ -921,7 +965,8 @@ chem_status chem_batch_init(const chem_config* cfgs, int32_t n_trains, chem_ctx*
   ctx->lc.stream_blocks = ctx->sms * 4;
   ctx->lc.search_blocks = ctx->sms * 4;  // resident CTAs (launch bounds 256 x 4); items are stolen
   ctx->lc.sort_blocks = ctx->sms * sort_occ;
-  ctx->lc.persistent_blocks = ctx->sms * pers_occ;
+  ctx->lc.persistent_blocks = ctx->sms;
+  ctx->lc.cluster_blocks = cluster;
   ctx->lc.small = n_trains == 1 && cap <= static_cast<uint64_t>(SMALL_SPECIES) ? 1 : 0;
 
   // ---- device allocations
@@ -1235,7 +1280,8 @@ chem_status chem_set_profiling(chem_ctx* ctx, int32_t on) {
     ctx->stats.phase_ms[i] = 0.0;
     ctx->stats.phase_launches[i] = 0;
   }
-  return capture_graph(ctx);
+  drop_graph(ctx);
+  return ctx->launch_mode == CHEM_LAUNCH_PHASES ? capture_graph(ctx) : CHEM_OK;
 }
 
 chem_status chem_autotune(chem_ctx* ctx, double budget_ms, int32_t* chosen) {
@@ -1292,9 +1338,10 @@ chem_status chem_autotune(chem_ctx* ctx, double budget_ms, int32_t* chosen) {
   for (int nm : {n_alloc, (3 * n_alloc) / 4, n_alloc / 2 - 1, (2 * n_alloc) / 5}) n_cands.push_back(std::max(3, nm));
   const int ih_cands[1] = {ctx->item_home};
   const int spl_cands[2] = {8, 32};
-  const bool mode_cands[2] = {false, true};  // per-phase graph, persistent launch
-  const bool saved_persistent = ctx->persistent;
-  bool best_persistent = saved_persistent;
+  const int mode_cands[2] = {CHEM_LAUNCH_PHASES, CHEM_LAUNCH_PERSISTENT};
+  const int saved_mode = ctx->launch_mode;
+  int best_mode = saved_mode;
+  const uint32_t n_ahead = ctx->g_pinned->n_ahead;
   cudaEvent_t e0, e1;
   CK(cudaEventCreate(&e0));
   CK(cudaEventCreate(&e1));
@@ -1307,10 +1354,11 @@ chem_status chem_autotune(chem_ctx* ctx, double budget_ms, int32_t* chosen) {
   // each trial's graph sorts the key bits its grid limit needs
   ctx->pass_cbref = tr0[0].n_ref != 0 ? tr0[0].cb_ref : 0;
   for (int combo = 0; combo < 4; ++combo) {
-    const bool pers = mode_cands[combo / 2];
+    const int mode = mode_cands[combo / 2];
     const int spl = spl_cands[combo % 2];
     const int ih = ih_cands[0];
-    ctx->persistent = pers;
+    ctx->launch_mode = mode;
+    const Form form = choose_form(ctx, n_ahead);
     ctx->steps_per_launch = spl;
     ctx->item_home = ih;  // selects the search kernel of the captured graph
     {
@@ -1327,7 +1375,8 @@ chem_status chem_autotune(chem_ctx* ctx, double budget_ms, int32_t* chosen) {
         s = upload_trains(ctx, tr);
         if (s) break;
         ctx->pass_nmax = tr[0].n_max;
-        s = capture_graph(ctx);
+        drop_graph(ctx);
+        if (form == FORM_PHASES) s = capture_graph(ctx);
         if (s) break;
         Global& gfix = *ctx->g_pinned;
         CK(cudaMemcpyAsync(&gfix, d.g, sizeof(Global), cudaMemcpyDeviceToHost, ctx->stream));
@@ -1337,9 +1386,11 @@ chem_status chem_autotune(chem_ctx* ctx, double budget_ms, int32_t* chosen) {
         CK(cudaMemcpyAsync(d.g, &gfix, sizeof(Global), cudaMemcpyHostToDevice, ctx->stream));
         CK(cudaStreamSynchronize(ctx->stream));
         const int reps = std::max(1, 24 / spl);
-        CK(cudaGraphLaunch(ctx->graph, ctx->stream));  // settle
+        s = launch_steps(ctx, form);  // settle
+        if (s) break;
         CK(cudaEventRecord(e0, ctx->stream));
-        for (int r = 0; r < reps; ++r) CK(cudaGraphLaunch(ctx->graph, ctx->stream));
+        for (int r = 0; r < reps && !s; ++r) s = launch_steps(ctx, form);
+        if (s) break;
         CK(cudaEventRecord(e1, ctx->stream));
         CK(cudaMemcpyAsync(ctx->g_pinned, d.g, sizeof(Global), cudaMemcpyDeviceToHost, ctx->stream));
         CK(cudaStreamSynchronize(ctx->stream));
@@ -1359,7 +1410,7 @@ chem_status chem_autotune(chem_ctx* ctx, double budget_ms, int32_t* chosen) {
         // the timed part by counting the timed replays' share
         const double timed_frac = static_cast<double>(reps) / (reps + 1);
         const double rate = ms > 0.f ? (static_cast<double>(ss - [&] { long long z = 0; for (int b = 0; b < ctx->B; ++b) z += tr0[b].species_steps; return z; }()) * timed_frac) / (ms * 1e-3) : 0.0;
-        if (rate > best_rate) { best_rate = rate; best_n = nm; best_ih = ih; best_spl = spl; best_persistent = pers; }
+        if (rate > best_rate) { best_rate = rate; best_n = nm; best_ih = ih; best_spl = spl; best_mode = mode; }
       }
     }
     if (s) break;
@@ -1396,15 +1447,16 @@ chem_status chem_autotune(chem_ctx* ctx, double budget_ms, int32_t* chosen) {
   if (s2) return s2;
   ctx->item_home = best_ih;
   ctx->steps_per_launch = best_rate > 0.0 ? best_spl : saved_spl;
-  ctx->persistent = best_rate > 0.0 ? best_persistent : saved_persistent;
+  ctx->launch_mode = best_rate > 0.0 ? best_mode : saved_mode;
   ctx->profiling = saved_prof;
-  s = capture_graph(ctx);
+  drop_graph(ctx);
+  if (ctx->launch_mode == CHEM_LAUNCH_PHASES) s = capture_graph(ctx);
   if (s) return s;
   if (chosen) {
-    chosen[0] = ctx->steps_per_launch;
+    chosen[0] = steps_of(ctx, FORM_PHASES);
     chosen[1] = best_n;
     chosen[2] = best_ih;
-    chosen[3] = ctx->persistent ? CHEM_LAUNCH_PERSISTENT : CHEM_LAUNCH_PHASES;
+    chosen[3] = ctx->launch_mode == CHEM_LAUNCH_PERSISTENT ? CHEM_LAUNCH_PERSISTENT : CHEM_LAUNCH_PHASES;
   }
   return ctx->status;
 }
@@ -1429,8 +1481,9 @@ chem_status chem_set_tuning(chem_ctx* ctx, const int32_t* tuning) {
   if (s) return s;
   ctx->item_home = ih;
   ctx->steps_per_launch = spl;
-  ctx->persistent = mode == CHEM_LAUNCH_PERSISTENT;
-  s = capture_graph(ctx);
+  ctx->launch_mode = mode;
+  drop_graph(ctx);
+  if (mode == CHEM_LAUNCH_PHASES) s = capture_graph(ctx);
   if (s) return s;
   return ctx->status;
 }

@@ -1,64 +1,24 @@
 // Kernels of one SBS step: one kernel per phase (captured into a CUDA graph of several
-// steps), and a persistent cooperative kernel that runs the same phases for several
-// steps of every train with grid barriers in between.
+// steps), and a kernel that runs the same phases for several steps of every train with
+// barriers in between.
 #pragma once
+#include <type_traits>
+
 #include "launch.h"
 #include "phases.cuh"
 #include "search_cells.cuh"
 
 namespace chem {
 
-union PhaseSmem {
-  BeginSmem begin;
-  SerialSmem serial;
-  ProductsSmem products;
-  EndSmem end;
-  ScSmem<8> cells;
-  TpsSmem<true, 8> tps32;
-  TpsSmem<false, 8> tps64;
-  uint32_t hist[MAX_PASSES][RADIX];
-  SortSmemP sort;
-};
-
-// Grid-wide barrier of the persistent kernel. The wait is bounded: past the limit the
-// kernel raises CHEM_ETIMEOUT, and once any error is raised the barrier stops waiting
-// (every phase then skips its work), so a launch always ends.
-__device__ __forceinline__ void grid_sync(const Dev& d) {
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    Global* g = d.g;
-    const uint32_t gen = ld_acquire_u32(&g->bar_gen);
-    __threadfence();
-    const uint32_t arrived = atomicAdd(&g->bar_count, 1u) + 1u;
-    if (arrived == gridDim.x) {
-      g->bar_count = 0;
-      __threadfence();
-      atomicAdd(&g->bar_gen, 1u);
-    } else {
-      const long long t0 = clock64();
-      while (ld_acquire_u32(&g->bar_gen) == gen) {
-        if (*reinterpret_cast<volatile int*>(&g->status) != 0) break;
-        if (clock64() - t0 > SPIN_LIMIT_CYCLES) {
-          raise_status(g, CHEM_ETIMEOUT);
-          break;
-        }
-        __nanosleep(32);
-      }
-    }
-    __threadfence();
-  }
-  __syncthreads();
-}
-
 template <bool F32L>
 __global__ void __launch_bounds__(256) k_diffuse(const __grid_constant__ Dev d) {
   __shared__ uint32_t hist[MAX_PASSES][RADIX];
-  phase_diffuse<F32L>(d, hist);
+  phase_diffuse<F32L>(d, hist, whole_grid());
 }
 
 template <bool F32L>
 __global__ void __launch_bounds__(256) k_gather(const __grid_constant__ Dev d) {
-  phase_gather<F32L>(d);
+  phase_gather<F32L>(d, whole_grid());
 }
 
 template <bool F32L>
@@ -111,9 +71,11 @@ __global__ void __launch_bounds__(256) k_products(const __grid_constant__ Dev d)
 
 // Reaction resolution, the step's end and (begin_next) the next step's begin, one CTA.
 struct alignas(16) ReactEndSmem {
-  ReactAllSmem react;
+  union {
+    ReactAllSmem react;
+    BeginSmem begin;
+  };
   EndSmem end;
-  BeginSmem begin;
 };
 constexpr int REACT_END_THREADS = 512;
 constexpr size_t REACT_END_BYTES = sizeof(ReactEndSmem) + react_all_bytes(RC_CAP);
@@ -124,45 +86,141 @@ template <bool F32L>
 __global__ void __launch_bounds__(REACT_END_THREADS) k_react_end(const __grid_constant__ Dev d, int begin_next) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   ReactEndSmem& sm = *reinterpret_cast<ReactEndSmem*>(smem_raw);
-  phase_react_all<F32L>(d, sm.react, reinterpret_cast<uint32_t*>(smem_raw + sizeof(ReactEndSmem)), RC_CAP);
+  phase_react_all<F32L>(d, sm.react, reinterpret_cast<uint32_t*>(smem_raw + sizeof(ReactEndSmem)), RC_CAP,
+                        *d.tables);
   phase_end_step(d, sm.end);
   if (begin_next) phase_begin(d, sm.begin);
+  else phase_look_ahead(d, sm.end);
 }
 
-template <bool F32L>
-__global__ void __launch_bounds__(PERSIST_THREADS) k_persistent(const __grid_constant__ Dev d, int n_steps) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  PhaseSmem& sm = *reinterpret_cast<PhaseSmem*>(smem_raw);
-  if (blockIdx.x == 0) phase_begin(d, sm.begin);
-  grid_sync(d);
-  for (int step = 0; step < n_steps; ++step) {
-    phase_diffuse<F32L>(d, sm.hist);  // includes the release
-    grid_sync(d);
-    for (int p = 0; p < d.passes; ++p) {
-      phase_sort_pass(d, p, sm.sort);
-      grid_sync(d);
+// ---- several steps in one launch
+// The steps of few species are launches and latency: seven to eleven kernels, each a chain of a
+// few dependent L2 accesses. Here CTAs that are resident together run the phases of many steps
+// with a barrier in between: 16 CTAs of one cluster with the hardware's cluster barrier for a
+// few thousand species, or one CTA per SM with a barrier in global memory. The search gives
+// every home at least two lanes; reaction resolution, the step's end and the next step's
+// begin are CTA 0's. A launch ends by itself when no train has anything left to do. A step of
+// 2,000 species takes 27 to 30 us (as kernels 52 to 60), of 32,000 track species 73 (105);
+// at 31,000 species the sort takes 19 us, the search 13 to 35, reaction resolution 10.
+constexpr int STEP_WARPS = PERSIST_THREADS / 32;
+constexpr uint32_t STEP_REACT_CAP = 1024;  // accepted pairs of a step resolved in shared memory
+
+union StepSmem {
+  uint32_t hist[MAX_PASSES][RADIX];
+  SortSmemP sort;
+  struct { SortOneSmem one; BlockSortSmem bs; ScanSmem ss; } sort_one;
+  GrpSmem<STEP_WARPS> grp;
+  ScSmem<STEP_WARPS> cells;
+  struct {
+    PlanSmem plan;
+    ReactAllSmem react;
+    EndSmem end;
+    alignas(16) uint32_t sbuf[react_all_bytes(STEP_REACT_CAP) / 4];
+  } react;
+};
+static_assert(sizeof(StepSmem) <= 200 * 1024, "shared memory of one CTA");
+
+// Barrier over all CTAs of a cooperative launch: arrivals are counted up over the whole launch
+// (the last CTA to leave clears the count). The wait is bounded: past the limit CHEM_ETIMEOUT is
+// raised and this CTA waits no more, so a launch always ends.
+struct GridBarrier {
+  uint32_t target = 0;
+  bool broken = false;
+  __device__ __forceinline__ void sync(const Dev& d) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      target += gridDim.x;
+      __threadfence();
+      atomicAdd(&d.g->bar_count, 1u);
+      if (!broken) {
+        const long long t0 = clock64();
+        while (static_cast<int32_t>(ld_acquire_u32(&d.g->bar_count) - target) < 0) {
+          if (clock64() - t0 > SPIN_LIMIT_CYCLES) {
+            raise_status(d.g, CHEM_ETIMEOUT);
+            broken = true;
+            break;
+          }
+        }
+      }
+      __threadfence();
     }
-    phase_gather<F32L>(d);
-    grid_sync(d);
-    if (d.g->search_cells_now) {
-      phase_search_cells<F32L, 8>(d, sm.cells);
-    } else {
-      if constexpr (F32L) phase_search_tps<true, 8>(d, sm.tps32);
-      else phase_search_tps<false, 8>(d, sm.tps64);
-    }
-    grid_sync(d);
-    phase_match_fast(d, blockIdx.x, gridDim.x);
-    grid_sync(d);
-    if (blockIdx.x == 0) phase_react_serial(d, sm.serial, nullptr);
-    grid_sync(d);
-    phase_products<F32L>(d, sm.products, blockIdx.x, gridDim.x);
-    grid_sync(d);
-    if (blockIdx.x == 0) {
-      phase_end_step(d, sm.end);
-      if (step + 1 < n_steps) phase_begin(d, sm.begin);  // the next step's begin
-    }
-    grid_sync(d);
+    __syncthreads();
   }
+  __device__ __forceinline__ void leave(const Dev& d) {
+    if (threadIdx.x == 0 && atomicAdd(&d.g->bar_left, 1u) + 1u == gridDim.x) {
+      d.g->bar_count = 0u;
+      d.g->bar_left = 0u;
+    }
+  }
+};
+
+// Barrier over the CTAs of one cluster (release / acquire of all memory among them).
+struct ClusterBarrier {
+  __device__ __forceinline__ void sync(const Dev&) {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  }
+  __device__ __forceinline__ void leave(const Dev&) {}
+};
+
+template <bool F32L, bool CLUSTER>
+__global__ void __launch_bounds__(PERSIST_THREADS, 1) k_steps(const __grid_constant__ Dev d, int n_steps, int align) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  StepSmem& sm = *reinterpret_cast<StepSmem*>(smem_raw);
+  typename std::conditional<CLUSTER, ClusterBarrier, GridBarrier>::type bar;
+  const Span sp = whole_grid();
+  const bool lead = sp.block == 0u;
+  if (lead) phase_begin(d, sm.react.plan.begin);
+  bar.sync(d);
+  for (int step = 0; step < n_steps; ++step) {
+    // CTA 0 alone writes these between the barriers: every CTA takes the same branches
+    const bool idle = d.g->any_active == 0u;
+    // (the order of the species after a run is that of launches of `align` steps: one that ends
+    // early re-sorts them once more, which removes the reacted and places the last products)
+    if (idle && (d.n_trains > 1u || (step != 0 && step % align == 0))) break;
+    const bool one = d.g->n_total <= SORT_ONE_CTA;
+    phase_diffuse<F32L>(d, one ? nullptr : sm.hist, sp);  // includes the release
+    bar.sync(d);
+    if (one) {
+      if (lead) phase_sort_one(d, sm.sort_one.one, sm.sort_one.bs, sm.sort_one.ss);
+      bar.sync(d);
+    } else {
+      const uint32_t n = d.g->n_total, active = active_passes(d, n);
+      for (int p = 0; p < d.passes; ++p) {
+        if (!((active >> p) & 1u) && p + 1 < d.passes) continue;  // the same for every CTA
+        const uint32_t tile = threadIdx.x == 0 ? atomicAdd(&d.g->tile_ctr[p], 1u) : 0u;
+        if (block_status_ok(d)) phase_sort_pass(d, p, active, n, tile, sm.sort, lead);
+        bar.sync(d);
+      }
+    }
+    phase_gather<F32L>(d, sp);
+    bar.sync(d);
+    if (idle) {
+      if (lead) phase_end_step(d, sm.react.end);
+      break;
+    }
+    // CTA 0 plans the next step while the others search
+    const bool plan = d.n_trains <= PLAN_TRAINS && step + 1 < n_steps;
+    if (plan && lead) {
+      stage_next(d, sm.react.plan);
+    } else if (d.g->search_cells_now) {
+      phase_search_cells<F32L, STEP_WARPS>(d, sm.cells);
+    } else {
+      const Span others = plan ? Span{sp.block - 1u, sp.blocks - 1u} : sp;
+      const int lg = lanes_per_home_lg(d.g->n_total - d.g->n_dead, others.stride());
+      phase_search_groups<F32L, STEP_WARPS>(d, sm.grp, lg > 0 ? lg : 1, others.warp(), others.warps());
+    }
+    bar.sync(d);
+    if (lead) {
+      phase_react_all<F32L>(d, sm.react.react, sm.react.sbuf, STEP_REACT_CAP, plan ? sm.react.plan.begin.tb : *d.tables);
+      if (!(plan && commit_next(d, sm.react.plan, sm.react.react))) {
+        phase_end_step(d, sm.react.end);
+        if (step + 1 < n_steps) phase_begin(d, sm.react.plan.begin);
+      }
+    }
+    bar.sync(d);
+  }
+  if (lead) phase_look_ahead(d, sm.react.end);
+  bar.leave(d);
 }
 
 // One step as one kernel per phase. With ev != nullptr, CUDA events are recorded
@@ -259,31 +317,66 @@ cudaError_t enqueue_check_accept(const Dev& d, uint32_t n, uint32_t step, double
   return cudaGetLastError();
 }
 
+// Up to n_steps steps (a multiple of `align`) in one launch: one cluster, or one CTA per SM
+// (cooperative).
 template <bool F32L>
-cudaError_t enqueue_persistent(const Dev& d, const LaunchCfg& lc, int n_steps, cudaStream_t s) {
+cudaError_t enqueue_steps(const Dev& d, const LaunchCfg& lc, bool cluster, int n_steps, int align, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(lc.persistent_blocks);
+  cfg.gridDim = dim3(cluster ? lc.cluster_blocks : lc.persistent_blocks);
   cfg.blockDim = dim3(PERSIST_THREADS);
-  cfg.dynamicSmemBytes = sizeof(PhaseSmem);
+  cfg.dynamicSmemBytes = sizeof(StepSmem);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeCooperative;
-  attr[0].val.cooperative = 1;
+  if (cluster) {
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = static_cast<unsigned>(lc.cluster_blocks);
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+  } else {
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+  }
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_persistent<F32L>, d, n_steps);
+  return cluster ? cudaLaunchKernelEx(&cfg, k_steps<F32L, true>, d, n_steps, align)
+                 : cudaLaunchKernelEx(&cfg, k_steps<F32L, false>, d, n_steps, align);
 }
 
+// Shared-memory limits of the precision's kernels; resident CTAs per SM of the persistent form
+// and the CTAs of its one-cluster form (0 when no cluster of STEP_CLUSTER or 8 fits).
 template <bool F32L>
-cudaError_t persistent_occupancy(int* blocks_per_sm) {
+cudaError_t step_kernel_limits(int* blocks_per_sm, int* cluster_blocks) {
   cudaError_t e = cudaFuncSetAttribute(k_react_end<F32L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(REACT_END_BYTES));
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_persistent<F32L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           static_cast<int>(sizeof(PhaseSmem)));
+  const int smem = static_cast<int>(sizeof(StepSmem));
+  e = cudaFuncSetAttribute(k_steps<F32L, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_persistent<F32L>, PERSIST_THREADS,
-                                                       sizeof(PhaseSmem));
+  e = cudaFuncSetAttribute(k_steps<F32L, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(k_steps<F32L, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e != cudaSuccess) return e;
+  *cluster_blocks = 0;
+  for (int c = STEP_CLUSTER; c >= 8 && *cluster_blocks == 0; c /= 2) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(c);
+    cfg.blockDim = dim3(PERSIST_THREADS);
+    cfg.dynamicSmemBytes = sizeof(StepSmem);
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = static_cast<unsigned>(c);
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int clusters = 0;
+    if (cudaOccupancyMaxActiveClusters(&clusters, k_steps<F32L, true>, &cfg) == cudaSuccess && clusters > 0)
+      *cluster_blocks = c;
+    else
+      cudaGetLastError();
+  }
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_steps<F32L, false>, PERSIST_THREADS,
+                                                       sizeof(StepSmem));
 }
 
 }  // namespace chem

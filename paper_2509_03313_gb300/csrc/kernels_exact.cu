@@ -12,7 +12,12 @@ __global__ void __launch_bounds__(256) k_begin(const __grid_constant__ Dev d) {
 
 __global__ void __launch_bounds__(SORT_THREADS) k_sort_pass(const __grid_constant__ Dev d, int pass) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  phase_sort_pass(d, pass, *reinterpret_cast<SortSmem*>(smem_raw));
+  // everything the pass starts from is read in one round: the tile, the status, the histograms
+  const uint32_t tile = threadIdx.x == 0 ? atomicAdd(&d.g->tile_ctr[pass], 1u) : 0u;
+  const uint32_t n = d.g->n_total;
+  const uint32_t active = active_passes(d, n);
+  if (!block_status_ok(d)) return;
+  phase_sort_pass(d, pass, active, n, tile, *reinterpret_cast<SortSmem*>(smem_raw), blockIdx.x == 0);
 }
 
 __global__ void __launch_bounds__(256) k_match_fast(const __grid_constant__ Dev d) {
@@ -31,6 +36,7 @@ __global__ void __launch_bounds__(REACT_THREADS) k_react_serial(const __grid_con
 __global__ void __launch_bounds__(256) k_end_step(const __grid_constant__ Dev d) {
   __shared__ EndSmem sm;
   phase_end_step(d, sm);
+  phase_look_ahead(d, sm);
 }
 
 cudaError_t enqueue_react_head(const Dev& d, const LaunchCfg& lc, cudaStream_t s) {
@@ -56,8 +62,10 @@ cudaError_t enqueue_end_begin(const Dev& d, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-__global__ void k_set_t_end(const __grid_constant__ Dev d, const double* t_end) {
+__global__ void __launch_bounds__(256) k_set_t_end(const __grid_constant__ Dev d, const double* t_end) {
+  __shared__ EndSmem sm;
   for (uint32_t b = threadIdx.x; b < d.n_trains; b += blockDim.x) d.trains[b].t_end = t_end[b];
+  phase_look_ahead(d, sm);
 }
 
 cudaError_t enqueue_begin(const Dev& d, cudaStream_t s) {
@@ -115,11 +123,14 @@ cudaError_t enqueue_step_f64(const Dev& d, const LaunchCfg& lc, cudaStream_t s, 
   return enqueue_phases<false>(d, lc, s, ev, first, last);
 }
 
-cudaError_t enqueue_persistent_f64(const Dev& d, const LaunchCfg& lc, int n_steps, cudaStream_t s) {
-  return enqueue_persistent<false>(d, lc, n_steps, s);
+cudaError_t enqueue_steps_f64(const Dev& d, const LaunchCfg& lc, bool cluster, int n_steps, int align,
+                              cudaStream_t s) {
+  return enqueue_steps<false>(d, lc, cluster, n_steps, align, s);
 }
 
-cudaError_t persistent_occupancy_f64(int* blocks_per_sm) { return persistent_occupancy<false>(blocks_per_sm); }
+cudaError_t step_kernel_limits_f64(int* blocks_per_sm, int* cluster_blocks) {
+  return step_kernel_limits<false>(blocks_per_sm, cluster_blocks);
+}
 
 cudaError_t enqueue_check_accept_f64(const Dev& d, uint32_t n, uint32_t step, double dt, const double* d0sq,
                                      const double* d1sq, const int32_t* rxn, const uint32_t* id_lo,

@@ -9,11 +9,14 @@ cudaError_t enqueue_step_f32l(const Dev& d, const LaunchCfg& lc, cudaStream_t s,
   return enqueue_phases<true>(d, lc, s, ev, first, last);
 }
 
-cudaError_t enqueue_persistent_f32l(const Dev& d, const LaunchCfg& lc, int n_steps, cudaStream_t s) {
-  return enqueue_persistent<true>(d, lc, n_steps, s);
+cudaError_t enqueue_steps_f32l(const Dev& d, const LaunchCfg& lc, bool cluster, int n_steps, int align,
+                              cudaStream_t s) {
+  return enqueue_steps<true>(d, lc, cluster, n_steps, align, s);
 }
 
-cudaError_t persistent_occupancy_f32l(int* blocks_per_sm) { return persistent_occupancy<true>(blocks_per_sm); }
+cudaError_t step_kernel_limits_f32l(int* blocks_per_sm, int* cluster_blocks) {
+  return step_kernel_limits<true>(blocks_per_sm, cluster_blocks);
+}
 
 cudaError_t enqueue_check_accept_f32l(const Dev& d, uint32_t n, uint32_t step, double dt, const double* d0sq,
                                      const double* d1sq, const int32_t* rxn, const uint32_t* id_lo,

@@ -15,7 +15,8 @@ struct LaunchCfg {
   int stream_blocks;      // grid of the grid-stride phases (release, diffuse, gather)
   int search_blocks;      // grid of the pair search
   int sort_blocks;        // resident CTAs of a sort pass
-  int persistent_blocks;  // resident CTAs of the persistent step kernel
+  int persistent_blocks;  // CTAs of the persistent step kernel (resident together)
+  int cluster_blocks;     // CTAs of its one-cluster form (0: not available)
   int search_tps;         // pair search: 1 one thread per home species, 0 cell tiles,
                           // 2 both launched, the step's choice runs (adaptive)
   int small;              // few species: one search kernel and one reaction kernel per step
@@ -35,9 +36,12 @@ cudaError_t sort_pass_occupancy(int* blocks_per_sm);
 // kernel also begins the next step).
 cudaError_t enqueue_step_f64(const Dev& d, const LaunchCfg& lc, cudaStream_t s, cudaEvent_t* ev, bool first,
                              bool last);
-cudaError_t enqueue_persistent_f64(const Dev& d, const LaunchCfg& lc, int n_steps, cudaStream_t s);
-// (also sets the shared-memory limits of the precision's kernels)
-cudaError_t persistent_occupancy_f64(int* blocks_per_sm);
+// Up to n_steps steps in one launch (one cluster, or one CTA per SM).
+// n_steps is a multiple of `align`, whose multiples the species' order follows.
+cudaError_t enqueue_steps_f64(const Dev& d, const LaunchCfg& lc, bool cluster, int n_steps, int align,
+                              cudaStream_t s);
+// Sets the shared-memory limits of the precision's kernels; CTAs of the two forms above.
+cudaError_t step_kernel_limits_f64(int* blocks_per_sm, int* cluster_blocks);
 cudaError_t enqueue_set_t_end(const Dev& d, const double* t_end_dev, cudaStream_t s);
 // one device thread waits, up to limit_s, for a word nothing writes (then CHEM_ETIMEOUT)
 cudaError_t enqueue_bounded_wait(const Dev& d, double limit_s, cudaStream_t s);
@@ -56,7 +60,8 @@ cudaError_t enqueue_homogeneous(const Dev& d, int blocks, cudaStream_t s);
 // kernels_f32l.cu (FP32-local mode)
 cudaError_t enqueue_step_f32l(const Dev& d, const LaunchCfg& lc, cudaStream_t s, cudaEvent_t* ev, bool first,
                               bool last);
-cudaError_t enqueue_persistent_f32l(const Dev& d, const LaunchCfg& lc, int n_steps, cudaStream_t s);
-cudaError_t persistent_occupancy_f32l(int* blocks_per_sm);
+cudaError_t enqueue_steps_f32l(const Dev& d, const LaunchCfg& lc, bool cluster, int n_steps, int align,
+                               cudaStream_t s);
+cudaError_t step_kernel_limits_f32l(int* blocks_per_sm, int* cluster_blocks);
 
 }  // namespace chem

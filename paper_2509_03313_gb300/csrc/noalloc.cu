@@ -236,6 +236,10 @@ extern "C" chem_status chem_step_noalloc(const chem_config* cfg, uint32_t step, 
     tb.n_prod[r] = x.n_prod;
     for (int q = 0; q < 3; ++q) tb.prod[r][q] = q < x.n_prod ? x.prod[q] : 0;
     tb.water[r] = x.water_delta;
+    tb.rxn_a[r] = x.a;
+    tb.rxn_b[r] = x.b;
+    tb.w_ab[r][0] = tb.D[x.a] / (tb.D[x.a] + tb.D[x.b]);
+    tb.w_ab[r][1] = tb.D[x.b] / (tb.D[x.b] + tb.D[x.a]);
     const double room = cfg->L_nm / 3.0 - tb.R[r];
     if (!(room > 0.0)) return CHEM_EINVAL;
     if (cfg->cutoff_c > 0.0) {
@@ -328,10 +332,10 @@ extern "C" chem_status chem_step_noalloc(const chem_config* cfg, uint32_t step, 
   d.tables = reinterpret_cast<const Tables*>(b + LAYOUT.tables);
   d.g = reinterpret_cast<Global*>(b + LAYOUT.global);
 
-  int dev = 0, sms = 0, sort_occ = 0, pers_occ = 0;
+  int dev = 0, sms = 0, sort_occ = 0, pers_occ = 0, cluster = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-      sort_pass_occupancy(&sort_occ) != cudaSuccess || persistent_occupancy_f64(&pers_occ) != cudaSuccess || sms < 1 ||
+      sort_pass_occupancy(&sort_occ) != cudaSuccess || step_kernel_limits_f64(&pers_occ, &cluster) != cudaSuccess || sms < 1 ||
       sort_occ < 1) {
     cudaGetLastError();
     return CHEM_ECUDA;
@@ -340,7 +344,8 @@ extern "C" chem_status chem_step_noalloc(const chem_config* cfg, uint32_t step, 
   lc.stream_blocks = std::max(1, std::min(sms * 2, (n + 255) / 256 + 1));
   lc.search_blocks = sms * 4;
   lc.sort_blocks = std::min(sms * sort_occ, static_cast<int>(NA_TILES));
-  lc.persistent_blocks = 1;
+  lc.persistent_blocks = sms;
+  lc.cluster_blocks = cluster;
   lc.search_tps = 0;
   lc.small = 1;
   cudaStream_t s = static_cast<cudaStream_t>(cfg->cuda_stream);

@@ -38,6 +38,16 @@ struct SortSmemT {
 using SortSmem = SortSmemT<SORT_THREADS>;      // the per-pass kernel
 using SortSmemP = SortSmemT<PERSIST_THREADS>;  // the persistent kernel
 
+// Rows of NT keys in a tile of a sort of n keys: a tile's rows are ranked one after the other, a
+// tile's look-back covers its predecessors, so few keys take small tiles (6,000
+// species in one tile of 12 rows took longer than 8,000 in four tiles of 4).
+__host__ __device__ __forceinline__ uint32_t sort_rows(uint32_t n, uint32_t nt) {
+  const uint32_t all = (n + nt - 1u) / nt;  // rows in one tile of everything
+  if (all <= SORT_ROWS_MIN) return all ? all : 1u;
+  const uint32_t r = (all + SORT_MANY_TILES - 1u) / SORT_MANY_TILES;
+  return r < SORT_ROWS_MIN ? SORT_ROWS_MIN : (r > static_cast<uint32_t>(SORT_ITEMS) ? static_cast<uint32_t>(SORT_ITEMS) : r);
+}
+
 constexpr unsigned long long LB_AGG = 1ull, LB_INC = 2ull;
 
 __device__ __forceinline__ unsigned long long lb_pack(uint32_t epoch, unsigned long long flag,
@@ -64,14 +74,16 @@ __device__ __forceinline__ uint32_t block_exclusive_scan256(uint32_t v, uint32_t
 
 // One pass over n keys by digit (key >> shift) & 255. ghist = this digit's histogram
 // over all n keys; vin == nullptr means value = input index. Must be called by all NT
-// threads of every CTA.
+// threads of every CTA; first_tile is thread 0's own claim from *tile_ctr (made by the caller
+// so that it travels with its other loads).
 template <int NT>
 __device__ void onesweep_pass(const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin,
                               uint32_t* __restrict__ kout, uint32_t* __restrict__ vout, uint32_t n,
-                              int shift, const uint32_t* ghist, uint32_t* tile_ctr,
+                              int shift, const uint32_t* ghist, uint32_t first_tile, uint32_t* tile_ctr,
                               unsigned long long* lookback, uint32_t epoch, Global* g,
                               SortSmemT<NT>& sm) {
-  constexpr int SORT_TILE = SortSmemT<NT>::TILE;
+  const uint32_t rows = sort_rows(n, NT);
+  const uint32_t SORT_TILE = rows * NT;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const uint32_t lanemask_lt = (1u << lane) - 1u;
   {
@@ -80,28 +92,31 @@ __device__ void onesweep_pass(const uint32_t* __restrict__ kin, const uint32_t* 
     if (tid < RADIX) sm.gbase[tid] = e;
   }
   const uint32_t n_tiles = (n + SORT_TILE - 1) / SORT_TILE;
-  for (;;) {
-    if (tid == 0) sm.tile = atomicAdd(tile_ctr, 1u);
+  const bool one_each = n_tiles <= gridDim.x;  // no CTA will find a second tile
+  for (bool first = true;; first = false) {
+    if (one_each && !first) break;
+    if (tid == 0) sm.tile = first ? first_tile : atomicAdd(tile_ctr, 1u);
     __syncthreads();
     const uint32_t tile = sm.tile;
     if (tile >= n_tiles) break;
     const uint32_t tile_base = tile * SORT_TILE;
-    const uint32_t tile_n = min(static_cast<uint32_t>(SORT_TILE), n - tile_base);
+    const uint32_t tile_n = min(SORT_TILE, n - tile_base);
     // clear this warp's digit counters
 #pragma unroll
     for (int i = lane; i < RADIX; i += 32) sm.wcnt[w][i] = 0u;
     __syncwarp();
     uint32_t key[SORT_ITEMS], val[SORT_ITEMS], rank[SORT_ITEMS];
-    const uint32_t wbase = tile_base + w * (32 * SORT_ITEMS);
+    const uint32_t wbase = tile_base + static_cast<uint32_t>(w) * (32u * rows);
 #pragma unroll
     for (int r = 0; r < SORT_ITEMS; ++r) {
       const uint32_t idx = wbase + r * 32 + lane;
-      const bool valid = idx < n;
+      const bool valid = static_cast<uint32_t>(r) < rows && idx < n;
       key[r] = valid ? kin[idx] : 0xFFFFFFFFu;
       val[r] = valid ? (vin ? vin[idx] : idx) : 0u;
     }
 #pragma unroll
     for (int r = 0; r < SORT_ITEMS; ++r) {
+      if (static_cast<uint32_t>(r) >= rows) break;
       const uint32_t idx = wbase + r * 32 + lane;
       const bool valid = idx < n;
       const uint32_t d = (key[r] >> shift) & 255u;
@@ -146,7 +161,7 @@ __device__ void onesweep_pass(const uint32_t* __restrict__ kin, const uint32_t* 
         int32_t t = static_cast<int32_t>(tile) - 1;
         bool timed_out = false;
         while (t >= 0) {
-          constexpr int LB_BATCH = 8;
+          constexpr int LB_BATCH = 8;  // (twice as many: 9 % slower on 130 tiles)
           unsigned long long wv[LB_BATCH];
 #pragma unroll
           for (int q = 0; q < LB_BATCH; ++q)
@@ -178,7 +193,7 @@ __device__ void onesweep_pass(const uint32_t* __restrict__ kin, const uint32_t* 
 #pragma unroll
     for (int r = 0; r < SORT_ITEMS; ++r) {
       const uint32_t idx = wbase + r * 32 + lane;
-      if (idx < n) {
+      if (static_cast<uint32_t>(r) < rows && idx < n) {
         const uint32_t d = (key[r] >> shift) & 255u;
         const uint32_t p = sm.tile_off[d] + sm.wcnt[w][d] + rank[r];
         sm.k[p] = key[r];

@@ -21,6 +21,17 @@ namespace chem {
 constexpr double TWO_POW_M53 = 1.1102230246251565e-16;
 constexpr float TWO_POW_M24F = 5.9604644775390625e-08f;
 
+// The part of a phase's work that a CTA takes: CTA `block` of `blocks`. Warps of one CTA are
+// `blocks` warps apart, so that little work spreads over all CTAs.
+struct Span {
+  uint32_t block, blocks;
+  __device__ __forceinline__ uint32_t warp() const { return (threadIdx.x >> 5) * blocks + block; }
+  __device__ __forceinline__ uint32_t warps() const { return (blockDim.x >> 5) * blocks; }
+  __device__ __forceinline__ uint32_t first() const { return warp() * 32u + (threadIdx.x & 31u); }
+  __device__ __forceinline__ uint32_t stride() const { return blocks * blockDim.x; }
+};
+__device__ __forceinline__ Span whole_grid() { return Span{blockIdx.x, gridDim.x}; }
+
 __device__ __forceinline__ int status_of(const Dev& d) {
   return *reinterpret_cast<volatile int*>(&d.g->status);
 }
@@ -188,6 +199,15 @@ __device__ __forceinline__ void set_pair_constants(Train& tr, const Tables& tb, 
   tr.inv_ddt_f[r] = 1.0f / static_cast<float>(tr.ddt[r]);
 }
 
+// Lanes of the pair search that share a home species (phase_search_groups): 2^lg, for n species
+// on `lanes` lanes as many as there are spare, up to 16 (a lane per cell of the half shell). 0:
+// one thread per home species.
+constexpr int GRP_MAX_LG = 4;
+__device__ __forceinline__ int lanes_per_home_lg(uint32_t n, uint32_t lanes) {
+  const uint32_t per = lanes / (n ? n : 1u);
+  return per >= 2u ? min(GRP_MAX_LG, 31 - __clz(per)) : 0;
+}
+
 // ======================================================================== begin
 constexpr int BEGIN_TRAINS = 16;  // trains whose cutoffs pass through shared memory
 
@@ -197,6 +217,11 @@ struct BeginSmem {
   double dt[MAX_TRAINS];
   unsigned long long rcmax_bits[MAX_TRAINS];
   float hf[MAX_TRAINS];                   // this step's cell side
+  // between the two halves of the phase: whether the train advances, its releases (arrived,
+  // re-created, unparked) and its species before them
+  uint8_t act[MAX_TRAINS];
+  uint32_t rel_new[MAX_TRAINS], mat[MAX_TRAINS], parked[MAX_TRAINS];
+  long long live[MAX_TRAINS];
   double c[BEGIN_TRAINS];                 // cutoff factor ...
   double rc2[BEGIN_TRAINS][MAXR];         // ... and squared cutoffs of the first trains
   int cb0;                                // train 0: key bits per axis of its cells
@@ -213,43 +238,37 @@ struct BeginSmem {
 // start (a train's record stays in its thread's registers through (1) and (3)), later
 // stages read what earlier ones wrote from shared memory, and the pending queue is only
 // searched when its first arrival is due. With loads in every stage it took 8 us.
-static __device__ void phase_begin(const Dev& d, BeginSmem& sb) {
+//
+// The phase has two halves: begin_plan, (1) to (4), which needs nothing of the reactions of
+// the step before and works on the records `trains` (the context's, or a copy of them that
+// already stands at the end of that step), and begin_commit, the rest.
+static __device__ void begin_plan(const Dev& d, BeginSmem& sb, Train* trains, int st) {
   const int tid = threadIdx.x, nt = blockDim.x;
   {
     const uint32_t* src = reinterpret_cast<const uint32_t*>(d.tables);
     uint32_t* dst = reinterpret_cast<uint32_t*>(&sb.tb);
     for (int i = tid; i < static_cast<int>(sizeof(Tables) / 4); i += nt) dst[i] = src[i];
   }
-  for (int i = tid; i < MAX_PASSES * RADIX; i += nt) (&d.g->hist[0][0])[i] = 0u;
-  const int st = status_of(d);
-  // the counters thread 0 updates below, read with the tables
-  Global* g = d.g;
-  uint32_t g_total = 0, g_live = 0, g_adaptive = 0, g_home = 0, g_epoch = 0, g_cells = 0;
-  unsigned long long g_incut = 0, g_mark = 0;
-  if (tid == 0) {
-    g_total = g->n_total; g_live = g->n_live; g_adaptive = g->search_adaptive; g_home = g->item_home;
-    g_epoch = g->epoch; g_cells = g->cells_steps; g_incut = g->pairs_in_cutoff; g_mark = g->incut_mark;
-    sb.any = 0;
-  }
+  if (tid == 0) sb.any = 0;
   // train `tid`
   const uint32_t b = static_cast<uint32_t>(tid);
   const bool have = b < d.n_trains;
-  Train& tr = d.trains[have ? b : 0u];
+  Train& tr = trains[have ? b : 0u];
   double t = 0, t_end = 0, t_lr = 0, horizon = 0, dt_min = 0, dt_L = 0, dt_cur = 0, next_arr = 0, L = 0, inv_L = 0;
-  uint32_t p_head = 0, p_tail = 0, pend_base = 0, next_id = 0, id_limit = 0, mat = 0, parked = 0;
+  uint32_t p_head = 0, p_tail = 0, pend_base = 0, mat = 0, parked = 0;
   int reset = 0, tr_n_max = 0, cb_alloc = 0, n_ref = 0;
   long long live = 0;
   if (have) {
     t = tr.t; t_end = tr.t_end; t_lr = tr.t_last_release; horizon = tr.horizon;
     dt_min = tr.dt_min; dt_L = tr.dt_L; dt_cur = tr.dt_cur; next_arr = tr.next_arr;
     p_head = tr.p_head; p_tail = tr.p_tail; pend_base = tr.pend_base;
-    next_id = tr.next_id; id_limit = tr.id_limit;
     mat = tr.mat_n;      // survivors of a homogeneous stage (already counted)
     parked = tr.park_n;  // species parked while the train was idle (counted)
     reset = tr.reset_on_release;
     L = tr.L; inv_L = tr.inv_L; tr_n_max = tr.n_max; cb_alloc = tr.cb_alloc; n_ref = tr.n_ref;
 #pragma unroll
     for (int ty = 0; ty < MAXT; ++ty) live += tr.counts[ty];  // 0 past the context's types
+    sb.live[b] = live;
     if (b < BEGIN_TRAINS) sb.c[b] = tr.c;
     if (b == 0) {  // the removed species' key below needs train 0's grid, idle or not
       sb.cb0 = tr.cb;
@@ -262,8 +281,6 @@ static __device__ void phase_begin(const Dev& d, BeginSmem& sb) {
   int free_jump = 0;
   if (have) {
     const bool act = (st == 0) && (t < t_end);
-    // an idle train with species among the stepped slots parks them this step
-    tr.park_now = (!act && d.pk_cell != nullptr && live > static_cast<long long>(parked) + mat) ? 1u : 0u;
     uint32_t rel = 0;
     sb.rcmax_bits[b] = 0ull;
     if (act) {
@@ -313,13 +330,9 @@ static __device__ void phase_begin(const Dev& d, BeginSmem& sb) {
       tr.park_n = 0;
       tr.rel_mat = mat;
       tr.mat_n = 0;
-      tr.rel_id0 = next_id;
       tr.rel_p0 = p_head;
       tr.p_head = p_head + rel;
-      tr.next_id = next_id + rel + mat;
-      tr.n_live_step = live + rel;
       tr.n_events_step = 0;
-      if (static_cast<unsigned long long>(next_id) + rel + mat > id_limit) raise_status(d.g, CHEM_ECAPACITY);
       atomicOr(&sb.any, 1u);
     } else {
       sb.dt[b] = 0.0;
@@ -330,6 +343,10 @@ static __device__ void phase_begin(const Dev& d, BeginSmem& sb) {
     }
     tr.active = act ? 1 : 0;
     tr.free_jump = free_jump;
+    sb.act[b] = act ? 1 : 0;
+    sb.rel_new[b] = rel;
+    sb.mat[b] = mat;
+    sb.parked[b] = parked;
   }
   __syncthreads();
   // cutoffs R + c sqrt(2 D_AB dt), bridge constants, and sigma = sqrt(2 D dt)
@@ -339,7 +356,7 @@ static __device__ void phase_begin(const Dev& d, BeginSmem& sb) {
     const int q = static_cast<int>(w % per);
     const double wdt = sb.dt[wb];
     if (wdt <= 0.0) continue;  // train not advancing this step
-    Train& wt = d.trains[wb];
+    Train& wt = trains[wb];
     if (q < MAXR) {
       if (q >= tb.n_rxn) continue;
       const double c = wb < BEGIN_TRAINS ? sb.c[wb] : wt.c;
@@ -411,7 +428,7 @@ static __device__ void phase_begin(const Dev& d, BeginSmem& sb) {
     const uint32_t wb = w / (MAXT * MAXT);
     const int q = static_cast<int>(w % (MAXT * MAXT));
     if (sb.dt[wb] <= 0.0) continue;
-    Train& wt = d.trains[wb];
+    Train& wt = trains[wb];
     const int r = tb.pair_rxn[q / MAXT][q % MAXT];
     const double c2 = r >= 0 ? (wb < BEGIN_TRAINS ? sb.rc2[wb][r] : wt.rc2[r]) : -1.0;
     const float c2f = r >= 0 ? static_cast<float>(c2) : -1.f;
@@ -421,12 +438,44 @@ static __device__ void phase_begin(const Dev& d, BeginSmem& sb) {
     const float rw = rc * 1.00001f + 2e-6f * sb.hf[wb];
     wt.rc2w_tt[q] = rc >= 0.f ? rw * rw * 1.00001f : -1.f;
   }
+}
+
+// Lanes that a launch of one thread per home species has at least (the per-phase form).
+constexpr uint32_t SEARCH_LANES = 152u * 1024u;
+
+// The rest of the begin: ids, slots and counters of the step (sb.live: the species per train).
+static __device__ void begin_commit(const Dev& d, BeginSmem& sb, Train* trains) {
+  const int tid = threadIdx.x, nt = blockDim.x;
+  Global* g = d.g;
+  for (int i = tid; i < MAX_PASSES * RADIX; i += nt) (&g->hist[0][0])[i] = 0u;
+  uint32_t g_total = 0, g_live = 0, g_adaptive = 0, g_home = 0, g_epoch = 0, g_cells = 0;
+  unsigned long long g_incut = 0, g_mark = 0;
+  if (tid == 0) {  // (all in flight together)
+    g_total = g->n_total; g_live = g->n_live; g_adaptive = g->search_adaptive; g_home = g->item_home;
+    g_epoch = g->epoch; g_cells = g->cells_steps; g_incut = g->pairs_in_cutoff; g_mark = g->incut_mark;
+  }
+  const uint32_t b = static_cast<uint32_t>(tid);
+  if (b < d.n_trains) {
+    Train& tr = trains[b];
+    const long long live = sb.live[b];
+    const uint32_t rel = sb.rel_new[b], mat = sb.mat[b];
+    const bool act = sb.act[b] != 0;
+    // an idle train with species among the stepped slots parks them this step
+    tr.park_now = (!act && d.pk_cell != nullptr && live > static_cast<long long>(sb.parked[b]) + mat) ? 1u : 0u;
+    if (act) {
+      const uint32_t next_id = tr.next_id;
+      tr.rel_id0 = next_id;
+      tr.next_id = next_id + rel + mat;
+      tr.n_live_step = live + rel;
+      if (static_cast<unsigned long long>(next_id) + rel + mat > tr.id_limit) raise_status(g, CHEM_ECAPACITY);
+    }
+  }
   if (tid == 0) {
     uint32_t off = g_total;
     const uint32_t before = off;
     unsigned long long total = off;
     for (uint32_t q = 0; q < d.n_trains; ++q) {
-      d.trains[q].rel_off = off;
+      trains[q].rel_off = off;
       total += sb.rel[q];
       off += sb.rel[q];
     }
@@ -451,11 +500,16 @@ static __device__ void phase_begin(const Dev& d, BeginSmem& sb) {
     // the homes of a cell and test a pair only when the types react; one thread per
     // species has the shorter per-item latency chain. Adaptive: cell tiles when the last
     // step found more than 3 pairs inside the cutoffs per live species (the measured
-    // crossover on track workloads); results do not depend on the mapping.
+    // crossover on track workloads). Where the launch has several lanes for each home
+    // those share the pairs of a home, and tiles only pay for a few thousand species or very
+    // many pairs: at 31,000 species lanes take 43, 79 and 143 us where tiles take 95, 156
+    // and 207, at 6, 16 and 25 pairs per species. Results do not depend on the mapping.
     uint32_t cells_now;
     if (g_adaptive) {
       const unsigned long long inc = g_incut - g_mark;
-      cells_now = inc > 3ull * static_cast<unsigned long long>(g_live) ? 1u : 0u;
+      const int lg = lanes_per_home_lg(g_live, SEARCH_LANES);
+      const unsigned long long most = lg > 0 && lg < GRP_MAX_LG ? 48ull : 3ull;
+      cells_now = inc > most * static_cast<unsigned long long>(g_live) ? 1u : 0u;
     } else {
       cells_now = g_home != 0u ? 1u : 0u;
     }
@@ -471,6 +525,12 @@ static __device__ void phase_begin(const Dev& d, BeginSmem& sb) {
     g->sentinel_step = d.n_trains == 1 ? sb.base0 + (kb >= 32 ? 0xFFFFFFFFu : (1u << kb) - 1u) : d.sentinel;
   }
   __syncthreads();
+}
+
+static __device__ void phase_begin(const Dev& d, BeginSmem& sb) {
+  begin_plan(d, sb, d.trains, status_of(d));
+  __syncthreads();
+  begin_commit(d, sb, d.trains);
 }
 
 // Train whose release block holds `slot` (release offsets ascend with b).
@@ -527,15 +587,19 @@ __device__ __forceinline__ uint32_t recreated_type(const Train& tr, uint32_t k) 
 // Species marked dead by the last step's reactions get the sentinel key. Species
 // released this step (slots [n_total - n_released, n_total)) are first built from the
 // pending queue (the release of Sec. 2.1) by the thread that then diffuses them.
+// `hist` is the CTA's shared-memory histogram; nullptr when the sort of the step counts for
+// itself.
 template <bool F32L>
-__device__ void phase_diffuse(const Dev& d, uint32_t (*hist)[RADIX]) {
-  for (int i = threadIdx.x; i < MAX_PASSES * RADIX; i += blockDim.x) (&hist[0][0])[i] = 0u;
-  __syncthreads();
+__device__ void phase_diffuse(const Dev& d, uint32_t (*hist)[RADIX], const Span& sp) {
+  if (hist) {
+    for (int i = threadIdx.x; i < MAX_PASSES * RADIX; i += blockDim.x) (&hist[0][0])[i] = 0u;
+    __syncthreads();
+  }
   // the trip count below must be the same for a whole warp (count_add votes)
   const bool ok = __shfl_sync(0xffffffffu, status_of(d) == 0 ? 1 : 0, 0) != 0;
   const uint32_t n_total = d.g->n_total;
   const uint32_t rel_base = n_total - d.g->n_released;
-  const uint32_t stride = gridDim.x * blockDim.x;
+  const uint32_t stride = sp.stride(), first = sp.first();
   const uint32_t n_iter = ok ? (n_total + stride - 1) / stride : 0u;
   uint32_t n_dead_local = 0;
   // the next iteration's state of a stepped slot is loaded while this one is worked on
@@ -556,9 +620,9 @@ __device__ void phase_diffuse(const Dev& d, uint32_t (*hist)[RADIX]) {
       }
     }
   };
-  if (n_iter > 0) prefetch(blockIdx.x * blockDim.x + threadIdx.x);
+  if (n_iter > 0) prefetch(first);
   for (uint32_t it = 0; it < n_iter; ++it) {
-    const uint32_t s = it * stride + blockIdx.x * blockDim.x + threadIdx.x;
+    const uint32_t s = it * stride + first;
     const uint32_t c_cell = pf_cell, c_prev = pf_prev, c_tid = pf_tid;
     const bool c_dead = pf_dead;
     const float4 c_v = pf_v;
@@ -730,13 +794,15 @@ __device__ void phase_diffuse(const Dev& d, uint32_t (*hist)[RADIX]) {
         }
       }
       d.keys0[s] = key;  // the first radix pass takes the slot itself as the value
-      for (int p = 0; p < d.passes; ++p) atomicAdd(&hist[p][(key >> (8 * p)) & 255u], 1u);
+      if (hist)
+        for (int p = 0; p < d.passes; ++p) atomicAdd(&hist[p][(key >> (8 * p)) & 255u], 1u);
     }
     count_add(d, rel_b, rel_type, 1, rel_new);
   }
   // warp-aggregate the dead count
   for (int o = 16; o > 0; o >>= 1) n_dead_local += __shfl_xor_sync(0xffffffffu, n_dead_local, o);
   if ((threadIdx.x & 31) == 0 && n_dead_local) atomicAdd(&d.g->n_dead, n_dead_local);
+  if (!hist) return;
   __syncthreads();
   if (ok) {
     for (int i = threadIdx.x; i < d.passes * RADIX; i += blockDim.x) {
@@ -749,18 +815,16 @@ __device__ void phase_diffuse(const Dev& d, uint32_t (*hist)[RADIX]) {
 // ======================================================================== sort pass
 // A pass whose digit is the same for every key is the identity and is skipped; the
 // ping-pong buffers of the remaining passes follow from the histograms, which every CTA
-// reads identically. Returns the number of executed passes before `pass` in *before.
-__device__ __forceinline__ bool pass_active(const uint32_t (*hist)[RADIX], int pass, uint32_t n,
-                                            int* before) {
-  int cnt = 0;
-  bool act = false;
-  for (int q = 0; q <= pass; ++q) {
-    const int trivial = __syncthreads_or(static_cast<int>(hist[q][threadIdx.x & (RADIX - 1)] == n));
-    if (q < pass) cnt += trivial ? 0 : 1;
-    else act = !trivial;
-  }
-  *before = cnt;
-  return act;
+// reads identically. Bit p of the result: pass p of the n keys has something to do.
+__device__ __forceinline__ uint32_t active_passes(const Dev& d, uint32_t n) {
+  uint32_t h[MAX_PASSES];
+#pragma unroll
+  for (int p = 0; p < MAX_PASSES; ++p) h[p] = p < d.passes ? d.g->hist[p][threadIdx.x & (RADIX - 1)] : n;
+  uint32_t mask = 0u;
+#pragma unroll
+  for (int p = 0; p < MAX_PASSES; ++p)
+    if (p < d.passes && !__syncthreads_or(static_cast<int>(h[p] == n))) mask |= 1u << p;
+  return mask;
 }
 
 // Status read once per CTA so that every thread takes the same branch before barriers.
@@ -768,31 +832,39 @@ __device__ __forceinline__ bool block_status_ok(const Dev& d) {
   return __syncthreads_and(threadIdx.x == 0 ? (status_of(d) == 0) : 1) != 0;
 }
 
+// One pass of the sort, `active` from active_passes. `lead` marks the CTA that records the
+// buffers of the result (at the last pass). `first_tile`: thread 0's claim of a tile.
 template <int NT>
-__device__ void phase_sort_pass(const Dev& d, int pass, SortSmemT<NT>& sm) {
-  if (!block_status_ok(d)) return;
-  const uint32_t n = d.g->n_total;
-  int before = 0;
-  const bool act = pass_active(d.g->hist, pass, n, &before);
-  if (pass == d.passes - 1 && blockIdx.x == 0 && threadIdx.x == 0) {
-    d.g->sort_parity = static_cast<uint32_t>((before + (act ? 1 : 0)) & 1);
-    d.g->sort_any = (before + (act ? 1 : 0)) > 0 ? 1u : 0u;
+__device__ void phase_sort_pass(const Dev& d, int pass, uint32_t active, uint32_t n, uint32_t first_tile,
+                                SortSmemT<NT>& sm, bool lead) {
+  const int before = __popc(active & ((1u << pass) - 1u));
+  if (pass == d.passes - 1 && lead && threadIdx.x == 0) {
+    const uint32_t all = __popc(active);
+    d.g->sort_parity = all & 1u;
+    d.g->sort_any = all > 0u ? 1u : 0u;
   }
-  if (!act) return;
+  if (!((active >> pass) & 1u)) return;
   const bool odd = before & 1;
   const uint32_t* kin = odd ? d.keys1 : d.keys0;
   const uint32_t* vin = before == 0 ? nullptr : (odd ? d.vals1 : d.vals0);  // nullptr: value = index
   uint32_t* kout = odd ? d.keys0 : d.keys1;
   uint32_t* vout = odd ? d.vals0 : d.vals1;
-  onesweep_pass(kin, vin, kout, vout, n, 8 * pass, d.g->hist[pass], &d.g->tile_ctr[pass],
+  onesweep_pass(kin, vin, kout, vout, n, 8 * pass, d.g->hist[pass], first_tile, &d.g->tile_ctr[pass],
                 d.lookback, d.g->epoch * 2 * MAX_PASSES + pass, d.g, sm);
 }
+
+// The whole sort by one CTA in shared memory, for at most SORT_ONE_CTA keys: three passes over
+// the grid are three chains of look-back and barrier.
+constexpr uint32_t SORT_ONE_CTA = 4096;
+struct SortOneSmem {
+  uint32_t k0[SORT_ONE_CTA], v0[SORT_ONE_CTA], k1[SORT_ONE_CTA], v1[SORT_ONE_CTA];
+};
 
 // ======================================================================== gather
 // Reorder the diffused species into cell order, record each cell's slot range (stamped
 // with this step's epoch) and drop the dead (sentinel keys sort last).
 template <bool F32L>
-__device__ void phase_gather(const Dev& d) {
+__device__ void phase_gather(const Dev& d, const Span& sp) {
   if (status_of(d)) return;
   const uint32_t* kf = d.g->sort_parity ? d.keys1 : d.keys0;
   const uint32_t* vf = d.g->sort_any ? (d.g->sort_parity ? d.vals1 : d.vals0) : nullptr;
@@ -802,10 +874,10 @@ __device__ void phase_gather(const Dev& d) {
   const uint32_t sentinel = d.g->sentinel_step;
   const uint32_t item_home = d.g->item_home;
   const bool items_now = item_home != 0 && d.g->search_cells_now;
-  const uint32_t stride = gridDim.x * blockDim.x;
+  const uint32_t stride = sp.stride();
   // GATHER_BATCH slots per thread and iteration, their loads in flight together: the
   // permutation and neighbouring keys first, then the gathered state
-  for (uint32_t s0 = blockIdx.x * blockDim.x + threadIdx.x; s0 < n_live; s0 += stride * GATHER_BATCH) {
+  for (uint32_t s0 = sp.first(); s0 < n_live; s0 += stride * GATHER_BATCH) {
     uint32_t key[GATHER_BATCH], idx[GATHER_BATCH], prv[GATHER_BATCH], nxt[GATHER_BATCH];
     bool ok[GATHER_BATCH];
 #pragma unroll
@@ -879,7 +951,7 @@ __device__ void phase_gather(const Dev& d) {
       }
     }
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) d.g->n_live = n_live;
+  if (sp.block == 0 && threadIdx.x == 0) d.g->n_live = n_live;
 }
 
 // ======================================================================== search
@@ -1422,14 +1494,6 @@ __device__ void phase_search_tps(const Dev& d, TpsSmem<F32L, W>& sm) {
 // non-empty ranges of a home are laid end to end, and its lanes take every 2^lg-th neighbour
 // of that list. The same pairs are visited and queued.
 constexpr int GRP_UNROLL = 4;    // neighbours a lane keeps in flight
-constexpr int GRP_MAX_LG = 4;
-
-// lg of the lanes per home for n species on `lanes` lanes: as many as there are spare, up to
-// 16 (a lane per cell of the half shell). 0: one thread per home species.
-__device__ __forceinline__ int lanes_per_home_lg(uint32_t n, uint32_t lanes) {
-  const uint32_t per = lanes / (n ? n : 1u);
-  return per >= 2u ? min(GRP_MAX_LG, 31 - __clz(per)) : 0;
-}
 
 template <int W>
 struct GrpSmem {
@@ -1630,7 +1694,7 @@ struct ProductsSmem {
 };
 
 struct EndSmem {
-  uint32_t any, stepped;
+  uint32_t any, stepped, ahead;
 };
 
 // Exclusive block-wide prefix of v (one value per thread); `total` gets the block sum.
@@ -1820,7 +1884,7 @@ constexpr size_t RC_SMEM_BYTES = rc_smem_bytes(RC_CAP);
 // sm.n_conflict share a species with another), sbuf of rc_smem_bytes(n_c) or more:
 // sm.n_won winners, their pairs' indices in the returned list (in sbuf).
 static __device__ const uint32_t* match_rounds_in_smem(const Dev& d, MatchSmem& sm, uint32_t* sbuf, uint32_t n_c,
-                                                       const uint32_t* list) {
+                                                       const uint32_t* list, const Cand* first = nullptr) {
   const int tid = threadIdx.x, nt = blockDim.x;
   const uint32_t hash = rc_hash(n_c);
   // carve the buffer (8-byte arrays first)
@@ -1844,7 +1908,7 @@ static __device__ const uint32_t* match_rounds_in_smem(const Dev& d, MatchSmem& 
   // load the pairs, reset the accepted-pair counts for the next step, insert the slots
   for (uint32_t i = tid; i < n_c; i += nt) {
     const uint32_t c = list ? list[i] : i;
-    const Cand cd = d.cand[c];
+    const Cand cd = first && i == static_cast<uint32_t>(tid) ? *first : d.cand[c];  // (first: pair `tid`)
     d.touch[cd.s_lo] = 0u;
     d.touch[cd.s_hi] = 0u;
     cix[i] = c;
@@ -1974,25 +2038,31 @@ static __device__ bool phase_match_rounds_smem(const Dev& d, MatchSmem& sm, uint
 // by comparison with the bucket's other keys (buckets hold a handful of keys for the
 // id-like keys sorted here). The result is in (k0, v0); (k1, v1) is scratch. Returns
 // false, with nothing changed, when a bucket holds more than 64 keys (clustered keys)
-// or the CTA is not 1024 threads; the caller then uses block_sort_pairs.
+// or the CTA's threads do not divide the buckets; the caller then uses block_sort_pairs.
 constexpr int BUCKETS = 2048;
 static __device__ bool block_bucket_sort(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1, uint32_t n,
-                                         BlockSortSmem& sm, ScanSmem& ss) {
+                                         BlockSortSmem& sm, ScanSmem& ss, bool known = false, uint32_t lowest = 0,
+                                         uint32_t highest = 0) {
   const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, w = tid >> 5;
-  if (2 * nt != BUCKETS) return false;     // two buckets per thread in the scan below
+  if (BUCKETS % nt != 0) return false;     // whole numbers of buckets per thread in the scan below
   uint32_t* cnt = &sm.whist[0][0];         // BUCKETS counts, then exclusive starts
   uint32_t* cur = cnt + BUCKETS;           // scatter cursors, then bucket ends
   uint32_t* red = cnt + 2 * BUCKETS;       // per-warp min / max / largest bucket
-  // key range
-  uint32_t mn = 0xFFFFFFFFu, mx = 0u;
-  for (uint32_t i = tid; i < n; i += nt) { mn = min(mn, k0[i]); mx = max(mx, k0[i]); }
-  mn = __reduce_min_sync(0xffffffffu, mn);
-  mx = __reduce_max_sync(0xffffffffu, mx);
-  if (lane == 0) { red[w] = mn; red[32 + w] = mx; }
+  // key range (`known`: every key lies in [lowest, highest])
+  uint32_t mn = lowest, mx = highest;
   for (int i = tid; i < BUCKETS; i += nt) cnt[i] = 0u;
+  if (!known) {
+    mn = 0xFFFFFFFFu; mx = 0u;
+    for (uint32_t i = tid; i < n; i += nt) { mn = min(mn, k0[i]); mx = max(mx, k0[i]); }
+    mn = __reduce_min_sync(0xffffffffu, mn);
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if (lane == 0) { red[w] = mn; red[32 + w] = mx; }
+  }
   __syncthreads();
-  mn = 0xFFFFFFFFu; mx = 0u;
-  for (int q = 0; q < (nt >> 5); ++q) { mn = min(mn, red[q]); mx = max(mx, red[32 + q]); }
+  if (!known) {
+    mn = 0xFFFFFFFFu; mx = 0u;
+    for (int q = 0; q < (nt >> 5); ++q) { mn = min(mn, red[q]); mx = max(mx, red[32 + q]); }
+  }
   const uint32_t range = n ? mx - mn : 0u;
   const int bits = range ? 32 - __clz(range) : 0;
   const int shift = bits > 11 ? bits - 11 : 0;
@@ -2003,15 +2073,21 @@ static __device__ bool block_bucket_sort(uint32_t* k0, uint32_t* v0, uint32_t* k
   for (int i = tid; i < BUCKETS; i += nt) big = max(big, cnt[i]);
   big = __reduce_max_sync(0xffffffffu, big);
   if (lane == 0) red[64 + w] = big;
-  // exclusive starts: each thread scans two consecutive buckets
-  const uint32_t c0 = cnt[2 * tid], c1 = cnt[2 * tid + 1];
+  // exclusive starts: each thread scans a few consecutive buckets
+  const int per = BUCKETS / nt;
+  uint32_t mine = 0;
+  for (int i = 0; i < per; ++i) mine += cnt[per * tid + i];
   uint32_t tot;
-  const uint32_t ex = block_excl_scan(c0 + c1, ss.warp_tot, &ss.total, tot);
+  uint32_t ex = block_excl_scan(mine, ss.warp_tot, &ss.total, tot);
   big = 0u;
   for (int q = 0; q < (nt >> 5); ++q) big = max(big, red[64 + q]);
   if (big > 64u) return false;  // uniform: every thread read the same values
-  cnt[2 * tid] = ex; cnt[2 * tid + 1] = ex + c0;
-  cur[2 * tid] = ex; cur[2 * tid + 1] = ex + c0;
+  for (int i = 0; i < per; ++i) {
+    const uint32_t c = cnt[per * tid + i];
+    cnt[per * tid + i] = ex;
+    cur[per * tid + i] = ex;
+    ex += c;
+  }
   __syncthreads();
   for (uint32_t i = tid; i < n; i += nt) {
     const uint32_t b = (k0[i] - mn) >> shift;
@@ -2107,6 +2183,25 @@ static __device__ int block_sort_pairs(uint32_t* k0, uint32_t* v0, uint32_t* k1,
   return parity;
 }
 
+// See SortOneSmem. Called by one CTA, after the histogram-free diffusion. (Gathering the state in
+// the same CTA, without the barrier in between, took 2 us longer than all CTAs' gather.)
+static __device__ void phase_sort_one(const Dev& d, SortOneSmem& so, BlockSortSmem& bs, ScanSmem& ss) {
+  const int tid = threadIdx.x, nt = blockDim.x;
+  const uint32_t n = d.g->n_total, first = d.n_trains == 1 ? d.trains[0].cell_base : 0u, last = d.g->sentinel_step;
+  if (!block_status_ok(d)) return;
+  for (uint32_t i = tid; i < n; i += nt) { so.k0[i] = d.keys0[i]; so.v0[i] = i; }
+  __syncthreads();
+  const bool bucketed = block_bucket_sort(so.k0, so.v0, so.k1, so.v1, n, bs, ss, true, first, last);
+  const int p = bucketed ? 0 : block_sort_pairs(so.k0, so.v0, so.k1, so.v1, n, bs);
+  const uint32_t* k = p ? so.k1 : so.k0;
+  const uint32_t* v = p ? so.v1 : so.v0;
+  for (uint32_t i = tid; i < n; i += nt) { d.keys1[i] = k[i]; d.vals1[i] = v[i]; }
+  if (tid == 0) {
+    d.g->sort_parity = 1u;
+    d.g->sort_any = 1u;
+  }
+}
+
 // Product-count prefix over the ordered events (`order`, optionally copied to
 // `order_out`), written to `pref`, plus each train's first prefix, event and product
 // counts.
@@ -2161,12 +2256,12 @@ struct SerialSmem {
 };
 
 // The one-CTA part of the react phase: conflict rounds, event order, product prefix.
-// With `sbuf` (4 * EV_SMEM_CAP words of shared memory) and at most EV_SMEM_CAP events
-// the sort runs in shared memory; otherwise in the global event buffers.
+// With at most EV_SMEM_CAP events the sort runs in `sbuf` (4 * EV_SMEM_CAP words of shared
+// memory), otherwise in the global event buffers.
 static __device__ void phase_react_serial(const Dev& d, SerialSmem& sm, uint32_t* sbuf) {
   const int tid = threadIdx.x, nt = blockDim.x;
   const uint32_t n_conflict = d.g->n_conflict;  // read before the rounds (all threads, uniform)
-  const bool rounds_smem = sbuf != nullptr && phase_match_rounds_smem(d, sm.match, sbuf);
+  const bool rounds_smem = phase_match_rounds_smem(d, sm.match, sbuf);
   if (!rounds_smem) phase_match_rounds(d, sm.match);
   const bool ok = block_status_ok(d);
   const uint32_t E = ok ? min(d.g->n_events, d.cap_cand) : 0u;
@@ -2180,9 +2275,9 @@ static __device__ void phase_react_serial(const Dev& d, SerialSmem& sm, uint32_t
     if (n_conflict > g->max_conflict) g->max_conflict = n_conflict;
     g->pairs_accepted += min(g->n_cand, d.cap_cand);
     if (E > g->max_events) g->max_events = E;
-    if (E > 0 && (sbuf == nullptr || E > static_cast<uint32_t>(EV_SMEM_CAP))) g->react_order_global += 1;
+    if (E > static_cast<uint32_t>(EV_SMEM_CAP)) g->react_order_global += 1;
   }
-  if (sbuf != nullptr && E <= static_cast<uint32_t>(EV_SMEM_CAP)) {
+  if (E <= static_cast<uint32_t>(EV_SMEM_CAP)) {
     uint32_t* k0 = sbuf;
     uint32_t* v0 = sbuf + EV_SMEM_CAP;
     uint32_t* k1 = sbuf + 2 * EV_SMEM_CAP;
@@ -2248,10 +2343,11 @@ __device__ __forceinline__ void write_event(const Dev& d, const Tables& tb, Prod
     const double rx = min_image(__dsub_rn(d.sx[cd.s_hi], xa), tr.L, tr.halfL);
     const double ry = min_image(__dsub_rn(d.sy[cd.s_hi], ya), tr.L, tr.halfL);
     const double rz = min_image(__dsub_rn(d.sz[cd.s_hi], za), tr.L, tr.halfL);
-    const double w = __ddiv_rn(tb.D[tlo], __dadd_rn(tb.D[tlo], tb.D[thi]));
-    const double px = wrap_box(__dadd_rn(xa, __dmul_rn(w, rx)), tr.L, tr.halfL);
-    const double py = wrap_box(__dadd_rn(ya, __dmul_rn(w, ry)), tr.L, tr.halfL);
-    const double pz = wrap_box(__dadd_rn(za, __dmul_rn(w, rz)), tr.L, tr.halfL);
+    const double w = tb.w_ab[r][static_cast<int>(tlo) == tb.rxn_a[r] ? 0 : 1];  // D_lo / (D_lo + D_hi)
+    double from_corner;
+    const double px = wrap_box_diffused(__dadd_rn(xa, __dmul_rn(w, rx)), tr.L, tr.halfL, from_corner);
+    const double py = wrap_box_diffused(__dadd_rn(ya, __dmul_rn(w, ry)), tr.L, tr.halfL, from_corner);
+    const double pz = wrap_box_diffused(__dadd_rn(za, __dmul_rn(w, rz)), tr.L, tr.halfL, from_corner);
     for (uint32_t q = 0; q < np; ++q) {
       const uint32_t pt = static_cast<uint32_t>(tb.prod[r][q]);
       d.sx[slot0 + q] = px; d.sy[slot0 + q] = py; d.sz[slot0 + q] = pz;
@@ -2331,21 +2427,35 @@ struct ReactAllSmem {
   uint32_t prods_tr[MAX_TRAINS], evs_tr[MAX_TRAINS];
   uint32_t n_prod;
 };
-// Bytes of sbuf for steps of up to `cap` accepted pairs (the rounds and the winners' keys); a
-// crowded step uses it for its block sort and scan.
+// Bytes of sbuf for steps of up to `cap` accepted pairs (the rounds; the winners' order then
+// takes the place of the pairs' keys, 20 of their 48 bytes a pair); a crowded step uses it for
+// its block sort and scan.
 __host__ __device__ constexpr size_t react_all_bytes(uint32_t cap) {
-  const size_t a = rc_smem_bytes(cap) + static_cast<size_t>(cap) * 8, b = sizeof(BlockSortSmem) + sizeof(ScanSmem);
+  const size_t a = rc_smem_bytes(cap), b = sizeof(BlockSortSmem) + sizeof(ScanSmem);
   return a > b ? a : b;
 }
 
 template <bool F32L>
-__device__ void phase_react_all(const Dev& d, ReactAllSmem& sm, uint32_t* sbuf, uint32_t cap) {
+__device__ void phase_react_all(const Dev& d, ReactAllSmem& sm, uint32_t* sbuf, uint32_t cap, const Tables& tb) {
   const int tid = threadIdx.x, nt = blockDim.x;
-  const Tables& tb = *d.tables;
-  const bool ok = block_status_ok(d);
   Global* g = d.g;
-  const uint32_t n_c = ok ? min(g->n_cand, d.cap_cand) : 0u;
-  const uint32_t n_live = g->n_total - g->n_dead;
+  // this thread's first pair is read with the counters, before it is known to be there
+  Cand mine{};
+  if (static_cast<uint32_t>(tid) < d.cap_cand) mine = d.cand[tid];
+  const uint32_t n_cand = g->n_cand, n_live = g->n_total - g->n_dead;
+  const bool ok = block_status_ok(d);
+  const uint32_t n_c = ok ? min(n_cand, d.cap_cand) : 0u;
+  if (static_cast<uint32_t>(tid) < n_c) {  // what the winners' events will read
+    prefetch_l1(&d.s4[mine.s_lo]);
+    prefetch_l1(&d.s4[mine.s_hi]);
+    prefetch_l1(&d.cell_sorted[mine.s_lo]);
+    prefetch_l1(&d.cell_sorted[mine.s_hi]);
+    if (!F32L) {
+      prefetch_l1(&d.sx[mine.s_lo]); prefetch_l1(&d.sy[mine.s_lo]); prefetch_l1(&d.sz[mine.s_lo]);
+      prefetch_l1(&d.sx[mine.s_hi]); prefetch_l1(&d.sy[mine.s_hi]); prefetch_l1(&d.sz[mine.s_hi]);
+      prefetch_l1(&d.stid[mine.s_lo]); prefetch_l1(&d.stid[mine.s_hi]);
+    }
+  }
   if (n_c > cap) {  // uniform
     phase_match_fast(d, 0u, 1u);
     __syncthreads();
@@ -2366,6 +2476,10 @@ __device__ void phase_react_all(const Dev& d, ReactAllSmem& sm, uint32_t* sbuf, 
     }
     products_prefix(d, scan, p ? d.ev_k1 : d.ev_k0, p ? d.ev_v1 : d.ev_v0, nullptr, p ? d.ev_k0 : d.ev_k1, E, ok2);
     phase_products<F32L>(d, sm.products, 0u, 1u);
+    for (uint32_t b = tid; b < d.n_trains; b += nt) {
+      sm.prods_tr[b] = d.trains[b].prods_step;
+      sm.evs_tr[b] = d.trains[b].n_events_step;
+    }
     __syncthreads();
     return;
   }
@@ -2375,10 +2489,10 @@ __device__ void phase_react_all(const Dev& d, ReactAllSmem& sm, uint32_t* sbuf, 
   __syncthreads();
   uint32_t E = 0u;
   if (n_c) {
-    const uint32_t* won = match_rounds_in_smem(d, sm.match, sbuf, n_c, nullptr);
+    const uint32_t* won = match_rounds_in_smem(d, sm.match, sbuf, n_c, nullptr, &mine);
     E = sm.match.n_won;
-    uint32_t* key = sbuf + rc_smem_bytes(cap) / 4;  // winners' (train, id_lo) keys and
-    uint32_t* np = key + cap;                       // product counts | train << 8
+    uint32_t* key = sbuf;       // winners' (train, id_lo) keys and
+    uint32_t* np = key + n_c;   // product counts | train << 8
     for (uint32_t q = tid; q < E; q += nt) {
       const Cand cd = d.cand[won[q]];
       const uint32_t b = cd.rxn_train >> 8, n = static_cast<uint32_t>(tb.n_prod[cd.rxn_train & 255u]);
@@ -2391,17 +2505,39 @@ __device__ void phase_react_all(const Dev& d, ReactAllSmem& sm, uint32_t* sbuf, 
       d.dead[cd.s_hi] = 1;
     }
     __syncthreads();
-    for (uint32_t q = tid; q < E; q += nt) {
-      const uint32_t mine = key[q], b = np[q] >> 8;
+    // eight lanes count a winner's smaller keys; then the events are written by consecutive
+    // threads in their order (FP64 instructions cost a warp the same for one lane as for 32)
+    uint32_t* at = np + n_c;        // winner at each place of the order,
+    uint32_t* pre = at + n_c;       // products before it, in all and
+    uint32_t* pre_tr = pre + n_c;   // of its train
+    for (uint32_t q0 = 0; q0 < E; q0 += static_cast<uint32_t>(nt) / 8u) {  // uniform (shuffles)
+      const uint32_t q = q0 + static_cast<uint32_t>(tid) / 8u;
+      const bool have = q < E;
+      const uint32_t k = have ? key[q] : 0u, b = have ? np[q] >> 8 : 0u;
       uint32_t rank = 0, before = 0, before_tr = 0;
-      for (uint32_t o = 0; o < E; ++o) {
-        const bool less = key[o] < mine;
+      for (uint32_t o = static_cast<uint32_t>(tid) & 7u; o < E; o += 8u) {
+        const bool less = key[o] < k;
         const uint32_t n = less ? np[o] : 0xFFFFFF00u;
         rank += less ? 1u : 0u;
         before += n & 255u;
         before_tr += (n >> 8) == b ? (n & 255u) : 0u;
       }
-      write_event<F32L>(d, tb, sm.products, d.cand[won[q]], n_live + before, d.trains[b].next_id + before_tr, rank);
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) {
+        rank += __shfl_xor_sync(0xffffffffu, rank, o);
+        before += __shfl_xor_sync(0xffffffffu, before, o);
+        before_tr += __shfl_xor_sync(0xffffffffu, before_tr, o);
+      }
+      if (have && (tid & 7) == 0) {
+        at[rank] = won[q];
+        pre[rank] = before;
+        pre_tr[rank] = before_tr;
+      }
+    }
+    __syncthreads();
+    for (uint32_t k = tid; k < E; k += nt) {
+      const Cand cd = d.cand[at[k]];
+      write_event<F32L>(d, tb, sm.products, cd, n_live + pre[k], d.trains[cd.rxn_train >> 8].next_id + pre_tr[k], k);
     }
     __syncthreads();
     add_tallies(d, sm.products);
@@ -2420,29 +2556,122 @@ __device__ void phase_react_all(const Dev& d, ReactAllSmem& sm, uint32_t* sbuf, 
   __syncthreads();
 }
 
+// The end of a step and the begin of the next, most of it ahead of time: while the other CTAs
+// search, one CTA takes a copy of the trains' records to the end of the step and plans the
+// next one on it (stage_next), and after reaction resolution only adds what depends on it and
+// writes the records back (commit_next). On the critical path the two took 6 us.
+constexpr uint32_t PLAN_TRAINS = 8;
+struct PlanSmem {
+  BeginSmem begin;
+  Train tr[PLAN_TRAINS];
+};
+
+static __device__ void stage_next(const Dev& d, PlanSmem& pl) {
+  const int tid = threadIdx.x, nt = blockDim.x;
+  const uint32_t words = d.n_trains * static_cast<uint32_t>(sizeof(Train) / 4);
+  const uint32_t* src = reinterpret_cast<const uint32_t*>(d.trains);
+  uint32_t* dst = reinterpret_cast<uint32_t*>(pl.tr);
+  for (uint32_t i = tid; i < words; i += nt) dst[i] = src[i];
+  __syncthreads();
+  if (static_cast<uint32_t>(tid) < d.n_trains) {
+    Train& tr = pl.tr[tid];
+    if (tr.active) {
+      tr.species_steps += tr.n_live_step;
+      tr.t = tr.t_next;
+      tr.step += 1;
+      tr.dt_cur = fmin(__dmul_rn(tr.dt_cur, tr.dt_growth), tr.dt_max);
+      tr.n_ref = tr.n;
+      tr.h_ref = tr.h;
+      tr.cb_ref = tr.cb;
+    }
+  }
+  __syncthreads();
+  begin_plan(d, pl.begin, pl.tr, 0);
+}
+
+// Step record of an advancing train (before its record moves on).
+__device__ __forceinline__ void log_step(const Dev& d, const Train& tr, uint32_t b, uint32_t n_events) {
+  const uint32_t e = atomicAdd(&d.g->step_log_n, 1u);
+  if (e >= d.cap_step_log) {
+    raise_status(d.g, CHEM_ECAPACITY);
+    return;
+  }
+  chem_step_record rec;
+  rec.step = tr.step; rec.train = b; rec.t_start_s = tr.t_start; rec.dt_s = tr.dt;
+  rec.n_live = tr.n_live_step; rec.n_events = n_events;
+  for (int q = 0; q < 8; ++q) rec.counts[q] = q < d.tables->n_types ? tr.counts[q] : 0;
+  d.step_log[e] = rec;
+}
+
+// After phase_react_all; false, with nothing done, when an error is raised.
+static __device__ bool commit_next(const Dev& d, PlanSmem& pl, const ReactAllSmem& ra) {
+  const int tid = threadIdx.x, nt = blockDim.x;
+  if (!block_status_ok(d)) return false;
+  Global* g = d.g;
+  const uint32_t b = static_cast<uint32_t>(tid);
+  bool stepped = false;
+  if (b < d.n_trains && d.trains[b].active) {
+    stepped = true;
+    if (d.cap_step_log) log_step(d, d.trains[b], b, ra.evs_tr[b]);
+    pl.begin.live[b] += static_cast<long long>(ra.prods_tr[b]) - 2ll * static_cast<long long>(ra.evs_tr[b]);
+    pl.tr[b].next_id += ra.prods_tr[b];
+  }
+  const bool any = __syncthreads_or(stepped ? 1 : 0) != 0;
+  if (tid == 0) {
+    if (any) g->steps_active += 1;
+    g->n_total = g->n_total - g->n_dead + g->n_products;
+    if (d.cap_ev_log) g->ev_log_n += g->n_events;
+  }
+  __syncthreads();
+  begin_commit(d, pl.begin, pl.tr);  // (ends with a barrier)
+  // everything but the tallies, which the reactions added to
+  constexpr uint32_t W = sizeof(Train) / 4, T0 = offsetof(Train, water) / 4, T1 = offsetof(Train, n_ref) / 4;
+  const uint32_t* src = reinterpret_cast<const uint32_t*>(pl.tr);
+  uint32_t* dst = reinterpret_cast<uint32_t*>(d.trains);
+  for (uint32_t i = tid; i < d.n_trains * W; i += nt) {
+    const uint32_t w = i % W;
+    if (w < T0 || w >= T1) dst[i] = src[i];
+  }
+  return true;
+}
+
+// Species the next step will work on (stepped slots and what its begin will release), for the
+// host's choice of the launch form; between steps, one CTA of at least MAX_TRAINS threads.
+static __device__ void phase_look_ahead(const Dev& d, EndSmem& sm) {
+  const uint32_t b = threadIdx.x;
+  __syncthreads();
+  if (b == 0) sm.ahead = d.g->n_total;
+  __syncthreads();
+  if (b < d.n_trains) {
+    const Train& tr = d.trains[b];
+    if (tr.t < tr.t_end) {
+      uint32_t lo = tr.p_head, hi = tr.p_tail;
+      if (tr.next_arr <= tr.t) {
+        const double* pt = d.pt + tr.pend_base;
+        while (lo < hi) {
+          const uint32_t mid = (lo + hi) >> 1;
+          if (pt[mid] <= tr.t) lo = mid + 1; else hi = mid;
+        }
+      }
+      const uint32_t more = tr.park_n + tr.mat_n + (lo - tr.p_head);
+      if (more) atomicAdd(&sm.ahead, more);
+    }
+  }
+  __syncthreads();
+  if (b == 0) d.g->n_ahead = sm.ahead;
+}
+
 static __device__ void phase_end_step(const Dev& d, EndSmem& sm) {
   const int tid = threadIdx.x, nt = blockDim.x;
   if (tid == 0) { sm.any = 0; sm.stepped = 0; }
   const bool ok = block_status_ok(d);
-  const Tables& tb = *d.tables;
   for (uint32_t b = tid; b < d.n_trains; b += nt) {
     Train& tr = d.trains[b];
     if (tr.active && ok) {
       atomicOr(&sm.stepped, 1u);
       tr.next_id += tr.prods_step;
       tr.species_steps += tr.n_live_step;
-      if (d.cap_step_log) {
-        const uint32_t e = atomicAdd(&d.g->step_log_n, 1u);
-        if (e < d.cap_step_log) {
-          chem_step_record rec;
-          rec.step = tr.step; rec.train = b; rec.t_start_s = tr.t_start; rec.dt_s = tr.dt;
-          rec.n_live = tr.n_live_step; rec.n_events = tr.n_events_step;
-          for (int q = 0; q < 8; ++q) rec.counts[q] = q < tb.n_types ? tr.counts[q] : 0;
-          d.step_log[e] = rec;
-        } else {
-          raise_status(d.g, CHEM_ECAPACITY);
-        }
-      }
+      if (d.cap_step_log) log_step(d, tr, b, tr.n_events_step);
       tr.t = tr.t_next;
       tr.step += 1;
       tr.dt_cur = fmin(__dmul_rn(tr.dt_cur, tr.dt_growth), tr.dt_max);

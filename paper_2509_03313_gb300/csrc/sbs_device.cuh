@@ -17,6 +17,7 @@
 //    pair search tests it before reading an entry. A stale bit only costs a lookup:
 //    the entry's epoch stamp still decides.
 #pragma once
+#include <cstddef>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -30,12 +31,17 @@ constexpr int MAX_TRAINS = 256;
 constexpr int RADIX = 256;
 constexpr int MAX_PASSES = 4;
 constexpr int SORT_THREADS = 512;    // threads of the per-pass sort kernel
-constexpr int PERSIST_THREADS = 256; // threads of the persistent step kernel
+constexpr int PERSIST_THREADS = 512; // threads of the persistent step kernel, one CTA per SM
+constexpr int STEP_CLUSTER = 16;     // CTAs of its one-cluster form
 constexpr int SORT_ITEMS = 15;
 constexpr int GATHER_BATCH = 4;   // slots per thread and iteration of the gather
 constexpr int S4_SPARE = 8;       // spare entries of s4 past its end: the search loads whole batches
-// the smallest sort tile (persistent kernel): sizes the look-back buffer
-constexpr int SORT_TILE_MIN = PERSIST_THREADS * SORT_ITEMS;
+// sorts of several tiles: tiles of at least SORT_ROWS_MIN rows of keys (a row is a key per
+// thread), about SORT_MANY_TILES of them until a tile is full
+constexpr uint32_t SORT_ROWS_MIN = 4;
+constexpr uint32_t SORT_MANY_TILES = 24;
+// the smallest such tile (persistent kernel): sizes the look-back buffer
+constexpr int SORT_TILE_MIN = PERSIST_THREADS * static_cast<int>(SORT_ROWS_MIN);
 constexpr int REACT_THREADS = 1024;
 constexpr int ITEM_HOME = 32;   // most home species per pair-search work item (one cell)
 // Contexts of at most this many species run a step as few launches (one search kernel, one
@@ -61,6 +67,7 @@ struct Tables {
   int prod[MAXR][3];
   int water[MAXR];
   int rxn_a[MAXR], rxn_b[MAXR]; // reactant types of each reaction
+  double w_ab[MAXR][2];         // D_a / (D_a + D_b) and D_b / (D_b + D_a): encounter point from a, from b
   double k_tab[MAXR];           // rate constant as tabulated (L mol^-1 s^-1; self: 2k)
 };
 
@@ -150,7 +157,7 @@ struct Global {
   uint32_t ev_log_n, step_log_n;
   uint32_t hist[MAX_PASSES][RADIX];
   uint32_t tile_ctr[MAX_PASSES];
-  uint32_t bar_count, bar_gen;  // grid barrier of the persistent launch
+  uint32_t bar_count, bar_left;  // grid barrier of the persistent launch: arrivals, CTAs that left
   uint32_t err_where;
   uint32_t steps_active;  // steps in which at least one train advanced
   uint32_t n_items;       // pair-search work items emitted by the gather
@@ -174,6 +181,7 @@ struct Global {
   unsigned long long pairs_in_cutoff;  // of them, reacting type pairs inside the cutoff
   unsigned long long pairs_accepted;   // of them, accepted (the steps' reactive pairs)
   unsigned long long incut_mark;       // pairs_in_cutoff when the last step began
+  uint32_t n_ahead;                    // species the next step will work on (launch form)
   uint32_t cells_steps;                // steps searched with cell tiles (cumulative)
   uint32_t sentinel_step;              // key of removed species this step: above every cell
                                        // key of the step (one train: the unused all-ones cell)
@@ -231,6 +239,8 @@ struct Dev {
 __device__ __forceinline__ void raise_status(Global* g, int code) {
   atomicCAS(&g->status, 0, code);
 }
+
+__device__ __forceinline__ void prefetch_l1(const void* p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
 
 __device__ __forceinline__ uint32_t tid_type(uint32_t tid) { return tid & 7u; }
 __device__ __forceinline__ uint32_t tid_id(uint32_t tid) { return tid >> 3; }
