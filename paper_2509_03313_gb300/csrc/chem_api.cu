@@ -64,13 +64,6 @@ struct PendingHost {
   void release() { buf[0].release(); buf[1].release(); n = 0; }
 };
 
-// Launch form by the species the next steps will work on. 64 steps of a uniform mixture and
-// whole track trajectories, ms as one cluster / one CTA per SM / per-phase kernels:
-//   2,000 species 2.04 / 2.19 / 3.36, 4,000 2.96 / 2.76 / 4.12, 32,000 7.1 / 4.3 / 5.2,
-//   200,000 - / 9.7 / 10.2; tracks 32,000 14.8 / 6.9 / 8.1, 176,000 - / 17.3 / 19.4.
-constexpr uint32_t CLUSTER_SPECIES = 2560;
-constexpr uint32_t GRID_SPECIES = 1u << 18;
-
 struct TrainHost {
   chem_config cfg;
   double E_dep = 0.0;
@@ -256,13 +249,16 @@ chem_status upload_mapping(chem_ctx* ctx, int ih) {
   return CHEM_OK;
 }
 
-chem_status init_global(chem_ctx* ctx) {
+// All counters to 0 but the step epoch, which goes on from `epoch`.
+chem_status init_global(chem_ctx* ctx, uint32_t epoch) {
   ctx->seen_rounds_global = ctx->seen_order_global = ctx->seen_order_radix = 0;
   ctx->seen_tested = ctx->seen_in_cut = ctx->seen_accepted = 0;
   ctx->seen_steps = 0;
   ctx->seen_cells_steps = 0;
   CK(cudaMemsetAsync(ctx->d.g, 0, sizeof(Global), ctx->stream));
-  return upload_mapping(ctx, ctx->item_home);
+  if (epoch)
+    CK(cudaMemcpyAsync(&ctx->d.g->epoch, &epoch, sizeof(epoch), cudaMemcpyHostToDevice, ctx->stream));
+  return upload_mapping(ctx, ctx->item_home);  // (synchronises)
 }
 
 // Fold the device's counters (reaction-resolution branches, pair-search work, steps;
@@ -354,10 +350,11 @@ int sort_passes(const chem_ctx* ctx) {
 enum Form { FORM_PHASES, FORM_GRID, FORM_CLUSTER };
 Form choose_form(const chem_ctx* ctx, uint32_t n) {
   if (ctx->launch_mode == CHEM_LAUNCH_PHASES) return FORM_PHASES;
-  if (ctx->launch_mode == CHEM_LAUNCH_AUTO && (ctx->profiling || n > GRID_SPECIES)) return FORM_PHASES;
-  return ctx->lc.cluster_blocks > 0 && n <= CLUSTER_SPECIES ? FORM_CLUSTER : FORM_GRID;
+  if (ctx->launch_mode == CHEM_LAUNCH_AUTO && (ctx->profiling || n > static_cast<uint32_t>(GRID_SPECIES))) return FORM_PHASES;
+  return ctx->lc.cluster_blocks > 0 && n <= static_cast<uint32_t>(CLUSTER_SPECIES) ? FORM_CLUSTER : FORM_GRID;
 }
 
+constexpr uint32_t EPOCH_MAX = 1u << 26;  // look-back words hold 30 bits of 8 x the epoch
 constexpr int AUTO_STEPS = 16;
 int steps_of(const chem_ctx* ctx, Form f) {
   if (ctx->steps_per_launch > 0) return ctx->steps_per_launch;
@@ -1070,7 +1067,7 @@ chem_status chem_batch_init(const chem_config* cfgs, int32_t n_trains, chem_ctx*
   CK(cudaMemsetAsync(d.occ, 0, static_cast<size_t>(d.occ_vec4) * 16, ctx->stream));
   CK(cudaMemsetAsync(d.lookback, 0, static_cast<size_t>(d.max_tiles) * RADIX * 8, ctx->stream));
   CK(cudaMemcpyAsync(tables_dev, &T, sizeof(Tables), cudaMemcpyHostToDevice, ctx->stream));
-  chem_status gs = init_global(ctx);
+  chem_status gs = init_global(ctx, 0u);
   if (gs) return gs;
   return upload_trains(ctx, tr);
 }
@@ -1243,13 +1240,22 @@ chem_status chem_batch_reset(chem_ctx* ctx, const uint64_t* seeds) {
     h.pend.clear();
     init_train_dynamic(tr[b], h.cfg, tr[b].n_alloc);
   }
-  s = init_global(ctx);
+  // The step epoch goes on, so stale hash stamps and look-back words never match and the large
+  // tables (2 GB of hash cells for a million species, 0.37 ms) keep their contents. After an
+  // error, or towards the end of the epoch's range, everything is cleared.
+  uint32_t epoch = 0;
+  CK(cudaMemcpyAsync(&epoch, &ctx->d.g->epoch, sizeof(epoch), cudaMemcpyDeviceToHost, ctx->stream));
+  CK(cudaStreamSynchronize(ctx->stream));
+  const bool clear = ctx->status != CHEM_OK || epoch >= EPOCH_MAX;
+  s = init_global(ctx, clear ? 0u : epoch + 1u);
   if (s) return s;
   CK(cudaMemsetAsync(ctx->d.dead, 0, ctx->d.cap, ctx->stream));
   CK(cudaMemsetAsync(ctx->d.touch, 0, static_cast<size_t>(ctx->d.cap) * 4, ctx->stream));
-  CK(cudaMemsetAsync(ctx->d.cell_info, 0xFF, (static_cast<size_t>(ctx->d.total_cells) + 1) * 16, ctx->stream));
   CK(cudaMemsetAsync(ctx->d.occ, 0, static_cast<size_t>(ctx->d.occ_vec4) * 16, ctx->stream));
-  CK(cudaMemsetAsync(ctx->d.lookback, 0, static_cast<size_t>(ctx->d.max_tiles) * RADIX * 8, ctx->stream));
+  if (clear) {
+    CK(cudaMemsetAsync(ctx->d.cell_info, 0xFF, (static_cast<size_t>(ctx->d.total_cells) + 1) * 16, ctx->stream));
+    CK(cudaMemsetAsync(ctx->d.lookback, 0, static_cast<size_t>(ctx->d.max_tiles) * RADIX * 8, ctx->stream));
+  }
   s = upload_trains(ctx, tr);
   if (s) return s;
   ctx->status = CHEM_OK;

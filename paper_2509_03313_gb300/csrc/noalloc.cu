@@ -33,7 +33,7 @@ constexpr size_t align256(size_t x) { return (x + 255) & ~static_cast<size_t>(25
 struct Layout {
   size_t sx, sy, sz, stid, tx, ty, tz, ttid, tdx, tdy, tdz, s4, t4, items, touch, cell_sorted, sortbuf, dead, cell_info, occ, lookback, cand,
       ev_list, alive0, alive1, ev_k0, ev_k1, ev_v0, ev_v1, ev_log, step_log, pend, trains, tables,
-      global, total;
+      global, last_epoch, total;
 };
 
 constexpr Layout make_layout() {
@@ -62,6 +62,7 @@ constexpr Layout make_layout() {
   L.trains = take(sizeof(Train));
   L.tables = take(sizeof(Tables));
   L.global = take(sizeof(Global));
+  L.last_epoch = take(4);
   L.total = o;
   return L;
 }
@@ -76,19 +77,39 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[NOALLOC_SCRATCH
 
 namespace {
 
-// Device address of g_noalloc_scratch per device, looked up once per device.
-std::mutex g_addr_mu;
-void* g_addr[64] = {};
+// Per device, looked up once: the address of g_noalloc_scratch, the multiprocessors and the
+// launch shapes of the step's kernel.
+struct DeviceInfo {
+  void* scratch = nullptr;
+  int sms = 0, per_sm = 0, cluster = 0;
+};
+std::mutex g_info_mu;
+DeviceInfo g_info[64];
 
-__global__ void k_noalloc_setup(Dev d, Tables tb, Train tr) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    *const_cast<Tables*>(d.tables) = tb;
-    *d.trains = tr;
-    Global g;
-    std::memset(&g, 0, sizeof(g));
-    g.item_home = 0;  // several lanes per home species (few species)
-    *d.g = g;
+// Leftovers of the previous call: its step epoch goes on (stale hash stamps and look-back words
+// then never match, so the large tables are not cleared), the occupancy bits and the accepted
+// pairs per slot are cleared. `last_epoch` keeps the epoch of the last call; near the end of
+// its range everything is cleared and it starts again.
+constexpr uint32_t NA_EPOCH_MAX = 1u << 26;
+__global__ void k_noalloc_setup(const __grid_constant__ Dev d, const __grid_constant__ Tables tb,
+                                const __grid_constant__ Train tr, const uint32_t* last_epoch) {
+  const uint32_t i0 = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
+  const uint32_t epoch = *last_epoch;
+  const bool again = epoch >= NA_EPOCH_MAX;
+  for (uint32_t i = i0; i < 4u * d.occ_vec4; i += stride) d.occ[i] = 0u;
+  for (uint32_t i = i0; i < NA_MAX_SPECIES; i += stride) d.touch[i] = 0u;
+  if (again) {
+    for (uint32_t i = i0; i <= NA_CELLS; i += stride) d.cell_info[i] = make_int4(-1, -1, -1, -1);
+    for (uint32_t i = i0; i < NA_TILES * RADIX; i += stride) d.lookback[i] = 0ull;
   }
+  // the records, a word per thread (all fields of Global start at 0 but the epoch; item_home 0:
+  // several lanes per home species)
+  const uint32_t* tb_w = reinterpret_cast<const uint32_t*>(&tb);
+  const uint32_t* tr_w = reinterpret_cast<const uint32_t*>(&tr);
+  for (uint32_t i = i0; i < sizeof(Tables) / 4; i += stride) reinterpret_cast<uint32_t*>(const_cast<Tables*>(d.tables))[i] = tb_w[i];
+  for (uint32_t i = i0; i < sizeof(Train) / 4; i += stride) reinterpret_cast<uint32_t*>(d.trains)[i] = tr_w[i];
+  for (uint32_t i = i0; i < sizeof(Global) / 4; i += stride)
+    reinterpret_cast<uint32_t*>(d.g)[i] = i == offsetof(Global, epoch) / 4 ? (again ? 0u : epoch) : 0u;
 }
 
 // Copy the caller's species into the scratch state. The inputs live on the device, so
@@ -96,10 +117,11 @@ __global__ void k_noalloc_setup(Dev d, Tables tb, Train tr) {
 // would overlap the type bits) or a position that is not finite and inside [-L/2, L/2)^3
 // raises CHEM_EINVAL and is not written; every later phase then does nothing and the
 // store kernel reports no species and no events.
-__global__ void k_noalloc_load(Dev d, int32_t n, const uint32_t* id, const int32_t* type,
-                               const double* xyz) {
+__global__ void k_noalloc_load(const __grid_constant__ Dev d, int32_t n, const uint32_t* id, const int32_t* type,
+                               const double* xyz, uint32_t* last_epoch) {
   const Train& tr = d.trains[0];
   const int n_types = d.tables->n_types;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *last_epoch = d.g->epoch + 1u;  // (the step's)
   for (int32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x) {
     const int32_t ty = type[s];
     const uint32_t ids = id[s];
@@ -123,7 +145,7 @@ __global__ void k_noalloc_load(Dev d, int32_t n, const uint32_t* id, const int32
 }
 
 // Copy the live species (slot order) and this step's events to the caller's buffers.
-__global__ void k_noalloc_store(Dev d, uint32_t* id_out, int32_t* type_out, double* xyz_out,
+__global__ void __launch_bounds__(1024) k_noalloc_store(const __grid_constant__ Dev d, uint32_t* id_out, int32_t* type_out, double* xyz_out,
                                 int32_t* n_out, uint32_t* next_id_out, chem_event* ev_out,
                                 int32_t* n_ev_out) {
   __shared__ uint32_t warp_tot[32];
@@ -169,22 +191,26 @@ __global__ void k_noalloc_store(Dev d, uint32_t* id_out, int32_t* type_out, doub
   }
 }
 
-chem_status scratch_address(void** out) {
+chem_status device_info(DeviceInfo* out) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
     cudaGetLastError();
     return CHEM_ECUDA;
   }
-  std::lock_guard<std::mutex> lock(g_addr_mu);
-  if (!g_addr[dev]) {
+  std::lock_guard<std::mutex> lock(g_info_mu);
+  if (!g_info[dev].scratch) {
+    DeviceInfo f;
     void* p = nullptr;
-    if (cudaGetSymbolAddress(&p, g_noalloc_scratch) != cudaSuccess || !p) {
+    if (cudaGetSymbolAddress(&p, g_noalloc_scratch) != cudaSuccess || !p ||
+        cudaDeviceGetAttribute(&f.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || f.sms < 1 ||
+        step_kernel_limits_f64(&f.per_sm, &f.cluster) != cudaSuccess || f.per_sm < 1) {
       cudaGetLastError();
       return CHEM_ECUDA;
     }
-    g_addr[dev] = p;
+    f.scratch = p;
+    g_info[dev] = f;
   }
-  *out = g_addr[dev];
+  *out = g_info[dev];
   return CHEM_OK;
 }
 
@@ -273,9 +299,9 @@ extern "C" chem_status chem_step_noalloc(const chem_config* cfg, uint32_t step, 
   tr.n_ref = NA_CELLS_AXIS;
   tr.h_ref = cfg->L_nm / NA_CELLS_AXIS;
 
-  void* base = nullptr;
-  if (scratch_address(&base) != CHEM_OK) return CHEM_ECUDA;
-  unsigned char* b = static_cast<unsigned char*>(base);
+  DeviceInfo info;
+  if (device_info(&info) != CHEM_OK) return CHEM_ECUDA;
+  unsigned char* b = static_cast<unsigned char*>(info.scratch);
   Dev d;
   std::memset(&d, 0, sizeof(d));
   d.cap = NA_MAX_SPECIES;
@@ -332,33 +358,18 @@ extern "C" chem_status chem_step_noalloc(const chem_config* cfg, uint32_t step, 
   d.tables = reinterpret_cast<const Tables*>(b + LAYOUT.tables);
   d.g = reinterpret_cast<Global*>(b + LAYOUT.global);
 
-  int dev = 0, sms = 0, sort_occ = 0, pers_occ = 0, cluster = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-      sort_pass_occupancy(&sort_occ) != cudaSuccess || step_kernel_limits_f64(&pers_occ, &cluster) != cudaSuccess || sms < 1 ||
-      sort_occ < 1) {
-    cudaGetLastError();
-    return CHEM_ECUDA;
-  }
   LaunchCfg lc;
-  lc.stream_blocks = std::max(1, std::min(sms * 2, (n + 255) / 256 + 1));
-  lc.search_blocks = sms * 4;
-  lc.sort_blocks = std::min(sms * sort_occ, static_cast<int>(NA_TILES));
-  lc.persistent_blocks = sms;
-  lc.cluster_blocks = cluster;
-  lc.search_tps = 0;
-  lc.small = 1;
+  std::memset(&lc, 0, sizeof(lc));
+  lc.persistent_blocks = info.sms;
+  lc.cluster_blocks = info.cluster;
   cudaStream_t s = static_cast<cudaStream_t>(cfg->cuda_stream);
-  // leftovers of the previous call: stale hash cells and look-back words must not match
-  bool ok = cudaMemsetAsync(d.cell_info, 0xFF, (NA_CELLS + 1) * 16, s) == cudaSuccess &&
-            cudaMemsetAsync(d.occ, 0, (NA_CELLS + 127) / 128 * 16, s) == cudaSuccess &&
-            cudaMemsetAsync(d.touch, 0, NA_MAX_SPECIES * 4, s) == cudaSuccess &&
-            cudaMemsetAsync(d.lookback, 0, static_cast<size_t>(NA_TILES) * RADIX * 8, s) == cudaSuccess;
-  if (ok) {
-    k_noalloc_setup<<<1, 1, 0, s>>>(d, tb, tr);
-    k_noalloc_load<<<lc.stream_blocks, 256, 0, s>>>(d, n, id, type, xyz);
-    ok = cudaGetLastError() == cudaSuccess && enqueue_step_f64(d, lc, s, nullptr, true, true) == cudaSuccess;
-  }
+  uint32_t* last_epoch = reinterpret_cast<uint32_t*>(b + LAYOUT.last_epoch);
+  const int blocks = std::max(8, std::min(info.sms, (n + 255) / 256));
+  k_noalloc_setup<<<info.sms, 256, 0, s>>>(d, tb, tr, last_epoch);
+  k_noalloc_load<<<blocks, 256, 0, s>>>(d, n, id, type, xyz, last_epoch);
+  // one step of the persistent kernel: one cluster, or one CTA per multiprocessor
+  const bool cluster = info.cluster > 0 && n <= CLUSTER_SPECIES;
+  bool ok = cudaGetLastError() == cudaSuccess && enqueue_steps_f64(d, lc, cluster, 1, 1, s) == cudaSuccess;
   if (ok) {
     k_noalloc_store<<<1, 1024, 0, s>>>(d, id_out, type_out, xyz_out, n_out, next_id_out, events_out,
                                        n_events_out);

@@ -49,6 +49,12 @@ constexpr int ITEM_HOME = 32;   // most home species per pair-search work item (
 // resolution to the next begin took 22 to 33 us as four kernels and takes 10 to 24 as one; the
 // 1e6-species benchmark has up to 6,800 events a step, more than one CTA should order.
 constexpr long long SMALL_SPECIES = 1ll << 18;
+// Launch form by the species the next steps will work on. 64 steps of a uniform mixture and
+// whole track trajectories, ms as one cluster / one CTA per SM / per-phase kernels:
+//   2,000 species 2.04 / 2.19 / 3.36, 4,000 2.96 / 2.76 / 4.12, 32,000 7.1 / 4.3 / 5.2,
+//   200,000 - / 9.7 / 10.2; tracks 32,000 14.8 / 6.9 / 8.1, 176,000 - / 17.3 / 19.4.
+constexpr int32_t CLUSTER_SPECIES = 2560;
+constexpr int32_t GRID_SPECIES = 1 << 18;
 constexpr int N_FWD = 14;       // own cell + 13 forward neighbour cells (half shell)
 constexpr double END_SLACK = 1.0 + 1e-6;    // last-step trim slack (relative)
 constexpr float CELL_SLACK_F = 1.0001f;    // hash cell >= cutoff * CELL_SLACK_F
