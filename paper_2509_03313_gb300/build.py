@@ -25,6 +25,7 @@ UNITS = {
     "kernels_f32l.cu": [],
     "noalloc.cu": ["--fmad=false"],
     "homog.cu": [],
+    "state.cu": ["--fmad=false"],
 }
 
 

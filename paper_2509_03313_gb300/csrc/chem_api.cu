@@ -706,77 +706,49 @@ chem_status state_one(chem_ctx* ctx, int b, int64_t cap, int32_t* type, uint32_t
   std::vector<Train> tr;
   s = download_trains(ctx, tr);
   if (s) return s;
-  const uint32_t n_slots = ctx->g_pinned->n_total;
   // the stepped slots, then the train's parked species (idle trains of a batch)
-  const uint32_t np = ctx->d.pk_cell ? tr[b].park_n : 0u, pb = tr[b].park_base;
-  const uint32_t n = n_slots + np;
-  std::vector<uint8_t> dead(n, 0);
-  std::vector<uint32_t> cell(n), tid(n);
-  std::vector<double> x(n), y(n), z(n);
-  std::vector<float4> v4;
-  if (ctx->precision != CHEM_FP64) v4.resize(n);
-  if (n_slots) {
-    CK(cudaMemcpy(dead.data(), ctx->d.dead, n_slots, cudaMemcpyDeviceToHost));
-    CK(cudaMemcpy(cell.data(), ctx->d.cell_sorted, n_slots * 4, cudaMemcpyDeviceToHost));
-    if (ctx->precision == CHEM_FP64) {
-      CK(cudaMemcpy(tid.data(), ctx->d.stid, n_slots * 4, cudaMemcpyDeviceToHost));
-      CK(cudaMemcpy(x.data(), ctx->d.sx, n_slots * 8, cudaMemcpyDeviceToHost));
-      CK(cudaMemcpy(y.data(), ctx->d.sy, n_slots * 8, cudaMemcpyDeviceToHost));
-      CK(cudaMemcpy(z.data(), ctx->d.sz, n_slots * 8, cudaMemcpyDeviceToHost));
-    } else {
-      CK(cudaMemcpy(v4.data(), ctx->d.s4, n_slots * 16, cudaMemcpyDeviceToHost));
-    }
+  const uint32_t n_slots = ctx->g_pinned->n_total;
+  const uint32_t n = n_slots + (ctx->d.pk_cell ? tr[b].park_n : 0u);
+  // between steps the diffused state and the sort's buffers hold nothing: the packed species
+  // and the chunks' counts go there
+  const Dev& d = ctx->d;
+  const size_t cap_slots = d.cap;
+  auto rows_of = [](size_t bytes) { return static_cast<uint32_t>(((bytes + 255) & ~static_cast<size_t>(255)) / 24); };
+  PackOut out{};
+  out.id = d.vals0;
+  out.type = reinterpret_cast<int32_t*>(d.vals1);
+  out.xyz[0] = reinterpret_cast<double*>(d.t4);
+  out.rows[0] = rows_of(cap_slots * 16);
+  if (ctx->precision == CHEM_FP64) {
+    out.xyz[1] = d.tx;
+    out.xyz[2] = d.ty;
+    out.rows[1] = out.rows[2] = rows_of(cap_slots * 8);
+  } else {
+    out.xyz[1] = reinterpret_cast<double*>(d.td4);
+    out.rows[1] = rows_of(cap_slots * 16);
   }
-  if (np) {
-    CK(cudaMemcpy(cell.data() + n_slots, ctx->d.pk_cell + pb, np * 4, cudaMemcpyDeviceToHost));
-    if (ctx->precision == CHEM_FP64) {
-      CK(cudaMemcpy(tid.data() + n_slots, ctx->d.pk_tid + pb, np * 4, cudaMemcpyDeviceToHost));
-      CK(cudaMemcpy(x.data() + n_slots, ctx->d.pkx + pb, np * 8, cudaMemcpyDeviceToHost));
-      CK(cudaMemcpy(y.data() + n_slots, ctx->d.pky + pb, np * 8, cudaMemcpyDeviceToHost));
-      CK(cudaMemcpy(z.data() + n_slots, ctx->d.pkz + pb, np * 8, cudaMemcpyDeviceToHost));
-    } else {
-      CK(cudaMemcpy(v4.data() + n_slots, ctx->d.pk4 + pb, np * 16, cudaMemcpyDeviceToHost));
+  uint32_t* counts = d.keys0;  // (a word per 1,024 slots: keys0 and keys1 hold two per slot)
+  const uint32_t chunks = pack_counts(n);
+  CK(enqueue_pack_count(d, static_cast<uint32_t>(b), n_slots, n, counts, ctx->stream));
+  uint32_t live = 0;
+  CK(cudaMemcpyAsync(&live, counts + chunks, sizeof(live), cudaMemcpyDeviceToHost, ctx->stream));
+  CK(cudaStreamSynchronize(ctx->stream));
+  const uint32_t k = static_cast<uint32_t>(std::min<int64_t>(live, cap));
+  if (k && (type || id || xyz)) {
+    CK(enqueue_pack_write(d, static_cast<uint32_t>(b), n_slots, n, counts, out, ctx->stream));
+    if (type) CK(cudaMemcpyAsync(type, out.type, k * sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
+    if (id) CK(cudaMemcpyAsync(id, out.id, k * sizeof(uint32_t), cudaMemcpyDeviceToHost, ctx->stream));
+    uint32_t row = 0;
+    for (uint32_t q = 0; xyz && q < PackOut::SEGS && row < k; ++q) {
+      const uint32_t m = std::min(k - row, out.rows[q]);
+      if (m) CK(cudaMemcpyAsync(xyz + 3 * static_cast<size_t>(row), out.xyz[q], m * 3 * sizeof(double),
+                                cudaMemcpyDeviceToHost, ctx->stream));
+      row += m;
     }
+    CK(cudaStreamSynchronize(ctx->stream));
   }
-  int64_t k = 0;
-  for (uint32_t i = 0; i < n; ++i) {
-    if (dead[i]) continue;
-    // train of the slot from its cell
-    int tb = 0;
-    for (int q = ctx->B - 1; q >= 0; --q)
-      if (tr[q].cell_base <= cell[i]) { tb = q; break; }
-    if (tb != b) continue;
-    const Train& t = tr[b];
-    uint32_t tt;
-    double px, py, pz;
-    if (ctx->precision == CHEM_FP64) {
-      tt = tid[i]; px = x[i]; py = y[i]; pz = z[i];
-    } else {
-      std::memcpy(&tt, &v4[i].w, 4);
-      const uint32_t loc = cell[i] - t.cell_base;
-      const uint32_t m = (1u << t.cb_ref) - 1u;  // the grid of the last step
-      const double h = t.h_ref;
-      const int ix = static_cast<int>(loc & m), iy = static_cast<int>((loc >> t.cb_ref) & m),
-                iz = static_cast<int>(loc >> (2 * t.cb_ref));
-      auto wrapb = [&](double q) {
-        q -= t.L * std::floor((q + t.halfL) / t.L);
-        if (q >= t.halfL) q -= t.L;
-        if (q < -t.halfL) q += t.L;
-        return q;
-      };
-      px = wrapb(ix * h - t.halfL + v4[i].x);
-      py = wrapb(iy * h - t.halfL + v4[i].y);
-      pz = wrapb(iz * h - t.halfL + v4[i].z);
-    }
-    if (k < cap) {
-      if (type) type[k] = static_cast<int32_t>(tt & 7u);
-      if (id) id[k] = tt >> 3;
-      if (xyz) { xyz[3 * k] = px; xyz[3 * k + 1] = py; xyz[3 * k + 2] = pz; }
-    }
-    ++k;
-  }
-  if (n_out) *n_out = k;
-  if (k > cap) return CHEM_EINVAL;
+  if (n_out) *n_out = live;
+  if (static_cast<int64_t>(live) > cap) return CHEM_EINVAL;
   return ctx->status;
 }
 

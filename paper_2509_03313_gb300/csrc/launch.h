@@ -57,6 +57,22 @@ cudaError_t enqueue_check_accept_f32l(const Dev& d, uint32_t n, uint32_t step, d
 // homog.cu: homogeneous (beam-off) stage of the trains with Train::hx_sel set
 cudaError_t enqueue_homogeneous(const Dev& d, int blocks, cudaStream_t s);
 
+// state.cu: the live species of one train packed in device order. The positions' rows lie in up
+// to three buffers one after the other (working memory that is idle between steps).
+struct PackOut {
+  static constexpr uint32_t SEGS = 3;
+  int32_t* type;
+  uint32_t* id;
+  double* xyz[SEGS];
+  uint32_t rows[SEGS];
+};
+// counts: one word per chunk of slots and one for the total (counts[pack_counts(n)]).
+uint32_t pack_counts(uint32_t n);
+cudaError_t enqueue_pack_count(const Dev& d, uint32_t train, uint32_t n_slots, uint32_t n, uint32_t* counts,
+                               cudaStream_t s);
+cudaError_t enqueue_pack_write(const Dev& d, uint32_t train, uint32_t n_slots, uint32_t n, const uint32_t* counts,
+                               const PackOut& out, cudaStream_t s);
+
 // kernels_f32l.cu (FP32-local mode)
 cudaError_t enqueue_step_f32l(const Dev& d, const LaunchCfg& lc, cudaStream_t s, cudaEvent_t* ev, bool first,
                               bool last);
