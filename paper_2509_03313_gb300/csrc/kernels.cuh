@@ -47,7 +47,7 @@ __device__ __forceinline__ void search_species(const Dev& d, SearchSmem<F32L, W>
 }
 
 template <bool F32L>
-__global__ void __launch_bounds__(32 * TPS_WARPS, F32L ? 6 : 5) k_search_tps(const __grid_constant__ Dev d) {
+__global__ void __launch_bounds__(32 * TPS_WARPS, F32L ? 8 : 7) k_search_tps(const __grid_constant__ Dev d) {
   __shared__ SearchSmem<F32L, TPS_WARPS> sm;
   if (d.g->search_cells_now) return;  // this step runs the cell tiles (grid-uniform)
   search_species<F32L, TPS_WARPS>(d, sm);
@@ -57,7 +57,7 @@ __global__ void __launch_bounds__(32 * TPS_WARPS, F32L ? 6 : 5) k_search_tps(con
 // their launches more than their work (on 1e6 species two kernels are the faster form: the
 // cell tiles want larger CTAs).
 template <bool F32L>
-__global__ void __launch_bounds__(32 * TPS_WARPS, F32L ? 6 : 5) k_search_any(const __grid_constant__ Dev d) {
+__global__ void __launch_bounds__(32 * TPS_WARPS, F32L ? 8 : 7) k_search_any(const __grid_constant__ Dev d) {
   __shared__ SearchSmem<F32L, TPS_WARPS> sm;
   if (d.g->search_cells_now) phase_search_cells<F32L, TPS_WARPS>(d, sm.cells);
   else search_species<F32L, TPS_WARPS>(d, sm);

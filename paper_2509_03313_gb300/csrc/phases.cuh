@@ -499,8 +499,9 @@ static __device__ void begin_commit(const Dev& d, BeginSmem& sb, Train* trains) 
     // Search mapping of this step. Cell tiles amortise the neighbour-cell lookups over
     // the homes of a cell and test a pair only when the types react; one thread per
     // species has the shorter per-item latency chain. Adaptive: cell tiles when the last
-    // step found more than 3 pairs inside the cutoffs per live species (the measured
-    // crossover on track workloads). Where the launch has several lanes for each home
+    // step found more than 4 pairs inside the cutoffs per live species (1e6 track species, one
+    // thread per species against tiles: 145 / 168 us at 2.9 pairs, 173 / 178 at 4.1, 240 / 213
+    // at 6.8). Where the launch has several lanes for each home
     // those share the pairs of a home, and tiles only pay for a few thousand species or very
     // many pairs: at 31,000 species lanes take 43, 79 and 143 us where tiles take 95, 156
     // and 207, at 6, 16 and 25 pairs per species. Results do not depend on the mapping.
@@ -508,7 +509,7 @@ static __device__ void begin_commit(const Dev& d, BeginSmem& sb, Train* trains) 
     if (g_adaptive) {
       const unsigned long long inc = g_incut - g_mark;
       const int lg = lanes_per_home_lg(g_live, SEARCH_LANES);
-      const unsigned long long most = lg > 0 && lg < GRP_MAX_LG ? 48ull : 3ull;
+      const unsigned long long most = lg == 0 ? 4ull : (lg < GRP_MAX_LG ? 48ull : 3ull);
       cells_now = inc > most * static_cast<unsigned long long>(g_live) ? 1u : 0u;
     } else {
       cells_now = g_home != 0u ? 1u : 0u;
@@ -1263,40 +1264,42 @@ __device__ __forceinline__ uint32_t resolve_queue(const Dev& d, const Tables& tb
   return rest;
 }
 
-// Neighbours whose loads one iteration of the per-species walk keeps in flight together. A
-// finished lane's next batch may start up to TPS_UNROLL - 1 past the last species.
+// Neighbours whose loads one batch of the per-species walk keeps in flight together (the whole
+// batch is loaded, past a range's end too).
 constexpr int TPS_UNROLL = 4;
-static_assert(2 * TPS_UNROLL <= S4_SPARE, "a batch past the last range stays inside s4");
+static_assert(TPS_UNROLL <= S4_SPARE, "a batch past the last range stays inside s4");
 constexpr int TPS_QCAP = 32 * (TPS_UNROLL + 1);  // fewer than 32 kept pairs and one batch of a warp
 
 // ---- one thread per home species
-// Each lane takes one home species (warps take 32 consecutive sorted slots by work
-// stealing), keeps the forward cells its largest cutoff can reach (a 13-bit mask from
-// per-axis face gaps), collects their non-empty ranges after its own cell's later slots,
-// and walks them one range at a time, TPS_UNROLL neighbours per iteration. Lanes of one
-// cell walk the same ranges in step, so their neighbour loads are broadcasts; the loops
-// are warp-uniform (trip count = the longest walk among the lanes) and pairs inside the
-// cutoff go to the warp's pair queue, a whole batch with one vote per neighbour. The walk is
-// bound by instruction issue: a batch is one address and four loads at fixed offsets, and the
-// queue holds three words a pair (the separation is formed again when it is resolved). With
-// the push per neighbour, the eight-word queue and an address and zero fill per neighbour the
-// search of the 1e6-species FP32-local run (mean of 102 steps) took 146 us, now 126.
+// Each lane takes one home species (warps take 32 consecutive sorted slots by work stealing),
+// keeps the forward cells its largest cutoff can reach (a 13-bit mask from per-axis face gaps)
+// and looks up the occupied ones. What bounds the walk over the neighbours found is instruction
+// issue, and the homes' walks differ widely (a cell's first home has all others later, its
+// last none): with a lane walking its own ranges, the longest walk of a warp took nine
+// batches of TPS_UNROLL neighbours where the mean is three. The lanes' ranges are therefore
+// cut into batches that go to one list per warp, and every lane takes every 32nd batch
+// whosever it is (its home's offsets come from shared memory). A batch is one address and
+// four loads at fixed offsets; pairs inside the cutoff go to the warp's pair queue, a whole
+// batch with one vote per neighbour, three words a pair. On 1e6 FP32-local track species the
+// search took 84, 87, 94, 103 us a step up to 1e-11, 1e-10, 1e-9, 1e-8 s with a walk per
+// lane, and takes 64, 65, 69, 81 (with 64 registers, for 32 warps per SM, of it 3 %).
+constexpr int TPS_EMIT = 8;                        // batches a lane lists at a time
+constexpr int TPS_LIST = 32 * (TPS_EMIT + 1);      // fewer than 32 waiting and one round's
 
 template <bool F32L, int W>
 struct TpsSmem {
-  using T = float;            // FP32 cutoffs (FP64 mode: widened, for its FP32 prefilter)
-  T ct[W][MAXT * MAXT];       // per warp: squared cutoffs of one train (-1: no reaction) ...
-  int ct_b[W];                // ... that train
-  uint32_t rs[W][N_FWD][32];  // per lane: its non-empty neighbour ranges [rs, re) ...
-  uint32_t re[W][N_FWD][32];
-  uint8_t rk[W][N_FWD][32];   // ... and their half-shell offsets
+  float ct[W][MAXT * MAXT];  // per warp: squared cutoffs of one train (-1: no reaction) ...
+  int ct_b[W];               // ... that train
+  float4 hv[W][32];          // the homes' cell offsets and id/type bits
+  uint2 list[W][TPS_LIST];   // batches: first slot; home lane | half-shell index << 5 | slots << 9
+  uint16_t pl[W][32 * (N_FWD - 1)];  // (home, forward cell) pairs: home lane | half-shell index << 5
   PairQueue<TPS_QCAP> q[W];
-  FwdSmem fo;                 // half-shell offsets
+  FwdSmem fo;                // half-shell offsets
 };
 
 template <bool F32L, int W>
 __device__ void phase_search_tps(const Dev& d, TpsSmem<F32L, W>& sm) {
-  using T = typename TpsSmem<F32L, W>::T;
+  constexpr uint32_t FULL = 0xffffffffu;
   if (d.g->search_cells_now) return;  // this step runs the cell tiles (grid-uniform)
   const uint32_t n_live = d.g->n_total - d.g->n_dead;
   const uint32_t epoch = d.g->epoch;
@@ -1315,172 +1318,166 @@ __device__ void phase_search_tps(const Dev& d, TpsSmem<F32L, W>& sm) {
   uint32_t n_tested = 0, n_in_cut = 0;  // pair-search counters of this lane
   uint32_t c_next = 0;
   if (lane == 0) c_next = atomicAdd(&d.g->item_ctr, 1u);
-  c_next = __shfl_sync(0xffffffffu, c_next, 0);
+  c_next = __shfl_sync(FULL, c_next, 0);
   while (c_next < n_chunks) {
     const uint32_t c = c_next;
     if (lane == 0) c_next = atomicAdd(&d.g->item_ctr, 1u);  // the next chunk, used at the end
     const uint32_t s = c * 32u + static_cast<uint32_t>(lane);
     bool home = s < n_live;
-    uint32_t tid_i = 0, cell = 0;
+    uint32_t cell = 0;
     float4 vi = make_float4(0.f, 0.f, 0.f, 0.f);
     if (home) {
       cell = d.cell_sorted[s];
       vi = d.s4[s];  // FP64 mode tests pairs first on these FP32 cell offsets
-      tid_i = __float_as_uint(vi.w);
     }
     const int b = (d.n_trains == 1 || !home) ? 0 : train_of_cell(d.trains, d.n_trains, cell);
     const Train& tr = d.trains[b];
-    const uint32_t ti = tid_type(tid_i);
+    const uint32_t ti = tid_type(__float_as_uint(vi.w));
     home = home && tr.active && !tr.free_jump && tb.reactive_mask[ti] != 0u;
-    // cutoff row of this lane's type: from the warp's table of its train when every
-    // lane of the chunk is in one train (refilled only when the train changes), else
-    // from a per-lane row
-    const int b0 = __shfl_sync(0xffffffffu, b, 0);
-    const T* rc2;
-    if (__all_sync(0xffffffffu, b == b0)) {
-      if (sm.ct_b[wib] != b0) {
-        const Train& t0 = d.trains[b0];
-        for (int qq = lane; qq < MAXT * MAXT; qq += 32) {
-          if constexpr (F32L) sm.ct[wib][qq] = t0.rc2f_tt[qq];
-          else sm.ct[wib][qq] = t0.rc2w_tt[qq];
-        }
-        __syncwarp();
-        if (lane == 0) sm.ct_b[wib] = b0;
-        __syncwarp();
-      }
-      rc2 = &sm.ct[wib][ti * MAXT];
-    } else {  // the rare chunk spanning several trains reads its rows from global memory
-      if constexpr (F32L) rc2 = &tr.rc2f_tt[ti * MAXT];
-      else rc2 = &tr.rc2w_tt[ti * MAXT];
+    if (!__any_sync(FULL, home)) {
+      c_next = __shfl_sync(FULL, c_next, 0);
+      continue;
     }
-    if (__any_sync(0xffffffffu, home)) {
-      // this lane's non-empty ranges: the own cell's later slots, then the forward cells
-      // within reach that are occupied (bit test in the L2-resident bitmap, then their
-      // 16-byte entries), collected (at most N_FWD ranges) and walked
-      uint32_t* rs_l = &sm.rs[wib][0][lane];
-      uint32_t* re_l = &sm.re[wib][0][lane];
-      uint8_t* rk_l = &sm.rk[wib][0][lane];
-      // bit 0: the own cell's later slots; bits 1..13: forward cells within reach
-      uint32_t kmask = 0u;
-      if (home) {
-        int ix, iy, iz;
-        cell_decode(cell - tr.cell_base, tr.cb, ix, iy, iz);
-        if (s + 1u < static_cast<uint32_t>(d.cell_info[cell].y)) kmask = 1u;
-        float rcmax2 = -1.f;
+    // cutoffs from the warp's table of its train when every lane of the chunk is in one train
+    // (refilled only when the train changes), else from the trains' records
+    const int b0 = __shfl_sync(FULL, b, 0);
+    const bool mixed = !__all_sync(FULL, b == b0);
+    if (!mixed && sm.ct_b[wib] != b0) {
+      const Train& t0 = d.trains[b0];
+      for (int qq = lane; qq < MAXT * MAXT; qq += 32) sm.ct[wib][qq] = F32L ? t0.rc2f_tt[qq] : t0.rc2w_tt[qq];
+      __syncwarp();
+      if (lane == 0) sm.ct_b[wib] = b0;
+    }
+    __syncwarp();  // (the last chunk's homes are no longer read)
+    sm.hv[wib][lane] = vi;
+    __syncwarp();
+    const float hf = tr.hf;
+    // the lane's range: first its own cell's later slots, then one of the warp's forward cells
+    uint32_t ja = 0u, ea = 0u, meta = static_cast<uint32_t>(lane), kmask = 0u;
+    if (home) {
+      ja = s + 1u;
+      ea = static_cast<uint32_t>(d.cell_info[cell].y);
+      float rcmax2 = -1.f;
 #pragma unroll
-        for (int t = 0; t < MAXT; ++t) rcmax2 = fmaxf(rcmax2, static_cast<float>(rc2[t]));
-        kmask |= cells_in_reach(vi, tr.hf, rcmax2);
+      for (int t = 0; t < MAXT; ++t)
+        rcmax2 = fmaxf(rcmax2, mixed ? (F32L ? tr.rc2f_tt[ti * MAXT + t] : tr.rc2w_tt[ti * MAXT + t])
+                                     : sm.ct[wib][ti * MAXT + t]);
+      kmask = cells_in_reach(vi, hf, rcmax2);
+    }
+    // the (home, forward cell) pairs within reach go to a list too: one round of lookups covers
+    // what a few homes close to their cells' faces would else do in several
+    uint32_t pairs, pair_at;
+    {
+      const uint32_t mine = __popc(kmask);
+      uint32_t incl = mine;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(FULL, incl, o);
+        if (lane >= o) incl += y;
       }
-      // (ranges are not moved between lanes: on clustered tracks, taking over half of a busy
-      // lane's range cost more issue slots than the idle lanes it saved; dense cells go to the
-      // cell-tile mapping instead)
-      const float hf = tr.hf;
-      int nr = 0;
-      // look up only the cells within reach (warp-uniform loop over each lane's set bits:
-      // at most N_FWD of them, so one pass collects them all)
-      {
-      // two cells per iteration, their bitmap words and then their entries loaded together
-      while (__any_sync(0xffffffffu, kmask != 0u)) {
-        int kk[2] = {-1, -1};
-        if (kmask != 0u) {
-          kk[0] = __ffs(kmask) - 1;
-          kmask &= kmask - 1u;
-        }
-        if (kmask != 0u) {
-          kk[1] = __ffs(kmask) - 1;
-          kmask &= kmask - 1u;
-        }
-        uint32_t nc[2] = {0u, 0u}, word[2] = {0u, 0u};
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          if (kk[q] > 0) {
-            const int k = kk[q], n = tr.n;
-            int ix, iy, iz;
-            cell_decode(cell - tr.cell_base, tr.cb, ix, iy, iz);
-            nc[q] = tr.cell_base + cell_encode(step_cell(ix, fo.i[0][k], n), step_cell(iy, fo.i[1][k], n),
-                                               step_cell(iz, fo.i[2][k], n), tr.cb);
-            word[q] = d.occ[nc[q] >> 5];
-          }
-        }
-        int4 ci[2];
-        bool occ[2];
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          occ[q] = kk[q] > 0 && ((word[q] >> (nc[q] & 31u)) & 1u);
-          ci[q] = occ[q] ? d.cell_info[nc[q]] : make_int4(0, 0, 0, 0);
-        }
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          if (kk[q] == 0) {
-            rs_l[0] = s + 1u;
-            re_l[0] = static_cast<uint32_t>(d.cell_info[cell].y);
-            rk_l[0] = 0;
-            nr = 1;
-          } else if (occ[q] && static_cast<uint32_t>(ci[q].z) == epoch && ci[q].y > ci[q].x) {
-            rs_l[32 * nr] = static_cast<uint32_t>(ci[q].x);
-            re_l[32 * nr] = static_cast<uint32_t>(ci[q].y);
-            rk_l[32 * nr] = static_cast<uint8_t>(kk[q]);
-            ++nr;
-          }
-        }
+      pairs = __shfl_sync(FULL, incl, 31);
+      pair_at = incl - mine;
+      while (kmask != 0u) {
+        const uint32_t k = static_cast<uint32_t>(__ffs(kmask)) - 1u;
+        kmask &= kmask - 1u;
+        sm.pl[wib][pair_at++] = static_cast<uint16_t>(static_cast<uint32_t>(lane) | (k << 5));
       }
-      }
-      // walk the ranges one after the other, TPS_UNROLL neighbours per iteration whose loads
-      // are in flight together; lanes of one cell stay in step (broadcast loads)
-      int ri = 0;
-      uint32_t j = 0, je = 0;
-      uint32_t kb_cur = 0;
-      float cx = 0.f, cy = 0.f, cz = 0.f;
-      auto open = [&](int r) {
-        j = rs_l[32 * r];
-        je = re_l[32 * r];
-        const int k = rk_l[32 * r];
-        cx = fo.f[0][k]; cy = fo.f[1][k]; cz = fo.f[2][k];  // in cells
-        kb_cur = static_cast<uint32_t>(k) | (static_cast<uint32_t>(b) << 8);
-      };
-      if (nr > 0) open(0);
-      while (__any_sync(0xffffffffu, ri < nr)) {
-        // the next TPS_UNROLL neighbours of the lane's current range (one cell offset for the
-        // batch). The whole batch is loaded, from one address; entries past the range's end
-        // belong to other cells and do not count
-        const bool act = ri < nr;
-        const uint32_t j0 = j, kb = kb_cur, left = act ? je - j : 0u;
-        const float bx = cx, by = cy, bz = cz;
-        const float4* src = d.s4 + j;
-        float4 vj[TPS_UNROLL];
+      __syncwarp();
+    }
+    uint32_t ln = 0;  // listed batches (warp-uniform)
+    // batches list[at, at + n), one per lane
+    auto take = [&](uint32_t at, uint32_t n) {
+      uint2 e = make_uint2(0u, 0u);
+      if (static_cast<uint32_t>(lane) < n) e = sm.list[wib][at + static_cast<uint32_t>(lane)];
+      const uint32_t h = e.y & 31u, k = (e.y >> 5) & 15u, left = e.y >> 9;
+      const float4* src = d.s4 + e.x;
+      float4 vj[TPS_UNROLL];
 #pragma unroll
-        for (int u = 0; u < TPS_UNROLL; ++u) vj[u] = src[u];
-        if (act) {
-          j += TPS_UNROLL;
-          if (j >= je && ++ri < nr) open(ri);
-        }
-        uint32_t bal[TPS_UNROLL];
+      for (int u = 0; u < TPS_UNROLL; ++u) vj[u] = src[u];
+      const float4 vh = sm.hv[wib][h];
+      const float* row = &sm.ct[wib][tid_type(__float_as_uint(vh.w)) * MAXT];
+      float hfh = hf;
+      int bh = b0;
+      if (mixed) {
+        bh = __shfl_sync(FULL, b, static_cast<int>(h));
+        const Train& th = d.trains[bh];
+        hfh = th.hf;
+        row = (F32L ? th.rc2f_tt : th.rc2w_tt) + tid_type(__float_as_uint(vh.w)) * MAXT;
+      }
+      const float bx = fo.f[0][k], by = fo.f[1][k], bz = fo.f[2][k];
+      uint32_t bal[TPS_UNROLL], any = 0u;
+#pragma unroll
+      for (int u = 0; u < TPS_UNROLL; ++u) {
+        float fx, fy, fz;
+        const float rc2u = static_cast<uint32_t>(u) < left ? row[__float_as_uint(vj[u].w) & 7u] : -1.f;
+        const bool pass = sep_f32(bx, by, bz, hfh, vj[u], vh, fx, fy, fz) < rc2u;  // -1: the types do not react
+        n_tested += rc2u >= 0.f ? 1u : 0u;  // reacting type pairs only
+        if constexpr (F32L) n_in_cut += pass ? 1u : 0u;
+        bal[u] = __ballot_sync(FULL, pass);
+        any |= bal[u];
+      }
+      if (any != 0u) {  // the same for every lane
 #pragma unroll
         for (int u = 0; u < TPS_UNROLL; ++u) {
-          float fx, fy, fz;
-          const float rc2u = static_cast<uint32_t>(u) < left ? rc2[__float_as_uint(vj[u].w) & 7u] : -1.f;
-          const bool pass = sep_f32(bx, by, bz, hf, vj[u], vi, fx, fy, fz) < rc2u;  // -1: the types do not react
-          n_tested += rc2u >= 0.f ? 1u : 0u;  // reacting type pairs only
-          if constexpr (F32L) n_in_cut += pass ? 1u : 0u;
-          bal[u] = __ballot_sync(0xffffffffu, pass);
-        }
-        uint32_t any = 0u;
-#pragma unroll
-        for (int u = 0; u < TPS_UNROLL; ++u) any |= bal[u];
-        if (any != 0u) {  // the same for every lane
-#pragma unroll
-          for (int u = 0; u < TPS_UNROLL; ++u) {
-            if ((bal[u] >> lane) & 1u) {
-              const uint32_t pos = qn + __popc(bal[u] & lanemask_lt);
-              q.si[pos] = s; q.j[pos] = j0 + static_cast<uint32_t>(u); q.kb[pos] = kb;
-            }
-            qn += __popc(bal[u]);
+          if ((bal[u] >> lane) & 1u) {
+            const uint32_t pos = qn + __popc(bal[u] & lanemask_lt);
+            q.si[pos] = c * 32u + h;
+            q.j[pos] = e.x + static_cast<uint32_t>(u);
+            q.kb[pos] = k | (static_cast<uint32_t>(bh) << 8);
           }
-          if (qn >= 32u) qn = resolve_queue<F32L>(d, tb, fo, q, qn, false, vf, lane, n_in_cut);
+          qn += __popc(bal[u]);
+        }
+        if (qn >= 32u) qn = resolve_queue<F32L>(d, tb, fo, q, qn, false, vf, lane, n_in_cut);
+      }
+    };
+    for (uint32_t p0 = 0;; p0 += 32u) {
+      // list the ranges' batches, up to TPS_EMIT of a lane at a time, and take them 32 by 32
+      while (__any_sync(FULL, ja < ea)) {
+        const uint32_t nb = ja < ea ? min((ea - ja + (TPS_UNROLL - 1u)) / TPS_UNROLL, static_cast<uint32_t>(TPS_EMIT)) : 0u;
+        uint32_t incl = nb;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const uint32_t y = __shfl_up_sync(FULL, incl, o);
+          if (lane >= o) incl += y;
+        }
+        const uint32_t at = ln + incl - nb;
+        for (uint32_t i = 0; i < nb; ++i) {
+          sm.list[wib][at + i] = make_uint2(ja, meta | (min(ea - ja, static_cast<uint32_t>(TPS_UNROLL)) << 9));
+          ja += TPS_UNROLL;
+        }
+        ln += __shfl_sync(FULL, incl, 31);
+        __syncwarp();
+        while (ln >= 32u) {
+          ln -= 32u;
+          take(ln, 32u);
+        }
+        __syncwarp();  // the places taken are listed anew
+      }
+      if (p0 >= pairs) break;
+      // the next 32 pairs: the cell's bitmap word and, when it is occupied, its entry
+      const uint32_t p = p0 + static_cast<uint32_t>(lane);
+      meta = p < pairs ? sm.pl[wib][p] : 0u;
+      const int h = static_cast<int>(meta & 31u), k = static_cast<int>(meta >> 5);
+      const uint32_t hcell = __shfl_sync(FULL, cell, h);
+      const Train& th = mixed ? d.trains[__shfl_sync(FULL, b, h)] : tr;
+      ja = ea = 0u;
+      if (p < pairs) {
+        const int n = th.n;
+        int ix, iy, iz;
+        cell_decode(hcell - th.cell_base, th.cb, ix, iy, iz);
+        const uint32_t nc = th.cell_base + cell_encode(step_cell(ix, fo.i[0][k], n), step_cell(iy, fo.i[1][k], n),
+                                                       step_cell(iz, fo.i[2][k], n), th.cb);
+        if ((d.occ[nc >> 5] >> (nc & 31u)) & 1u) {
+          const int4 ci = d.cell_info[nc];
+          if (static_cast<uint32_t>(ci.z) == epoch) {
+            ja = static_cast<uint32_t>(ci.x);
+            ea = static_cast<uint32_t>(ci.y);
+          }
         }
       }
     }
-    c_next = __shfl_sync(0xffffffffu, c_next, 0);
+    if (ln != 0u) take(0u, ln);
+    c_next = __shfl_sync(FULL, c_next, 0);
   }
   resolve_queue<F32L>(d, tb, fo, q, qn, true, vf, lane, n_in_cut);
   add_pair_counts(d, n_tested, n_in_cut);
