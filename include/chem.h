@@ -284,7 +284,9 @@ typedef struct chem_stats {
    * conflict rounds run in shared memory for up to 1,536 conflicting accepted pairs and
    * in global memory beyond; the events of a step are
    * ordered in shared memory for up to 8,192 events (bucket sort, or a block radix sort
-   * when the keys cluster) and in global memory beyond. Single trains of at most 262,144
+   * when the keys cluster) and in global memory beyond; contexts of more than 262,144
+   * species order more than 1,024 events by buckets of their ids, unless one overflows.
+   * Single trains of at most 262,144
    * species and the persistent launches resolve up to 1,536 (persistent: 1,024) accepted
    * pairs of a step at once in shared memory. The results do not depend on the
    * branch; these counters let tests show that each branch ran. */

@@ -331,11 +331,10 @@ void init_train_dynamic(Train& t, const chem_config& c, int n_max) {
 }
 
 // Kernels of one captured step: diffusion, the sort passes, gather, the search (one or
-// both mappings), fast matching, the one-CTA reaction kernel, products, and the end (or
-// end-and-next-begin) kernel; small contexts have one search kernel and one kernel for all
-// that follows it.
+// both mappings; small contexts have one kernel for either) and one kernel from the matching
+// to the next step's begin.
 int kernels_per_step(const chem_ctx* ctx) {
-  return ctx->lc.small ? 4 + ctx->d.passes : 6 + ctx->d.passes + (ctx->lc.search_tps == 2 ? 2 : 1);
+  return ctx->lc.small ? 4 + ctx->d.passes : 3 + ctx->d.passes + (ctx->lc.search_tps == 2 ? 2 : 1);
 }
 
 // Radix passes for the captured graph (see chem_ctx::passes_alloc).
@@ -998,6 +997,22 @@ chem_status chem_batch_init(const chem_config* cfgs, int32_t n_trains, chem_ctx*
     d.keys1 = sortbuf + cap;
     d.vals0 = sortbuf + 2 * cap;
     d.vals1 = sortbuf + 3 * cap;
+  }
+  if (cap > static_cast<uint64_t>(SMALL_SPECIES)) {  // event buckets, shared out by capacity
+    uint32_t nb = 1;
+    while (static_cast<uint64_t>(nb) * EV_BUCKET_OF < cap) nb <<= 1;
+    uint32_t base = 0;
+    for (int b = 0; b < n_trains; ++b) {
+      const uint64_t share = static_cast<uint64_t>(nb) * static_cast<uint64_t>(cfgs[b].capacity_species) / cap;
+      tr[b].bk_base = base;
+      tr[b].bk_n = static_cast<uint32_t>(std::max<uint64_t>(1, share / EV_GROUP) * EV_GROUP);
+      base += tr[b].bk_n;
+    }
+    d.n_buckets = base;
+    d.bk_cnt = static_cast<uint32_t*>(A(static_cast<size_t>(base) * 4));
+    d.bk_slot = static_cast<unsigned long long*>(A(static_cast<size_t>(base) * EV_SLOTS * 8));
+    d.bk_group = static_cast<uint32_t*>(A(static_cast<size_t>(base) / EV_GROUP * 4));
+    d.bk_start = static_cast<uint2*>(A((static_cast<size_t>(base) / EV_GROUP + 1) * 8));
   }
   d.dead = static_cast<uint8_t*>(A(cap));
   d.touch = static_cast<uint32_t*>(A(cap * 4));

@@ -20,48 +20,6 @@ __global__ void __launch_bounds__(SORT_THREADS) k_sort_pass(const __grid_constan
   phase_sort_pass(d, pass, active, n, tile, *reinterpret_cast<SortSmem*>(smem_raw), blockIdx.x == 0);
 }
 
-__global__ void __launch_bounds__(256) k_match_fast(const __grid_constant__ Dev d) {
-  phase_match_fast(d, blockIdx.x, gridDim.x);
-}
-
-constexpr size_t REACT_SERIAL_DYN_SMEM = (4 * EV_SMEM_CAP * sizeof(uint32_t) > RC_SMEM_BYTES)
-                                           ? 4 * EV_SMEM_CAP * sizeof(uint32_t) : RC_SMEM_BYTES;
-
-__global__ void __launch_bounds__(REACT_THREADS) k_react_serial(const __grid_constant__ Dev d) {
-  __shared__ SerialSmem sm;
-  extern __shared__ __align__(16) uint32_t sbuf[];
-  phase_react_serial(d, sm, sbuf);
-}
-
-__global__ void __launch_bounds__(256) k_end_step(const __grid_constant__ Dev d) {
-  __shared__ EndSmem sm;
-  phase_end_step(d, sm);
-  phase_look_ahead(d, sm);
-}
-
-cudaError_t enqueue_react_head(const Dev& d, const LaunchCfg& lc, cudaStream_t s) {
-  k_match_fast<<<lc.stream_blocks, 256, 0, s>>>(d);
-  k_react_serial<<<1, REACT_THREADS, REACT_SERIAL_DYN_SMEM, s>>>(d);
-  return cudaGetLastError();
-}
-
-cudaError_t enqueue_end_step(const Dev& d, cudaStream_t s) {
-  k_end_step<<<1, 256, 0, s>>>(d);
-  return cudaGetLastError();
-}
-
-__global__ void __launch_bounds__(256) k_end_begin(const __grid_constant__ Dev d) {
-  __shared__ EndSmem se;
-  __shared__ BeginSmem sb;
-  phase_end_step(d, se);
-  phase_begin(d, sb);
-}
-
-cudaError_t enqueue_end_begin(const Dev& d, cudaStream_t s) {
-  k_end_begin<<<1, 256, 0, s>>>(d);
-  return cudaGetLastError();
-}
-
 __global__ void __launch_bounds__(256) k_set_t_end(const __grid_constant__ Dev d, const double* t_end) {
   __shared__ EndSmem sm;
   for (uint32_t b = threadIdx.x; b < d.n_trains; b += blockDim.x) d.trains[b].t_end = t_end[b];
@@ -81,9 +39,6 @@ cudaError_t enqueue_sort_pass(const Dev& d, int pass, int blocks, cudaStream_t s
 cudaError_t sort_pass_occupancy(int* blocks_per_sm) {
   cudaError_t e = cudaFuncSetAttribute(k_sort_pass, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(sizeof(SortSmem)));
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_react_serial, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           static_cast<int>(REACT_SERIAL_DYN_SMEM));
   if (e != cudaSuccess) return e;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_sort_pass, SORT_THREADS,
                                                        sizeof(SortSmem));

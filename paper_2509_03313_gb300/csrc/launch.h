@@ -25,15 +25,9 @@ struct LaunchCfg {
 // kernels_exact.cu (FP64 arithmetic without contraction)
 cudaError_t enqueue_begin(const Dev& d, cudaStream_t s);
 cudaError_t enqueue_sort_pass(const Dev& d, int pass, int blocks, cudaStream_t s);
-// matching (fast path + conflict rounds), event ordering, product prefix
-cudaError_t enqueue_react_head(const Dev& d, const LaunchCfg& lc, cudaStream_t s);
-cudaError_t enqueue_end_step(const Dev& d, cudaStream_t s);
-// end of one step and begin of the next in one one-CTA kernel
-cudaError_t enqueue_end_begin(const Dev& d, cudaStream_t s);
 cudaError_t sort_pass_occupancy(int* blocks_per_sm);
 // One SBS step. `first`: the step begins with its own begin kernel (else the previous
-// step's end kernel began it); `last`: it ends with a plain end kernel (else its end
-// kernel also begins the next step).
+// step's last kernel began it); `last`: its last kernel does not begin the next step.
 cudaError_t enqueue_step_f64(const Dev& d, const LaunchCfg& lc, cudaStream_t s, cudaEvent_t* ev, bool first,
                              bool last);
 // Up to n_steps steps in one launch (one cluster, or one CTA per SM).

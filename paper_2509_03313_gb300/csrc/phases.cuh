@@ -492,6 +492,7 @@ static __device__ void begin_commit(const Dev& d, BeginSmem& sb, Train* trains) 
     g->n_items = 0;
     g->item_ctr = 0;
     g->n_events = 0;
+    g->bk_overflow = 0;
     g->n_products = 0;
     g->n_dead = 0;
     g->epoch = g_epoch + 1u;
@@ -875,6 +876,11 @@ __device__ void phase_gather(const Dev& d, const Span& sp) {
   const uint32_t sentinel = d.g->sentinel_step;
   const uint32_t item_home = d.g->item_home;
   const bool items_now = item_home != 0 && d.g->search_cells_now;
+  if (d.bk_cnt)  // the last step's event buckets
+    for (uint32_t i = sp.first(); i < d.n_buckets; i += sp.stride()) {
+      d.bk_cnt[i] = 0u;
+      if (i < d.n_buckets / EV_GROUP) d.bk_group[i] = 0u;
+    }
   const uint32_t stride = sp.stride();
   // GATHER_BATCH slots per thread and iteration, their loads in flight together: the
   // permutation and neighbouring keys first, then the gathered state
@@ -1654,8 +1660,9 @@ __device__ void phase_search_groups(const Dev& d, GrpSmem<W>& sm, int lg, uint32
 //     remaining pair of both its species. Together with 1 this equals the greedy walk
 //     over all accepted pairs sorted by that key (closest first, lower ids first).
 //  3. phase_react_serial runs 2 and then, in the same CTA, orders the events by
-//     (train, id_lo) with a block radix sort (in shared memory when they fit) and forms
-//     the product-count prefix in that order;
+//     (train, id_lo) (a bucket or radix sort in shared memory when they fit, or in large
+//     contexts the prefix over their event buckets) and forms the product-count
+//     prefix in that order;
 //  4. phase_products (all CTAs): product ids and positions at the diffusion-weighted
 //     encounter point (Table 1 right-hand sides), tallies summed per CTA, event log;
 //  5. phase_end_step (one CTA): FP64 clock, step counter, dt growth, step records.
@@ -1745,20 +1752,39 @@ __device__ __forceinline__ uint32_t warp_reserve(uint32_t* counter, bool pred) {
   return base + static_cast<uint32_t>(__popc(m & ((1u << lane) - 1u)));
 }
 
+// Events of large contexts are ordered by (train, id_lo) with buckets: a train's ids up to its
+// next id, in equal parts (the FP32 product is monotonic, so the buckets ascend with the ids).
+// A step of 1e6 species has up to 7,000 events on 16,384 buckets; one CTA scans the counts of
+// groups of buckets, and the few events of a bucket are ranked where they are written. Sorting
+// them in one CTA took 10 us at 7,000 events and 90 us from 8,192 on (in global memory).
+__device__ __forceinline__ uint32_t event_bucket(const Dev& d, uint32_t b, uint32_t id_lo) {
+  const Train& tr = d.trains[b];
+  const float per_id = static_cast<float>(tr.bk_n) / static_cast<float>(tr.next_id);
+  return tr.bk_base + min(tr.bk_n - 1u, static_cast<uint32_t>(static_cast<float>(id_lo) * per_id));
+}
+
 // Record accepted pair c as event number e (reserved by the caller).
 __device__ __forceinline__ void commit_event(const Dev& d, uint32_t c, const Cand& cd, uint32_t e) {
   d.dead[cd.s_lo] = 1;
   d.dead[cd.s_hi] = 1;
-  d.ev_k0[e] = event_key(d, cd);
-  d.ev_v0[e] = c | (static_cast<uint32_t>(d.tables->n_prod[cd.rxn_train & 255u]) << 24);
+  const uint32_t key = event_key(d, cd), np = static_cast<uint32_t>(d.tables->n_prod[cd.rxn_train & 255u]);
+  d.ev_k0[e] = key;
+  d.ev_v0[e] = c | (np << 24);
+  if (d.bk_cnt) {
+    const uint32_t x = event_bucket(d, cd.rxn_train >> 8, cd.id_lo);
+    const uint32_t at = atomicAdd(&d.bk_cnt[x], 1u | (np << 16)) & 0xFFFFu;
+    atomicAdd(&d.bk_group[x / EV_GROUP], 1u | (np << 16));
+    if (at < EV_SLOTS) d.bk_slot[x * EV_SLOTS + at] = (static_cast<unsigned long long>(key) << 32) | c | (np << 24);
+    else d.g->bk_overflow = 1u;
+  }
 }
 
-static __device__ void phase_match_fast(const Dev& d, uint32_t block, uint32_t blocks) {
+static __device__ void phase_match_fast(const Dev& d, const Span& sp) {
   const bool ok = block_status_ok(d);  // includes a barrier
   const uint32_t n_c = ok ? min(d.g->n_cand, d.cap_cand) : 0u;
-  const uint32_t stride = blocks * blockDim.x;
-  for (uint32_t c0 = block * blockDim.x; c0 < n_c; c0 += stride) {  // uniform per block
-    const uint32_t c = c0 + threadIdx.x;
+  const uint32_t lane = threadIdx.x & 31u;
+  for (uint32_t c0 = sp.first() - lane; c0 < n_c; c0 += sp.stride()) {  // uniform per warp
+    const uint32_t c = c0 + lane;
     const bool valid = c < n_c;
     Cand cd{};
     bool lone = false;
@@ -2250,7 +2276,51 @@ struct SerialSmem {
   MatchSmem match;
   BlockSortSmem sort;
   ScanSmem scan;
+  unsigned long long warp_tot64[REACT_THREADS / 32];
 };
+
+// Events and products before every group of EV_GROUP buckets (d.bk_start) and each train's, by
+// one CTA. (The prefix over all buckets took 8 us at 16,384 buckets and 25 us at 65,536; the
+// groups are few, and an event adds up the buckets before its own itself.)
+static __device__ void bucket_prefix(const Dev& d, SerialSmem& sm) {
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, w = tid >> 5, nw = nt >> 5;
+  const uint32_t n = d.n_buckets / EV_GROUP;
+  unsigned long long carry = 0;  // events | products << 32
+  for (uint32_t i0 = 0; i0 < n; i0 += nt) {
+    const uint32_t i = i0 + tid, c = i < n ? d.bk_group[i] : 0u;
+    const unsigned long long mine = static_cast<unsigned long long>(c & 0xFFFFu) | (static_cast<unsigned long long>(c >> 16) << 32);
+    unsigned long long incl = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned long long y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += y;
+    }
+    if (lane == 31) sm.warp_tot64[w] = incl;
+    __syncthreads();
+    unsigned long long at = carry + incl - mine;
+    for (int q = 0; q < nw; ++q) {
+      const unsigned long long t = sm.warp_tot64[q];
+      if (q < w) at += t;
+      carry += t;
+    }
+    if (i < n) d.bk_start[i] = make_uint2(static_cast<uint32_t>(at), static_cast<uint32_t>(at >> 32));
+    __syncthreads();
+  }
+  if (tid == 0) {
+    d.bk_start[n] = make_uint2(static_cast<uint32_t>(carry), static_cast<uint32_t>(carry >> 32));
+    d.g->n_products = static_cast<uint32_t>(carry >> 32);
+  }
+  __syncthreads();
+  for (uint32_t b = tid; b < d.n_trains; b += nt) {
+    Train& tr = d.trains[b];
+    const uint2 lo = d.bk_start[tr.bk_base / EV_GROUP];
+    const uint2 hi = d.bk_start[(b + 1u < d.n_trains ? d.trains[b + 1u].bk_base : d.n_buckets) / EV_GROUP];
+    tr.pref0 = lo.y;
+    tr.prods_step = hi.y - lo.y;
+    tr.n_events_step = hi.x - lo.x;
+  }
+  __syncthreads();
+}
 
 // The one-CTA part of the react phase: conflict rounds, event order, product prefix.
 // With at most EV_SMEM_CAP events the sort runs in `sbuf` (4 * EV_SMEM_CAP words of shared
@@ -2272,7 +2342,13 @@ static __device__ void phase_react_serial(const Dev& d, SerialSmem& sm, uint32_t
     if (n_conflict > g->max_conflict) g->max_conflict = n_conflict;
     g->pairs_accepted += min(g->n_cand, d.cap_cand);
     if (E > g->max_events) g->max_events = E;
-    if (E > static_cast<uint32_t>(EV_SMEM_CAP)) g->react_order_global += 1;
+    if (E > static_cast<uint32_t>(EV_SMEM_CAP) && (d.bk_cnt == nullptr || g->bk_overflow != 0u)) g->react_order_global += 1;
+  }
+  const bool buckets = d.bk_cnt != nullptr && d.g->bk_overflow == 0u;
+  if (tid == 0) d.g->ev_bucketed = buckets ? 1u : 0u;
+  if (buckets) {
+    bucket_prefix(d, sm);
+    return;
   }
   if (E <= static_cast<uint32_t>(EV_SMEM_CAP)) {
     uint32_t* k0 = sbuf;
@@ -2392,18 +2468,47 @@ __device__ __forceinline__ void add_tallies(const Dev& d, const ProductsSmem& sm
   }
 }
 
-// `block` of `blocks` CTAs.
+// sm is cleared (clear_products; a barrier follows below).
 template <bool F32L>
-__device__ void phase_products(const Dev& d, ProductsSmem& sm, uint32_t block, uint32_t blocks) {
-  const uint32_t nt = blockDim.x;
-  const Tables& tb = *d.tables;
-  clear_products(d, sm);
+__device__ void phase_products(const Dev& d, ProductsSmem& sm, const Tables& tb, const Span& sp) {
   const bool ok = block_status_ok(d);
   const uint32_t E = ok ? d.g->n_events : 0u;
   const uint32_t* order = d.g->ev_parity ? d.ev_v1 : d.ev_v0;
   const uint32_t* pref = d.g->ev_parity ? d.ev_k0 : d.ev_k1;
   const uint32_t n_live = d.g->n_total - d.g->n_dead;
-  for (uint32_t k = block * nt + threadIdx.x; k < E; k += blocks * nt) {
+  if (d.bk_cnt && d.g->ev_bucketed) {
+    // the events as they were recorded, each ranked among the few of its bucket
+    for (uint32_t e = sp.first(); e < E; e += sp.stride()) {
+      const uint32_t key = d.ev_k0[e];
+      const Cand cd = d.cand[d.ev_v0[e] & EV_CAND_MASK];
+      const uint32_t b = cd.rxn_train >> 8, x = event_bucket(d, b, cd.id_lo), n = d.bk_cnt[x] & 0xFFFFu;
+      uint2 at = d.bk_start[x / EV_GROUP];
+      const uint4* before = reinterpret_cast<const uint4*>(d.bk_cnt + x / EV_GROUP * EV_GROUP);
+      const uint32_t in_group = x % EV_GROUP;
+#pragma unroll
+      for (uint32_t i = 0; i < EV_GROUP / 4u; ++i) {
+        if (4u * i >= in_group) break;
+        const uint4 c = before[i];
+        const uint32_t left = in_group - 4u * i;
+        const uint32_t s4 = c.x + (left > 1u ? c.y : 0u) + (left > 2u ? c.z : 0u) + (left > 3u ? c.w : 0u);
+        at.x += s4 & 0xFFFFu;  // (at most EV_GROUP x EV_SLOTS events: the halves do not mix)
+        at.y += s4 >> 16;
+      }
+      for (uint32_t i = 0; i < n; ++i) {
+        const unsigned long long o = d.bk_slot[x * EV_SLOTS + i];
+        if (static_cast<uint32_t>(o >> 32) < key) {
+          at.x += 1u;
+          at.y += static_cast<uint32_t>(o) >> 24;
+        }
+      }
+      const Train& tr = d.trains[b];
+      write_event<F32L>(d, tb, sm, cd, n_live + at.y, tr.next_id + (at.y - tr.pref0), at.x);
+    }
+    __syncthreads();
+    add_tallies(d, sm);
+    return;
+  }
+  for (uint32_t k = sp.first(); k < E; k += sp.stride()) {
     const Cand cd = d.cand[order[k] & EV_CAND_MASK];
     const Train& tr = d.trains[cd.rxn_train >> 8];
     const uint32_t ex = pref[k];
@@ -2454,7 +2559,7 @@ __device__ void phase_react_all(const Dev& d, ReactAllSmem& sm, uint32_t* sbuf, 
     }
   }
   if (n_c > cap) {  // uniform
-    phase_match_fast(d, 0u, 1u);
+    phase_match_fast(d, Span{0u, 1u});
     __syncthreads();
     const uint32_t n_conflict = g->n_conflict;
     phase_match_rounds(d, sm.match);
@@ -2464,6 +2569,7 @@ __device__ void phase_react_all(const Dev& d, ReactAllSmem& sm, uint32_t* sbuf, 
     ScanSmem& scan = *reinterpret_cast<ScanSmem*>(sbuf + sizeof(BlockSortSmem) / 4);
     const int p = block_sort_pairs(d.ev_k0, d.ev_v0, d.ev_k1, d.ev_v1, E, sort);
     if (tid == 0 && ok2) {  // branch record (read by chem_get_stats)
+      g->ev_bucketed = 0u;
       g->ev_parity = static_cast<uint32_t>(p);
       g->react_rounds_global += n_conflict > 0u ? 1u : 0u;
       g->react_order_global += 1u;
@@ -2472,7 +2578,8 @@ __device__ void phase_react_all(const Dev& d, ReactAllSmem& sm, uint32_t* sbuf, 
       g->max_events = max(g->max_events, E);
     }
     products_prefix(d, scan, p ? d.ev_k1 : d.ev_k0, p ? d.ev_v1 : d.ev_v0, nullptr, p ? d.ev_k0 : d.ev_k1, E, ok2);
-    phase_products<F32L>(d, sm.products, 0u, 1u);
+    clear_products(d, sm.products);
+    phase_products<F32L>(d, sm.products, tb, Span{0u, 1u});
     for (uint32_t b = tid; b < d.n_trains; b += nt) {
       sm.prods_tr[b] = d.trains[b].prods_step;
       sm.evs_tr[b] = d.trains[b].n_events_step;
@@ -2557,13 +2664,14 @@ __device__ void phase_react_all(const Dev& d, ReactAllSmem& sm, uint32_t* sbuf, 
 // search, one CTA takes a copy of the trains' records to the end of the step and plans the
 // next one on it (stage_next), and after reaction resolution only adds what depends on it and
 // writes the records back (commit_next). On the critical path the two took 6 us.
-constexpr uint32_t PLAN_TRAINS = 8;
+template <uint32_t TRAINS>
 struct PlanSmem {
   BeginSmem begin;
-  Train tr[PLAN_TRAINS];
+  Train tr[TRAINS];
 };
 
-static __device__ void stage_next(const Dev& d, PlanSmem& pl) {
+template <uint32_t TRAINS>
+static __device__ void stage_next(const Dev& d, PlanSmem<TRAINS>& pl) {
   const int tid = threadIdx.x, nt = blockDim.x;
   const uint32_t words = d.n_trains * static_cast<uint32_t>(sizeof(Train) / 4);
   const uint32_t* src = reinterpret_cast<const uint32_t*>(d.trains);
@@ -2600,8 +2708,9 @@ __device__ __forceinline__ void log_step(const Dev& d, const Train& tr, uint32_t
   d.step_log[e] = rec;
 }
 
-// After phase_react_all; false, with nothing done, when an error is raised.
-static __device__ bool commit_next(const Dev& d, PlanSmem& pl, const ReactAllSmem& ra) {
+// After the step's products; false, with nothing done, when an error is raised.
+template <uint32_t TRAINS>
+static __device__ bool commit_next(const Dev& d, PlanSmem<TRAINS>& pl) {
   const int tid = threadIdx.x, nt = blockDim.x;
   if (!block_status_ok(d)) return false;
   Global* g = d.g;
@@ -2609,9 +2718,10 @@ static __device__ bool commit_next(const Dev& d, PlanSmem& pl, const ReactAllSme
   bool stepped = false;
   if (b < d.n_trains && d.trains[b].active) {
     stepped = true;
-    if (d.cap_step_log) log_step(d, d.trains[b], b, ra.evs_tr[b]);
-    pl.begin.live[b] += static_cast<long long>(ra.prods_tr[b]) - 2ll * static_cast<long long>(ra.evs_tr[b]);
-    pl.tr[b].next_id += ra.prods_tr[b];
+    const Train& tr = d.trains[b];
+    if (d.cap_step_log) log_step(d, tr, b, tr.n_events_step);
+    pl.begin.live[b] += static_cast<long long>(tr.prods_step) - 2ll * static_cast<long long>(tr.n_events_step);
+    pl.tr[b].next_id += tr.prods_step;
   }
   const bool any = __syncthreads_or(stepped ? 1 : 0) != 0;
   if (tid == 0) {

@@ -33,6 +33,8 @@ constexpr int MAX_PASSES = 4;
 constexpr int SORT_THREADS = 512;    // threads of the per-pass sort kernel
 constexpr int PERSIST_THREADS = 512; // threads of the persistent step kernel, one CTA per SM
 constexpr int STEP_CLUSTER = 16;     // CTAs of its one-cluster form
+constexpr uint32_t PLAN_TRAINS = 8;  // its batches of up to so many trains plan a step ahead
+constexpr uint32_t REACT_PLAN_TRAINS = 64;  // the same for k_react_grid
 constexpr int SORT_ITEMS = 15;
 constexpr int GATHER_BATCH = 4;   // slots per thread and iteration of the gather
 constexpr int S4_SPARE = 8;       // spare entries of s4 past its end: the search loads whole batches
@@ -43,6 +45,9 @@ constexpr uint32_t SORT_MANY_TILES = 24;
 // the smallest such tile (persistent kernel): sizes the look-back buffer
 constexpr int SORT_TILE_MIN = PERSIST_THREADS * static_cast<int>(SORT_ROWS_MIN);
 constexpr int REACT_THREADS = 1024;
+constexpr uint32_t EV_SLOTS = 8;       // places of an event bucket
+constexpr uint32_t EV_GROUP = 64;      // buckets of a group
+constexpr uint32_t EV_BUCKET_OF = 96;  // species capacity per bucket (a power of two of them)
 constexpr int ITEM_HOME = 32;   // most home species per pair-search work item (one cell)
 // Contexts of at most this many species run a step as few launches (one search kernel, one
 // kernel for reaction resolution and the step's end): at 2,000 to 140,000 species reaction
@@ -144,6 +149,7 @@ struct Train {
   uint32_t park_n;         // species parked
   uint32_t park_now;       // this step moves the train's species to the parking buffers
   uint32_t rel_park;       // of this step's releases, the unparked species (first)
+  uint32_t bk_base, bk_n;  // the train's event buckets
   double hx_t_end;
   double hx_e[MAXR];       // real extents of the last stage (events)
   long long hx_E[MAXR];    // whole events of the last stage
@@ -174,6 +180,8 @@ struct Global {
   uint32_t item_ctr;      // next pair-search work item (work stealing)
   uint32_t sort_parity;   // number of non-trivial passes of this step's cell sort, mod 2
   uint32_t sort_any;      // at least one pass executed (else the order is unchanged)
+  uint32_t ev_bucketed;   // this step's events are ordered by their buckets
+  uint32_t bk_overflow;   // a bucket got more events than it has places this step
   uint32_t ev_parity;     // event order in ev_v1 (1) or ev_v0 (0), prefix in the other key buffer
   uint32_t never_set;     // stays 0: the word chem_check_bounded_wait waits for
   // which branches reaction resolution took (cumulative since the last reset)
@@ -231,6 +239,11 @@ struct Dev {
   uint32_t max_tiles;
   Cand* cand;
   uint32_t* ev_list;     // committed candidate indices (cap_cand)
+  // event buckets of large contexts (nullptr otherwise), ascending in (train, id_lo): events |
+  // products << 16 of a bucket and of a group of EV_GROUP, the bucket's first EV_SLOTS events
+  // (key << 32 | value), and the events and products before a group
+  uint32_t* bk_cnt; uint32_t* bk_group; unsigned long long* bk_slot; uint2* bk_start;
+  uint32_t n_buckets;
   uint32_t* alive0; uint32_t* alive1;
   uint32_t* ev_k0; uint32_t* ev_k1; uint32_t* ev_v0; uint32_t* ev_v1;
   chem_event* ev_log;
