@@ -4,13 +4,13 @@
 //
 // For every train the host selected (Train::hx_sel):
 //  1. k_hx_remove marks every particle of the train removed (the next sort drops it);
-//  2. k_hx_integrate, one CTA per train, takes the train's species counts n0 as
+//  2. k_hx_integrate, a cluster of two CTAs per train, takes the train's species counts n0 as
 //     molecule numbers in the box volume V and integrates the reaction extents e_r
 //     (events): n(e) = n0 + nu e, de_r/dt = kappa_r n_a n_b, kappa_r = k_r / (N_A V), and
 //     (k_tab / 2) / (N_A V) for a self reaction whose tabulated value is 2k. This is Eq. 3
 //     multiplied through by N_A V. The integrator is the extrapolated linearly implicit
 //     Euler method (Deuflhard 1985; Hairer and Wanner, Solving ODEs II, Sec. IV.9) with
-//     the harmonic substep sequence 1..6 (a half warp per column) and an analytic
+//     the harmonic substep sequence 1..6 (a warp per column) and an analytic
 //     Jacobian: stiff rate equations
 //     (R9 at 1.1e11 L/mol/s) over 10 s take a few hundred steps;
 //  3. the extents are rounded to whole events without bias, E_r = floor(e_r) +
@@ -37,145 +37,179 @@ __device__ __forceinline__ int status_of_hx(const Dev& d) {
   return *reinterpret_cast<volatile int*>(&d.g->status);
 }
 
-// One train is integrated by one CTA of three warps: each of the six extrapolation columns
-// belongs to a half warp, lane r of it to reaction r. What bounds the stage is the length
-// of its dependent chain (a few hundred steps, each a factorisation and up to six
-// substeps) and the FP64 pipe, which a warp's instruction occupies for 16 cycles however
-// many lanes are active. Rows of the matrices therefore live in the lanes' registers and
-// travel by shuffles, and the columns run side by side (two per warp, of similar length).
-// Measured, 64 trains of 500 to 20,000 species over 10 s (a whole pass with its host calls):
-// 64.1 -> 16.2 ms against one lane per column with its matrices in local memory, an FP64
-// power for the step size and the table's divisions in one lane.
-constexpr int HX_THREADS = 16 * HX_K;  // one half warp per column
-static_assert(MAXR <= 16, "a half warp holds the rows of the matrix");
+// One train is integrated by a cluster of two CTAs of three warps, one warp per extrapolation
+// column. What bounds the stage is the length of its dependent chain (250 to 300 steps, each
+// an inverse and up to six substeps) and the FP64 pipe, which a warp's instruction occupies
+// for many cycles however many lanes are active. So the work of a column is spread over the
+// lanes of its warp (lane r + 16 h: reaction r, the matrix's columns of parity h), a substep
+// is one product with the inverse instead of two triangular sweeps, and no more than three
+// warps lie on an SM; the columns' end values go to both CTAs through distributed shared memory.
+// Measured, 64 trains of 500 to 20,000 species over 10 s (252 steps; the call): 2.9 ms, against
+// 6.1 ms with a half warp per column, LU factors and one CTA per train, and the same 6.1 ms
+// with those three warps on SMs of their own; a whole pass with its host calls 13.9 -> 11.2 ms
+// (64.1 with one lane per column and its matrices in local memory).
+constexpr int HX_CTAS = 2;
+constexpr int HX_WARPS = HX_K / HX_CTAS;
+constexpr int HX_THREADS = 32 * HX_WARPS;
+static_assert(HX_WARPS * HX_CTAS == HX_K, "a warp per column");
+static_assert(MAXR == 16 && MAXT == 8, "a half warp holds the rows of the matrix, twice the species");
+
+// Extrapolation of the columns FIRST+1..HX_K (step sizes H / j, errors in h, h^2, ...) to
+// h = 0: the weight of column j is the product of j / (j - i) over the other columns i.
+__host__ __device__ constexpr double hx_weight(int j, int first) {
+  double w = 1.0;
+  for (int i = first + 1; i <= HX_K; ++i)
+    if (i != j) w *= static_cast<double>(j) / static_cast<double>(j - i);
+  return w;
+}
 
 // Kinetics of one train in molecule numbers, and the columns' end values.
 struct HxSmem {
-  double n0[MAXT];
   double nu[MAXR][MAXT];      // change of species x per event of reaction r
   double nu_ab[MAXR][MAXR][2];  // [s][r]: change of r's two reactants per event of s
-  double col[HX_K][MAXR];
+  double col[2][HX_K][MAXR];  // (alternating, so that one barrier a step is enough)
   double e[MAXR];             // extents at the end of the integration
+  int go;                     // the train is to be integrated
 };
 
-// What a lane keeps of its reaction (lanes past the reactions: kappa 0, reactants 0).
+// Barrier over a train's CTAs (release / acquire of all memory among them).
+__device__ __forceinline__ void hx_sync() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// Address of CTA q's copy of the shared variable p.
+__device__ __forceinline__ uint32_t hx_peer(const void* p, uint32_t q) {
+  uint32_t a;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(p))), "r"(q));
+  return a;
+}
+
+// What a lane keeps: its reaction r (lanes past the reactions: kappa 0, reactants 0), its half
+// h, and the entries of parity h for species r mod 8.
 struct HxLane {
-  int nr, nt, r, col;
+  int nr, nt, r, h, col;
   int a, b;
   double kappa;
+  double n0;           // of the species, in half 0
+  double nu[MAXR / 2];  // change of the species per event of reaction 2j + h
 };
 
 __device__ __forceinline__ double hx_shfl(double v, int src) {
   return __shfl_sync(0xffffffffu, v, src, 16);
 }
 
-// kappa n_a and kappa n_b of this lane's reaction and its rate, at extents y (one per lane).
-__device__ __forceinline__ double hx_rate(const HxLane& k, const HxSmem& sm, double y, double& na, double& nb) {
-  const int x = k.r & (MAXT - 1);  // lane x also carries species x (and lane x + 8 a copy)
-  double n = sm.n0[x], n2 = 0.0;
+// kappa n_a and kappa n_b of this lane's reaction and its rate, at extents y (one per row).
+__device__ __forceinline__ double hx_rate(const HxLane& k, double y, double& na, double& nb) {
+  double n = k.n0;
 #pragma unroll
-  for (int s = 0; s < MAXR; s += 2) {
-    if (s < k.nr) n += sm.nu[s][x] * hx_shfl(y, s);
-    if (s + 1 < k.nr) n2 += sm.nu[s + 1][x] * hx_shfl(y, s + 1);
-  }
-  n += n2;
+  for (int j = 0; j < MAXR / 2; ++j)
+    if (2 * j < k.nr) n += k.nu[j] * hx_shfl(y, 2 * j + k.h);
+  n += __shfl_xor_sync(0xffffffffu, n, 16);
   na = hx_shfl(n, k.a);
   nb = hx_shfl(n, k.b);
   return k.kappa * na * nb;
 }
 
-// One extrapolated step of length H from y0 (one extent per lane, the same in every half
-// warp): column j takes j linearly implicit Euler substeps (I - hJ) d = h f(y), y += d,
-// h = H / j, with the Jacobian J of y0; then lane r forms the Aitken-Neville table of
-// component r, which removes the error terms in h, h^2, ... (the method's expansion is in
-// powers of h). The matrix is factored once by elimination with a pivot row per column
-// (largest element to 1 part in 2^16, rows stay where they are); a substep is one forward
-// and one backward sweep. Returns false (for the whole CTA) when a matrix is singular or
-// the result is not finite; else y1 and the scaled error estimate.
-__device__ bool hx_step(const HxLane& k, HxSmem& sm, double y0, double H, double& y1, double& err) {
+// 1 / x for normal x with 1 / x normal, within 2 units in the last place: the FP32 reciprocal
+// of the significand (off by less than 2^-22) and one Newton step of third order.
+__device__ __forceinline__ double hx_recip(double x) {
+  const int hi = __double2hiint(x);
+  const double m = __hiloint2double((hi & static_cast<int>(0x800FFFFFu)) | 0x3FF00000, __double2loint(x));
+  const double y = static_cast<double>(__frcp_rn(static_cast<float>(m)));
+  const double e = fma(-m, y, 1.0);
+  const double z = fma(y, fma(e, e, e), y);
+  return __hiloint2double(__double2hiint(z) + (0x3FF00000 - (hi & 0x7FF00000)), __double2loint(z));
+}
+
+// One extrapolated step of length H from y0 (one extent per row, the same in every half
+// warp): column j takes j linearly implicit Euler substeps y += (I - hJ)^-1 h f(y), h = H / j,
+// with the Jacobian J of y0; then each lane extrapolates its component, which removes the
+// error terms in h, h^2, ... (the method's expansion is in powers of h). The inverse is formed
+// in place by Gauss-Jordan elimination with a pivot row per column (largest element to 1 part
+// in 2^16, rows stay where they are). Returns false (in every CTA of the train) when a matrix
+// is singular, which makes its column not a number, or the result is not finite; else y1,
+// whether every error estimate is within its tolerance, and the largest ratio of the two.
+__device__ bool hx_step(const HxLane& k, HxSmem& sm, int odd, double y0, double H, double& y1, bool& within,
+                        float& err) {
   const int nr = k.nr;
   const double h = H / static_cast<double>(k.col + 1);
   double na, nb;
-  double f = hx_rate(k, sm, y0, na, nb);
-  const double ka = k.kappa * nb, kb = k.kappa * na;
-  // row r of I - hJ: d rate_r / d e_s = kappa_r (n_b nu[a][s] + n_a nu[b][s])
-  double M[MAXR];
+  double f = hx_rate(k, y0, na, nb);
+  const double ka = -h * (k.kappa * nb), kb = -h * (k.kappa * na);
+  // row r of I - hJ: d rate_r / d e_s = kappa_r (n_b nu[a][s] + n_a nu[b][s]); s = 2j + h
+  double M[MAXR / 2];
 #pragma unroll
-  for (int s = 0; s < MAXR; ++s) {
-    M[s] = 0.0;
-    if (s < nr) M[s] = (s == k.r ? 1.0 : 0.0) - h * (ka * sm.nu_ab[s][k.r][0] + kb * sm.nu_ab[s][k.r][1]);
+  for (int j = 0; j < MAXR / 2; ++j) {
+    const int s = 2 * j + k.h;
+    M[j] = 0.0;
+    if (2 * j < nr)
+      M[j] = fma(kb, sm.nu_ab[s][k.r][1], fma(ka, sm.nu_ab[s][k.r][0], s == k.r && s < nr ? 1.0 : 0.0));
   }
-  int pos = MAXR;                // elimination order of this lane's row (MAXR: not yet)
-  double inv_own = 0.0;          // 1 / pivot of this lane's row
-  unsigned long long perm = 0;   // pivot lane of column c in bits 4c
+  bool free_row = k.r < nr;
+  unsigned long long perm = 0;  // pivot row of column c in bits 4c
   bool ok = true;
 #pragma unroll
   for (int c = 0; c < MAXR; ++c) {
     if (c >= nr) break;
-    const unsigned hi = static_cast<unsigned>(__double2hiint(M[c])) & 0x7FFFFFF0u;
-    const bool free_row = pos == MAXR && k.r < nr;
-    const unsigned key = free_row ? (hi | static_cast<unsigned>(15 - k.r)) : 0u;
-    const unsigned best0 = __reduce_max_sync(0xffffffffu, (k.col & 1) ? 0u : key);
-    const unsigned best1 = __reduce_max_sync(0xffffffffu, (k.col & 1) ? key : 0u);
-    const unsigned best = (k.col & 1) ? best1 : best0;
+    const double m = __shfl_sync(0xffffffffu, M[c / 2], k.r + 16 * (c & 1));
+    const unsigned hi = static_cast<unsigned>(__double2hiint(m)) & 0x7FFFFFF0u;
+    const unsigned best = __reduce_max_sync(0xffffffffu, free_row ? (hi | static_cast<unsigned>(15 - k.r)) : 0u);
     const int p = 15 - static_cast<int>(best & 15u);
-    ok = ok && best >= 16u && best < 0x7FF00000u;
+    ok = ok && best >= 0x00100000u && best < 0x7FD00000u;
     perm |= static_cast<unsigned long long>(p) << (4 * c);
-    const double inv = 1.0 / hx_shfl(M[c], p);
+    const double inv = hx_shfl(hx_recip(m), p);  // (every row's, beside the search for the pivot)
     const bool mine = k.r == p;
-    if (mine) { pos = c; inv_own = inv; }
-    const double l = (free_row && !mine) ? M[c] * inv : 0.0;
-    if (free_row && !mine) M[c] = l;
+    if (mine) free_row = false;
+    const double g = mine ? -inv : m * inv;
 #pragma unroll
-    for (int q = c + 1; q < MAXR; ++q)
-      if (q < nr) M[q] -= l * hx_shfl(M[q], p);
+    for (int j = 0; j < MAXR / 2; ++j)
+      if (2 * j < nr) M[j] = fma(-g, hx_shfl(M[j], p), mine ? 0.0 : M[j]);
+    if (k.h == (c & 1)) M[c / 2] = -g;
   }
+  // the solution's component c is the sum over c' of M[pivot row of c][c'] v[pivot row of c']
+  int from[MAXR / 2];
+#pragma unroll
+  for (int j = 0; j < MAXR / 2; ++j) from[j] = static_cast<int>(perm >> (4 * (2 * j + k.h))) & 15;
+  const int row = static_cast<int>(perm >> (4 * k.r)) & 15;
   double y = y0;
-  for (int i = 0; i <= (k.col | 1); ++i) {  // warp-uniform: as many as its longer column takes
-    if (i > 0) f = hx_rate(k, sm, y, na, nb);
-    double v = h * f, x = 0.0;
+  for (int i = 0; i <= k.col; ++i) {
+    if (i > 0) f = hx_rate(k, y, na, nb);
+    const double v = h * f;
+    double x = 0.0;
 #pragma unroll
-    for (int c = 0; c < MAXR; ++c) {
-      if (c >= nr) break;
-      const double xc = hx_shfl(v, static_cast<int>(perm >> (4 * c)) & 15);
-      if (pos > c) v -= M[c] * xc;
-    }
-#pragma unroll
-    for (int c = MAXR - 1; c >= 0; --c) {
-      if (c >= nr) continue;
-      const double xc = hx_shfl(v * inv_own, static_cast<int>(perm >> (4 * c)) & 15);
-      if (pos < c) v -= M[c] * xc;
-      if (k.r == c) x = xc;
-    }
-    if (i <= k.col) y += x;
+    for (int j = 0; j < MAXR / 2; ++j)
+      if (2 * j < nr) x += M[j] * hx_shfl(v, from[j]);
+    x += __shfl_xor_sync(0xffffffffu, x, 16);
+    x = hx_shfl(x, row);
+    if (k.r < nr) y += x;
   }
-  sm.col[k.col][k.r] = y;
-  ok = __syncthreads_and(ok ? 1 : 0) != 0;
-  // every half warp forms the same table, so that all go on with the same values
-  double prev[HX_K], cur[HX_K];
+  if (!ok) y = nan("");
+  static_assert(HX_CTAS == 2, "half h writes to CTA h");
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(hx_peer(&sm.col[odd][k.col][k.r], k.h)), "d"(y) : "memory");
+  hx_sync();
+  // every half warp extrapolates, so that all go on with the same values
+  const double last = sm.col[odd][HX_K - 1][k.r];
+  double all = 0.0, but_one = 0.0;
 #pragma unroll
-  for (int j = 1; j <= HX_K; ++j) {
-    cur[0] = sm.col[j - 1][k.r];
-#pragma unroll
-    for (int l = 0; l + 1 < j; ++l)  // the weight is 1 / (j / (j - l - 1) - 1)
-      cur[l + 1] = cur[l] + (cur[l] - prev[l]) * (static_cast<double>(j - l - 1) / static_cast<double>(l + 1));
-#pragma unroll
-    for (int l = 0; l < j; ++l) prev[l] = cur[l];
+  for (int j = 1; j < HX_K; ++j) {
+    const double dv = sm.col[odd][j - 1][k.r] - last;  // (the weights' sum is 1)
+    all += hx_weight(j, 0) * dv;
+    if (j > 1) but_one += hx_weight(j, 1) * dv;
   }
-  y1 = cur[HX_K - 1];
+  y1 = last + all;
   const double sc = HX_ATOL + HX_RTOL * fmax(fabs(y0), fabs(y1));
-  double e = k.r < nr ? fabs(y1 - cur[HX_K - 2]) / sc : 0.0;
-  bool fin = k.r >= nr || isfinite(y1);
-#pragma unroll
-  for (int o = 8; o > 0; o >>= 1) e = fmax(e, __shfl_xor_sync(0xffffffffu, e, o, 16));
-  fin = __all_sync(0xffffffffu, fin);  // (both halves hold the same components)
-  err = e;
-  if (k.r >= nr) y1 = 0.0;
-  __syncthreads();  // the columns are rewritten by the next step
-  return ok && fin;
+  const double de = fabs(all - but_one);
+  const bool mine = k.r < nr;
+  const bool fin = __all_sync(0xffffffffu, !mine || isfinite(y1));
+  within = __all_sync(0xffffffffu, !mine || de <= sc);
+  const float ratio = mine && fin ? static_cast<float>(de) / static_cast<float>(sc) : 0.f;
+  err = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(ratio)));
+  if (!mine) y1 = 0.0;
+  return fin;
 }
 
-// Extents after T seconds from e = 0, one per lane (identical control flow on every
+// Extents after T seconds from e = 0, one per row (identical control flow on every
 // thread). Returns the accepted steps, or -1 on failure.
 __device__ long long hx_integrate(const HxLane& k, HxSmem& sm, double T, double& e) {
   e = 0.0;
@@ -186,11 +220,13 @@ __device__ long long hx_integrate(const HxLane& k, HxSmem& sm, double T, double&
     if (t >= T) return accepted;
     const bool last = H >= T - t;
     const double Hs = last ? T - t : H;
-    double err = 0.0, y1;
-    const bool ok = hx_step(k, sm, e, Hs, y1, err);
+    double y1;
+    bool within;
+    float err;
+    const bool ok = hx_step(k, sm, it & 1, e, Hs, y1, within, err);
     // the step-size factor needs a few digits only: FP32 power
-    const float root = (ok && err > 0.0) ? 0.9f * powf(fminf(static_cast<float>(err), 1e30f), -1.0f / HX_K) : 4.f;
-    if (ok && err <= 1.0) {
+    const float root = (ok && err > 0.f) ? 0.9f * powf(fminf(err, 1e30f), -1.0f / HX_K) : 4.f;
+    if (ok && within) {
       e = y1;
       t = last ? T : t + Hs;
       ++accepted;
@@ -212,20 +248,26 @@ __global__ void k_hx_remove(Dev d) {
   }
 }
 
-__global__ void __launch_bounds__(HX_THREADS) k_hx_integrate(Dev d) {
+__global__ void __cluster_dims__(HX_CTAS, 1, 1) __launch_bounds__(HX_THREADS) k_hx_integrate(Dev d) {
   __shared__ HxSmem sm;
   const int tid = threadIdx.x;
-  const uint32_t b = blockIdx.x;
-  // one answer for the CTA (another train's CTA may raise the status meanwhile)
-  if (__syncthreads_or(status_of_hx(d))) return;
+  const uint32_t b = blockIdx.x / HX_CTAS, rank = blockIdx.x % HX_CTAS;
   Train& tr = d.trains[b];
-  if (!tr.hx_sel) return;
+  // one answer for the train's CTAs (another train's may raise the status meanwhile)
+  hx_sync();
+  if (rank == 0 && tid < HX_CTAS) {
+    const int go = status_of_hx(d) == 0 && tr.hx_sel ? 1 : 0;
+    asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(hx_peer(&sm.go, tid)), "r"(go) : "memory");
+  }
+  hx_sync();
+  if (!sm.go) return;
   const Tables& tb = *d.tables;
   HxLane k;
   k.nt = tb.n_types;
   k.nr = tb.n_rxn;
   k.r = tid & 15;
-  k.col = tid >> 4;
+  k.h = (tid >> 4) & 1;
+  k.col = HX_WARPS * static_cast<int>(rank) + (tid >> 5);
   const double NV = HX_N_AVOGADRO * (tr.L * tr.L * tr.L * 1e-24);
   for (int q = tid; q < MAXT * MAXR; q += HX_THREADS) {
     const int x = q % MAXT, r = q / MAXT;
@@ -237,21 +279,25 @@ __global__ void __launch_bounds__(HX_THREADS) k_hx_integrate(Dev d) {
     }
     sm.nu[r][x] = v;
   }
-  if (tid < MAXT) sm.n0[tid] = tid < k.nt ? static_cast<double>(tr.counts[tid]) : 0.0;
   __syncthreads();
+  const int x = k.r & (MAXT - 1);  // the species this lane sums (lane x + 8 a copy)
+  k.n0 = k.h == 0 && x < k.nt ? static_cast<double>(tr.counts[x]) : 0.0;
+#pragma unroll
+  for (int j = 0; j < MAXR / 2; ++j) k.nu[j] = sm.nu[2 * j + k.h][x];
   k.a = k.r < k.nr ? tb.rxn_a[k.r] : 0;
   k.b = k.r < k.nr ? tb.rxn_b[k.r] : 0;
   k.kappa = k.r < k.nr ? (k.a == k.b ? 0.5 * tb.k_tab[k.r] : tb.k_tab[k.r]) / NV : 0.0;
-  for (int s = k.col; s < MAXR; s += HX_K) {
+  for (int s = tid >> 4; s < MAXR; s += HX_THREADS / 16) {
     sm.nu_ab[s][k.r][0] = sm.nu[s][k.a];
     sm.nu_ab[s][k.r][1] = sm.nu[s][k.b];
   }
-  __syncthreads();
   double own;
-  const long long steps = hx_integrate(k, sm, tr.hx_t_end - tr.t, own);
+  const double T = tr.hx_t_end - tr.t;
+  hx_sync();  // (both have read the train's record)
+  const long long steps = hx_integrate(k, sm, T, own);
   if (tid < MAXR) sm.e[tid] = own;
-  __syncthreads();
-  if (tid != 0) return;  // the rounding and the train's record: one thread
+  __syncwarp();
+  if (rank != 0 || tid != 0) return;  // the rounding and the train's record: one thread
   const double* e = sm.e;
   if (steps < 0) {
     raise_status(d.g, CHEM_ECAPACITY);
@@ -319,7 +365,7 @@ cudaError_t enqueue_homogeneous(const Dev& d, int blocks, cudaStream_t s) {
   k_hx_remove<<<blocks, 256, 0, s>>>(d);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k_hx_integrate<<<static_cast<int>(d.n_trains), HX_THREADS, 0, s>>>(d);
+  k_hx_integrate<<<static_cast<int>(d.n_trains) * HX_CTAS, HX_THREADS, 0, s>>>(d);
   return cudaGetLastError();
 }
 
