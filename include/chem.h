@@ -248,9 +248,10 @@ chem_status chem_batch_homogeneous_report(chem_ctx* ctx, int32_t train, double* 
  * and the hash resolution limit (cells per axis at small cutoffs, i.e. the cell size).
  * The pair-search mapping is kept (set it with chem_set_tuning): 0 = one thread per
  * home species; 1..32 = cell tiles, the number of home species one warp takes per work
- * item of a cell; -1 = chosen per step (cell tiles when the last step found more than 3
- * pairs inside the cutoffs per live species; the default). The device state is saved
- * before and restored after every trial; trials run past the end time. FP64 results do not depend on the choice; FP32-local results
+ * item of a cell; -1 = chosen per step (cell tiles when the last step found more than 4
+ * pairs inside the cutoffs per live species, or more where several lanes share a home
+ * species; the default). The device state is saved before and restored after every trial;
+ * trials run past the end time. FP64 results do not depend on the choice; FP32-local results
  * depend on the hash resolution only through rounding. budget_ms bounds the time spent
  * (at least one trial runs). chosen[4] = {steps_per_launch, cells_per_axis_limit,
  * species_per_item, launch_mode} when chosen is not NULL. */

@@ -1069,7 +1069,6 @@ chem_status chem_batch_init(const chem_config* cfgs, int32_t n_trains, chem_ctx*
   d.lookback = static_cast<unsigned long long*>(A(static_cast<size_t>(d.max_tiles) * RADIX * 8));
   d.cand = static_cast<Cand*>(A(cand * sizeof(Cand)));
   const uint64_t evn = std::max<uint64_t>(cand, RADIX);
-  d.ev_list = static_cast<uint32_t*>(A(evn * 4));
   d.alive0 = static_cast<uint32_t*>(A(evn * 4));
   d.alive1 = static_cast<uint32_t*>(A(evn * 4));
   d.ev_k0 = static_cast<uint32_t*>(A(evn * 4));

@@ -32,7 +32,7 @@ constexpr size_t align256(size_t x) { return (x + 255) & ~static_cast<size_t>(25
 // Byte layout of the scratch array.
 struct Layout {
   size_t sx, sy, sz, stid, tx, ty, tz, ttid, tdx, tdy, tdz, s4, t4, items, touch, cell_sorted, sortbuf, dead, cell_info, occ, lookback, cand,
-      ev_list, alive0, alive1, ev_k0, ev_k1, ev_v0, ev_v1, ev_log, step_log, pend, trains, tables,
+      alive0, alive1, ev_k0, ev_k1, ev_v0, ev_v1, ev_log, step_log, pend, trains, tables,
       global, last_epoch, total;
 };
 
@@ -54,7 +54,7 @@ constexpr Layout make_layout() {
   L.occ = take((NA_CELLS + 127) / 128 * 16);
   L.lookback = take(static_cast<size_t>(NA_TILES) * RADIX * 8);
   L.cand = take(C * sizeof(Cand));
-  L.ev_list = take(C * 4); L.alive0 = take(C * 4); L.alive1 = take(C * 4);
+  L.alive0 = take(C * 4); L.alive1 = take(C * 4);
   L.ev_k0 = take(C * 4); L.ev_k1 = take(C * 4); L.ev_v0 = take(C * 4); L.ev_v1 = take(C * 4);
   L.ev_log = take(NA_MAX_EVENTS * sizeof(chem_event));
   L.step_log = take(sizeof(chem_step_record));
@@ -343,7 +343,6 @@ extern "C" chem_status chem_step_noalloc(const chem_config* cfg, uint32_t step, 
   d.lookback = reinterpret_cast<unsigned long long*>(b + LAYOUT.lookback);
   d.max_tiles = NA_TILES;
   d.cand = reinterpret_cast<Cand*>(b + LAYOUT.cand);
-  d.ev_list = reinterpret_cast<uint32_t*>(b + LAYOUT.ev_list);
   d.alive0 = reinterpret_cast<uint32_t*>(b + LAYOUT.alive0);
   d.alive1 = reinterpret_cast<uint32_t*>(b + LAYOUT.alive1);
   d.ev_k0 = reinterpret_cast<uint32_t*>(b + LAYOUT.ev_k0);

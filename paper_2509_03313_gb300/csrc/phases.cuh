@@ -45,16 +45,6 @@ __device__ __forceinline__ double wrap_box(double x, double L, double halfL) {
   return x;
 }
 
-// The same shift computed with 1/L instead of a division (FP32-local regrid only; the
-// FP64 mode keeps wrap_box, whose rounding is the reference's).
-__device__ __forceinline__ double wrap_box_fast(double x, double L, double halfL, double inv_L) {
-  const double k = floor((x + halfL) * inv_L);
-  x -= k * L;
-  if (x >= halfL) x -= L;
-  if (x < -halfL) x += L;
-  return x;
-}
-
 // A coordinate measured from the box corner folded into [0, L) (FP32-local regrid).
 __device__ __forceinline__ double rebase_corner(double a, double L, double inv_L) {
   if (a >= L || a < 0.0) a -= L * floor(a * inv_L);

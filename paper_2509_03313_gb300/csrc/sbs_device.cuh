@@ -238,7 +238,6 @@ struct Dev {
   unsigned long long* lookback;
   uint32_t max_tiles;
   Cand* cand;
-  uint32_t* ev_list;     // committed candidate indices (cap_cand)
   // event buckets of large contexts (nullptr otherwise), ascending in (train, id_lo): events |
   // products << 16 of a bucket and of a group of EV_GROUP, the bucket's first EV_SLOTS events
   // (key << 32 | value), and the events and products before a group
