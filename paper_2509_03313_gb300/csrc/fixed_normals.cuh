@@ -6,10 +6,13 @@
 // integers (the uniforms of the Philox block), which suits fixed point: no argument
 // reduction is rounded, and every result carries at least 58 correct bits before its one
 // rounding to double, so the errors stay below those of the double-precision functions
-// (half an ulp in all; the angle 2 pi u itself is never rounded). Against 160-bit arithmetic
-// the largest errors are 5.6e-17 (sine, cosine) and 7.6e-16 (radius), those of the
-// double-precision formulas 6.9e-16 and 1.24e-15. The diffusion of 1e6 FP64 species, with the
-// cells and offsets taken on the FP32 pipe (cell_index_split), went from 313 to 62 us.
+// (half an ulp in all). The angle is 2 pi u rounded to double, as every FP64 evaluation of
+// the transform has it: its difference from 2 pi u is formed exactly from the integers and
+// added to the folded angle to first order. (Positions after 1,000 steps of 2,000 species are
+// 2.0e-16 from an FP64 evaluation's as with double-precision functions, 6.9e-16 with the
+// unrounded angle; it costs the FP64 mode's passes 1 to 3 %.) The diffusion of 1e6 FP64
+// species, with the cells and offsets taken on the FP32 pipe (cell_index_split), went from
+// 313 to some 65 us.
 //
 // Methods, from the mathematics: octant folding and the Taylor polynomials of sine and
 // cosine on [0, pi/4] by Horner's rule; the logarithm by a table of ln(R_i / 512), R_i =
@@ -75,8 +78,27 @@ struct Folded {
   uint64_t xn;  // x 2^se, its leading bits kept however small x is
   int se;
   uint64_t z;   // x^2 2^64
+  int64_t d;    // what the rounding of 2 pi u to double adds to x, 2^103 units
   bool swap, neg_s, neg_c;  // sine and cosine change places; their signs
 };
+
+// fl(fl(2 pi) fl(m / 2^53)) - 2 pi m / 2^53 in units of 2^-103, below 2^53 in magnitude.
+FN_FN int64_t angle_rounding(uint64_t m) {
+  constexpr uint64_t TWO_PI = 0x1921fb54442d18ull;  // the double nearest 2 pi, 2^50 units
+  const uint64_t lo = TWO_PI * m;
+#ifdef __CUDACC__
+  const uint64_t hi = __umul64hi(TWO_PI, m);
+#else
+  const uint64_t hi = static_cast<uint64_t>((static_cast<unsigned __int128>(TWO_PI) * m) >> 64);
+#endif
+  const int n = hi ? 128 - clz64(hi) : 64 - clz64(lo | 1u);  // bits of the product
+  const int drop = n > 53 ? n - 53 : 0;                      // at most 53 go, to nearest, ties to even
+  const uint64_t one = 1ull << drop, rem = lo & (one - 1u), half = one >> 1;
+  const bool up = drop > 0 && (rem > half || (rem == half && (lo & one) != 0u));
+  const int64_t e = static_cast<int64_t>(up ? rem - one : rem);
+  // (2 pi minus its double) u: 2^103 units
+  return -e - static_cast<int64_t>(mh64(m << 11, 0x8d313198a2e03ull));
+}
 
 FN_FN Folded fold(uint64_t m) {
   Folded f;
@@ -89,10 +111,37 @@ FN_FN Folded fold(uint64_t m) {
   f.se = 63 + sh;
   const uint64_t x = f.xn >> sh;  // 2^63 units
   f.z = mh64(x, x) << 2;
+  const int64_t d = angle_rounding(m);
+  f.d = (q & 1u) ? -d : d;
   f.swap = ((q + 1u) >> 1) & 1u;
   f.neg_s = q >= 4u;
   f.neg_c = ((q + 2u) >> 2) & 1u;
   return f;
+}
+
+// sin(x + d) from v = sin x in 2^f.se units: v + d cos x.
+FN_FN double sine_at(const Folded& f, uint64_t v) {
+  const int sh = f.se - 63;
+  // (below 2^-45, two draws in 2^45, in double: d may be as large as x)
+  if (sh > 45) return to_double(v, f.se) + static_cast<double>(f.d) * 0x1p-103;
+  const uint64_t a = static_cast<uint64_t>(f.d < 0 ? -f.d : f.d);
+  uint64_t D = sh <= 40 ? a >> (40 - sh) : a << (sh - 40);
+  const uint32_t zh = hi32(f.z);
+  if (zh >= 16u) {  // cos x to z^3 / 6!, 2^31 units
+    const uint32_t z2 = mh32(zh, zh);
+    const uint32_t c = 0x80000000u - (zh >> 2) + mh32(z2, 0x05555555u) - mh32(mh32(z2, zh), 0x002d82d8u);
+    D = mh64(D, static_cast<uint64_t>(c) << 33);
+  }
+  return to_double(f.d < 0 ? v - D : v + D, f.se);
+}
+
+// cos(x + d) from v = cos x in 2^63 units: v - d sin x.
+FN_FN double cosine_at(const Folded& f, uint64_t v) {
+  const uint64_t a = static_cast<uint64_t>(f.d < 0 ? -f.d : f.d) >> 40;  // 2^63 units, below 2^13
+  const uint32_t zh = hi32(f.z), x = hi32(f.xn >> (f.se - 63));         // 2^31 units
+  const uint32_t sn = x - mh32(x, mh32(zh, 0x2aaaaaabu) - mh32(mh32(zh, zh), 0x02222222u));
+  const uint64_t D = mul_wide(static_cast<uint32_t>(a), sn) >> 31;
+  return to_double(f.d < 0 ? v + D : v - D, 63);
 }
 
 // sin x = x (1 - z/3! + z^2/5! - ...), to z^8 / 17!.
@@ -106,7 +155,7 @@ FN_FN double sine(const Folded& f) {
   s = 0x0222222222222222ull - mh64(f.z, s);
   s = 0x2aaaaaaaaaaaaaabull - mh64(f.z, s);
   s = mh64(f.z, s);
-  return to_double(f.xn - mh64(f.xn, s), f.se);
+  return sine_at(f, f.xn - mh64(f.xn, s));
 }
 
 // cos x = 1 - (z/2! - z^2/4! + ...), to z^9 / 18!.
@@ -121,12 +170,12 @@ FN_FN double cosine(const Folded& f) {
   c = 0x0aaaaaaaaaaaaaabull - mh64(f.z, c);
   c = 0x8000000000000000ull - mh64(f.z, c);
   c = mh64(f.z, c);
-  return to_double(0x8000000000000000ull - (c >> 1), 63);
+  return cosine_at(f, 0x8000000000000000ull - (c >> 1));
 }
 
 FN_FN double with_sign(double v, bool neg) { return neg ? -v : v; }
 
-// sin and cos of 2 pi m / 2^53.
+// sin and cos of 2 pi m / 2^53 (rounded to double).
 FN_FN void sincos_2pi(uint64_t m, double& s, double& c) {
   const Folded f = fold(m);
   const double a = sine(f), b = cosine(f);
@@ -134,7 +183,7 @@ FN_FN void sincos_2pi(uint64_t m, double& s, double& c) {
   c = with_sign(f.swap ? a : b, f.neg_c);
 }
 
-// cos of 2 pi m / 2^53: one polynomial, the coefficients chosen by the octant.
+// cos of 2 pi m / 2^53 (rounded to double): one polynomial, the coefficients chosen by the octant.
 FN_FN double cos_2pi(uint64_t m) {
   const Folded f = fold(m);
   const uint32_t zh = hi32(f.z);
@@ -149,7 +198,7 @@ FN_FN double cos_2pi(uint64_t m) {
   s = w ? s : 0x8000000000000000ull - mh64(f.z, s);
   s = mh64(f.z, s);
   const uint64_t v = w ? f.xn - mh64(f.xn, s) : 0x8000000000000000ull - (s >> 1);
-  return with_sign(to_double(v, w ? f.se : 63), f.neg_c);
+  return with_sign(w ? sine_at(f, v) : cosine_at(f, v), f.neg_c);
 }
 
 struct alignas(16) LogRow {
