@@ -2094,6 +2094,7 @@ static __device__ bool block_bucket_sort(uint32_t* k0, uint32_t* v0, uint32_t* k
   uint32_t ex = block_excl_scan(mine, ss.warp_tot, &ss.total, tot);
   big = 0u;
   for (int q = 0; q < (nt >> 5); ++q) big = max(big, red[64 + q]);
+  __syncthreads();               // all have read `red`, which the caller's radix sort clears next
   if (big > 64u) return false;  // uniform: every thread read the same values
   for (int i = 0; i < per; ++i) {
     const uint32_t c = cnt[per * tid + i];
