@@ -155,9 +155,11 @@ struct GridBarrier {
   }
 };
 
-// Barrier over the CTAs of one cluster (release / acquire of all memory among them).
+// Barrier over the CTAs of one cluster (release / acquire of all memory among them). The aligned
+// instructions need the warp together, which the phases' ends (work of lane or thread 0) leave open.
 struct ClusterBarrier {
   __device__ __forceinline__ void sync(const Dev&) {
+    __syncwarp();
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
   }
   __device__ __forceinline__ void leave(const Dev&) {}
