@@ -99,7 +99,8 @@ typedef struct chem_config {
   int32_t cells_per_axis_max;  /* spatial-hash resolution limit; 0 = automatic         */
   int32_t steps_per_launch;    /* steps per captured graph replay; 0 = automatic       */
   int32_t launch_mode;         /* CHEM_LAUNCH_AUTO: by the number of species, persistent up
-                                  to some 260,000 and one kernel per phase beyond;
+                                  to some 260,000 and one kernel per phase beyond, chosen
+                                  again when species that arrive outgrow it;
                                   CHEM_LAUNCH_PHASES; CHEM_LAUNCH_PERSISTENT (many steps
                                   per launch, CTAs resident together with barriers)    */
   void* cuda_stream;           /* cudaStream_t to run on; NULL = library-owned stream  */

@@ -361,6 +361,14 @@ Form choose_form(const chem_ctx* ctx, uint32_t n) {
   return ctx->lc.cluster_blocks > 0 && n <= static_cast<uint32_t>(CLUSTER_SPECIES) ? FORM_CLUSTER : FORM_GRID;
 }
 
+// Most species that a launch of the form f takes a step on: a pulse may arrive during a launch.
+// (1e6 track species due 1 ps into a fresh context: 23.1 ms to 1 us, as when due at 0; in the
+// form of the first, empty step, one cluster, 260 ms. 32,000 species: 6.2 and 14.4 ms.)
+uint32_t most_species(const chem_ctx* ctx, Form f) {
+  if (f == FORM_CLUSTER) return static_cast<uint32_t>(CLUSTER_SPECIES);
+  return ctx->launch_mode == CHEM_LAUNCH_AUTO ? static_cast<uint32_t>(GRID_SPECIES) : 0xFFFFFFFFu;
+}
+
 constexpr uint32_t EPOCH_MAX = 1u << 26;  // look-back words hold 30 bits of 8 x the epoch
 constexpr int AUTO_STEPS = 16;
 int steps_of(const chem_ctx* ctx, Form f) {
@@ -415,9 +423,13 @@ chem_status capture_graph(chem_ctx* ctx) {
   return CHEM_OK;
 }
 
-// Queues the next steps in the form f.
-chem_status launch_steps(chem_ctx* ctx, Form f) {
-  if (f == FORM_PHASES) {
+// Queues the next steps in the form f. The `done` steps since the last multiple of the graph's
+// steps were another form's, which its species outgrew: the per-phase form then takes the rest
+// up to the next multiple without a graph, so that runs end in the same order of species as
+// with graphs alone.
+chem_status launch_steps(chem_ctx* ctx, Form f, int done) {
+  const int align = steps_of(ctx, FORM_PHASES);
+  if (f == FORM_PHASES && done == 0) {
     if (!ctx->graph) {
       chem_status s = capture_graph(ctx);
       if (s) return s;
@@ -426,10 +438,16 @@ chem_status launch_steps(chem_ctx* ctx, Form f) {
     return CHEM_OK;
   }
   set_launch_params(ctx);
-  const bool cluster = f == FORM_CLUSTER;
-  CK(ctx->precision == CHEM_FP64
-         ? enqueue_steps_f64(ctx->d, ctx->lc, cluster, steps_of(ctx, f), steps_of(ctx, FORM_PHASES), ctx->stream)
-         : enqueue_steps_f32l(ctx->d, ctx->lc, cluster, steps_of(ctx, f), steps_of(ctx, FORM_PHASES), ctx->stream));
+  if (f == FORM_PHASES) {
+    for (int s = done; s < align; ++s)
+      CK(ctx->precision == CHEM_FP64
+             ? enqueue_step_f64(ctx->d, ctx->lc, ctx->stream, nullptr, s == done, s + 1 == align)
+             : enqueue_step_f32l(ctx->d, ctx->lc, ctx->stream, nullptr, s == done, s + 1 == align));
+    return CHEM_OK;
+  }
+  const StepRun r{f == FORM_CLUSTER, steps_of(ctx, f) - done, align, done, most_species(ctx, f)};
+  CK(ctx->precision == CHEM_FP64 ? enqueue_steps_f64(ctx->d, ctx->lc, r, ctx->stream)
+                                 : enqueue_steps_f32l(ctx->d, ctx->lc, r, ctx->stream));
   return CHEM_OK;
 }
 
@@ -444,9 +462,11 @@ chem_status run_loop(chem_ctx* ctx) {
     if (s0) return s0;
   }
   uint32_t active_before = ctx->g_pinned->steps_active;
+  const int align = steps_of(ctx, FORM_PHASES);
+  int done = 0;  // steps since the run's last multiple of `align`
   for (long long it = 0;; ++it) {
     const Form form = choose_form(ctx, ctx->g_pinned->n_ahead);
-    chem_status ls = launch_steps(ctx, form);
+    chem_status ls = launch_steps(ctx, form, done);
     if (ls) return ls;
     CK(cudaMemcpyAsync(ctx->g_pinned, ctx->d.g, sizeof(Global), cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
@@ -462,11 +482,13 @@ chem_status run_loop(chem_ctx* ctx) {
     } else {
       // per replay: one begin kernel, then every step's kernels (the end kernel of each step
       // but the last also begins the next)
-      ctx->stats.graph_replays += 1;
-      ctx->stats.steps_launched += ctx->graph_steps;
-      ctx->stats.kernel_launches += 1 + static_cast<int64_t>(ctx->graph_steps) * kernels_per_step(ctx);
+      ctx->stats.graph_replays += done == 0 ? 1 : 0;
+      ctx->stats.steps_launched += align - done;
+      ctx->stats.kernel_launches += 1 + static_cast<int64_t>(align - done) * kernels_per_step(ctx);
     }
-    if (form == FORM_PHASES && ctx->graph_events) {
+    const bool timed = form == FORM_PHASES && done == 0 && ctx->graph_events;
+    done = form == FORM_PHASES ? 0 : static_cast<int>((static_cast<uint32_t>(done) + stepped) % static_cast<uint32_t>(align));
+    if (timed) {
       for (uint32_t st = 0; st < stepped && st < static_cast<uint32_t>(ctx->graph_steps); ++st) {
         for (int ph = 0; ph < PH_PERSISTENT; ++ph) {
           float ms = 0.f;
@@ -1425,10 +1447,10 @@ chem_status chem_autotune(chem_ctx* ctx, double budget_ms, int32_t* chosen) {
         CK(cudaMemcpyAsync(d.g, &gfix, sizeof(Global), cudaMemcpyHostToDevice, ctx->stream));
         CK(cudaStreamSynchronize(ctx->stream));
         const int reps = std::max(1, 24 / spl);
-        s = launch_steps(ctx, form);  // settle
+        s = launch_steps(ctx, form, 0);  // settle
         if (s) break;
         CK(cudaEventRecord(e0, ctx->stream));
-        for (int r = 0; r < reps && !s; ++r) s = launch_steps(ctx, form);
+        for (int r = 0; r < reps && !s; ++r) s = launch_steps(ctx, form, 0);
         if (s) break;
         CK(cudaEventRecord(e1, ctx->stream));
         CK(cudaMemcpyAsync(ctx->g_pinned, d.g, sizeof(Global), cudaMemcpyDeviceToHost, ctx->stream));

@@ -84,7 +84,6 @@ __global__ void __launch_bounds__(REACT_END_THREADS) k_react_end(const __grid_co
                         *d.tables);
   phase_end_step(d, sm.end);
   if (begin_next) phase_begin(d, sm.begin);
-  else phase_look_ahead(d, sm.end);
 }
 
 // ---- several steps in one launch
@@ -93,7 +92,8 @@ __global__ void __launch_bounds__(REACT_END_THREADS) k_react_end(const __grid_co
 // with a barrier in between: 16 CTAs of one cluster with the hardware's cluster barrier for a
 // few thousand species, or one CTA per SM with a barrier in global memory. The search gives
 // every home at least two lanes; reaction resolution, the step's end and the next step's
-// begin are CTA 0's. A launch ends by itself when no train has anything left to do. A step of
+// begin are CTA 0's. A launch ends by itself when no train has anything left to do, or before
+// a step whose species (what arrives included) are more than its form is for. A step of
 // 2,000 species takes 27 to 30 us (as kernels 52 to 60), of 32,000 track species 73 (105);
 // at 31,000 species the sort takes 19 us, the search 13 to 35, reaction resolution 10.
 constexpr int STEP_WARPS = PERSIST_THREADS / 32;
@@ -213,18 +213,22 @@ __global__ void __launch_bounds__(REACT_THREADS, 1) k_react_grid(const __grid_co
     phase_products<F32L>(d, sm.many.products, sm.many.tb, Span{block - 1u, plan ? blocks - 2u : blocks - 1u});
   bar.sync(d);
   if (planner || (!plan && block == 0u)) {
-    if (!(plan && commit_next(d, sm.plan))) {
+    if (!(plan && commit_next(d, sm.plan, ~0u))) {
       __syncthreads();
       phase_end_step(d, end);
       if (begin_next) phase_begin(d, sm.begin);
-      else phase_look_ahead(d, end);
     }
   }
   bar.leave(d);
 }
 
+constexpr uint32_t ANY_OUTGROWN = 2u;  // Global::any_active: there is more to do, but not in this launch
+
+// The first step is `done` steps into a group of `align`; a step of more than `most` species is
+// left to the next launch (the first is taken whatever its size: the host chose it).
 template <bool F32L, bool CLUSTER>
-__global__ void __launch_bounds__(PERSIST_THREADS, 1) k_steps(const __grid_constant__ Dev d, int n_steps, int align) {
+__global__ void __launch_bounds__(PERSIST_THREADS, 1) k_steps(const __grid_constant__ Dev d, int n_steps, int align,
+                                                              int done, uint32_t most) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   StepSmem& sm = *reinterpret_cast<StepSmem*>(smem_raw);
   typename std::conditional<CLUSTER, ClusterBarrier, GridBarrier>::type bar;
@@ -234,10 +238,12 @@ __global__ void __launch_bounds__(PERSIST_THREADS, 1) k_steps(const __grid_const
   bar.sync(d);
   for (int step = 0; step < n_steps; ++step) {
     // CTA 0 alone writes these between the barriers: every CTA takes the same branches
-    const bool idle = d.g->any_active == 0u;
+    const uint32_t any = d.g->any_active;
+    const bool idle = any != 1u;
     // (the order of the species after a run is that of launches of `align` steps: one that ends
-    // early re-sorts them once more, which removes the reacted and places the last products)
-    if (idle && (d.n_trains > 1u || (step != 0 && step % align == 0))) break;
+    // early re-sorts them once more, which removes the reacted and places the last products; an
+    // outgrown launch has not begun this step)
+    if (idle && (any == ANY_OUTGROWN || d.n_trains > 1u || (step != 0 && (done + step) % align == 0))) break;
     const bool one = d.g->n_total <= SORT_ONE_CTA;
     phase_diffuse<F32L>(d, one ? nullptr : sm.hist, sp);  // includes the release
     bar.sync(d);
@@ -273,14 +279,16 @@ __global__ void __launch_bounds__(PERSIST_THREADS, 1) k_steps(const __grid_const
     bar.sync(d);
     if (lead) {
       phase_react_all<F32L>(d, sm.react.react, sm.react.sbuf, STEP_REACT_CAP, plan ? sm.react.plan.begin.tb : *d.tables);
-      if (!(plan && commit_next(d, sm.react.plan))) {
+      if (!(plan && commit_next(d, sm.react.plan, most))) {
         phase_end_step(d, sm.react.end);
-        if (step + 1 < n_steps) phase_begin(d, sm.react.plan.begin);
+        const bool leave = d.g->any_active != 0u && d.g->n_ahead > most;
+        __syncthreads();  // (all have read it)
+        if (leave && threadIdx.x == 0) d.g->any_active = ANY_OUTGROWN;
+        if (step + 1 < n_steps && !leave) phase_begin(d, sm.react.plan.begin);
       }
     }
     bar.sync(d);
   }
-  if (lead) phase_look_ahead(d, sm.react.end);
   bar.leave(d);
 }
 
@@ -385,10 +393,10 @@ cudaError_t enqueue_check_accept(const Dev& d, uint32_t n, uint32_t step, double
   return cudaGetLastError();
 }
 
-// Up to n_steps steps (a multiple of `align`) in one launch: one cluster, or one CTA per SM
-// (cooperative).
+// Steps in one launch (StepRun): one cluster, or one CTA per SM (cooperative).
 template <bool F32L>
-cudaError_t enqueue_steps(const Dev& d, const LaunchCfg& lc, bool cluster, int n_steps, int align, cudaStream_t s) {
+cudaError_t enqueue_steps(const Dev& d, const LaunchCfg& lc, const StepRun& r, cudaStream_t s) {
+  const bool cluster = r.cluster;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(cluster ? lc.cluster_blocks : lc.persistent_blocks);
   cfg.blockDim = dim3(PERSIST_THREADS);
@@ -406,8 +414,8 @@ cudaError_t enqueue_steps(const Dev& d, const LaunchCfg& lc, bool cluster, int n
   }
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cluster ? cudaLaunchKernelEx(&cfg, k_steps<F32L, true>, d, n_steps, align)
-                 : cudaLaunchKernelEx(&cfg, k_steps<F32L, false>, d, n_steps, align);
+  return cluster ? cudaLaunchKernelEx(&cfg, k_steps<F32L, true>, d, r.n_steps, r.align, r.done, r.most)
+                 : cudaLaunchKernelEx(&cfg, k_steps<F32L, false>, d, r.n_steps, r.align, r.done, r.most);
 }
 
 // Shared-memory limits of the precision's kernels; resident CTAs per SM of the persistent form

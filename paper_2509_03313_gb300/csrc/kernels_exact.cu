@@ -78,9 +78,8 @@ cudaError_t enqueue_step_f64(const Dev& d, const LaunchCfg& lc, cudaStream_t s, 
   return enqueue_phases<false>(d, lc, s, ev, first, last);
 }
 
-cudaError_t enqueue_steps_f64(const Dev& d, const LaunchCfg& lc, bool cluster, int n_steps, int align,
-                              cudaStream_t s) {
-  return enqueue_steps<false>(d, lc, cluster, n_steps, align, s);
+cudaError_t enqueue_steps_f64(const Dev& d, const LaunchCfg& lc, const StepRun& r, cudaStream_t s) {
+  return enqueue_steps<false>(d, lc, r, s);
 }
 
 cudaError_t step_kernel_limits_f64(int* blocks_per_sm, int* cluster_blocks) {

@@ -9,9 +9,8 @@ cudaError_t enqueue_step_f32l(const Dev& d, const LaunchCfg& lc, cudaStream_t s,
   return enqueue_phases<true>(d, lc, s, ev, first, last);
 }
 
-cudaError_t enqueue_steps_f32l(const Dev& d, const LaunchCfg& lc, bool cluster, int n_steps, int align,
-                              cudaStream_t s) {
-  return enqueue_steps<true>(d, lc, cluster, n_steps, align, s);
+cudaError_t enqueue_steps_f32l(const Dev& d, const LaunchCfg& lc, const StepRun& r, cudaStream_t s) {
+  return enqueue_steps<true>(d, lc, r, s);
 }
 
 cudaError_t step_kernel_limits_f32l(int* blocks_per_sm, int* cluster_blocks) {

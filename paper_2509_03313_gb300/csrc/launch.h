@@ -22,6 +22,15 @@ struct LaunchCfg {
   int small;              // few species: one search kernel and one reaction kernel per step
 };
 
+// Up to n_steps steps in one launch of one cluster, or of one CTA per SM. They are the steps from
+// `done` on of a group of `align` (whose ends the species' order follows; done + n_steps is
+// a multiple of it), and end before a step on more than `most` species.
+struct StepRun {
+  bool cluster;
+  int n_steps, align, done;
+  uint32_t most;
+};
+
 // kernels_exact.cu (FP64 arithmetic without contraction)
 cudaError_t enqueue_begin(const Dev& d, cudaStream_t s);
 cudaError_t enqueue_sort_pass(const Dev& d, int pass, int blocks, cudaStream_t s);
@@ -30,10 +39,7 @@ cudaError_t sort_pass_occupancy(int* blocks_per_sm);
 // step's last kernel began it); `last`: its last kernel does not begin the next step.
 cudaError_t enqueue_step_f64(const Dev& d, const LaunchCfg& lc, cudaStream_t s, cudaEvent_t* ev, bool first,
                              bool last);
-// Up to n_steps steps in one launch (one cluster, or one CTA per SM).
-// n_steps is a multiple of `align`, whose multiples the species' order follows.
-cudaError_t enqueue_steps_f64(const Dev& d, const LaunchCfg& lc, bool cluster, int n_steps, int align,
-                              cudaStream_t s);
+cudaError_t enqueue_steps_f64(const Dev& d, const LaunchCfg& lc, const StepRun& r, cudaStream_t s);
 // Sets the shared-memory limits of the precision's kernels; CTAs of the two forms above.
 cudaError_t step_kernel_limits_f64(int* blocks_per_sm, int* cluster_blocks);
 cudaError_t enqueue_set_t_end(const Dev& d, const double* t_end_dev, cudaStream_t s);
@@ -70,8 +76,7 @@ cudaError_t enqueue_pack_write(const Dev& d, uint32_t train, uint32_t n_slots, u
 // kernels_f32l.cu (FP32-local mode)
 cudaError_t enqueue_step_f32l(const Dev& d, const LaunchCfg& lc, cudaStream_t s, cudaEvent_t* ev, bool first,
                               bool last);
-cudaError_t enqueue_steps_f32l(const Dev& d, const LaunchCfg& lc, bool cluster, int n_steps, int align,
-                               cudaStream_t s);
+cudaError_t enqueue_steps_f32l(const Dev& d, const LaunchCfg& lc, const StepRun& r, cudaStream_t s);
 cudaError_t step_kernel_limits_f32l(int* blocks_per_sm, int* cluster_blocks);
 
 }  // namespace chem

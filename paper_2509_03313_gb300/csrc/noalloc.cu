@@ -367,8 +367,8 @@ extern "C" chem_status chem_step_noalloc(const chem_config* cfg, uint32_t step, 
   k_noalloc_setup<<<info.sms, 256, 0, s>>>(d, tb, tr, last_epoch);
   k_noalloc_load<<<blocks, 256, 0, s>>>(d, n, id, type, xyz, last_epoch);
   // one step of the persistent kernel: one cluster, or one CTA per multiprocessor
-  const bool cluster = info.cluster > 0 && n <= CLUSTER_SPECIES;
-  bool ok = cudaGetLastError() == cudaSuccess && enqueue_steps_f64(d, lc, cluster, 1, 1, s) == cudaSuccess;
+  const StepRun run{info.cluster > 0 && n <= CLUSTER_SPECIES, 1, 1, 0, 0xFFFFFFFFu};
+  bool ok = cudaGetLastError() == cudaSuccess && enqueue_steps_f64(d, lc, run, s) == cudaSuccess;
   if (ok) {
     k_noalloc_store<<<1, 1024, 0, s>>>(d, id_out, type_out, xyz_out, n_out, next_id_out, events_out,
                                        n_events_out);

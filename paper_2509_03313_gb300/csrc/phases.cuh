@@ -2659,6 +2659,7 @@ template <uint32_t TRAINS>
 struct PlanSmem {
   BeginSmem begin;
   Train tr[TRAINS];
+  uint32_t rel_all;  // releases of the planned step
 };
 
 template <uint32_t TRAINS>
@@ -2683,6 +2684,11 @@ static __device__ void stage_next(const Dev& d, PlanSmem<TRAINS>& pl) {
   }
   __syncthreads();
   begin_plan(d, pl.begin, pl.tr, 0);
+  if (tid == 0) {  // (read after a barrier, in commit_next)
+    uint32_t n = 0;
+    for (uint32_t b = 0; b < d.n_trains; ++b) n += pl.begin.rel[b];
+    pl.rel_all = n;
+  }
 }
 
 // Step record of an advancing train (before its record moves on).
@@ -2699,12 +2705,19 @@ __device__ __forceinline__ void log_step(const Dev& d, const Train& tr, uint32_t
   d.step_log[e] = rec;
 }
 
-// After the step's products; false, with nothing done, when an error is raised.
+// After the step's products; false, with nothing done, when an error is raised or the planned step
+// would work on more than `most` species.
 template <uint32_t TRAINS>
-static __device__ bool commit_next(const Dev& d, PlanSmem<TRAINS>& pl) {
+static __device__ bool commit_next(const Dev& d, PlanSmem<TRAINS>& pl, uint32_t most) {
   const int tid = threadIdx.x, nt = blockDim.x;
-  if (!block_status_ok(d)) return false;
   Global* g = d.g;
+  uint32_t n_slots = 0;
+  bool go = true;
+  if (tid == 0) {
+    n_slots = g->n_total - g->n_dead + g->n_products;
+    go = status_of(d) == 0 && (pl.begin.any == 0u || n_slots + pl.rel_all <= most);
+  }
+  if (!__syncthreads_and(go ? 1 : 0)) return false;
   const uint32_t b = static_cast<uint32_t>(tid);
   bool stepped = false;
   if (b < d.n_trains && d.trains[b].active) {
@@ -2717,7 +2730,7 @@ static __device__ bool commit_next(const Dev& d, PlanSmem<TRAINS>& pl) {
   const bool any = __syncthreads_or(stepped ? 1 : 0) != 0;
   if (tid == 0) {
     if (any) g->steps_active += 1;
-    g->n_total = g->n_total - g->n_dead + g->n_products;
+    g->n_total = n_slots;
     if (d.cap_ev_log) g->ev_log_n += g->n_events;
   }
   __syncthreads();
@@ -2733,35 +2746,38 @@ static __device__ bool commit_next(const Dev& d, PlanSmem<TRAINS>& pl) {
   return true;
 }
 
-// Species the next step will work on (stepped slots and what its begin will release), for the
-// host's choice of the launch form; between steps, one CTA of at least MAX_TRAINS threads.
-static __device__ void phase_look_ahead(const Dev& d, EndSmem& sm) {
-  const uint32_t b = threadIdx.x;
-  __syncthreads();
-  if (b == 0) sm.ahead = d.g->n_total;
-  __syncthreads();
-  if (b < d.n_trains) {
-    const Train& tr = d.trains[b];
-    if (tr.t < tr.t_end) {
-      uint32_t lo = tr.p_head, hi = tr.p_tail;
-      if (tr.next_arr <= tr.t) {
-        const double* pt = d.pt + tr.pend_base;
-        while (lo < hi) {
-          const uint32_t mid = (lo + hi) >> 1;
-          if (pt[mid] <= tr.t) lo = mid + 1; else hi = mid;
-        }
-      }
-      const uint32_t more = tr.park_n + tr.mat_n + (lo - tr.p_head);
-      if (more) atomicAdd(&sm.ahead, more);
+// Species that the begin of the train's next step will release.
+__device__ __forceinline__ uint32_t releases_ahead(const Dev& d, const Train& tr) {
+  uint32_t lo = tr.p_head, hi = tr.p_tail;
+  if (tr.next_arr <= tr.t) {
+    const double* pt = d.pt + tr.pend_base;
+    while (lo < hi) {
+      const uint32_t mid = (lo + hi) >> 1;
+      if (pt[mid] <= tr.t) lo = mid + 1; else hi = mid;
     }
   }
-  __syncthreads();
-  if (b == 0) d.g->n_ahead = sm.ahead;
+  return tr.park_n + tr.mat_n + (lo - tr.p_head);
 }
 
+// Species the next step will work on (stepped slots and what its begin will release), for the
+// choice of the launch form; between steps, one CTA.
+static __device__ void phase_look_ahead(const Dev& d, EndSmem& sm) {
+  __syncthreads();
+  if (threadIdx.x == 0) sm.ahead = d.g->n_total;
+  __syncthreads();
+  for (uint32_t b = threadIdx.x; b < d.n_trains; b += blockDim.x) {
+    const Train& tr = d.trains[b];
+    const uint32_t more = tr.t < tr.t_end ? releases_ahead(d, tr) : 0u;
+    if (more) atomicAdd(&sm.ahead, more);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) d.g->n_ahead = sm.ahead;
+}
+
+// The end of a step; the species ahead are counted with it (phase_look_ahead).
 static __device__ void phase_end_step(const Dev& d, EndSmem& sm) {
   const int tid = threadIdx.x, nt = blockDim.x;
-  if (tid == 0) { sm.any = 0; sm.stepped = 0; }
+  if (tid == 0) { sm.any = 0; sm.stepped = 0; sm.ahead = 0; }
   const bool ok = block_status_ok(d);
   for (uint32_t b = tid; b < d.n_trains; b += nt) {
     Train& tr = d.trains[b];
@@ -2777,14 +2793,19 @@ static __device__ void phase_end_step(const Dev& d, EndSmem& sm) {
       tr.h_ref = tr.h;
       tr.cb_ref = tr.cb;
     }
-    if (tr.t < tr.t_end) atomicOr(&sm.any, 1u);
+    if (tr.t < tr.t_end) {
+      atomicOr(&sm.any, 1u);
+      const uint32_t more = releases_ahead(d, tr);
+      if (more) atomicAdd(&sm.ahead, more);
+    }
   }
   __syncthreads();
   if (tid == 0) {
     if (sm.stepped) d.g->steps_active += 1;
     if (ok) {
-      const uint32_t n_live = d.g->n_total - d.g->n_dead;
-      d.g->n_total = n_live + d.g->n_products;
+      const uint32_t n_total = d.g->n_total - d.g->n_dead + d.g->n_products;
+      d.g->n_total = n_total;
+      d.g->n_ahead = n_total + sm.ahead;
       if (d.cap_ev_log) d.g->ev_log_n += d.g->n_events;
     }
     d.g->any_active = sm.any;
