@@ -245,8 +245,10 @@ chem_status chem_batch_homogeneous_report(chem_ctx* ctx, int32_t train, double* 
                                           int64_t* integrator_steps);
 
 /* Choose, by timing short runs from the current state, the launch form (one kernel per
- * phase in a graph, or the persistent cooperative kernel), the steps per graph replay
- * and the hash resolution limit (cells per axis at small cutoffs, i.e. the cell size).
+ * phase in a graph, or many steps per launch as for the species at hand), the steps per
+ * graph replay and the hash resolution limit (cells per axis at small cutoffs, i.e. the
+ * cell size). A context in the automatic launch mode stays in it when the faster form is
+ * the one that mode takes.
  * The pair-search mapping is kept (set it with chem_set_tuning): 0 = one thread per
  * home species; 1..32 = cell tiles, the number of home species one warp takes per work
  * item of a cell; -1 = chosen per step (cell tiles when the last step found more than 4

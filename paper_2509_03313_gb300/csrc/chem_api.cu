@@ -372,8 +372,10 @@ uint32_t most_species(const chem_ctx* ctx, Form f) {
 constexpr uint32_t EPOCH_MAX = 1u << 26;  // look-back words hold 30 bits of 8 x the epoch
 constexpr int AUTO_STEPS = 16;
 int steps_of(const chem_ctx* ctx, Form f) {
-  if (ctx->steps_per_launch > 0) return ctx->steps_per_launch;
-  return f == FORM_PHASES ? AUTO_STEPS : 8 * AUTO_STEPS;  // (the persistent kernel ends by itself)
+  // (the persistent kernel ends by itself: where it was not asked for, its launches are longer)
+  const bool asked = ctx->steps_per_launch > 0 && ctx->launch_mode == CHEM_LAUNCH_PERSISTENT;
+  const int steps = ctx->steps_per_launch > 0 ? ctx->steps_per_launch : AUTO_STEPS;
+  return f == FORM_PHASES || asked ? steps : 8 * steps;
 }
 
 // Drops the captured graph after a change of what it holds.
@@ -1402,7 +1404,12 @@ chem_status chem_autotune(chem_ctx* ctx, double budget_ms, int32_t* chosen) {
   const int mode_cands[2] = {CHEM_LAUNCH_PHASES, CHEM_LAUNCH_PERSISTENT};
   const int saved_mode = ctx->launch_mode;
   int best_mode = saved_mode;
-  const uint32_t n_ahead = ctx->g_pinned->n_ahead;
+  // species the next step works on, what is due included: the forms are timed as a run from here
+  // takes them (from the counters alone a fresh context seemed empty, its persistent trials
+  // ran as one cluster, and 32,000 tracks were tuned to 6.7 ms where the default takes 6.2)
+  uint32_t n_ahead = 0;
+  for (int b = 0; b < ctx->B; ++b) ctx->t_end_pinned[b] = std::numeric_limits<double>::infinity();
+  CK(cudaMemcpyAsync(ctx->t_end_dev, ctx->t_end_pinned, sizeof(double) * ctx->B, cudaMemcpyHostToDevice, ctx->stream));
   cudaEvent_t e0, e1;
   CK(cudaEventCreate(&e0));
   CK(cudaEventCreate(&e1));
@@ -1419,7 +1426,6 @@ chem_status chem_autotune(chem_ctx* ctx, double budget_ms, int32_t* chosen) {
     const int spl = spl_cands[combo % 2];
     const int ih = ih_cands[0];
     ctx->launch_mode = mode;
-    const Form form = choose_form(ctx, n_ahead);
     ctx->steps_per_launch = spl;
     ctx->item_home = ih;  // selects the search kernel of the captured graph
     {
@@ -1432,12 +1438,13 @@ chem_status chem_autotune(chem_ctx* ctx, double budget_ms, int32_t* chosen) {
         CK(cudaMemcpyAsync(d.g, snap + global_off, sizeof(Global), cudaMemcpyDeviceToDevice, ctx->stream));
         CK(cudaStreamSynchronize(ctx->stream));
         std::vector<Train> tr = tr0;
-        for (auto& t : tr) { t.n_max = std::min(nm, t.n_alloc); t.t_end = std::numeric_limits<double>::infinity(); }
+        for (auto& t : tr) t.n_max = std::min(nm, t.n_alloc);
         s = upload_trains(ctx, tr);
         if (s) break;
+        CK(enqueue_set_t_end(d, ctx->t_end_dev, ctx->stream));  // (counts the species ahead)
         ctx->pass_nmax = tr[0].n_max;
         drop_graph(ctx);
-        if (form == FORM_PHASES) s = capture_graph(ctx);
+        if (mode == CHEM_LAUNCH_PHASES) s = capture_graph(ctx);
         if (s) break;
         Global& gfix = *ctx->g_pinned;
         CK(cudaMemcpyAsync(&gfix, d.g, sizeof(Global), cudaMemcpyDeviceToHost, ctx->stream));
@@ -1446,9 +1453,17 @@ chem_status chem_autotune(chem_ctx* ctx, double budget_ms, int32_t* chosen) {
         set_mapping(gfix, ih);
         CK(cudaMemcpyAsync(d.g, &gfix, sizeof(Global), cudaMemcpyHostToDevice, ctx->stream));
         CK(cudaStreamSynchronize(ctx->stream));
+        n_ahead = gfix.n_ahead;
         const int reps = std::max(1, 24 / spl);
-        s = launch_steps(ctx, form, 0);  // settle
+        s = launch_steps(ctx, choose_form(ctx, n_ahead), 0);  // settle
         if (s) break;
+        std::vector<Train> after;
+        CK(cudaMemcpyAsync(ctx->g_pinned, d.g, sizeof(Global), cudaMemcpyDeviceToHost, ctx->stream));
+        s = download_trains(ctx, after);  // (synchronises)
+        if (s) break;
+        long long ss = 0;
+        for (const Train& t : after) ss -= t.species_steps;
+        const Form form = choose_form(ctx, ctx->g_pinned->n_ahead);  // (as a run would)
         CK(cudaEventRecord(e0, ctx->stream));
         for (int r = 0; r < reps && !s; ++r) s = launch_steps(ctx, form, 0);
         if (s) break;
@@ -1457,7 +1472,6 @@ chem_status chem_autotune(chem_ctx* ctx, double budget_ms, int32_t* chosen) {
         CK(cudaStreamSynchronize(ctx->stream));
         float ms = 0.f;
         CK(cudaEventElapsedTime(&ms, e0, e1));
-        std::vector<Train> after;
         s = download_trains(ctx, after);
         if (s) break;
         if (ctx->g_pinned->status != 0) {
@@ -1465,12 +1479,8 @@ chem_status chem_autotune(chem_ctx* ctx, double budget_ms, int32_t* chosen) {
           CK(cudaMemsetAsync(&d.g->status, 0, sizeof(int), ctx->stream));
           continue;
         }
-        long long ss = 0;
-        for (int b = 0; b < ctx->B; ++b) ss += after[b].species_steps;
-        // steps of the settle replay are included in ss; subtract them with the rate of
-        // the timed part by counting the timed replays' share
-        const double timed_frac = static_cast<double>(reps) / (reps + 1);
-        const double rate = ms > 0.f ? (static_cast<double>(ss - [&] { long long z = 0; for (int b = 0; b < ctx->B; ++b) z += tr0[b].species_steps; return z; }()) * timed_frac) / (ms * 1e-3) : 0.0;
+        for (const Train& t : after) ss += t.species_steps;
+        const double rate = ms > 0.f ? static_cast<double>(ss) / (ms * 1e-3) : 0.0;
         if (rate > best_rate) { best_rate = rate; best_n = nm; best_ih = ih; best_spl = spl; best_mode = mode; }
       }
     }
@@ -1504,20 +1514,24 @@ chem_status chem_autotune(chem_ctx* ctx, double budget_ms, int32_t* chosen) {
       break;
     }
   }
-  if (s) return s;
-  if (s2) return s2;
   ctx->item_home = best_ih;
   ctx->steps_per_launch = best_rate > 0.0 ? best_spl : saved_spl;
-  ctx->launch_mode = best_rate > 0.0 ? best_mode : saved_mode;
+  // a context in the automatic mode keeps it where the mode's form was the faster one, and with it
+  // the choice by the species of later steps
+  ctx->launch_mode = saved_mode;
+  const int taken = choose_form(ctx, n_ahead) == FORM_PHASES ? CHEM_LAUNCH_PHASES : CHEM_LAUNCH_PERSISTENT;
+  if (best_rate > 0.0 && best_mode != taken) ctx->launch_mode = best_mode;
   ctx->profiling = saved_prof;
   drop_graph(ctx);
+  if (s) return s;
+  if (s2) return s2;
   if (ctx->launch_mode == CHEM_LAUNCH_PHASES) s = capture_graph(ctx);
   if (s) return s;
   if (chosen) {
     chosen[0] = steps_of(ctx, FORM_PHASES);
     chosen[1] = best_n;
     chosen[2] = best_ih;
-    chosen[3] = ctx->launch_mode == CHEM_LAUNCH_PERSISTENT ? CHEM_LAUNCH_PERSISTENT : CHEM_LAUNCH_PHASES;
+    chosen[3] = best_rate > 0.0 ? best_mode : taken;
   }
   return ctx->status;
 }
