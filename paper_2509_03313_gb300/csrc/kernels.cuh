@@ -170,11 +170,18 @@ struct ClusterBarrier {
 // part in CTA 0 while the last CTA plans the next step, products over the others, commit. It
 // takes 30 us on 1e6 FP32-local species and 40 on 4.1e6; as four kernels (matching, serial,
 // products, end and begin) with the events sorted by one CTA it took 42 and 131.
+struct ReactLeadSmem {
+  SerialSmem serial;
+  alignas(16) uint32_t sbuf[(RC_SMEM_BYTES > 16u * EV_SMEM_CAP ? RC_SMEM_BYTES : 16u * EV_SMEM_CAP) / 4];
+};
+// Batches of up to so many trains plan a step ahead: the records that fit into the shared memory
+// that CTA 0's part of the launch takes anyway (more would leave the products less L1). Whole sweeps
+// of 5,836 steps planned / begun after the reactions: 16 trains 117 / 122 ms, 80 trains 175 / 176.
+constexpr uint32_t REACT_PLAN_TRAINS =
+    static_cast<uint32_t>((sizeof(ReactLeadSmem) - sizeof(PlanSmem<1>)) / sizeof(Train)) + 1u;
+static_assert(sizeof(PlanSmem<REACT_PLAN_TRAINS>) <= sizeof(ReactLeadSmem), "no more than CTA 0's part");
 union ReactGridSmem {
-  struct {
-    SerialSmem serial;
-    alignas(16) uint32_t sbuf[(RC_SMEM_BYTES > 16u * EV_SMEM_CAP ? RC_SMEM_BYTES : 16u * EV_SMEM_CAP) / 4];
-  } lead;
+  ReactLeadSmem lead;
   struct {
     ProductsSmem products;
     Tables tb;

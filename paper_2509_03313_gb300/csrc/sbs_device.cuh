@@ -34,7 +34,6 @@ constexpr int SORT_THREADS = 512;    // threads of the per-pass sort kernel
 constexpr int PERSIST_THREADS = 512; // threads of the persistent step kernel, one CTA per SM
 constexpr int STEP_CLUSTER = 16;     // CTAs of its one-cluster form
 constexpr uint32_t PLAN_TRAINS = 8;  // its batches of up to so many trains plan a step ahead
-constexpr uint32_t REACT_PLAN_TRAINS = 64;  // the same for k_react_grid
 constexpr int SORT_ITEMS = 15;
 constexpr int GATHER_BATCH = 4;   // slots per thread and iteration of the gather
 constexpr int S4_SPARE = 8;       // spare entries of s4 past its end: the search loads whole batches
