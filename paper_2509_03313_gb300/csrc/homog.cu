@@ -111,17 +111,6 @@ __device__ __forceinline__ double hx_rate(const HxLane& k, double y, double& na,
   return k.kappa * na * nb;
 }
 
-// 1 / x for normal x with 1 / x normal, within 2 units in the last place: the FP32 reciprocal
-// of the significand (off by less than 2^-22) and one Newton step of third order.
-__device__ __forceinline__ double hx_recip(double x) {
-  const int hi = __double2hiint(x);
-  const double m = __hiloint2double((hi & static_cast<int>(0x800FFFFFu)) | 0x3FF00000, __double2loint(x));
-  const double y = static_cast<double>(__frcp_rn(static_cast<float>(m)));
-  const double e = fma(-m, y, 1.0);
-  const double z = fma(y, fma(e, e, e), y);
-  return __hiloint2double(__double2hiint(z) + (0x3FF00000 - (hi & 0x7FF00000)), __double2loint(z));
-}
-
 // One extrapolated step of length H from y0 (one extent per row, the same in every half
 // warp): column j takes j linearly implicit Euler substeps y += (I - hJ)^-1 h f(y), h = H / j,
 // with the Jacobian J of y0; then each lane extrapolates its component, which removes the
@@ -158,7 +147,9 @@ __device__ bool hx_step(const HxLane& k, HxSmem& sm, int odd, double y0, double 
     const int p = 15 - static_cast<int>(best & 15u);
     ok = ok && best >= 0x00100000u && best < 0x7FD00000u;
     perm |= static_cast<unsigned long long>(p) << (4 * c);
-    const double inv = hx_shfl(hx_recip(m), p);  // (every row's, beside the search for the pivot)
+    // (every row's, beside the search for the pivot; 1 where none could be, off CUDA's slow path)
+    const unsigned mag = static_cast<unsigned>(__double2hiint(m)) & 0x7FFFFFFFu;
+    const double inv = hx_shfl(__drcp_rn(mag >= 0x00100000u && mag < 0x7FD00000u ? m : 1.0), p);
     const bool mine = k.r == p;
     if (mine) free_row = false;
     const double g = mine ? -inv : m * inv;
