@@ -44,9 +44,9 @@ __device__ __forceinline__ int status_of_hx(const Dev& d) {
 // lanes of its warp (lane r + 16 h: reaction r, the matrix's columns of parity h), a substep
 // is one product with the inverse instead of two triangular sweeps, and no more than three
 // warps lie on an SM; the columns' end values go to both CTAs through distributed shared memory.
-// Measured, 64 trains of 500 to 20,000 species over 10 s (252 steps; the call): 2.9 ms, against
+// Measured, 64 trains of 500 to 20,000 species over 10 s (252 steps; the call): 3.1 ms, against
 // 6.1 ms with a half warp per column, LU factors and one CTA per train, and the same 6.1 ms
-// with those three warps on SMs of their own; a whole pass with its host calls 13.9 -> 11.2 ms
+// with those three warps on SMs of their own; a whole pass with its host calls 13.9 -> 11.4 ms
 // (64.1 with one lane per column and its matrices in local memory).
 constexpr int HX_CTAS = 2;
 constexpr int HX_WARPS = HX_K / HX_CTAS;
@@ -111,6 +111,21 @@ __device__ __forceinline__ double hx_rate(const HxLane& k, double y, double& na,
   return k.kappa * na * nb;
 }
 
+// (de / sc)^(-1 / HX_K) in FP64 for a quotient of 1e-4 to 1e4, and that of the nearer end beyond
+// (past the step-size factor's limits anyway). r from FP32 and the reciprocal of sc from FP32 with
+// one Newton step; then de / sc = (1 - t) r^-6 with |t| below 1e-5, and two terms of the binomial
+// series of (1 - t)^(-1/6), whose third is below 1e-16. (The call of 64 trains below takes 3.14 ms
+// with it, 3.32 with a division, a square root and a cube root, 2.9 with a factor in FP32.)
+__device__ __forceinline__ double hx_root(double de, double sc) {
+  static_assert(HX_K == 6, "the power of r and the series' terms");
+  const float scf = static_cast<float>(sc), q = static_cast<float>(de) / scf, cut = fminf(fmaxf(q, 1e-4f), 1e4f);
+  const double r = static_cast<double>(powf(cut, -1.0f / HX_K)), r3 = r * r * r;
+  double inv = static_cast<double>(1.0f / scf);
+  inv = fma(inv, fma(-sc, inv, 1.0), inv);
+  const double t = q == cut ? fma(-de, r3 * r3, sc) * inv : 0.0;
+  return fma(r, t * fma(t, 7.0 / 72.0, 1.0 / 6.0), r);
+}
+
 // One extrapolated step of length H from y0 (one extent per row, the same in every half
 // warp): column j takes j linearly implicit Euler substeps y += (I - hJ)^-1 h f(y), h = H / j,
 // with the Jacobian J of y0; then each lane extrapolates its component, which removes the
@@ -118,9 +133,9 @@ __device__ __forceinline__ double hx_rate(const HxLane& k, double y, double& na,
 // in place by Gauss-Jordan elimination with a pivot row per column (largest element to 1 part
 // in 2^16, rows stay where they are). Returns false (in every CTA of the train) when a matrix
 // is singular, which makes its column not a number, or the result is not finite; else y1,
-// whether every error estimate is within its tolerance, and the largest ratio of the two.
+// whether every error estimate is within its tolerance, and the smallest hx_root of the two.
 __device__ bool hx_step(const HxLane& k, HxSmem& sm, int odd, double y0, double H, double& y1, bool& within,
-                        float& err) {
+                        double& root) {
   const int nr = k.nr;
   const double h = H / static_cast<double>(k.col + 1);
   double na, nb;
@@ -194,8 +209,11 @@ __device__ bool hx_step(const HxLane& k, HxSmem& sm, int odd, double y0, double 
   const bool mine = k.r < nr;
   const bool fin = __all_sync(0xffffffffu, !mine || isfinite(y1));
   within = __all_sync(0xffffffffu, !mine || de <= sc);
-  const float ratio = mine && fin ? static_cast<float>(de) / static_cast<float>(sc) : 0.f;
-  err = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(ratio)));
+  // the smallest by its bits (none is negative): the high words, then the low words with that one
+  const double own = mine ? hx_root(de, sc) : 8.0;
+  const unsigned hi = static_cast<unsigned>(__double2hiint(own)), top = __reduce_min_sync(0xffffffffu, hi);
+  const unsigned low = __reduce_min_sync(0xffffffffu, hi == top ? static_cast<unsigned>(__double2loint(own)) : ~0u);
+  root = __hiloint2double(static_cast<int>(top), static_cast<int>(low));
   if (!mine) y1 = 0.0;
   return fin;
 }
@@ -212,18 +230,17 @@ __device__ long long hx_integrate(const HxLane& k, HxSmem& sm, double T, double&
     const bool last = H >= T - t;
     const double Hs = last ? T - t : H;
     double y1;
+    double root;
     bool within;
-    float err;
-    const bool ok = hx_step(k, sm, it & 1, e, Hs, y1, within, err);
-    // the step-size factor needs a few digits only: FP32 power
-    const float root = (ok && err > 0.f) ? 0.9f * powf(fminf(err, 1e30f), -1.0f / HX_K) : 4.f;
+    const bool ok = hx_step(k, sm, it & 1, e, Hs, y1, within, root);
+    root *= 0.9;
     if (ok && within) {
       e = y1;
       t = last ? T : t + Hs;
       ++accepted;
-      H = Hs * static_cast<double>(fminf(4.f, fmaxf(0.2f, root)));
+      H = Hs * fmin(4.0, fmax(0.2, root));
     } else {
-      H = Hs * static_cast<double>(ok ? fminf(0.5f, fmaxf(0.2f, root)) : 0.2f);
+      H = Hs * (ok ? fmin(0.5, fmax(0.2, root)) : 0.2);
     }
   }
   return -1;
