@@ -102,12 +102,12 @@ __device__ __forceinline__ void gauss3_f64(uint32_t id, uint32_t step, uint32_t 
                                            double& g0, double& g1, double& g2) {
   const uint4 a = philox4x32_10(make_uint4(id, step, 0u, 0u), k0, k1);
   const uint4 b = philox4x32_10(make_uint4(id, step, 0u, 1u), k0, k1);
-  const double r = fixedn::radius(u53(a.x, a.y));
+  const double r = fixedn::radius_fp64(u53(a.x, a.y));
   double s, c;
   fixedn::sincos_2pi(u53(a.z, a.w), s, c);
   g0 = __dmul_rn(r, c);
   g1 = __dmul_rn(r, s);
-  g2 = __dmul_rn(fixedn::radius(u53(b.x, b.y)), fixedn::cos_2pi(u53(b.z, b.w)));
+  g2 = __dmul_rn(fixedn::radius_fp64(u53(b.x, b.y)), fixedn::cos_2pi(u53(b.z, b.w)));
 }
 
 // Three standard normals (FP32-local mode): one Philox block, 24-bit uniforms.
