@@ -5,12 +5,13 @@
 // while the integer multipliers run 32 to 64 lanes per clock. The arguments are 53-bit
 // integers (the uniforms of the Philox block), which suits fixed point: no argument
 // reduction is rounded, and every result carries at least 58 correct bits before its one
-// rounding to double, so the errors stay below those of the double-precision functions
-// (half an ulp in all). The angle is 2 pi u rounded to double, as every FP64 evaluation of
-// the transform has it: its difference from 2 pi u is formed exactly from the integers and
-// added to the folded angle to first order. (Positions after 1,000 steps of 2,000 species are
-// 2.0e-16 from an FP64 evaluation's as with double-precision functions, 6.9e-16 with the
-// unrounded angle; it costs the FP64 mode's passes 1 to 3 %.) The diffusion of 1e6 FP64
+// rounding to double, so the errors stay below those of the double-precision functions.
+// An FP64 evaluation of the transform rounds the angle 2 pi u and the logarithm to double before
+// it goes on, and so do these: the angle's difference from 2 pi u is formed exactly from the
+// integers and added to the folded angle to first order, the logarithm is rounded before the
+// root. (Positions after 1,000 steps of 2,000 species are 4.7e-17 from an FP64 evaluation's,
+// 2.0e-16 with the logarithm unrounded or with double-precision functions, 6.9e-16 with the
+// angle unrounded too; the roundings cost the FP64 mode's passes 1 to 3 %.) The diffusion of 1e6 FP64
 // species, with the cells and offsets taken on the FP32 pipe (cell_index_split), went from
 // 313 to some 65 us.
 //
