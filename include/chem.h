@@ -370,7 +370,10 @@ chem_status chem_check_bounded_wait(chem_ctx* ctx, double limit_s);
  * id_hi, 2), 53 bits) is below the touch probability p of chem_run_until. The search
  * decides most pairs on an FP32 estimate of p with a rigorous error band and forms p in
  * FP64 only when u falls inside the band; this call lets a test check, with u placed
- * within a few ulp of p, that the tiered decision always equals the FP64 one.
+ * within a few ulp of p, that the tiered decision always equals the FP64 one. (In FP64
+ * mode the search first rejects pairs on FP32 distances with a bound of their error, before
+ * the squared separations that this test starts from are formed; that tier is not part of
+ * this call.)
  * precision: CHEM_FP64 runs the FP64 mode's test on the squared separations as given;
  * CHEM_FP32_LOCAL runs the FP32-local mode's test on their FP32 roundings. Output
  * (host, n bytes): accept[i] bit 0 = the tiered decision, bit 1 = u < p evaluated in

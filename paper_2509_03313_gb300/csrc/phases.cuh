@@ -1157,10 +1157,27 @@ __device__ __forceinline__ bool surely_rejected(float d0f, float d1f, float eps,
   const float ea = __expf(-x);
   const float ulo = static_cast<float>(w.x >> 8) * 5.9604645e-8f;
   if (ulo >= ea * (1.f + 2.f * err)) return true;  // p <= exp(-a)
+  // the quotient's bound below, (1 + 2 z) (1 + z)^2 <= 1 + 8 z for z = eps / R, ends at z = 0.63
+  if (!(eps <= 0.25f * Rf)) return false;
   const float cb = d0f * d1f * inv, cc = Rf * (d0f + d1f - Rf) * inv;
   const float p = ea * (expm1f(-cc) / expm1f(-cb));
-  // a relative error of cb or cc is at most passed on: each has at most 2 eps / R
+  // a relative error of cb or cc is at most passed on
   return ulo >= p * (1.f + 2.f * (err + 4.f * eps / Rf));
+}
+
+// FP64 mode: FP32 start separation of a pair, from its end separation f and the displacements ei, ej.
+// `margin` bounds its error past that of f: the displacements are truncated to 24 bits, an error
+// that grows with each of them and not with their difference (3.1e-7 of `size` in all), and the
+// sums and squares are rounded (3e-7 of the result).
+__device__ __forceinline__ float start_distance_f32(float fx, float fy, float fz, double eix, double eiy, double eiz,
+                                                    double ejx, double ejy, double ejz, float& margin) {
+  const float ix = truncate_double(eix), iy = truncate_double(eiy), iz = truncate_double(eiz);
+  const float jx = truncate_double(ejx), jy = truncate_double(ejy), jz = truncate_double(ejz);
+  const float rx = fx - (jx - ix), ry = fy - (jy - iy), rz = fz - (jz - iz);
+  const float d0 = sqrtf(rx * rx + ry * ry + rz * rz);
+  const float size = fmaxf(fmaxf(fabsf(ix) + fabsf(jx), fabsf(iy) + fabsf(jy)), fabsf(iz) + fabsf(jz));
+  margin = 1e-6f * (size + d0);
+  return d0;
 }
 
 // Acceptance of one queued pair (home slot si, neighbour slot j in the forward cell k of
@@ -1204,13 +1221,9 @@ __device__ __forceinline__ void resolve_pair(const Dev& d, const Tables& tb, con
     const bool sure_in = d1f < sqrtf(tr.rc2f_tt[ti * MAXT + tj]) * 0.99999f - eps;
     if (sure_in) {
       ++n_in_cut;
-      const float r0x = fx - (truncate_double(ejx) - truncate_double(eix));
-      const float r0y = fy - (truncate_double(ejy) - truncate_double(eiy));
-      const float r0z = fz - (truncate_double(ejz) - truncate_double(eiz));
-      const float d0f = sqrtf(r0x * r0x + r0y * r0y + r0z * r0z);
-      // the displacements' truncation is relative to them, which no pair's distance bounds
-      const float big = fmaxf(fmaxf(fabsf(r0x - fx), fabsf(r0y - fy)), fabsf(r0z - fz));
-      if (surely_rejected(d0f, d1f, eps + 1e-6f * (big + d0f), r, tb, tr, id_lo, id_hi)) return;
+      float margin;
+      const float d0f = start_distance_f32(fx, fy, fz, eix, eiy, eiz, ejx, ejy, ejz, margin);
+      if (surely_rejected(d0f, d1f, eps + margin, r, tb, tr, id_lo, id_hi)) return;
     }
     // minimum image of x_j - x_i (Eq. 2), exactly as the reference forms it up to the
     // orientation, which is negated below without rounding
