@@ -102,7 +102,12 @@ typedef struct chem_config {
                                   to some 260,000 and one kernel per phase beyond, chosen
                                   again when species that arrive outgrow it;
                                   CHEM_LAUNCH_PHASES; CHEM_LAUNCH_PERSISTENT (many steps
-                                  per launch, CTAs resident together with barriers)    */
+                                  per launch, CTAs resident together with barriers).
+                                  Beyond some 2,500 species a persistent launch takes every
+                                  multiprocessor for up to 128 steps: it starts when all are
+                                  free, and other streams' kernels (another context's too)
+                                  run before or after it. CHEM_LAUNCH_PHASES lets the
+                                  kernels of several streams share the GPU              */
   void* cuda_stream;           /* cudaStream_t to run on; NULL = library-owned stream  */
   chem_alloc_fn dev_alloc;     /* NULL = cudaMalloc / cudaFree                         */
   chem_free_fn dev_free;
@@ -288,11 +293,11 @@ typedef struct chem_stats {
    * conflict rounds run in shared memory for up to 1,536 conflicting accepted pairs and
    * in global memory beyond; the events of a step are
    * ordered in shared memory for up to 8,192 events (bucket sort, or a block radix sort
-   * when the keys cluster) and in global memory beyond; contexts of more than 262,144
-   * species order more than 1,024 events by buckets of their ids, unless one overflows.
-   * Single trains of at most 262,144
-   * species and the persistent launches resolve up to 1,536 (persistent: 1,024) accepted
-   * pairs of a step at once in shared memory. The results do not depend on the
+   * when the keys cluster) and in global memory beyond. Contexts of more than 262,144
+   * species order any number of events by buckets of their ids, and as above in a step
+   * where one of the buckets overflows. Single trains of at most 262,144 species and the
+   * persistent launches resolve up to 1,536 (persistent: 1,024) accepted pairs of a step at
+   * once in shared memory, more in global memory. The results do not depend on the
    * branch; these counters let tests show that each branch ran. */
   int64_t react_rounds_global;  /* steps whose conflict rounds ran in global memory     */
   int64_t react_order_global;   /* steps whose event order ran in global memory         */

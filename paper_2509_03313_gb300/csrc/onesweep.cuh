@@ -5,7 +5,8 @@
 //  * the digit histogram of the whole input comes precomputed (it is accumulated for
 //    every pass at once while the keys are produced), so each CTA derives the global
 //    digit bases with a 256-wide exclusive scan;
-//  * tiles of 3840 keys are claimed in order through an atomic counter; inside a tile
+//  * tiles of up to 15 keys per thread (7,680 of 512 threads; fewer where there would be few
+//    tiles, sort_rows) are claimed in order through an atomic counter; inside a tile
 //    each warp ranks its keys with __match_any_sync (warp-private digit counters keep
 //    the pass stable; the keys of a tile are nearly sorted, so few digits are distinct),
 //    warps are combined through shared memory;
@@ -21,7 +22,7 @@
 
 namespace chem {
 
-// NT threads per CTA, tiles of NT * SORT_ITEMS keys.
+// NT threads per CTA, tiles of up to NT * SORT_ITEMS keys.
 template <int NT>
 struct SortSmemT {
   static constexpr int TILE = NT * SORT_ITEMS;

@@ -954,9 +954,9 @@ __device__ void phase_gather(const Dev& d, const Span& sp) {
 // ======================================================================== search
 // For every unordered pair of live species whose types react (Table 1), separated by
 // less than the reaction's cutoff under the minimum image (Eq. 2), evaluate the
-// encounter probability and keep the pair if its uniform falls below it. Two mappings
-// visit the same pairs: one thread per home species (below) and cell tiles
-// (search_cells.cuh). With at least 3 cells per axis each unordered pair is visited
+// encounter probability and keep the pair if its uniform falls below it. Three mappings
+// visit the same pairs: one thread per home species, several lanes per home (both below) and
+// cell tiles (search_cells.cuh). With at least 3 cells per axis each unordered pair is visited
 // once: the own cell's later slots and the forward half of the surrounding cells.
 
 // Half-shell offsets: entry 0 is the own cell, 1..13 the cells one away in fwd_offset's
@@ -1181,7 +1181,7 @@ __device__ __forceinline__ float start_distance_f32(float fx, float fy, float fz
 }
 
 // Acceptance of one queued pair (home slot si, neighbour slot j in the forward cell k of
-// the home's cell) and, when accepted, its candidate record. kb = k | train << 8. Both
+// the home's cell) and, when accepted, its candidate record. kb = k | train << 8. All
 // search mappings queue pairs that passed the FP32 cutoff test and resolve them here, one
 // pair per lane. In FP64 mode that test is against a widened cutoff, the FP32 distances
 // (error below eps = 2e-6 of a cell, the same margin) reject most pairs, and the rest are
