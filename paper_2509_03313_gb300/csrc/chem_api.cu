@@ -778,13 +778,16 @@ chem_status state_one(chem_ctx* ctx, int b, int64_t cap, int32_t* type, uint32_t
   if (s) return s;
   // the stepped slots, then the train's parked species (idle trains of a batch)
   const uint32_t n_slots = ctx->g_pinned->n_total;
-  const uint32_t n = n_slots + (ctx->d.pk_cell ? tr[b].park_n : 0u);
+  // (a train that was to park more than its capacity, CHEM_ECAPACITY, has counted them all, and
+  // has those it parked among the slots too)
+  const uint32_t n = n_slots + (ctx->d.pk_cell ? std::min(tr[b].park_n, tr[b].park_cap) : 0u);
   // between steps the diffused state and the sort's buffers hold nothing: the packed species
   // and the chunks' counts go there
   const Dev& d = ctx->d;
   const size_t cap_slots = d.cap;
   auto rows_of = [](size_t bytes) { return static_cast<uint32_t>(((bytes + 255) & ~static_cast<size_t>(255)) / 24); };
   PackOut out{};
+  out.most = static_cast<uint32_t>(cap_slots);
   out.id = d.vals0;
   out.type = reinterpret_cast<int32_t*>(d.vals1);
   out.xyz[0] = reinterpret_cast<double*>(d.t4);
@@ -803,6 +806,7 @@ chem_status state_one(chem_ctx* ctx, int b, int64_t cap, int32_t* type, uint32_t
   uint32_t live = 0;
   CK(cudaMemcpyAsync(&live, counts + chunks, sizeof(live), cudaMemcpyDeviceToHost, ctx->stream));
   CK(cudaStreamSynchronize(ctx->stream));
+  live = std::min(live, out.most);
   const uint32_t k = static_cast<uint32_t>(std::min<int64_t>(live, cap));
   if (k && (type || id || xyz)) {
     CK(enqueue_pack_write(d, static_cast<uint32_t>(b), n_slots, n, counts, out, ctx->stream));

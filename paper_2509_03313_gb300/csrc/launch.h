@@ -58,9 +58,11 @@ cudaError_t enqueue_check_accept_f32l(const Dev& d, uint32_t n, uint32_t step, d
 cudaError_t enqueue_homogeneous(const Dev& d, int blocks, cudaStream_t s);
 
 // state.cu: the live species of one train packed in device order. The positions' rows lie in up
-// to three buffers one after the other (working memory that is idle between steps).
+// to three buffers one after the other (working memory that is idle between steps), which have
+// room for `most` species like the other two arrays; rows past it are not written.
 struct PackOut {
   static constexpr uint32_t SEGS = 3;
+  uint32_t most;
   int32_t* type;
   uint32_t* id;
   double* xyz[SEGS];

@@ -79,7 +79,7 @@ __global__ void __launch_bounds__(PACK_THREADS) k_pack_write(const __grid_consta
     uint32_t total;
     const uint32_t p = at + block_excl_scan(r.live ? 1u : 0u, warp_tot, &total_s, total);
     at += total;
-    if (!r.live) continue;
+    if (!r.live || p >= out.most) continue;
     uint32_t tid;
     double x, y, z;
     if (F32L) {
