@@ -99,7 +99,7 @@ typedef struct chem_config {
   int32_t cells_per_axis_max;  /* spatial-hash resolution limit; 0 = automatic         */
   int32_t steps_per_launch;    /* steps per captured graph replay; 0 = automatic       */
   int32_t launch_mode;         /* CHEM_LAUNCH_AUTO: by the number of species, persistent up
-                                  to some 260,000 and one kernel per phase beyond, chosen
+                                  to 65,536 (batches 131,072), one kernel per phase beyond, chosen
                                   again when species that arrive outgrow it;
                                   CHEM_LAUNCH_PHASES; CHEM_LAUNCH_PERSISTENT (many steps
                                   per launch, CTAs resident together with barriers).
@@ -293,11 +293,12 @@ typedef struct chem_stats {
    * conflict rounds run in shared memory for up to 1,536 conflicting accepted pairs and
    * in global memory beyond; the events of a step are
    * ordered in shared memory for up to 8,192 events (bucket sort, or a block radix sort
-   * when the keys cluster) and in global memory beyond. Contexts of more than 262,144
+   * when the keys cluster) and in global memory beyond. Contexts of more than 65,536
    * species order any number of events by buckets of their ids, and as above in a step
-   * where one of the buckets overflows. Single trains of at most 262,144 species and the
-   * persistent launches resolve up to 1,536 (persistent: 1,024) accepted pairs of a step at
-   * once in shared memory, more in global memory. The results do not depend on the
+   * where one of the buckets overflows. Single trains in steps of at most 65,536 species
+   * (contexts of at most 262,144) and the persistent launches resolve up to 1,536
+   * (persistent: 1,024) accepted pairs of a step at once in shared memory, more in global
+   * memory. The results do not depend on the
    * branch; these counters let tests show that each branch ran. */
   int64_t react_rounds_global;  /* steps whose conflict rounds ran in global memory     */
   int64_t react_order_global;   /* steps whose event order ran in global memory         */

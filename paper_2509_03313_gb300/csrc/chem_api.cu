@@ -86,7 +86,8 @@ struct chem_ctx {
   chem_free_fn dfree = nullptr;
   void* alloc_user = nullptr;
   std::vector<std::pair<void*, size_t>> allocs;
-  cudaGraphExec_t graph = nullptr;  // the per-phase form
+  cudaGraphExec_t graph[2] = {};    // the per-phase form; [1]: of few species (LaunchCfg::small)
+  bool may_be_small = false;        // a single train of at most SMALL_SPECIES
   int graph_steps = 0;
   bool graph_events = false;  // the captured graph records the phase events
   int steps_per_launch = 0;   // 0: automatic
@@ -153,8 +154,10 @@ void* dev_alloc(chem_ctx* ctx, size_t bytes) {
 }
 
 void release_all(chem_ctx* ctx) {
-  if (ctx->graph) cudaGraphExecDestroy(ctx->graph);
-  ctx->graph = nullptr;
+  for (cudaGraphExec_t& g : ctx->graph) {
+    if (g) cudaGraphExecDestroy(g);
+    g = nullptr;
+  }
   if (ctx->stream) cudaStreamSynchronize(ctx->stream);
   for (auto& a : ctx->allocs) {
     if (ctx->dfree) ctx->dfree(a.first, a.second, ctx->alloc_user);
@@ -355,9 +358,12 @@ int sort_passes(const chem_ctx* ctx) {
 
 // Launch form of the next steps, which will work on n species.
 enum Form { FORM_PHASES, FORM_GRID, FORM_CLUSTER };
+uint32_t grid_species(const chem_ctx* ctx) {
+  return static_cast<uint32_t>(ctx->B > 1 ? GRID_SPECIES_BATCH : GRID_SPECIES);
+}
 Form choose_form(const chem_ctx* ctx, uint32_t n) {
   if (ctx->launch_mode == CHEM_LAUNCH_PHASES) return FORM_PHASES;
-  if (ctx->launch_mode == CHEM_LAUNCH_AUTO && (ctx->profiling || n > static_cast<uint32_t>(GRID_SPECIES))) return FORM_PHASES;
+  if (ctx->launch_mode == CHEM_LAUNCH_AUTO && (ctx->profiling || n > grid_species(ctx))) return FORM_PHASES;
   return ctx->lc.cluster_blocks > 0 && n <= static_cast<uint32_t>(CLUSTER_SPECIES) ? FORM_CLUSTER : FORM_GRID;
 }
 
@@ -366,7 +372,7 @@ Form choose_form(const chem_ctx* ctx, uint32_t n) {
 // form of the first, empty step, one cluster, 260 ms. 32,000 species: 6.2 and 14.4 ms.)
 uint32_t most_species(const chem_ctx* ctx, Form f) {
   if (f == FORM_CLUSTER) return static_cast<uint32_t>(CLUSTER_SPECIES);
-  return ctx->launch_mode == CHEM_LAUNCH_AUTO ? static_cast<uint32_t>(GRID_SPECIES) : 0xFFFFFFFFu;
+  return ctx->launch_mode == CHEM_LAUNCH_AUTO ? grid_species(ctx) : 0xFFFFFFFFu;
 }
 
 constexpr uint32_t EPOCH_MAX = 1u << 26;  // look-back words hold 30 bits of 8 x the epoch
@@ -378,12 +384,17 @@ int steps_of(const chem_ctx* ctx, Form f) {
   return f == FORM_PHASES || asked ? steps : 8 * steps;
 }
 
-// Drops the captured graph after a change of what it holds.
+// Drops the captured graphs after a change of what they hold.
 void drop_graph(chem_ctx* ctx) {
-  if (ctx->graph) cudaGraphExecDestroy(ctx->graph);
-  ctx->graph = nullptr;
+  for (cudaGraphExec_t& g : ctx->graph) {
+    if (g) cudaGraphExecDestroy(g);
+    g = nullptr;
+  }
   ctx->graph_events = false;
 }
+
+// Whether steps on n species take the few launches of small ones in the per-phase form.
+int small_steps(const chem_ctx* ctx, uint64_t n) { return ctx->may_be_small && n <= ONE_CTA_SPECIES ? 1 : 0; }
 
 // Sort passes and search kernels of the next launches.
 void set_launch_params(chem_ctx* ctx) {
@@ -391,10 +402,10 @@ void set_launch_params(chem_ctx* ctx) {
   ctx->d.passes = sort_passes(ctx);
 }
 
-// Captures the per-phase form.
-chem_status capture_graph(chem_ctx* ctx) {
+// Captures the per-phase form for steps on n species.
+chem_status capture_graph(chem_ctx* ctx, uint64_t n) {
   set_launch_params(ctx);
-  drop_graph(ctx);
+  ctx->lc.small = small_steps(ctx, n);
   const int steps = steps_of(ctx, FORM_PHASES);
   const size_t n_ev = ctx->profiling ? static_cast<size_t>(steps) * 2 * N_PHASES : 0;
   while (ctx->events.size() < n_ev) {
@@ -417,7 +428,7 @@ chem_status capture_graph(chem_ctx* ctx) {
     return fail(ctx, CHEM_ECUDA, "kernel launch during capture failed: %s", cudaGetErrorString(e));
   }
   CK(e2);
-  e = cudaGraphInstantiate(&ctx->graph, g, 0);
+  e = cudaGraphInstantiate(&ctx->graph[ctx->lc.small], g, 0);
   cudaGraphDestroy(g);
   CK(e);
   ctx->graph_steps = steps;
@@ -425,18 +436,19 @@ chem_status capture_graph(chem_ctx* ctx) {
   return CHEM_OK;
 }
 
-// Queues the next steps in the form f. The `done` steps since the last multiple of the graph's
+// Queues the next steps, on n species, in the form f. The `done` steps since the last multiple of the graph's
 // steps were another form's, which its species outgrew: the per-phase form then takes the rest
 // up to the next multiple without a graph, so that runs end in the same order of species as
 // with graphs alone.
-chem_status launch_steps(chem_ctx* ctx, Form f, int done) {
+chem_status launch_steps(chem_ctx* ctx, Form f, int done, uint32_t n) {
   const int align = steps_of(ctx, FORM_PHASES);
+  ctx->lc.small = small_steps(ctx, n);
   if (f == FORM_PHASES && done == 0) {
-    if (!ctx->graph) {
-      chem_status s = capture_graph(ctx);
+    if (!ctx->graph[ctx->lc.small]) {
+      chem_status s = capture_graph(ctx, n);
       if (s) return s;
     }
-    CK(cudaGraphLaunch(ctx->graph, ctx->stream));
+    CK(cudaGraphLaunch(ctx->graph[ctx->lc.small], ctx->stream));
     return CHEM_OK;
   }
   set_launch_params(ctx);
@@ -468,7 +480,7 @@ chem_status run_loop(chem_ctx* ctx) {
   int done = 0;  // steps since the run's last multiple of `align`
   for (long long it = 0;; ++it) {
     const Form form = choose_form(ctx, ctx->g_pinned->n_ahead);
-    chem_status ls = launch_steps(ctx, form, done);
+    chem_status ls = launch_steps(ctx, form, done, ctx->g_pinned->n_ahead);
     if (ls) return ls;
     CK(cudaMemcpyAsync(ctx->g_pinned, ctx->d.g, sizeof(Global), cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
@@ -1010,7 +1022,8 @@ chem_status chem_batch_init(const chem_config* cfgs, int32_t n_trains, chem_ctx*
   ctx->lc.sort_blocks = ctx->sms * sort_occ;
   ctx->lc.persistent_blocks = ctx->sms;
   ctx->lc.cluster_blocks = cluster;
-  ctx->lc.small = n_trains == 1 && cap <= static_cast<uint64_t>(SMALL_SPECIES) ? 1 : 0;
+  ctx->may_be_small = n_trains == 1 && cap <= static_cast<uint64_t>(SMALL_SPECIES);
+  ctx->lc.small = small_steps(ctx, cap);
 
   // ---- device allocations
   Dev& d = ctx->d;
@@ -1073,7 +1086,7 @@ chem_status chem_batch_init(const chem_config* cfgs, int32_t n_trains, chem_ctx*
     d.vals0 = sortbuf + 2 * cap;
     d.vals1 = sortbuf + 3 * cap;
   }
-  if (cap > static_cast<uint64_t>(SMALL_SPECIES)) {  // event buckets, shared out by capacity
+  if (cap > static_cast<uint64_t>(ONE_CTA_SPECIES)) {  // event buckets, shared out by capacity
     uint32_t nb = 1;
     while (static_cast<uint64_t>(nb) * EV_BUCKET_OF < cap) nb <<= 1;
     uint32_t base = 0;
@@ -1348,7 +1361,7 @@ chem_status chem_set_profiling(chem_ctx* ctx, int32_t on) {
     ctx->stats.phase_launches[i] = 0;
   }
   drop_graph(ctx);
-  return ctx->launch_mode == CHEM_LAUNCH_PHASES ? capture_graph(ctx) : CHEM_OK;
+  return ctx->launch_mode == CHEM_LAUNCH_PHASES ? capture_graph(ctx, ctx->d.cap) : CHEM_OK;
 }
 
 chem_status chem_autotune(chem_ctx* ctx, double budget_ms, int32_t* chosen) {
@@ -1448,8 +1461,6 @@ chem_status chem_autotune(chem_ctx* ctx, double budget_ms, int32_t* chosen) {
         CK(enqueue_set_t_end(d, ctx->t_end_dev, ctx->stream));  // (counts the species ahead)
         ctx->pass_nmax = tr[0].n_max;
         drop_graph(ctx);
-        if (mode == CHEM_LAUNCH_PHASES) s = capture_graph(ctx);
-        if (s) break;
         Global& gfix = *ctx->g_pinned;
         CK(cudaMemcpyAsync(&gfix, d.g, sizeof(Global), cudaMemcpyDeviceToHost, ctx->stream));
         CK(cudaStreamSynchronize(ctx->stream));
@@ -1458,8 +1469,10 @@ chem_status chem_autotune(chem_ctx* ctx, double budget_ms, int32_t* chosen) {
         CK(cudaMemcpyAsync(d.g, &gfix, sizeof(Global), cudaMemcpyHostToDevice, ctx->stream));
         CK(cudaStreamSynchronize(ctx->stream));
         n_ahead = gfix.n_ahead;
+        if (mode == CHEM_LAUNCH_PHASES) s = capture_graph(ctx, n_ahead);
+        if (s) break;
         const int reps = std::max(1, 24 / spl);
-        s = launch_steps(ctx, choose_form(ctx, n_ahead), 0);  // settle
+        s = launch_steps(ctx, choose_form(ctx, n_ahead), 0, n_ahead);  // settle
         if (s) break;
         std::vector<Train> after;
         CK(cudaMemcpyAsync(ctx->g_pinned, d.g, sizeof(Global), cudaMemcpyDeviceToHost, ctx->stream));
@@ -1467,9 +1480,10 @@ chem_status chem_autotune(chem_ctx* ctx, double budget_ms, int32_t* chosen) {
         if (s) break;
         long long ss = 0;
         for (const Train& t : after) ss -= t.species_steps;
-        const Form form = choose_form(ctx, ctx->g_pinned->n_ahead);  // (as a run would)
+        const uint32_t n_next = ctx->g_pinned->n_ahead;
+        const Form form = choose_form(ctx, n_next);  // (as a run would)
         CK(cudaEventRecord(e0, ctx->stream));
-        for (int r = 0; r < reps && !s; ++r) s = launch_steps(ctx, form, 0);
+        for (int r = 0; r < reps && !s; ++r) s = launch_steps(ctx, form, 0, n_next);
         if (s) break;
         CK(cudaEventRecord(e1, ctx->stream));
         CK(cudaMemcpyAsync(ctx->g_pinned, d.g, sizeof(Global), cudaMemcpyDeviceToHost, ctx->stream));
@@ -1529,7 +1543,7 @@ chem_status chem_autotune(chem_ctx* ctx, double budget_ms, int32_t* chosen) {
   drop_graph(ctx);
   if (s) return s;
   if (s2) return s2;
-  if (ctx->launch_mode == CHEM_LAUNCH_PHASES) s = capture_graph(ctx);
+  if (ctx->launch_mode == CHEM_LAUNCH_PHASES) s = capture_graph(ctx, n_ahead);
   if (s) return s;
   if (chosen) {
     chosen[0] = steps_of(ctx, FORM_PHASES);
@@ -1562,7 +1576,7 @@ chem_status chem_set_tuning(chem_ctx* ctx, const int32_t* tuning) {
   ctx->steps_per_launch = spl;
   ctx->launch_mode = mode;
   drop_graph(ctx);
-  if (mode == CHEM_LAUNCH_PHASES) s = capture_graph(ctx);
+  if (mode == CHEM_LAUNCH_PHASES) s = capture_graph(ctx, ctx->d.cap);
   if (s) return s;
   return ctx->status;
 }

@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(32 * TPS_WARPS, F32L ? 8 : 7) k_search_tps(con
   search_species<F32L, TPS_WARPS>(d, sm);
 }
 
-// Either mapping in one launch, for contexts of at most SMALL_SPECIES species, whose steps cost
+// Either mapping in one launch, for steps of at most ONE_CTA_SPECIES species, which cost
 // their launches more than their work (on 1e6 species two kernels are the faster form: the
 // cell tiles want larger CTAs).
 template <bool F32L>
@@ -165,8 +165,8 @@ struct ClusterBarrier {
   __device__ __forceinline__ void leave(const Dev&) {}
 };
 
-// Reaction resolution, the step's end and (begin_next) the next step's begin of contexts that are
-// not small, as one cooperative launch of a CTA per SM: matching over all CTAs, the serial
+// Reaction resolution, the step's end and (begin_next) the next step's begin where one CTA does
+// not do it (LaunchCfg::small), as one cooperative launch of a CTA per SM: matching over all CTAs, the serial
 // part in CTA 0 while the last CTA plans the next step, products over the others, commit. It
 // takes 30 us on 1e6 FP32-local species and 40 on 4.1e6; as four kernels (matching, serial,
 // products, end and begin) with the events sorted by one CTA it took 42 and 131.

@@ -48,17 +48,27 @@ constexpr uint32_t EV_SLOTS = 8;       // places of an event bucket
 constexpr uint32_t EV_GROUP = 64;      // buckets of a group
 constexpr uint32_t EV_BUCKET_OF = 96;  // species capacity per bucket (a power of two of them)
 constexpr int ITEM_HOME = 32;   // most home species per pair-search work item (one cell)
-// Contexts of at most this many species run a step as few launches (one search kernel, one
-// kernel for reaction resolution and the step's end): at 2,000 to 140,000 species reaction
-// resolution to the next begin took 22 to 33 us as four kernels and takes 10 to 24 as one; the
-// 1e6-species benchmark has up to 6,800 events a step, more than one CTA should order.
+// Steps of at most ONE_CTA_SPECIES species of a single train, in contexts of at most SMALL_SPECIES,
+// have one search kernel and one CTA for reaction resolution up to the next begin in the per-phase
+// form; others search in kernels of their own and react on all SMs. ms of whole runs with one CTA /
+// all SMs: tracks 44,000 species 7.7 / 8.3, 64,000 8.7 / 8.7, 90,000 10.5 / 9.8, 160,000
+// 14.9 / 11.4; a mixture of 0.4 mM 45,000 3.1 / 3.4, 120,000 5.0 / 4.9; of 6.6 mM 20,000 3.3 / 3.3,
+// 90,000 5.9 / 4.4.
 constexpr long long SMALL_SPECIES = 1ll << 18;
+constexpr uint32_t ONE_CTA_SPECIES = 1u << 16;
 // Launch form by the species the next steps will work on. 64 steps of a uniform mixture and
 // whole track trajectories, ms as one cluster / one CTA per SM / per-phase kernels:
-//   2,000 species 2.04 / 2.19 / 3.36, 4,000 2.96 / 2.76 / 4.12, 32,000 7.1 / 4.3 / 5.2,
-//   200,000 - / 9.7 / 10.2; tracks 32,000 14.8 / 6.9 / 8.1, 176,000 - / 17.3 / 19.4.
+//   2,000 species 2.04 / 2.19 / 3.36, 4,000 2.96 / 2.76 / 4.12; tracks 32,000 14.8 / 6.9 / 8.1.
+// One CTA per SM / per-phase kernels (reacting on all SMs), single trains: tracks 64,000 8.4 / 8.7,
+// 90,000 10.8 / 9.8, 160,000 14.9 / 11.4, 250,000 17.8 / 12.9; volume study 65,000 15.3 / 13.5,
+// 160,000 22.5 / 19.4; a mixture of 6.6 mM 45,000 3.8 / 3.6, 90,000 5.4 / 4.4, of 0.4 mM 65,000
+// 2.9 / 3.6, 160,000 5.2 / 5.4, 250,000 7.4 / 6.1. Tracks and dense mixtures decide: beyond their
+// line the first form had also fallen behind the per-phase kernels that preceded both (13.3
+// for the 160,000 tracks). Batches, whose per-phase steps sort four passes, of 0.4 mM: 6 x 20,000
+// 4.2 / 4.9, 8 x 16,000 4.5 / 4.8, 8 x 24,000 6.1 / 5.7, 48 x 4,000 7.4 / 6.4, 6 x 40,000 7.3 / 6.0.
 constexpr int32_t CLUSTER_SPECIES = 2560;
-constexpr int32_t GRID_SPECIES = 1 << 18;
+constexpr int32_t GRID_SPECIES = 1 << 16;
+constexpr int32_t GRID_SPECIES_BATCH = 1 << 17;
 constexpr int N_FWD = 14;       // own cell + 13 forward neighbour cells (half shell)
 constexpr double END_SLACK = 1.0 + 1e-6;    // last-step trim slack (relative)
 constexpr float CELL_SLACK_F = 1.0001f;    // hash cell >= cutoff * CELL_SLACK_F

@@ -1,6 +1,6 @@
 """Species that arrive while a launch of many steps runs: the launch ends before the first step
-whose species are more than its form is for (2,560 for one cluster, 262,144 for one CTA per
-SM), and the next steps take the form for them. The results, the order of the species
+whose species are more than its form is for (2,560 for one cluster, 65,536 for one CTA per
+SM, 131,072 in batches), and the next steps take the form for them. The results, the order of the species
 included, are those of the per-phase form; the counters show which launches ran."""
 import dataclasses
 
@@ -62,6 +62,7 @@ def _same(a, b):
     ([(4000, 16)], 17, (2, 0)), ([(700, 0), (1800, 15)], 48, (1, 0)),
     ([(280_000, 1)], 40, (1, 2)), ([(300, 0), (264_000, 16)], 32, (1, 1)), ([(5000, 0), (270_000, 37)], 50, (1, 1)),
     ([(300, 0), (9000, 3), (270_000, 7)], 16, (2, 0)),
+    ([(60_000, 0), (9000, 17)], 50, (1, 2)),       # in the per-phase form: one CTA reacts, then all SMs
 ])
 def test_a_launch_ends_where_its_species_outgrow_it(pulses, steps, launches):
     wl = _growing(pulses, steps, 900 + steps)
@@ -89,3 +90,17 @@ def test_fp64_and_batches_equal_the_reference():
         outs = gpu_batch_run(wls, [50 + b for b in range(trains)])
         for b, (w, g) in enumerate(zip(wls, outs)):
             assert_fp64_parity(g, oracle_run(w, 50 + b, train_id=b, impl="cxx"), w.L)
+
+
+def test_a_batch_that_outgrows_its_form_equals_the_per_phase_form():
+    # 103,000 species, then 139,000 (one CTA per SM up to 131,072 in batches), and few after 40 steps: steps 0 to 5,
+    # then 10 without a graph and two of 16 with one, and the rest
+    wls = [_growing([(3000, 0), (2000, 9)], 50, 61), _growing([(100_000, 0), (34_000, 6)], 40, 62)]
+    stats = {}
+    got = gpu_batch_run(wls, [5, 6], precision=chem.CHEM_FP32_LOCAL, stats=stats)
+    ref = gpu_batch_run(wls, [5, 6], precision=chem.CHEM_FP32_LOCAL, launch_mode=PH)
+    assert (stats["phase_launches"]["persistent"], stats["graph_replays"]) == (2, 2)
+    for a, b in zip(got, ref):
+        _same(a["state"], b["state"])
+        _same([a["events"], a["tally"]["counts"], a["tally"]["events"]],
+              [b["events"], b["tally"]["counts"], b["tally"]["events"]])
