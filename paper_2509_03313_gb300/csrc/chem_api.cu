@@ -104,6 +104,7 @@ struct chem_ctx {
                                  // cell tiles of that many homes, -1 = chosen per step
   Global* g_pinned = nullptr;  // host copy of the global counters
   double* t_end_pinned = nullptr;
+  void* few_pinned = nullptr;  // chem_get_state of few species
   double* t_end_dev = nullptr;
   bool profiling = false;
   std::vector<cudaEvent_t> events;  // 2 * N_PHASES per captured step when profiling
@@ -167,6 +168,8 @@ void release_all(chem_ctx* ctx) {
   for (TrainHost& h : ctx->th) h.pend.release();
   if (ctx->g_pinned) cudaFreeHost(ctx->g_pinned);
   if (ctx->t_end_pinned) cudaFreeHost(ctx->t_end_pinned);
+  if (ctx->few_pinned) cudaFreeHost(ctx->few_pinned);
+  ctx->few_pinned = nullptr;
   ctx->g_pinned = nullptr;
   ctx->t_end_pinned = nullptr;
   for (cudaEvent_t e : ctx->events) cudaEventDestroy(e);
@@ -783,16 +786,19 @@ chem_status state_one(chem_ctx* ctx, int b, int64_t cap, int32_t* type, uint32_t
                       int64_t* n_out) {
   if (!ctx) return CHEM_EINVAL;
   if (b < 0 || b >= ctx->B || cap < 0) return CHEM_EINVAL;
-  chem_status s = download_global(ctx);
+  // (both copies before one synchronise, and the train's record alone: a state of few species is
+  // its synchronises)
+  Train tr;
+  ctx->stats.bytes_d2h += sizeof(Global);
+  CK(cudaMemcpyAsync(ctx->g_pinned, ctx->d.g, sizeof(Global), cudaMemcpyDeviceToHost, ctx->stream));
+  chem_status s = download_train(ctx, b, tr);
   if (s) return s;
-  std::vector<Train> tr;
-  s = download_trains(ctx, tr);
-  if (s) return s;
+  note_device_counters(ctx, *ctx->g_pinned);
   // the stepped slots, then the train's parked species (idle trains of a batch)
   const uint32_t n_slots = ctx->g_pinned->n_total;
   // (a train that was to park more than its capacity, CHEM_ECAPACITY, has counted them all, and
   // has those it parked among the slots too)
-  const uint32_t n = n_slots + (ctx->d.pk_cell ? std::min(tr[b].park_n, tr[b].park_cap) : 0u);
+  const uint32_t n = n_slots + (ctx->d.pk_cell ? std::min(tr.park_n, tr.park_cap) : 0u);
   // between steps the diffused state and the sort's buffers hold nothing: the packed species
   // and the chunks' counts go there
   const Dev& d = ctx->d;
@@ -811,6 +817,31 @@ chem_status state_one(chem_ctx* ctx, int b, int64_t cap, int32_t* type, uint32_t
   } else {
     out.xyz[1] = reinterpret_cast<double*>(d.td4);
     out.rows[1] = rows_of(cap_slots * 16);
+  }
+  if (n <= PACK_FEW && n <= out.rows[0]) {
+    // few: all of them to page-locked memory, behind the number that is live, and from there
+    if (!ctx->few_pinned &&
+        cudaMallocHost(&ctx->few_pinned, 16 + PACK_FEW * (sizeof(int32_t) + sizeof(uint32_t) + 3 * sizeof(double))) != cudaSuccess) {
+      cudaGetLastError();
+      return fail(ctx, CHEM_ENOMEM, "page-locked state buffer");
+    }
+    uint32_t* live_p = static_cast<uint32_t*>(ctx->few_pinned);
+    double* xyz_p = reinterpret_cast<double*>(static_cast<unsigned char*>(ctx->few_pinned) + 16);
+    int32_t* type_p = reinterpret_cast<int32_t*>(xyz_p + 3 * PACK_FEW);
+    uint32_t* id_p = reinterpret_cast<uint32_t*>(type_p + PACK_FEW);
+    const uint32_t m = static_cast<uint32_t>(std::min<int64_t>(n, cap));
+    CK(enqueue_pack_few(d, static_cast<uint32_t>(b), n_slots, n, d.keys0, out, ctx->stream));
+    CK(cudaMemcpyAsync(live_p, d.keys0, sizeof(uint32_t), cudaMemcpyDeviceToHost, ctx->stream));
+    if (type && m) CK(cudaMemcpyAsync(type_p, out.type, m * sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
+    if (id && m) CK(cudaMemcpyAsync(id_p, out.id, m * sizeof(uint32_t), cudaMemcpyDeviceToHost, ctx->stream));
+    if (xyz && m) CK(cudaMemcpyAsync(xyz_p, out.xyz[0], m * 3 * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
+    CK(cudaStreamSynchronize(ctx->stream));
+    const uint32_t live = std::min(*live_p, out.most), k = std::min(live, m);
+    if (type) std::memcpy(type, type_p, k * sizeof(int32_t));
+    if (id) std::memcpy(id, id_p, k * sizeof(uint32_t));
+    if (xyz) std::memcpy(xyz, xyz_p, k * 3 * sizeof(double));
+    if (n_out) *n_out = live;
+    return static_cast<int64_t>(live) > cap ? CHEM_EINVAL : ctx->status;
   }
   uint32_t* counts = d.keys0;  // (a word per 1,024 slots: keys0 and keys1 hold two per slot)
   const uint32_t chunks = pack_counts(n);

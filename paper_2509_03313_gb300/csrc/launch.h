@@ -72,6 +72,10 @@ struct PackOut {
 uint32_t pack_counts(uint32_t n);
 cudaError_t enqueue_pack_count(const Dev& d, uint32_t train, uint32_t n_slots, uint32_t n, uint32_t* counts,
                                cudaStream_t s);
+// Both at once by one CTA, for at most PACK_FEW slots; the number of live species in *live.
+constexpr uint32_t PACK_FEW = 4096;
+cudaError_t enqueue_pack_few(const Dev& d, uint32_t train, uint32_t n_slots, uint32_t n, uint32_t* live,
+                             const PackOut& out, cudaStream_t s);
 cudaError_t enqueue_pack_write(const Dev& d, uint32_t train, uint32_t n_slots, uint32_t n, const uint32_t* counts,
                                const PackOut& out, cudaStream_t s);
 
