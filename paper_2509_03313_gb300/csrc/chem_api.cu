@@ -439,10 +439,10 @@ chem_status capture_graph(chem_ctx* ctx, uint64_t n) {
   return CHEM_OK;
 }
 
-// Queues the next steps, on n species, in the form f. The `done` steps since the last multiple of the graph's
-// steps were another form's, which its species outgrew: the per-phase form then takes the rest
-// up to the next multiple without a graph, so that runs end in the same order of species as
-// with graphs alone.
+// Queues the next steps, on n species, in the form f. The `done` steps since the last multiple of
+// the graph's steps were another form's, which its species outgrew: the per-phase form then takes
+// the rest up to the next multiple without a graph, so that runs end in the same order of species
+// as with graphs alone.
 chem_status launch_steps(chem_ctx* ctx, Form f, int done, uint32_t n) {
   const int align = steps_of(ctx, FORM_PHASES);
   ctx->lc.small = small_steps(ctx, n);
